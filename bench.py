@@ -464,7 +464,7 @@ def main():
                      ms=float(e2e_t.item()), ms_without_cached_device_memory=e2e_uncached_ms,
                      what="hap_problem_create + hap_enumerate + hap_search_best from host buffers (median of 3; the "
                           "process keeps freed device memory and the classes' prefix trees between problems)"),
-            # per step: type_const, one decode and one tree-gather launch, one tree DP launch per PP class, argmin partial + final
+            # per step: type_const, records, the tree DP's launches, argmin partial + final
             gpu_launches=hap.hap_launches_per_pass(hp) * args.steps,
             **extra_modes,
             joint_recurrence_ms=joint_ms,
@@ -475,7 +475,7 @@ def main():
                                     n_evaluated=stats_pr["n_evaluated"]),
             best=dict(cost=best[0], index=best[1], search_index=plan["index"]),
             kernels_ms=dict(type_constants=lc_med, pipeline_dp=dp_med),
-            roofline=dict(bound="alu", kernel="trie_dp_kernel (one launch per PP class, concurrent streams)",
+            roofline=dict(bound="alu", kernel="tree_dp_kernel (two launches: deep pipelines, the others)",
                           achieved=achieved, peak=alu_peak, unit="Tops/s", frac=achieved / alu_peak,
                           traffic=None, ops_per_split=4, splits_executed=cells,
                           effective_finite=dict(cells=cells_finite, tops=4.0 * cells_finite / (dp_med * 1e-3) / 1e12),

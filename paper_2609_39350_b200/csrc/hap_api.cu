@@ -2,7 +2,8 @@
 // work partitioning, kernel launches.  Every step of the hot path runs in the kernels of
 // hap_device.cuh; nothing here evaluates a cost.
 #include "hap_device.cuh"
-#include "hap_trie.cuh"
+#include "hap_tree.cuh"
+#include "hap_tree_host.h"
 
 #include <algorithm>
 #include <cstdarg>
@@ -35,6 +36,23 @@ template <typename E> struct View {
     const E *end() const { return ptr + n; }
 };
 
+// Configuration table and prefix trees on a device, laid out once and shared by the problems of the process whose model
+// dimensions, cluster and search options are the same (they do not depend on the profiled tables).
+struct DeviceImage {
+    int device = 0;
+    unsigned char *base = nullptr;
+    hap_pconf *d_pconf = nullptr;
+    TreeClass *d_cls = nullptr;
+    std::vector<TreeClass> cls;            // the classes that walk a tree, deepest pipeline first (device pointers inside)
+    std::vector<int> tree_of;              // per PP class: its entry in cls, -1 for none
+    std::vector<unsigned> masks_used;      // per PP class: type masks that occur
+    size_t rec_total = 0, prep_smem = 0;
+    DeviceImage() = default;
+    DeviceImage(const DeviceImage &) = delete;
+    DeviceImage &operator=(const DeviceImage &) = delete;
+    ~DeviceImage();
+};
+
 struct hap_problem {
     int device = 0;
     // host copies
@@ -56,57 +74,56 @@ struct hap_problem {
     uint64_t n_cand = 0;
     View<WorkItem> items;                  // grouped by PP class, heaviest class first
     std::shared_ptr<const void> enum_ref;
-    std::shared_ptr<const void> tree_image;      // the page-locked image the trees were uploaded from (kept until the copy is known to be done)
-    // prefix tree of a class's mappings (trie_dp_kernel); ok = false: the class runs in pipeline_dp_kernel only
-    struct TriePartDev { TrieNode *d_nodes; TrieLeaf *d_leaves; TrieCell *d_cells; u32 *d_first_leaf, *d_gnode; uint8_t *d_depth;
-                         u32 n_nodes, n_cells, nmap, m_lo; uint8_t mrow_of[16]; };
-    struct Trie { bool ok = false; TrieMeta *d_metas = nullptr; u32 *d_plist = nullptr;       // both inside d_trie_arena
-                  std::vector<TriePartDev> parts; unsigned n_conf = 0; int threads = 0; size_t smem = 0; };
-    struct PpClass { int PP; int warps; size_t smem; size_t item_lo, item_hi; u64 map_base; bool has_tab; bool multiset; unsigned masks_used; cudaStream_t stream; cudaEvent_t done; Trie trie;
-                     mutable bool tab_valid = false;        // the device table of decoded mappings of this class has been filled
-                     size_t pslot_lo = 0, pslot_n = 0; };   // the class's slots in the per-block partial minima of a search
+    std::shared_ptr<const DeviceImage> image;
+    struct PpClass { int PP; int warps; size_t smem; size_t item_lo, item_hi; u64 map_base; bool has_tab; bool multiset; unsigned masks_used;
+                     int tree = -1;                          // entry in image->cls; -1: the class runs in pipeline_dp_kernel only
+                     cudaStream_t stream = nullptr; cudaEvent_t done = nullptr;
+                     mutable bool tab_valid = false; };      // the device table of decoded mappings of this class has been filled
     std::vector<PpClass> classes;
-    uint8_t *d_maptab = nullptr;           // decoded mappings of every class that is small enough
-    unsigned char *d_arena = nullptr;      // everything hap_enumerate sizes, in one allocation (the d_* pointers below point into it)
-    unsigned char *d_trie_arena = nullptr; // the prefix trees of all classes
+    bool all_trees = false;
+    u64 tab_bytes = 0;
     // device
     DevConst dc{};
-    double *d_tables = nullptr;            // all six tables in one allocation
-    hap_pconf *d_pconf = nullptr;
+    TreeArgs targs{};
+    LiveArgs largs{};
+    bool state_dirty = false;              // a pass was cut short between its kernels: its counters have to be cleared
+    double *d_tables = nullptr;            // all six tables in one allocation (behind the range flag's slot)
+    u64 *d_range = nullptr;                // sticky flag: a cost left the supported value range
+    unsigned char *d_arena = nullptr;      // what every pass needs, in one allocation
+    i64 *d_coef = nullptr;
+    TypeConst *d_tc = nullptr;             // scratch: per (configuration, type) constants of the layer costs
+    i64 *d_lb = nullptr;                   // scratch: per-configuration lower bound on the summed stage time
+    i64 *d_pcost = nullptr;                // per-block partial minima
+    u64 *d_pindex = nullptr;
+    PlanSlot *d_plans = nullptr;           // per block of a tree search the plan of its best candidate
+    u64 *d_counters = nullptr;             // general kernel: [0] evaluated [1] feasible [2] pruned [3] incumbent
+    i64 *d_best = nullptr;                 // (cost, index) of the search
+    void *d_single = nullptr;              // outputs of the one-candidate re-evaluation
+    size_t n_partial = 0;                  // allocated slots of the partial minima
+    // general kernel, layer-cost array (first use)
+    unsigned char *d_gen_arena = nullptr;
+    bool gen_ready = false;
     WorkItem *d_items = nullptr;
-    i64 *d_c2 = nullptr, *d_coef = nullptr;
-    double *d_c2f = nullptr, *d_coeff = nullptr;   // fp64-mode layer costs and coefficients (allocated on first use)
-    i64 *d_fcost = nullptr;                 // fp64-mode search: per-candidate costs (bit patterns), allocated on first use
-    u64 *d_range = nullptr;                 // sticky flag: a cost left the supported value range
+    i64 *d_c2 = nullptr;
+    uint8_t *d_maptab = nullptr;           // decoded mappings of every class that is small enough
+    double *d_c2f = nullptr, *d_coeff = nullptr;   // fp64-mode layer costs and coefficients (first use)
+    i64 *d_fcost = nullptr;                // fp64-mode search through the general kernel: per-candidate costs (bit patterns), first use
+    i64 *d_cand_lb = nullptr;              // scratch of the refinement searches: per-candidate bottleneck, then lower bound (first use)
     // joint device-state recurrence (built on first use)
     struct JointHost { JointClass jc; std::vector<unsigned> ids; unsigned *d_ids = nullptr; int *d_arrays = nullptr; size_t smem = 0; };
     std::vector<JointHost> joint;
     i64 *d_joint_scratch = nullptr;
     int joint_grid = 0;
     bool joint_ready = false;
-    i64 *d_lb = nullptr;                    // scratch: per-configuration lower bound on the summed stage time
-    PlanSlot *d_plans = nullptr;            // per partial-minimum slot the plan of the block's best candidate (searches over the prefix trees; first use)
-    i64 *d_cand_lb = nullptr;               // scratch of the refinement searches: per-candidate bottleneck, then lower bound (first use)
-    TypeConst *d_tc = nullptr;              // scratch: per (configuration, type) constants of the layer-cost kernels
-    i64 *d_pcost = nullptr;                // per-block partial minima
-    u64 *d_pindex = nullptr;
-    u64 *d_counters = nullptr;             // [0] evaluated [1] feasible [2] pruned [3] incumbent
-    i64 *d_best = nullptr;                 // (cost, index) of the search
-    void *d_single = nullptr;              // outputs of the one-candidate re-evaluation
-    size_t n_partial = 0;                  // allocated slots of the partial minima
-    size_t n_pslots = 0;                   // slots a search pass writes and reduces (sum of the classes' pslot_n)
-    bool timed = false;
-    cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
-    cudaEvent_t ev_upload = nullptr;       // the last host-to-device upload of this problem (tables, configuration table, trees)
-    bool upload_pending = false;           // that upload has not been waited for yet
-    cudaEvent_t ev_fork = nullptr;          // classes run on their own streams between this event and their `done` events
-    cudaEvent_t ev_pre = nullptr;           // start of a pass: the candidate decode of the classes waits for this one only
-    cudaEvent_t ev_dec = nullptr;           // the merged candidate decode of a pass has finished
-    DecodeJobs decode_jobs{};               // classes that walk a prefix tree: one merged decode launch per pass
-    GatherJob *d_gather_jobs = nullptr;     // inside d_trie_arena: one entry per part of every tree
-    int n_gather_jobs = 0;
-    unsigned gather_blocks = 0;
-    bool decoded_all = false;               // this pass's merged decode is already queued
+    TreeResult *host_result = nullptr;     // page-locked, mapped: the last block of a search writes the plan here
+    int timed = 0;                         // 1: events around the last pass, 2: the tree kernels' own time stamps
+    cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
+    cudaEvent_t ev_upload = nullptr;       // the upload of the tables
+    bool upload_pending = false;           // no completed call has waited for that upload yet
+    cudaEvent_t ev_fork = nullptr;         // general kernel: classes run on their own streams between this event and their `done` events
+    cudaEvent_t ev_done = nullptr;         // end of the last asynchronous call
+    bool in_flight = false;                // that call has not been waited for
+    cudaStream_t last_stream = nullptr;    // the stream it went to
     std::string err;
 };
 
@@ -144,7 +161,7 @@ static cudaStream_t pooled_stream(int device, size_t index)
 // that uses the data waits for the upload's event.  The staging buffers are kept per process (a page-locked
 // allocation costs more than a search); a buffer is reused once the copy that last read it has completed.
 namespace {
-struct PinnedBuf { void *ptr = nullptr; size_t cap = 0; cudaEvent_t done = nullptr; int device = -1; };
+struct PinnedBuf { void *ptr = nullptr; size_t cap = 0; cudaEvent_t done = nullptr; int device = -1; bool busy = false; };   // busy: being filled
 struct UploadState {
     std::mutex mu;
     std::vector<PinnedBuf> bufs;
@@ -152,6 +169,9 @@ struct UploadState {
 };
 UploadState &upload_state() { static UploadState *u = new UploadState(); return *u; }      // never destroyed
 constexpr size_t kPinnedBufs = 8;
+constexpr size_t kRangeSlot = 512;          // bytes in front of a problem's tables that hold its range flag and a pass's counters
+static_assert(16 + sizeof(TreeState) <= kRangeSlot, "flag, then counters");
+constexpr unsigned kTreeSlots = 4096;       // per-block minima of the tree kernel
 }  // namespace
 
 static cudaStream_t upload_stream(int device)
@@ -163,25 +183,26 @@ static cudaStream_t upload_stream(int device)
     return s;
 }
 
-// a page-locked buffer of at least `bytes` whose previous copy (if any) has completed; nullptr: use pageable memory
+// a page-locked buffer of at least `bytes` whose previous copy (if any) has completed, marked busy until pinned_put;
+// nullptr: use pageable memory
 static PinnedBuf *pinned_get(int device, size_t bytes)
 {
     UploadState &u = upload_state();
     std::lock_guard<std::mutex> lock(u.mu);
-    for (auto &b : u.bufs)
-        if (b.device == device && b.cap >= bytes && cudaEventQuery(b.done) == cudaSuccess) return &b;
-    cudaGetLastError();                                  // cudaErrorNotReady of a busy buffer is not an error
-    if (u.bufs.size() >= kPinnedBufs) {                  // reuse the oldest buffer of the device: wait for it, regrow it
-        for (auto &b : u.bufs)
-            if (b.device == device) {
-                cudaEventSynchronize(b.done);
-                if (b.cap >= bytes) return &b;
-                cudaFreeHost(b.ptr); b.ptr = nullptr; b.cap = 0;
-                if (cudaHostAlloc(&b.ptr, bytes, cudaHostAllocDefault) != cudaSuccess) { cudaGetLastError(); b.ptr = nullptr; return nullptr; }
-                b.cap = bytes;
-                return &b;
-            }
-        return nullptr;
+    PinnedBuf *small = nullptr;                             // an idle buffer of the device that is too small
+    for (auto &b : u.bufs) {
+        if (b.device != device || b.busy || cudaEventQuery(b.done) != cudaSuccess) continue;
+        if (b.cap >= bytes) { b.busy = true; return &b; }
+        small = &b;
+    }
+    cudaGetLastError();                                  // cudaErrorNotReady of a buffer in flight is not an error
+    if (u.bufs.size() >= kPinnedBufs) {                  // regrow an idle one
+        if (!small) return nullptr;
+        cudaFreeHost(small->ptr); small->ptr = nullptr; small->cap = 0;
+        if (cudaHostAlloc(&small->ptr, bytes, cudaHostAllocDefault) != cudaSuccess) { cudaGetLastError(); small->ptr = nullptr; return nullptr; }
+        small->cap = bytes;
+        small->busy = true;
+        return small;
     }
     u.bufs.reserve(kPinnedBufs);                          // pointers into the vector stay valid
     PinnedBuf b;
@@ -189,12 +210,82 @@ static PinnedBuf *pinned_get(int device, size_t bytes)
     b.cap = std::max<size_t>(bytes, 1 << 20);
     if (cudaHostAlloc(&b.ptr, b.cap, cudaHostAllocDefault) != cudaSuccess) { cudaGetLastError(); return nullptr; }
     if (cudaEventCreateWithFlags(&b.done, cudaEventDisableTiming) != cudaSuccess) { cudaFreeHost(b.ptr); cudaGetLastError(); return nullptr; }
+    b.busy = true;
     u.bufs.push_back(b);
     return &u.bufs.back();
 }
 
+static void pinned_put(PinnedBuf *b)
+{
+    std::lock_guard<std::mutex> lock(upload_state().mu);
+    b->busy = false;
+}
+
 // host -> device copy of `bytes` that `fill` writes into a staging buffer; asynchronous when a page-locked buffer
 // and the upload stream are available (the problem's upload event then marks its completion), synchronous otherwise
+// Events without timing are pooled per process: creating and destroying a handful per problem costs as much as a launch.
+namespace {
+struct EventPool { std::mutex mu; std::vector<cudaEvent_t> idle[64]; };
+EventPool &event_pool() { static EventPool *e = new EventPool(); return *e; }           // never destroyed
+constexpr size_t kPooledEvents = 64;
+}  // namespace
+
+static cudaEvent_t pooled_event(int device)
+{
+    EventPool &ep = event_pool();
+    {
+        std::lock_guard<std::mutex> lock(ep.mu);
+        auto &v = ep.idle[device & 63];
+        if (!v.empty()) { cudaEvent_t e = v.back(); v.pop_back(); return e; }
+    }
+    cudaEvent_t e = nullptr;
+    if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    return e;
+}
+
+static void pooled_event_put(int device, cudaEvent_t e)
+{
+    if (!e) return;
+    EventPool &ep = event_pool();
+    {
+        std::lock_guard<std::mutex> lock(ep.mu);
+        auto &v = ep.idle[device & 63];
+        if (v.size() < kPooledEvents) { v.push_back(e); return; }
+    }
+    cudaEventDestroy(e);
+}
+
+// Page-locked, mapped result slots of searches: one page per process, a slot per problem that has searched.
+namespace {
+constexpr int kResultSlots = 128;
+struct ResultPool { std::mutex mu; unsigned char *base = nullptr; bool failed = false; std::vector<int> idle; };
+ResultPool &result_pool() { static ResultPool *r = new ResultPool(); return *r; }       // never destroyed
+constexpr size_t kResultStride = (sizeof(TreeResult) + 255) / 256 * 256;
+}  // namespace
+
+static TreeResult *result_slot_get()
+{
+    ResultPool &rp = result_pool();
+    std::lock_guard<std::mutex> lock(rp.mu);
+    if (!rp.base && !rp.failed) {
+        void *ptr = nullptr;
+        if (cudaHostAlloc(&ptr, kResultSlots * kResultStride, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) { cudaGetLastError(); rp.failed = true; }
+        else { rp.base = static_cast<unsigned char *>(ptr); for (int i = kResultSlots; i-- > 0;) rp.idle.push_back(i); }
+    }
+    if (rp.idle.empty()) return nullptr;                     // the caller copies from the device instead
+    const int i = rp.idle.back();
+    rp.idle.pop_back();
+    return reinterpret_cast<TreeResult *>(rp.base + (size_t)i * kResultStride);
+}
+
+static void result_slot_put(TreeResult *r)
+{
+    if (!r) return;
+    ResultPool &rp = result_pool();
+    std::lock_guard<std::mutex> lock(rp.mu);
+    rp.idle.push_back((int)((reinterpret_cast<unsigned char *>(r) - rp.base) / (ptrdiff_t)kResultStride));
+}
+
 template <class Fill>
 static cudaError_t upload(hap_problem *p, void *dst, size_t bytes, Fill fill)
 {
@@ -205,56 +296,25 @@ static cudaError_t upload(hap_problem *p, void *dst, size_t bytes, Fill fill)
         if (!fill(stage.data())) return cudaErrorInvalidValue;
         return cudaMemcpy(dst, stage.data(), bytes, cudaMemcpyHostToDevice);
     }
+    struct Put { PinnedBuf *b; ~Put() { pinned_put(b); } } put{pb};
     if (!fill(static_cast<unsigned char *>(pb->ptr))) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemcpyAsync(dst, pb->ptr, bytes, cudaMemcpyHostToDevice, us);
     if (e != cudaSuccess) return e;
     if ((e = cudaEventRecord(pb->done, us)) != cudaSuccess) return e;
-    if (!p->ev_upload && (e = cudaEventCreateWithFlags(&p->ev_upload, cudaEventDisableTiming)) != cudaSuccess) return e;
+    if (!p->ev_upload && !(p->ev_upload = pooled_event(p->device))) return cudaErrorUnknown;
     if ((e = cudaEventRecord(p->ev_upload, us)) != cudaSuccess) return e;
     p->upload_pending = true;
     return cudaSuccess;
 }
 
-// A host image in page-locked memory that uploads read directly, without the pass through a staging buffer: what is
-// derived from the lists and the cluster alone (configuration table, prefix trees) is laid out once per process.
-struct PinnedImage {
-    void *ptr = nullptr;
-    size_t bytes = 0;
-    PinnedImage() = default;
-    PinnedImage(const PinnedImage &) = delete;
-    PinnedImage &operator=(const PinnedImage &) = delete;
-    ~PinnedImage() { if (ptr) { cudaFreeHost(ptr); cudaGetLastError(); } }
-};
-
-static std::shared_ptr<PinnedImage> pinned_image(size_t bytes)
-{
-    auto im = std::make_shared<PinnedImage>();
-    if (cudaHostAlloc(&im->ptr, std::max<size_t>(bytes, 1), cudaHostAllocPortable) != cudaSuccess) { cudaGetLastError(); im->ptr = nullptr; return nullptr; }
-    im->bytes = bytes;
-    return im;
-}
-
-// host -> device copy straight from such an image (the problem holds a reference to it until it is destroyed, which
-// waits for the copy)
-static cudaError_t upload_image(hap_problem *p, void *dst, const PinnedImage &im, size_t bytes)
-{
-    cudaStream_t us = upload_stream(p->device);
-    if (!us) return cudaMemcpy(dst, im.ptr, bytes, cudaMemcpyHostToDevice);
-    cudaError_t e = cudaMemcpyAsync(dst, im.ptr, bytes, cudaMemcpyHostToDevice, us);
-    if (e != cudaSuccess) return e;
-    if (!p->ev_upload && (e = cudaEventCreateWithFlags(&p->ev_upload, cudaEventDisableTiming)) != cudaSuccess) return e;
-    if ((e = cudaEventRecord(p->ev_upload, us)) != cudaSuccess) return e;
-    p->upload_pending = true;
-    return cudaSuccess;
-}
-
-// the first use of uploaded data waits for the upload (on the host: by then the copy has long finished)
+// a call that hands data to the host waits for the upload itself; every other one lets its stream wait
 static cudaError_t uploads_done(hap_problem *p)
 {
     if (!p->upload_pending) return cudaSuccess;
     p->upload_pending = false;
     return cudaEventSynchronize(p->ev_upload);
 }
+
 
 // Device memory of destroyed problems is kept for the next problem of the process: allocating and freeing the
 // three arenas of a problem costs about as much as the search itself.  A freed block serves a later request
@@ -321,8 +381,24 @@ static void cached_free(void *ptr)
     mc.idle_bytes += b.bytes;
 }
 
+
+DeviceImage::~DeviceImage() { cached_free(base); }
+
+// device images kept per process, by device and everything they are derived from
+namespace {
+struct ImageCache { std::mutex mu; std::map<std::string, std::shared_ptr<const DeviceImage>> map; };
+ImageCache &image_cache() { static ImageCache *c = new ImageCache(); return *c; }       // never destroyed
+constexpr size_t kImages = 16;
+}  // namespace
+
 extern "C" hap_status hap_release_cached_memory(void)
 {
+    {   // images that no problem holds go back to the cache of device memory first
+        ImageCache &ic = image_cache();
+        std::map<std::string, std::shared_ptr<const DeviceImage>> drop;
+        std::lock_guard<std::mutex> lock(ic.mu);
+        drop.swap(ic.map);
+    }
     MemCache &mc = mem_cache();
     std::lock_guard<std::mutex> lock(mc.mu);
     int prev = 0;
@@ -380,17 +456,15 @@ static void release_device(hap_problem *p)
 {
     // nothing of this problem may still be running when its memory goes back to the cache
     if (p->upload_pending) { cudaEventSynchronize(p->ev_upload); p->upload_pending = false; }
-    if (p->d_tables || p->d_arena) cudaDeviceSynchronize();
-    cached_free(p->d_tables); cached_free(p->d_arena); cached_free(p->d_trie_arena);
+    if (p->in_flight) { cudaEventSynchronize(p->ev_done); p->in_flight = false; }
+    cached_free(p->d_tables); cached_free(p->d_arena); cached_free(p->d_gen_arena);
     cached_free(p->d_joint_scratch);
     for (auto &j : p->joint) { cached_free(j.d_ids); cached_free(j.d_arrays); }
-    cached_free(p->d_c2f); cached_free(p->d_coeff); cached_free(p->d_fcost); cached_free(p->d_cand_lb); cached_free(p->d_plans);
+    cached_free(p->d_c2f); cached_free(p->d_coeff); cached_free(p->d_fcost); cached_free(p->d_cand_lb);
     for (auto &e : p->ev) if (e) cudaEventDestroy(e);
-    if (p->ev_fork) cudaEventDestroy(p->ev_fork);
-    if (p->ev_pre) cudaEventDestroy(p->ev_pre);
-    if (p->ev_dec) cudaEventDestroy(p->ev_dec);
-    if (p->ev_upload) cudaEventDestroy(p->ev_upload);
-    for (auto &cl : p->classes) { if (cl.done) cudaEventDestroy(cl.done); }      // the class streams belong to the pool
+    pooled_event_put(p->device, p->ev_fork); pooled_event_put(p->device, p->ev_done); pooled_event_put(p->device, p->ev_upload);
+    for (auto &cl : p->classes) pooled_event_put(p->device, cl.done);              // the class streams belong to the pool
+    result_slot_put(p->host_result);
 }
 
 extern "C" void hap_problem_destroy(hap_problem *p)
@@ -536,13 +610,17 @@ extern "C" hap_status hap_problem_create(const hap_model *mo, const hap_cluster 
 
     // ---- device ------------------------------------------------------------------------------
     if (cudaGetDevice(&p->device) != cudaSuccess) return HAP_E_CUDA;
-    if (cached_malloc(p->device, (void **)&p->d_tables, n_tab * sizeof(double)) != cudaSuccess) return HAP_E_NOMEM;
+    // the range flag and the counters travel in front of the tables, cleared
+    if (cached_malloc(p->device, (void **)&p->d_range, kRangeSlot + n_tab * sizeof(double)) != cudaSuccess) return HAP_E_NOMEM;
+    p->d_tables = reinterpret_cast<double *>(p->d_range);                   // (the allocation, until release)
     {
-        const cudaError_t e = upload(p, p->d_tables, n_tab * sizeof(double), fill_tables);
+        const cudaError_t e = upload(p, p->d_range, kRangeSlot + n_tab * sizeof(double), [&](unsigned char *dst) {
+            std::memset(dst, 0, kRangeSlot);
+            return fill_tables(dst + kRangeSlot); });
         if (e == cudaErrorInvalidValue) { cudaGetLastError(); return HAP_E_INVALID; }
         if (e != cudaSuccess) return HAP_E_CUDA;
     }
-    for (auto &e : p->ev) if (cudaEventCreate(&e) != cudaSuccess) return HAP_E_CUDA;
+    if (!(p->ev_done = pooled_event(p->device))) return HAP_E_CUDA;
 
     DevConst &dc = p->dc;
     std::memset(&dc, 0, sizeof(dc));
@@ -585,7 +663,7 @@ extern "C" hap_status hap_problem_create(const hap_model *mo, const hap_cluster 
     dc.kind_uniform_from = N - 1;
     while (dc.kind_uniform_from > 0 && p->kind[dc.kind_uniform_from - 1] == p->kind[N - 1]) --dc.kind_uniform_from;
     dc.kind_uniform = dc.kind_uniform_from == 0;
-    dc.tab4 = p->d_tables;
+    dc.tab4 = p->d_tables + kRangeSlot / sizeof(double);
     dc.tpre = dc.tab4 + 4 * n5; dc.tpost = dc.tpre + n4;
 
     guard.keep = true;
@@ -622,517 +700,67 @@ static uint64_t sequences_sat(const int *cnt, int T, uint64_t sat)
     return (uint64_t)r;
 }
 
-// Prefix tree of the decoded mappings of one PP class (host copy `tab`: nmap x PP x (mask, link) bytes).
-// A node is a distinct sequence of stage keys (types, link, load-balance window) of stages 1..d, d < PP;
-// mappings that are consecutive in enumeration order share the nodes of their common prefix.  The window
-// and the band of reachable end layers follow the same integer formulas as pipeline_dp_kernel; a node's
-// band is the union over the mappings below it, which only adds cells that hold their plain recurrence
-// value.  Returns false (and leaves the class on the general kernel) when the tree does not fit.
-struct TriePartHost {
-    TrieMeta meta;                          // device pointers are filled in after the upload
-    std::vector<unsigned char> blob;        // nodes | leaves | cells | first_leaf | cell_gnode | parent | depth
-    size_t o_nodes, o_leaves, o_cells, o_first, o_gnode, o_parent, o_depth;
-    u32 n_nodes, n_cells, nmap, max_level;
-    size_t smem;
-};
-
-// the tree of mappings [m0, m1) of the class
-// `limit`: largest acceptable dynamic shared memory; a tree that needs more is abandoned before its records are written
-static bool build_trie_part(hap_problem *p, const hap_problem::PpClass &cl, const uint8_t *tab_all, u64 m0, u64 m1, size_t limit,
-                            TriePartHost &part)
-{
-    const int N = p->model.N, PP = cl.PP, T = p->T, R = p->prof.R;
-    const u64 nmap = m1 - m0;
-    const uint8_t *tab = tab_all + m0 * (u64)PP * 2;
-    if (nmap == 0 || nmap > 65535) return false;
-    struct Key { uint8_t mask, link, nmin, nmax; };
-    struct HNode { u32 parent; Key k; int bl, bh; u32 first_leaf; };
-    std::vector<std::vector<HNode>> lv(PP + 1);               // lv[d], d = 1..PP-1
-    std::vector<TrieLeaf> leaves(nmap);
-    std::vector<u32> path(PP + 1, 0);
-    std::vector<Key> pkey(PP + 1);
-    bool have_prev = false;
-    i64 Pmin[1 << HAP_MAX_TYPES];
-    for (int mk = 1; mk < (1 << T); ++mk) {
-        i64 v = 0; bool seen = false;
-        for (int h = 0; h < T; ++h) if (mk >> h & 1) { if (!seen || p->P[h] < v) v = p->P[h]; seen = true; }
-        Pmin[mk] = v;
-    }
-    int capt_of[1 << HAP_MAX_TYPES] = {0};                      // type whose (smallest) memory binds a stage of these types
-    for (int mk = 1; mk < (1 << T); ++mk) {
-        i64 cap = 0; bool seen = false;
-        for (int h = 0; h < T; ++h) if (mk >> h & 1) { if (!seen || p->cap_eff[h] < cap) { cap = p->cap_eff[h]; capt_of[mk] = h; } seen = true; }
-    }
-    const int delta_q = p->opts.delta_q;
-    const bool uniform = (p->opts.flags & HAP_OPT_UNIFORM) != 0;
-    std::vector<int> nmin(PP + 1), nmax(PP + 1), bl(PP + 1), bh(PP + 1);
-    // the window of a stage depends on its type mask and on the mapping's summed compute power only: the two
-    // divisions are done once per mask while that sum stays the same (it does for all sequences of a multiset)
-    i64 win_Ps = -1;
-    int win_lo[1 << HAP_MAX_TYPES], win_hi[1 << HAP_MAX_TYPES];
-    for (u64 m = 0; m < nmap; ++m) {
-        const uint8_t *row = tab + m * (u64)PP * 2;
-        i64 Ps = 0;
-        for (int s = 0; s < PP; ++s) {
-            const int mk = row[s * 2];
-            if (mk < 1 || mk >= (1 << T)) return false;
-            Ps += Pmin[mk];
-        }
-        if (!uniform && delta_q >= 0 && Ps != win_Ps) {
-            const i64 den = 1024 * Ps;
-            for (int mk = 1; mk < (1 << T); ++mk) {
-                i64 a = ((i64)(1024 - delta_q) * Pmin[mk] * N) / den;
-                i64 b = ((i64)(1024 + delta_q) * Pmin[mk] * N + den - 1) / den;
-                if (a < 1) a = 1;
-                if (b > N - PP + 1) b = N - PP + 1;
-                win_lo[mk] = (int)a; win_hi[mk] = (int)b;
-            }
-            win_Ps = Ps;
-        }
-        for (int s = 1; s <= PP; ++s) {
-            int lo = 1, hi = N - PP + 1;
-            if (uniform) { lo = N / PP; hi = (N + PP - 1) / PP; }
-            else if (delta_q >= 0) { lo = win_lo[row[(s - 1) * 2]]; hi = win_hi[row[(s - 1) * 2]]; }
-            if (lo < 0 || lo > 255 || hi < 0 || hi > 255) return false;
-            nmin[s] = lo; nmax[s] = hi;
-        }
-        int tmin = 0, tmax = 0;
-        for (int s = 1; s <= PP; ++s) { tmin += nmin[s]; tmax += nmax[s]; }
-        bool dead = false;
-        int smin = 0, smax = 0;
-        for (int s = 1; s <= PP; ++s) {
-            smin += nmin[s]; smax += nmax[s];
-            int lo = smin > s ? smin : s, hi = smax < N - PP + s ? smax : N - PP + s;
-            const int rl = N - (tmax - smax), rh = N - (tmin - smin);
-            lo = lo > rl ? lo : rl; hi = hi < rh ? hi : rh;
-            bl[s] = lo; bh[s] = hi;
-            if (lo > hi) dead = true;
-        }
-        TrieLeaf &lf = leaves[m];
-        std::memset(&lf, 0, sizeof(lf));
-        lf.mask = row[(PP - 1) * 2]; lf.link = row[(PP - 1) * 2 + 1];
-        lf.nmin = (uint8_t)nmin[PP]; lf.nmax = (uint8_t)nmax[PP];
-        lf.dead = dead ? 1 : 0;
-        lf.capt = (uint8_t)capt_of[lf.mask];
-        if (dead) continue;
-        int d0 = 1;                                              // first depth at which a new node is needed
-        if (have_prev)
-            for (; d0 < PP; ++d0) {
-                const Key &k = pkey[d0];
-                if (k.mask != row[(d0 - 1) * 2] || k.link != row[(d0 - 1) * 2 + 1] || k.nmin != nmin[d0] || k.nmax != nmax[d0]) break;
-            }
-        for (int d = d0; d < PP; ++d) {
-            HNode nd;
-            nd.parent = d > 1 ? path[d - 1] : 0;
-            nd.k = Key{row[(d - 1) * 2], row[(d - 1) * 2 + 1], (uint8_t)nmin[d], (uint8_t)nmax[d]};
-            nd.bl = 1 << 20; nd.bh = -1; nd.first_leaf = (u32)(m0 + m);
-            pkey[d] = nd.k;
-            path[d] = (u32)lv[d].size();
-            lv[d].push_back(nd);
-        }
-        have_prev = true;
-        for (int d = 1; d < PP; ++d) {
-            HNode &nd = lv[d][path[d]];
-            nd.bl = std::min(nd.bl, bl[d]); nd.bh = std::max(nd.bh, bh[d]);
-        }
-        lf.parent = PP > 1 ? (uint16_t)path[PP - 1] : 0;
-    }
-    // nodes of a depth ordered by the width of their window (widest first, stable), so that the cells a warp works
-    // on have split loops of similar length
-    for (int d = 1; d < PP; ++d) {
-        std::vector<u32> ord(lv[d].size()), newidx(lv[d].size());
-        for (size_t i = 0; i < ord.size(); ++i) ord[i] = (u32)i;
-        std::stable_sort(ord.begin(), ord.end(), [&](u32 a, u32 b) {
-            return (int)lv[d][a].k.nmax - (int)lv[d][a].k.nmin > (int)lv[d][b].k.nmax - (int)lv[d][b].k.nmin; });
-        std::vector<HNode> sorted(lv[d].size());
-        for (size_t i = 0; i < ord.size(); ++i) { sorted[i] = lv[d][ord[i]]; newidx[ord[i]] = (u32)i; }
-        lv[d].swap(sorted);
-        if (d + 1 < PP) for (auto &ch : lv[d + 1]) ch.parent = newidx[ch.parent];
-        else for (u64 m = 0; m < nmap; ++m) if (!leaves[m].dead) leaves[m].parent = (uint16_t)newidx[leaves[m].parent];
-    }
-    // flat layout
-    TrieMeta &tm = part.meta;
-    std::memset(&tm, 0, sizeof(tm));
-    tm.PP = PP; tm.nmap = (u32)nmap; tm.m_lo = (u32)m0;
-    // row groups of the time rows: one per type mask that some stage has
-    std::memset(tm.mrow_of, 255, sizeof(tm.mrow_of));
-    {
-        unsigned used = 0;
-        for (int d = 1; d < PP; ++d) for (const auto &h : lv[d]) used |= 1u << h.k.mask;
-        for (u64 m = 0; m < nmap; ++m) used |= 1u << leaves[m].mask;
-        for (int mk = 1; mk < (1 << T); ++mk)
-            if ((used >> mk) & 1u) { tm.mrow_of[mk] = (uint8_t)tm.n_mrows; tm.mask_of_row[tm.n_mrows] = (uint8_t)mk; tm.n_mrows++; }
-    }
-    u32 n_nodes = 0, n_cells = 0, max_level = 0;
-    std::vector<std::vector<u32>> rowoff(PP + 1);
-    for (int d = 1; d < PP; ++d) {
-        if (lv[d].size() > 65535) return false;
-        tm.node_lo[d] = n_nodes; tm.cell_lo[d] = n_cells;
-        u32 c = 0;
-        rowoff[d].resize(lv[d].size());
-        for (size_t i = 0; i < lv[d].size(); ++i) { rowoff[d][i] = c; c += (u32)(lv[d][i].bh - lv[d][i].bl + 1); }
-        tm.buf_cells[d & 1] = std::max(tm.buf_cells[d & 1], c);
-        max_level = std::max(max_level, c);
-        n_nodes += (u32)lv[d].size(); n_cells += c;
-    }
-    for (int d = std::max(PP, 1); d <= HAP_MAX_PP; ++d) { tm.node_lo[d] = n_nodes; tm.cell_lo[d] = n_cells; }
-    {   // the shared memory the tree needs is known from the node bands: stop here if it is too much
-        int widest = 1;
-        for (int d = 1; d < PP; ++d) {
-            int lo = 1 << 20, hi = -1;
-            for (const auto &h : lv[d]) { lo = std::min(lo, h.bl); hi = std::max(hi, h.bh); }
-            if (hi >= lo) widest = std::max(widest, hi - lo + 1);
-        }
-        const u32 be = (tm.buf_cells[0] + 1) / 2 * 2, bo = (tm.buf_cells[1] + 1) / 2 * 2;
-        part.smem = trie_smem_bytes(N, PP, T, R, tm.n_mrows, p->dc.kind_uniform ? 1 : widest, be, bo, n_cells, n_nodes);
-        if (part.smem > limit) return false;
-    }
-    tm.buf_cells[0] = (tm.buf_cells[0] + 1) / 2 * 2; tm.buf_cells[1] = (tm.buf_cells[1] + 1) / 2 * 2;
-    if (n_cells >= (1u << 25)) return false;
-    std::vector<TrieNode> nodes(n_nodes);
-    std::vector<uint16_t> parent(n_nodes);
-    std::vector<TrieCell> cells(n_cells);
-    std::vector<u32> cell_gnode(n_cells);
-    int band_max = 1;
-    for (int d = 1; d <= PP; ++d) { tm.jlo[d] = 255; tm.jhi[d] = 0; tm.wmax[d] = 0; tm.tmask[d] = 0; tm.kmin[d] = 255; tm.kmax[d] = 0; }
-    tm.jlo[PP] = tm.jhi[PP] = (uint8_t)N;
-    for (u64 m = 0; m < nmap; ++m) {
-        if (leaves[m].dead) continue;
-        tm.wmax[PP] = std::max(tm.wmax[PP], leaves[m].nmax);
-        tm.tmask[PP] |= (uint8_t)(1u << leaves[m].capt);
-    }
-    std::vector<u32> first_leaf(n_nodes);
-    std::vector<uint8_t> depth(n_nodes);
-    for (int d = 1; d < PP; ++d) {
-        // per-depth extremes are gathered in locals (the description's byte fields alias everything the loop writes)
-        int d_jlo = 255, d_jhi = 0, d_wmax = 0, d_kmin = 255, d_kmax = 0;
-        unsigned d_tmask = 0;
-        const u32 node_lo = tm.node_lo[d], cell_lo = tm.cell_lo[d];
-        const u32 *ro = rowoff[d].data();
-        TrieCell *cd = cells.data();
-        u32 *gn = cell_gnode.data();
-        for (size_t i = 0; i < lv[d].size(); ++i) {
-            const HNode &h = lv[d][i];
-            TrieNode nd{};
-            nd.rowoff = ro[i];
-            nd.mask = h.k.mask; nd.link = h.k.link; nd.nmin = h.k.nmin; nd.nmax = h.k.nmax;
-            nd.bl = (uint8_t)h.bl; nd.bh = (uint8_t)h.bh;
-            if (d > 1) { const HNode &ph = lv[d - 1][h.parent]; nd.prowoff = rowoff[d - 1][h.parent]; nd.pbl = (uint8_t)ph.bl; nd.pbh = (uint8_t)ph.bh; }
-            else { nd.prowoff = 0; nd.pbl = 0; nd.pbh = 0; }
-            nodes[node_lo + i] = nd;
-            parent[node_lo + i] = (uint16_t)h.parent;
-            first_leaf[node_lo + i] = h.first_leaf;
-            depth[node_lo + i] = (uint8_t)d;
-            d_jlo = std::min<int>(d_jlo, nd.bl); d_jhi = std::max<int>(d_jhi, nd.bh);
-            d_wmax = std::max<int>(d_wmax, nd.nmax);
-            d_tmask |= 1u << capt_of[nd.mask];
-            const int cls = nd.link & 3, ha = (nd.link >> 2) & 3, hb = (nd.link >> 4) & 3;
-            const u32 kidx = d == 1 ? tm.mrow_of[nd.mask] : 16 + hb * 6 + (cls == HAP_CROSS ? 2 + ha : cls);
-            const u32 cx = (u32)((int)nd.prowoff - (int)nd.pbl + 256) | (kidx << 26);
-            const u32 cw = (u32)tm.mrow_of[nd.mask] * (u32)(R * (N + 1));
-            const u32 g = node_lo + (u32)i;
-            const int nmx = nd.nmax, nmn = nd.nmin, pbl = nd.pbl, pbh = nd.pbh;
-            u32 c = cell_lo + ro[i];
-            for (int j = h.bl; j <= h.bh; ++j, ++c) {
-                int klo = std::max(j - nmx, pbl), khi = std::min(j - nmn, pbh);
-                if (klo > khi) { klo = 1; khi = 0; }
-                else { d_kmin = std::min(d_kmin, klo); d_kmax = std::max(d_kmax, khi); }
-                TrieCell cc;
-                cc.x = cx;
-                cc.y = (u32)j | ((u32)klo << 8) | ((u32)khi << 16);
-                cc.z = 0;                                         // threshold index: needs the depth's first end layer, set below
-                cc.w = cw;
-                cd[c] = cc;
-                gn[c] = g;
-            }
-        }
-        tm.jlo[d] = (uint8_t)d_jlo; tm.jhi[d] = (uint8_t)d_jhi; tm.wmax[d] = (uint8_t)d_wmax;
-        tm.tmask[d] = (uint8_t)d_tmask; tm.kmin[d] = (uint8_t)d_kmin; tm.kmax[d] = (uint8_t)d_kmax;
-    }
-    for (int d = 1; d <= PP; ++d) if (tm.jlo[d] <= tm.jhi[d]) band_max = std::max(band_max, tm.jhi[d] - tm.jlo[d] + 1);
-    for (u64 m = 0; m < nmap; ++m) {
-        TrieLeaf &lf = leaves[m];
-        if (lf.dead || PP == 1) { lf.prowoff = 0; lf.pbl = 0; lf.pbh = 0; continue; }
-        const HNode &ph = lv[PP - 1][lf.parent];
-        lf.prowoff = rowoff[PP - 1][lf.parent]; lf.pbl = (uint8_t)ph.bl; lf.pbh = (uint8_t)ph.bh;
-    }
-    for (u64 m = 0; m < nmap; ++m) {
-        const TrieLeaf &lf = leaves[m];
-        if (lf.dead) continue;
-        const int klo = std::max(N - (int)lf.nmax, (int)lf.pbl), khi = std::min(N - (int)lf.nmin, (int)lf.pbh);
-        if (klo <= khi) { tm.kmin[PP] = std::min<uint8_t>(tm.kmin[PP], (uint8_t)klo); tm.kmax[PP] = std::max<uint8_t>(tm.kmax[PP], (uint8_t)khi); }
-    }
-    // A depth whose cells only look at splits behind the last change of layer kind sees spans of one kind only:
-    // their memory depends on the length alone and a threshold row of that depth is one number.  All depths of a
-    // model whose layers are all of one kind; every depth but the first few of a model with a dense prefix.
-    bool all_flat = true;
-    for (int d = 1; d <= PP; ++d) {
-        tm.flat[d] = (tm.kmin[d] > tm.kmax[d] || (int)tm.kmin[d] >= p->dc.kind_uniform_from) ? 1 : 0;
-        all_flat = all_flat && tm.flat[d];
-    }
-    tm.all_flat = all_flat ? 1 : 0;
-    const int thr_w = all_flat ? 1 : band_max;
-    tm.thr_w = thr_w;
-    for (u32 c = 0; c < n_cells; ++c) {
-        const u32 g = cell_gnode[c];
-        const int d = depth[g], j = (int)(cells[c].y & 255);
-        cells[c].z = (u32)((((d - 1) * T + capt_of[nodes[g].mask]) * R) * thr_w + ((thr_w == 1 || tm.flat[d]) ? 0 : j - (int)tm.jlo[d]));
-    }
-    tm.band_max = band_max;
-    const size_t smem = trie_smem_bytes(N, PP, T, R, tm.n_mrows, thr_w, tm.buf_cells[0], tm.buf_cells[1], n_cells, n_nodes);
-    if (smem > limit) return false;
-    // one blob: nodes | leaves | cells | first_leaf | cell_gnode | parent | depth
-    auto up = [](size_t v) { return (v + 255) / 256 * 256; };
-    part.o_nodes = 0; part.o_leaves = up(part.o_nodes + (size_t)n_nodes * sizeof(TrieNode));
-    part.o_cells = up(part.o_leaves + nmap * sizeof(TrieLeaf));
-    part.o_first = up(part.o_cells + (size_t)n_cells * sizeof(TrieCell)); part.o_gnode = up(part.o_first + (size_t)n_nodes * 4);
-    part.o_parent = up(part.o_gnode + (size_t)n_cells * 4); part.o_depth = up(part.o_parent + (size_t)n_nodes * 2);
-    const size_t total = up(part.o_depth + n_nodes) + 256;
-    part.blob.assign(total, 0);
-    unsigned char *blob = part.blob.data();
-    if (n_nodes) std::memcpy(blob + part.o_nodes, nodes.data(), (size_t)n_nodes * sizeof(TrieNode));
-    std::memcpy(blob + part.o_leaves, leaves.data(), nmap * sizeof(TrieLeaf));
-    if (n_cells) std::memcpy(blob + part.o_cells, cells.data(), (size_t)n_cells * sizeof(TrieCell));
-    if (n_nodes) std::memcpy(blob + part.o_first, first_leaf.data(), (size_t)n_nodes * 4);
-    if (n_cells) std::memcpy(blob + part.o_gnode, cell_gnode.data(), (size_t)n_cells * 4);
-    if (n_nodes) std::memcpy(blob + part.o_parent, parent.data(), (size_t)n_nodes * 2);
-    if (n_nodes) std::memcpy(blob + part.o_depth, depth.data(), n_nodes);
-    part.n_nodes = n_nodes; part.n_cells = n_cells; part.nmap = (u32)nmap; part.max_level = max_level; part.smem = smem;
-    return true;
-}
-
-// Builds the class's tree, as one part or, when one part would leave room for only one block per SM, as up to
-// eight parts over contiguous ranges of mappings (the few nodes near the root that two parts share are computed by
-// both).  Returns false (the class stays on the general kernel) when nothing fits.
-struct TrieClassHost { std::vector<TriePartHost> parts; unsigned masks_used = 0xffffffffu; };
-// what upload_tries gets per class: the class, its (shared) host tree and the class's configurations
-struct TrieBuilt { hap_problem::PpClass *cl; std::shared_ptr<const TrieClassHost> tree; std::vector<u32> plist; };
-
-static bool build_trie(hap_problem *p, hap_problem::PpClass &cl, const uint8_t *tab, u64 nmap, size_t n_conf, TrieClassHost &out)
-{
-    if (nmap == 0 || n_conf == 0) return false;
-    constexpr size_t kTwoPerSm = 108 * 1024;                 // dynamic shared memory that lets two blocks share an SM
-    const size_t slots = (cl.item_hi - cl.item_lo) / n_conf;             // work items per configuration
-    std::vector<TriePartHost> parts;
-    // The number of parts that worked for a class of this shape before is tried first (a hint kept per process: a
-    // wrong hint costs one failed attempt, the sequence below then runs as usual).
-    static std::mutex hint_mu;
-    static std::map<std::array<long long, 6>, int> hint;
-    const std::array<long long, 6> key = {cl.PP, (long long)nmap, p->model.N, p->T * 16 + p->prof.R, p->opts.delta_q, (long long)(p->opts.flags & HAP_OPT_UNIFORM)};
-    int first_np = 0;
-    { std::lock_guard<std::mutex> lock(hint_mu); auto it = hint.find(key); if (it != hint.end()) first_np = it->second; }
-    auto attempt = [&](int np) {
-        if ((u64)np > nmap || (np > 1 && (size_t)np > slots)) return false;
-        std::vector<TriePartHost> cand(np);
-        bool ok = true;
-        for (int q = 0; q < np && ok; ++q) ok = build_trie_part(p, cl, tab, nmap * q / np, nmap * (q + 1) / np, kTwoPerSm, cand[q]);
-        if (ok) parts.swap(cand);
-        return ok;
-    };
-    int used_np = 0;
-    if (first_np > 1 && attempt(first_np)) used_np = first_np;
-    if (!used_np)
-        for (int np : {1, 2, 3, 4, 6, 8}) {
-            if ((u64)np > nmap || (np > 1 && (size_t)np > slots)) break;
-            if (np == first_np) continue;
-            if (attempt(np)) { used_np = np; break; }
-        }
-    if (used_np) { std::lock_guard<std::mutex> lock(hint_mu); hint[key] = used_np; }
-    if (parts.empty()) {                                     // no split lets two blocks share an SM: one block per SM
-        parts.resize(1);
-        if (!build_trie_part(p, cl, tab, 0, nmap, 220 * 1024, parts[0])) parts.clear();
-    }
-    if (parts.empty()) return false;
-    out.parts.swap(parts);
-    return true;
-}
-
-// One allocation for the trees of all classes.  Its head holds what does not depend on where it lies -- per class the
-// parts' blobs and the list of the class's configurations -- and is copied from an image kept per process under
-// `image_key` (the classes' tree keys and the enumeration's key); behind it lie the part descriptions and the job
-// list of the gather kernel, which hold device addresses and are staged for every problem.
-namespace {
-std::mutex g_tree_image_mu;
-std::map<std::string, std::shared_ptr<PinnedImage>> g_tree_images;
-constexpr size_t kTreeImages = 16;
-}
-
-static bool upload_tries(hap_problem *p, std::vector<TrieBuilt> &built, const std::string &image_key)
-{
-    constexpr size_t kTwoPerSm = 108 * 1024;
-    auto up = [](size_t v) { return (v + 255) / 256 * 256; };
-    size_t head = 0, tail = 0, n_parts_all = 0;
-    for (auto &bc : built) {
-        for (const auto &pt : bc.tree->parts) head += up(pt.blob.size());
-        head += up(bc.plist.size() * sizeof(u32));
-        tail += up(bc.tree->parts.size() * sizeof(TrieMeta));
-        n_parts_all += bc.tree->parts.size();
-    }
-    if (!head) return true;
-    const size_t o_jobs = head + tail;
-    const size_t total = o_jobs + up(n_parts_all * sizeof(GatherJob));
-    std::vector<GatherJob> gjobs;
-    DecodeJobs dj{};
-    unsigned dblk = 0, gblk = 0;
-    if (cached_malloc(p->device, (void **)&p->d_trie_arena, total) != cudaSuccess) { p->d_trie_arena = nullptr; cudaGetLastError(); return false; }
-    // the head: blobs and configuration lists (`stage` may be null: only the offsets are wanted then)
-    auto fill_head = [&](unsigned char *stage) {
-        size_t off = 0;
-        for (auto &bc : built) {
-            for (const auto &pt : bc.tree->parts) {
-                if (stage) std::memcpy(stage + off, pt.blob.data(), pt.blob.size());
-                off += up(pt.blob.size());
-            }
-            if (stage) std::memcpy(stage + off, bc.plist.data(), bc.plist.size() * sizeof(u32));
-            off += up(bc.plist.size() * sizeof(u32));
-        }
-    };
-    // the tail: part descriptions and gather jobs, with this arena's addresses; also fills the per-class records
-    auto fill_tail = [&](unsigned char *stage) -> bool {          // (stage = start of the tail)
-    size_t off = 0, toff = 0;
-    for (auto &bc : built) {
-        hap_problem::Trie &tr = bc.cl->trie;
-        const TrieClassHost &h = *bc.tree;
-        std::vector<TrieMeta> metas;
-        size_t smem = 0;
-        u32 want = 0;
-        for (const auto &pt : h.parts) {
-            unsigned char *base = p->d_trie_arena + off;
-            hap_problem::TriePartDev pd{};
-            pd.d_nodes = reinterpret_cast<TrieNode *>(base + pt.o_nodes);
-            pd.d_leaves = reinterpret_cast<TrieLeaf *>(base + pt.o_leaves);
-            pd.d_cells = reinterpret_cast<TrieCell *>(base + pt.o_cells);
-            pd.d_first_leaf = reinterpret_cast<u32 *>(base + pt.o_first);
-            pd.d_gnode = reinterpret_cast<u32 *>(base + pt.o_gnode);
-            pd.d_depth = base + pt.o_depth;
-            pd.n_nodes = pt.n_nodes; pd.n_cells = pt.n_cells; pd.nmap = pt.nmap; pd.m_lo = pt.meta.m_lo;
-            std::memcpy(pd.mrow_of, pt.meta.mrow_of, sizeof(pd.mrow_of));
-            TrieMeta meta = pt.meta;                 // the host tree is shared between problems: the device pointers go into a copy
-            meta.nodes = pd.d_nodes; meta.leaves = pd.d_leaves; meta.cells = pd.d_cells;
-            meta.parent = reinterpret_cast<const uint16_t *>(base + pt.o_parent);
-            tr.parts.push_back(pd);
-            metas.push_back(meta);
-            GatherJob gj{};
-            gj.first_leaf = pd.d_first_leaf; gj.gnode = pd.d_gnode; gj.depth = pd.d_depth;
-            gj.nodes = pd.d_nodes; gj.cells = pd.d_cells; gj.leaves = pd.d_leaves;
-            gj.tab_off = bc.cl->map_base; gj.n_nodes = pd.n_nodes; gj.n_cells = pd.n_cells; gj.nmap = pd.nmap; gj.m_lo = pd.m_lo;
-            gj.blk_lo = gblk; gj.PP = bc.cl->PP;
-            std::memcpy(gj.rm.mrow_of, pd.mrow_of, sizeof(gj.rm.mrow_of));
-            gblk += (pd.n_nodes + pd.n_cells + pd.nmap + 255) / 256;
-            gjobs.push_back(gj);
-            smem = std::max(smem, pt.smem);
-            want = std::max(want, std::max(pt.max_level, pt.nmap));
-            off += up(pt.blob.size());
-        }
-        tr.d_plist = reinterpret_cast<u32 *>(p->d_trie_arena + off);
-        off += up(bc.plist.size() * sizeof(u32));
-        tr.d_metas = reinterpret_cast<TrieMeta *>(p->d_trie_arena + head + toff);
-        std::memcpy(stage + toff, metas.data(), metas.size() * sizeof(TrieMeta));
-        toff += up(metas.size() * sizeof(TrieMeta));
-        tr.n_conf = (unsigned)bc.plist.size(); tr.smem = smem;
-        if (dj.n <= HAP_MAX_PP) {
-            const hap_problem::PpClass &cl = *bc.cl;
-            const u32 rep = p->items[cl.item_lo].p;
-            const u64 nmap_cl = p->pconfs[rep].nmap;
-            dj.blk_lo[dj.n] = dblk; dj.p_rep[dj.n] = rep; dj.nmap[dj.n] = (u32)nmap_cl; dj.tab_off[dj.n] = cl.map_base;
-            dblk += (unsigned)((nmap_cl + 3) / 4);
-            dj.n++;
-            dj.blk_lo[dj.n] = dblk;
-        }
-        // a thread takes about four cells of the widest depth (measured: smaller blocks, more of them per SM)
-        const int th = (int)(((want + 3) / 4 + 31) / 32 * 32);
-        tr.threads = std::min(smem <= kTwoPerSm ? 512 : 1024, std::max(128, th));
-        tr.ok = true;
-    }
-    std::memcpy(stage + tail, gjobs.data(), gjobs.size() * sizeof(GatherJob));
-    return true;
-    };
-    // head: from the process's image of these trees when there is one (made on first use)
-    std::shared_ptr<PinnedImage> image;
-    if (upload_stream(p->device)) {
-        std::lock_guard<std::mutex> lock(g_tree_image_mu);
-        auto it = g_tree_images.find(image_key);
-        if (it != g_tree_images.end() && it->second->bytes == head) image = it->second;
-        else if ((image = pinned_image(head))) {
-            std::memset(image->ptr, 0, head);
-            fill_head(static_cast<unsigned char *>(image->ptr));
-            if (g_tree_images.size() >= kTreeImages) g_tree_images.clear();
-            g_tree_images[image_key] = image;
-        }
-    }
-    cudaError_t e = image ? upload_image(p, p->d_trie_arena, *image, head)
-                          : upload(p, p->d_trie_arena, head, [&](unsigned char *stage) { fill_head(stage); return true; });
-    if (e == cudaSuccess) e = upload(p, p->d_trie_arena + head, total - head, fill_tail);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        for (auto &bc : built) bc.cl->trie = hap_problem::Trie{};
-        return false;
-    }
-    p->tree_image = image;
-    p->decode_jobs = dj;
-    p->d_gather_jobs = reinterpret_cast<GatherJob *>(p->d_trie_arena + o_jobs);
-    p->n_gather_jobs = (int)gjobs.size();
-    p->gather_blocks = gblk;
-    return true;
-}
-
-// ---- per-process cache of the classes' prefix trees ------------------------------------------------------
-namespace {
-std::mutex g_trie_cache_mu;
-std::map<std::string, std::shared_ptr<const TrieClassHost>> g_trie_cache;
-constexpr size_t kTrieCacheEntries = 256;
-}
-
 template <class V> static void key_put(std::string &k, const V &v) { k.append(reinterpret_cast<const char *>(&v), sizeof(v)); }
 
-// everything the decoded mappings, the windows, the bands, the cell records and the split into parts depend on
-static std::string trie_cache_key(const hap_problem *p, const hap_problem::PpClass &cl)
+// ---- per-process cache of the classes' prefix trees (host side) ------------------------------------------
+namespace {
+struct TreeCache { std::mutex mu; std::map<std::string, std::shared_ptr<const TreeClassHost>> map; };
+TreeCache &tree_cache() { static TreeCache *c = new TreeCache(); return *c; }
+constexpr size_t kTreeCacheEntries = 256;
+}
+
+// everything the mappings, the windows, the bands, the task lists and the split into parts depend on
+static std::string tree_cache_key(const hap_problem *p, const hap_problem::PpClass &cl, bool want_tree)
 {
-    std::string k("hap-trie-1");
+    std::string k("hap-tree-2");
     const hap_pconf &rep = p->pconfs[p->items[cl.item_lo].p];
     const size_t n_conf = p->items[cl.item_hi - 1].p - p->items[cl.item_lo].p + 1;
     const int32_t head[] = {p->model.N, p->T, p->prof.R, cl.PP, rep.G, rep.mode, p->opts.delta_q, (int32_t)(p->opts.flags & HAP_OPT_UNIFORM),
-                            p->dc.kind_uniform, p->dc.kind_uniform_from, (int32_t)((cl.item_hi - cl.item_lo) / n_conf)};
+                            p->dc.kind_uniform, p->dc.kind_uniform_from, (int32_t)n_conf, p->dc.tau_linear, (int32_t)want_tree};
     key_put(k, head);
     key_put(k, rep.nmap);
     for (int h = 0; h < p->T; ++h) { key_put(k, p->P[h]); key_put(k, p->cap_eff[h]); key_put(k, p->dc.m[h]); key_put(k, p->dc.node_size[h]); }
     return k;
 }
 
-static std::shared_ptr<const TrieClassHost> trie_cache_find(const std::string &key)
+static std::shared_ptr<const TreeClassHost> tree_of_class(const hap_problem *p, const hap_problem::PpClass &cl, bool want_tree)
 {
-    std::lock_guard<std::mutex> lock(g_trie_cache_mu);
-    auto it = g_trie_cache.find(key);
-    return it == g_trie_cache.end() ? nullptr : it->second;
-}
-
-static void trie_cache_insert(const std::string &key, std::shared_ptr<const TrieClassHost> tree)
-{
-    std::lock_guard<std::mutex> lock(g_trie_cache_mu);
-    if (g_trie_cache.size() >= kTrieCacheEntries) g_trie_cache.clear();
-    g_trie_cache[key] = std::move(tree);
-}
-
-// the configurations of a class (contiguous: PP is the outermost loop of the enumeration)
-static std::vector<u32> class_plist(const hap_problem *p, const hap_problem::PpClass &cl)
-{
-    std::vector<u32> plist;
-    for (size_t pi = p->items[cl.item_lo].p; pi <= p->items[cl.item_hi - 1].p; ++pi) plist.push_back((u32)pi);
-    return plist;
+    const std::string key = tree_cache_key(p, cl, want_tree);
+    TreeCache &tc = tree_cache();
+    {
+        std::lock_guard<std::mutex> lock(tc.mu);
+        auto it = tc.map.find(key);
+        if (it != tc.map.end()) return it->second;
+    }
+    auto th = std::make_shared<TreeClassHost>();
+    TreeInputs in{};
+    in.dc = &p->dc; in.rep = p->pconfs[p->items[cl.item_lo].p];
+    in.n_conf = p->items[cl.item_hi - 1].p - p->items[cl.item_lo].p + 1;
+    in.want_tree = want_tree;
+    TreeBuilder(in).build(*th);
+    if (th->ok) {
+        th->cls.n_conf = (u32)in.n_conf;
+        tree_items(th->cls);
+        // (a record or a part that does not leave room for one block on an SM: the class runs one warp per candidate)
+        th->ok = tree_smem_bytes(th->cls) <= 200 * 1024 && tree_prep_smem_bytes(th->cls, p->model.N, p->T) <= 200 * 1024;
+    }
+    std::lock_guard<std::mutex> lock(tc.mu);
+    if (tc.map.size() >= kTreeCacheEntries) tc.map.clear();
+    tc.map[key] = th;
+    return th;
 }
 
 // ---- per-process cache of enumerations -----------------------------------------------------------------------
 struct EnumResult {
     std::vector<hap_pconf> rows;
     std::vector<WorkItem> items;
-    std::vector<hap_problem::PpClass> classes;       // streams, events and trees are per problem: empty here
+    std::vector<hap_problem::PpClass> classes;       // streams and events are per problem: empty here
     uint64_t n_cand = 0;
     u64 tab_bytes = 0;
-    std::shared_ptr<PinnedImage> image;             // rows | padding to 256 bytes | items | padding: the head of a problem's arena (may be null)
 };
 namespace {
-std::mutex g_enum_cache_mu;
-std::map<std::string, std::shared_ptr<const EnumResult>> g_enum_cache;
+struct EnumCache { std::mutex mu; std::map<std::string, std::shared_ptr<const EnumResult>> map; };
+EnumCache &enum_cache() { static EnumCache *c = new EnumCache(); return *c; }
 constexpr size_t kEnumCacheEntries = 64;
 }
 
@@ -1152,16 +780,105 @@ static std::string enum_cache_key(const hap_problem *p)
 
 static std::shared_ptr<const EnumResult> enum_cache_find(const std::string &key)
 {
-    std::lock_guard<std::mutex> lock(g_enum_cache_mu);
-    auto it = g_enum_cache.find(key);
-    return it == g_enum_cache.end() ? nullptr : it->second;
+    EnumCache &ec = enum_cache();
+    std::lock_guard<std::mutex> lock(ec.mu);
+    auto it = ec.map.find(key);
+    return it == ec.map.end() ? nullptr : it->second;
 }
 
 static void enum_cache_insert(const std::string &key, std::shared_ptr<const EnumResult> r)
 {
-    std::lock_guard<std::mutex> lock(g_enum_cache_mu);
-    if (g_enum_cache.size() >= kEnumCacheEntries) g_enum_cache.clear();
-    g_enum_cache[key] = std::move(r);
+    EnumCache &ec = enum_cache();
+    std::lock_guard<std::mutex> lock(ec.mu);
+    if (ec.map.size() >= kEnumCacheEntries) ec.map.clear();
+    ec.map[key] = std::move(r);
+}
+
+// Configuration table and trees on the problem's device: from the process's images when one of the same key exists, else
+// laid out and copied now (once per cluster, model dimensions and search options).
+static hap_status image_for(hap_problem *p, const std::string &ekey)
+{
+    // the tree kernel holds times as doubles: exact while every prefix row stays below 2^52, which the per-layer limit of
+    // 2^36 ns guarantees when N (2 + max tau) <= 2^16; rows that are not combined by level also form tau x forward time
+    int tau_max = 0;
+    for (int r = 0; r < p->prof.R; ++r) tau_max = std::max(tau_max, p->tau_q[r]);
+    const int64_t N = p->model.N;
+    const bool exact = N * (2 + (tau_max >> 10)) <= 65536 && (p->dc.tau_linear || N * tau_max < (1 << 17));
+    // and the split pointer of the scan needs levels that repeat no less forward work the higher they are
+    bool ordered = true;
+    for (uint32_t mk : p->rc_masks) {
+        int last = -1;
+        for (int r = 0; r < p->prof.R; ++r)
+            if ((mk >> r) & 1u) { ordered = ordered && p->tau_q[r] >= last; last = p->tau_q[r]; }
+    }
+    const bool want_tree = !(p->opts.flags & (HAP_OPT_NO_TRIE | HAP_OPT_NO_MAPTAB)) && exact && ordered;
+    std::string key = ekey;
+    const int32_t head[] = {p->device, want_tree, p->prof.R, p->opts.delta_q, (int32_t)(p->opts.flags & HAP_OPT_UNIFORM), p->dc.kind_uniform,
+                            p->dc.kind_uniform_from, p->dc.tau_linear};
+    key_put(key, head);
+    for (int h = 0; h < p->T; ++h) { key_put(key, p->P[h]); key_put(key, p->cap_eff[h]); key_put(key, p->dc.node_size[h]); }
+    ImageCache &ic = image_cache();
+    {
+        std::lock_guard<std::mutex> lock(ic.mu);
+        auto it = ic.map.find(key);
+        if (it != ic.map.end()) { p->image = it->second; return HAP_OK; }
+    }
+    auto im = std::make_shared<DeviceImage>();
+    im->device = p->device;
+    auto up = [](size_t v) { return (v + 255) / 256 * 256; };
+    std::vector<std::shared_ptr<const TreeClassHost>> trees;
+    size_t o = up(p->pconfs.size() * sizeof(hap_pconf));
+    for (const auto &cl : p->classes) {
+        std::shared_ptr<const TreeClassHost> th = tree_of_class(p, cl, want_tree);
+        im->masks_used.push_back(th->masks_used);
+        im->tree_of.push_back(th->ok ? (int)trees.size() : -1);
+        if (!th->ok) continue;
+        TreeClass c = th->cls;
+        c.p_lo = p->items[cl.item_lo].p;
+        c.rec_off = im->rec_total;
+        im->rec_total += up((size_t)c.n_conf * c.rec_bytes);
+        im->prep_smem = std::max(im->prep_smem, tree_prep_smem_bytes(c, p->model.N, p->T));
+        im->cls.push_back(c);
+        trees.push_back(th);
+    }
+    const size_t o_cls = o;
+    o = up(o + trees.size() * sizeof(TreeClass));
+    std::vector<size_t> o_parts;
+    for (const auto &th : trees) {
+        o_parts.push_back(o);
+        o = up(o + th->parts.size() * sizeof(TreePart));
+        for (const auto &pt : th->parts) o = up(up(up(o + pt.tasks.size() * sizeof(TreeTask)) + pt.path.size() * 4) + pt.leaf.size() * 4);
+    }
+    CUDA_TRY(p, cached_malloc(p->device, (void **)&im->base, o));
+    std::vector<unsigned char> stage(o, 0);
+    std::memcpy(stage.data(), p->pconfs.data(), p->pconfs.size() * sizeof(hap_pconf));
+    for (size_t t = 0; t < trees.size(); ++t) {
+        size_t at = up(o_parts[t] + trees[t]->parts.size() * sizeof(TreePart));
+        TreePart *parts = reinterpret_cast<TreePart *>(stage.data() + o_parts[t]);
+        for (size_t q = 0; q < trees[t]->parts.size(); ++q) {
+            const TreePartHost &ph = trees[t]->parts[q];
+            parts[q] = ph.meta;
+            parts[q].tasks = reinterpret_cast<const TreeTask *>(im->base + at);
+            if (!ph.tasks.empty()) std::memcpy(stage.data() + at, ph.tasks.data(), ph.tasks.size() * sizeof(TreeTask));
+            at = up(at + ph.tasks.size() * sizeof(TreeTask));
+            parts[q].path = reinterpret_cast<const u32 *>(im->base + at);
+            std::memcpy(stage.data() + at, ph.path.data(), ph.path.size() * 4);
+            at = up(at + ph.path.size() * 4);
+            parts[q].leaf = reinterpret_cast<const u32 *>(im->base + at);
+            std::memcpy(stage.data() + at, ph.leaf.data(), ph.leaf.size() * 4);
+            at = up(at + ph.leaf.size() * 4);
+        }
+        im->cls[t].parts = reinterpret_cast<const TreePart *>(im->base + o_parts[t]);
+    }
+    if (!im->cls.empty()) std::memcpy(stage.data() + o_cls, im->cls.data(), im->cls.size() * sizeof(TreeClass));
+    CUDA_TRY(p, cudaMemcpy(im->base, stage.data(), o, cudaMemcpyHostToDevice));
+    im->d_pconf = reinterpret_cast<hap_pconf *>(im->base);
+    im->d_cls = reinterpret_cast<TreeClass *>(im->base + o_cls);
+    p->image = im;
+    std::lock_guard<std::mutex> lock(ic.mu);
+    if (ic.map.size() >= kImages) ic.map.clear();
+    ic.map[key] = im;
+    return HAP_OK;
 }
 
 extern "C" hap_status hap_enumerate(hap_problem *p, uint64_t *n_pconf, uint64_t *n_candidates)
@@ -1286,17 +1003,6 @@ extern "C" hap_status hap_enumerate(hap_problem *p, uint64_t *n_pconf, uint64_t 
 
             fresh->rows.swap(rows); fresh->items.swap(items); fresh->classes.swap(classes);
             fresh->n_cand = off; fresh->tab_bytes = tab_bytes;
-            {   // the table and the items as every problem with these lists uploads them
-                auto up = [](size_t v) { return (v + 255) / 256 * 256; };
-                const size_t o_items = up(fresh->rows.size() * sizeof(hap_pconf)), total = up(o_items + fresh->items.size() * sizeof(WorkItem));
-                fresh->image = pinned_image(total);
-                if (fresh->image) {
-                    unsigned char *im = static_cast<unsigned char *>(fresh->image->ptr);
-                    std::memset(im, 0, total);
-                    std::memcpy(im, fresh->rows.data(), fresh->rows.size() * sizeof(hap_pconf));
-                    std::memcpy(im + o_items, fresh->items.data(), fresh->items.size() * sizeof(WorkItem));
-                }
-            }
             return HAP_OK;
             }();
             if (es != HAP_OK) return es;
@@ -1307,134 +1013,81 @@ extern "C" hap_status hap_enumerate(hap_problem *p, uint64_t *n_pconf, uint64_t 
         p->pconfs.ptr = er->rows.data(); p->pconfs.n = er->rows.size();
         p->items.ptr = er->items.data(); p->items.n = er->items.size();
         p->classes = er->classes;
-        const uint64_t off = er->n_cand;
-        const u64 tab_bytes = er->tab_bytes;
-        p->n_cand = off;
+        p->tab_bytes = er->tab_bytes;
+        p->n_cand = er->n_cand;
         const size_t np = p->pconfs.size();
-        // one allocation for everything whose size the enumeration fixes (an allocation costs far more than the
-        // microseconds a pass takes): configuration table | work items | layer costs | coefficients | per-type
-        // constants | lower bounds | partial minima | mapping tables | small scalars
-        // partial minima of a search: one slot per block; a class's tree kernel may run up to 8 parts per configuration
-        // (the exact count is fixed below, once the trees are built)
-        p->n_partial = 1024;
-        for (const auto &cl : p->classes) {
-            const size_t n_conf = p->items[cl.item_hi - 1].p - p->items[cl.item_lo].p + 1;
-            p->n_partial += std::max(cl.item_hi - cl.item_lo, n_conf * 8);
+        {
+            hap_status is = image_for(p, ekey);
+            if (is != HAP_OK) return is;
         }
+        const DeviceImage &im = *p->image;
+        p->all_trees = true;
+        for (size_t ci = 0; ci < p->classes.size(); ++ci) {
+            p->classes[ci].tree = im.tree_of[ci];
+            p->classes[ci].masks_used = im.masks_used[ci];
+            p->all_trees = p->all_trees && im.tree_of[ci] >= 0;
+        }
+        // one allocation for everything a pass needs (an allocation costs far more than the microseconds a pass takes):
+        // coefficients | per-type constants | lower bounds | partial minima | plans | records | small scalars; partial
+        // minima: one slot per block of the tree kernel, then one per block of the general one
+        p->n_partial = std::max<size_t>(1024, kTreeSlots + p->items.size());
         {
             auto up = [](size_t v) { return (v + 255) / 256 * 256; };
             size_t o = 0;
-            const size_t o_pconf = o; o = up(o + np * sizeof(hap_pconf));
-            const size_t o_items = o; o = up(o + p->items.size() * sizeof(WorkItem));
-            const size_t o_c2 = o; o = up(o + np * T * N * 2 * sizeof(i64));
             const size_t o_coef = o; o = up(o + np * T * HAP_NCOEF * sizeof(i64));
             const size_t o_tc = o; o = up(o + np * T * sizeof(TypeConst));
             const size_t o_lb = o; o = up(o + np * sizeof(i64));
             const size_t o_pcost = o; o = up(o + p->n_partial * sizeof(i64));
             const size_t o_pindex = o; o = up(o + p->n_partial * sizeof(u64));
-            const size_t o_maptab = o; o = up(o + tab_bytes);
-            const size_t o_range = o; o = up(o + sizeof(u64));
+            const size_t o_plans = o; o = up(o + (im.cls.empty() ? 0 : kTreeSlots) * sizeof(PlanSlot));
+            const size_t o_rec = o; o = up(o + im.rec_total);
             const size_t o_counters = o; o = up(o + 8 * sizeof(u64));
             const size_t o_best = o; o = up(o + 2 * sizeof(i64));
             const size_t o_single = o; o = up(o + sizeof(SingleOut));
+            const size_t o_report = o; o = up(o + sizeof(TreeReport));
+            const size_t o_live = o; o = up(o + np * sizeof(u32));
+            const size_t o_dead = o; o = up(o + np * sizeof(u32));
+            const size_t o_hist = o; o = up(o + (p->opts.prune ? kOrderBuckets * sizeof(u64) : 0));
+            const size_t o_key = o; o = up(o + (p->opts.prune ? np * sizeof(uint4) : 0));
+            const size_t o_order = o; o = up(o + (p->opts.prune ? (np + 1) * sizeof(uint4) : 0));
+            const size_t o_res = o; o = up(o + sizeof(TreeResult));
             CUDA_TRY(p, cached_malloc(p->device, (void **)&p->d_arena, o));
             unsigned char *base = p->d_arena;
-            p->d_pconf = reinterpret_cast<hap_pconf *>(base + o_pconf); p->d_items = reinterpret_cast<WorkItem *>(base + o_items);
-            p->d_c2 = reinterpret_cast<i64 *>(base + o_c2); p->d_coef = reinterpret_cast<i64 *>(base + o_coef);
+            p->d_coef = reinterpret_cast<i64 *>(base + o_coef);
             p->d_tc = reinterpret_cast<TypeConst *>(base + o_tc); p->d_lb = reinterpret_cast<i64 *>(base + o_lb);
             p->d_pcost = reinterpret_cast<i64 *>(base + o_pcost); p->d_pindex = reinterpret_cast<u64 *>(base + o_pindex);
-            p->d_maptab = tab_bytes ? base + o_maptab : nullptr;
-            p->d_range = reinterpret_cast<u64 *>(base + o_range); p->d_counters = reinterpret_cast<u64 *>(base + o_counters);
+            p->d_plans = reinterpret_cast<PlanSlot *>(base + o_plans);
+            p->d_counters = reinterpret_cast<u64 *>(base + o_counters);
             p->d_best = reinterpret_cast<i64 *>(base + o_best); p->d_single = base + o_single;
-            // configuration table and work items travel in one copy (they are adjacent up to padding)
-            if (er->image && er->image->bytes == o_c2) CUDA_TRY(p, upload_image(p, base, *er->image, o_c2));
-            else CUDA_TRY(p, upload(p, base, o_c2, [&](unsigned char *stage) {
-                std::memcpy(stage + o_pconf, p->pconfs.data(), np * sizeof(hap_pconf));
-                std::memcpy(stage + o_items, p->items.data(), p->items.size() * sizeof(WorkItem));
-                return true; }));
-            if (p->upload_pending) {
-                cudaStream_t us = upload_stream(p->device);
-                CUDA_TRY(p, cudaMemsetAsync(p->d_range, 0, sizeof(u64), us));
-                CUDA_TRY(p, cudaEventRecord(p->ev_upload, us));
-            } else CUDA_TRY(p, cudaMemset(p->d_range, 0, sizeof(u64)));
+            TreeArgs &ta = p->targs;
+            ta.rec = base + o_rec;
+            ta.state = reinterpret_cast<TreeState *>(reinterpret_cast<unsigned char *>(p->d_range) + 16);
+            ta.report = reinterpret_cast<TreeReport *>(base + o_report);
+            ta.live_list = reinterpret_cast<const u32 *>(base + o_live); ta.dead_list = reinterpret_cast<const u32 *>(base + o_dead);
+            ta.hist = reinterpret_cast<u64 *>(base + o_hist);
+            ta.order_key = reinterpret_cast<uint4 *>(base + o_key); ta.order = reinterpret_cast<uint4 *>(base + o_order);
+            LiveArgs &la = p->largs;
+            la.hist = ta.hist; la.n_hist = 0;
+            la.state = ta.state; la.report = ta.report;
+            la.live_list = reinterpret_cast<u32 *>(base + o_live); la.dead_list = reinterpret_cast<u32 *>(base + o_dead);
+            la.n_cls = ta.n_cls = (int)im.cls.size();
+            for (size_t c = 0; c < im.cls.size(); ++c) {
+                la.p_lo[c] = ta.p_lo[c] = im.cls[c].p_lo; la.p_hi[c] = im.cls[c].p_lo + im.cls[c].n_conf;
+                ta.nmap[c] = (u32)p->pconfs[im.cls[c].p_lo].nmap;
+                la.first_min[c] = 0;
+                for (int h = 0; h < HAP_MAX_TYPES; ++h) la.first_min[c] |= (u32)im.cls[c].first_min[h] << (8 * h);
+            }
+            ta.res_dev = reinterpret_cast<TreeResult *>(base + o_res);
+            ta.N = N; ta.T = T; ta.R = p->prof.R; ta.n_rc = p->opts.n_rc; ta.RW = p->dc.tau_linear ? p->prof.R : 2;
+            ta.eta_q = p->dc.eta_q; ta.kind_uniform = p->dc.kind_uniform; ta.kind0 = p->kind[0];
+            for (int i = 0; i < p->opts.n_rc; ++i) { ta.rc_masks[i] = p->dc.rc_masks[i]; ta.rc_sup[i] = p->dc.rc_sup[i]; ta.rc_order[i] = p->dc.rc_order[i]; }
+            for (int r = 0; r < p->prof.R; ++r) ta.tau[r] = p->tau_q[r] / 1024.0;
+            ta.cls = im.d_cls;
+            ta.range_flag = p->d_range;
+            ta.slots = p->d_plans; ta.slot_cost = p->d_pcost; ta.slot_index = p->d_pindex;
         }
-        p->dc.pconf = p->d_pconf;
+        p->dc.pconf = im.d_pconf;
         p->dc.n_pconf = np;
-        CUDA_TRY(p, cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming));
-        CUDA_TRY(p, cudaEventCreateWithFlags(&p->ev_pre, cudaEventDisableTiming));
-        CUDA_TRY(p, cudaEventCreateWithFlags(&p->ev_dec, cudaEventDisableTiming));
-        for (size_t ci = 0; ci < p->classes.size(); ++ci) {
-            auto &cl = p->classes[ci];
-            cl.stream = pooled_stream(p->device, ci);
-            if (!cl.stream) return fail(p, HAP_E_CUDA, "cudaStreamCreateWithFlags");
-            CUDA_TRY(p, cudaEventCreateWithFlags(&cl.done, cudaEventDisableTiming));
-        }
-        if (tab_bytes) {
-            // The prefix tree of a class depends on the cluster, the stage count, the model's layer kinds and the
-            // window, not on the profiled tables: trees are kept per process under a key of exactly those inputs, so
-            // that planning again on the same cluster (new tables, new batch) neither decodes the mappings for the
-            // host nor rebuilds a tree.
-            // the tree kernel holds times as doubles: exact while every prefix row stays below 2^52, which the
-            // per-layer limit of 2^36 ns guarantees when N (2 + max tau) <= 2^16
-            int tau_max = 0;
-            for (int r = 0; r < p->prof.R; ++r) tau_max = std::max(tau_max, p->tau_q[r] >> 10);
-            const bool rows_exact = (int64_t)N * (2 + tau_max) <= 65536;
-            const bool want_trees = !(p->opts.flags & HAP_OPT_NO_TRIE) && p->dc.tau_linear && rows_exact;
-            std::vector<TrieBuilt> built;
-            std::vector<hap_problem::PpClass *> missing;
-            std::vector<std::string> keys(p->classes.size());
-            for (size_t ci = 0; ci < p->classes.size(); ++ci) {
-                auto &cl = p->classes[ci];
-                if (!cl.has_tab) continue;
-                keys[ci] = trie_cache_key(p, cl);
-                std::shared_ptr<const TrieClassHost> hit = trie_cache_find(keys[ci]);
-                if (!hit) { missing.push_back(&cl); continue; }
-                cl.masks_used = hit->masks_used;
-                if (want_trees && !hit->parts.empty()) built.push_back(TrieBuilt{&cl, hit, class_plist(p, cl)});
-            }
-            if (!missing.empty()) {
-                CUDA_TRY(p, uploads_done(p));                 // the decode below reads the configuration table
-                for (const hap_problem::PpClass *cl : missing) {
-                    const WorkItem &rep = p->items[cl->item_lo];
-                    const u64 nmap = p->pconfs[rep.p].nmap;
-                    maptab_kernel<<<(unsigned)((nmap + 3) / 4), 128>>>(p->dc, rep.p, nmap, p->d_maptab + cl->map_base);
-                    CUDA_TRY(p, cudaGetLastError());
-                    cl->tab_valid = true;
-                }
-                CUDA_TRY(p, cudaDeviceSynchronize());
-                std::vector<uint8_t> tab(tab_bytes);
-                CUDA_TRY(p, cudaMemcpy(tab.data(), p->d_maptab, tab_bytes, cudaMemcpyDeviceToHost));
-                for (hap_problem::PpClass *clp : missing) {
-                    auto &cl = *clp;
-                    const u64 nmap = p->pconfs[p->items[cl.item_lo].p].nmap;
-                    auto th = std::make_shared<TrieClassHost>();
-                    // which type masks occur in a class: the DP kernel builds stage rows for those only
-                    unsigned used = 0;
-                    for (u64 e = 0; e < nmap * (u64)cl.PP; ++e) used |= 1u << tab[cl.map_base + e * 2];
-                    th->masks_used = used;
-                    cl.masks_used = used;
-                    const std::vector<u32> plist = class_plist(p, cl);
-                    const bool ok = want_trees && build_trie(p, cl, tab.data() + cl.map_base, nmap, plist.size(), *th);
-                    if (!ok) th->parts.clear();
-                    // a class whose tree was not wanted this time is not remembered as "has no tree"
-                    if (want_trees) trie_cache_insert(keys[clp - p->classes.data()], th);
-                    if (ok) built.push_back(TrieBuilt{&cl, th, plist});
-                }
-            }
-            // the launch order of the merged decode / gather jobs follows the class order
-            std::sort(built.begin(), built.end(), [](const TrieBuilt &x, const TrieBuilt &y) { return x.cl < y.cl; });
-            std::string image_key = ekey;
-            for (const auto &bc : built) image_key += keys[bc.cl - p->classes.data()];
-            upload_tries(p, built, image_key);
-        }
-        p->n_pslots = 0;
-        for (auto &cl : p->classes) {
-            cl.pslot_lo = p->n_pslots;
-            cl.pslot_n = cl.item_hi - cl.item_lo;
-            if (cl.trie.ok) cl.pslot_n = std::max(cl.pslot_n, (size_t)cl.trie.n_conf * cl.trie.parts.size());
-            p->n_pslots += cl.pslot_n;
-        }
-        if (p->n_pslots > p->n_partial) return fail(p, HAP_E_STATE, "partial-minimum slots exceed their allocation");
         p->enumerated = true;
     }
     if (n_pconf) *n_pconf = p->pconfs.size();
@@ -1451,12 +1104,33 @@ extern "C" hap_status hap_get_pconfs(const hap_problem *p, hap_pconf *host_out, 
     return HAP_OK;
 }
 
-static hap_status enter(hap_problem *p)
+// Every call that launches work starts here.  The tables' upload is waited for by the stream; a call on another stream
+// than the last one waits for that one's work, because a problem's passes share its scratch memory.
+static hap_status enter(hap_problem *p, cudaStream_t st)
 {
     if (!p) return HAP_E_INVALID;
     if (!p->enumerated) return fail(p, HAP_E_STATE, "hap_enumerate has not run");
     if (cudaSetDevice(p->device) != cudaSuccess) return fail(p, HAP_E_CUDA, "cudaSetDevice");
-    if (uploads_done(p) != cudaSuccess) return fail(p, HAP_E_CUDA, "upload of the problem's tables");
+    if (p->upload_pending) CUDA_TRY(p, cudaStreamWaitEvent(st, p->ev_upload, 0));
+    if (p->in_flight && st != p->last_stream) CUDA_TRY(p, cudaStreamWaitEvent(st, p->ev_done, 0));
+    return HAP_OK;
+}
+
+// ... and ends here: the work it queued on `st` is in flight
+static hap_status leave_async(hap_problem *p, cudaStream_t st)
+{
+    CUDA_TRY(p, cudaEventRecord(p->ev_done, st));
+    p->in_flight = true;
+    p->last_stream = st;
+    return HAP_OK;
+}
+
+// ... or here, with everything it queued done
+static hap_status leave_synced(hap_problem *p, cudaStream_t st)
+{
+    CUDA_TRY(p, cudaStreamSynchronize(st));
+    p->in_flight = false;
+    p->upload_pending = false;
     return HAP_OK;
 }
 
@@ -1476,7 +1150,7 @@ static hap_status check_range(hap_problem *p, uint64_t first, uint64_t count)
 
 extern "C" hap_status hap_decode(hap_problem *p, uint64_t first, uint64_t count, hap_candidate *dev_out, void *stream)
 {
-    hap_status s = enter(p);
+    hap_status s = enter(p, (cudaStream_t)stream);
     if (s != HAP_OK) return s;
     if ((s = check_range(p, first, count)) != HAP_OK) return s;
     if (count == 0) return HAP_OK;
@@ -1485,6 +1159,33 @@ extern "C" hap_status hap_decode(hap_problem *p, uint64_t first, uint64_t count,
     if (blocks > 0x7fffffffull) return fail(p, HAP_E_RANGE, "count too large for one launch");
     decode_kernel<<<(unsigned)blocks, 128, 0, (cudaStream_t)stream>>>(p->dc, first, count, dev_out, nullptr);
     CUDA_TRY(p, cudaGetLastError());
+    return leave_async(p, (cudaStream_t)stream);
+}
+
+
+// work items, layer-cost array and mapping table of the general kernel, with its streams and events (first use)
+static hap_status ensure_general(hap_problem *p)
+{
+    if (p->gen_ready) return HAP_OK;
+    const size_t np = p->pconfs.size();
+    auto up = [](size_t v) { return (v + 255) / 256 * 256; };
+    size_t o = 0;
+    const size_t o_items = o; o = up(o + p->items.size() * sizeof(WorkItem));
+    const size_t o_c2 = o; o = up(o + np * p->T * p->model.N * 2 * sizeof(i64));
+    const size_t o_maptab = o; o = up(o + p->tab_bytes);
+    CUDA_TRY(p, cached_malloc(p->device, (void **)&p->d_gen_arena, o));
+    p->d_items = reinterpret_cast<WorkItem *>(p->d_gen_arena + o_items);
+    p->d_c2 = reinterpret_cast<i64 *>(p->d_gen_arena + o_c2);
+    p->d_maptab = p->tab_bytes ? p->d_gen_arena + o_maptab : nullptr;
+    CUDA_TRY(p, cudaMemcpy(p->d_items, p->items.data(), p->items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice));
+    if (!(p->ev_fork = pooled_event(p->device))) return fail(p, HAP_E_CUDA, "cudaEventCreate");
+    for (auto &e : p->ev) CUDA_TRY(p, cudaEventCreate(&e));
+    for (size_t ci = 0; ci < p->classes.size(); ++ci) {
+        auto &cl = p->classes[ci];
+        if (!(cl.stream = pooled_stream(p->device, ci))) return fail(p, HAP_E_CUDA, "cudaStreamCreateWithFlags");
+        if (!(cl.done = pooled_event(p->device))) return fail(p, HAP_E_CUDA, "cudaEventCreate");
+    }
+    p->gen_ready = true;
     return HAP_OK;
 }
 
@@ -1530,41 +1231,47 @@ static void configs_of_range(const hap_problem *p, u64 first, u64 count, unsigne
     lo = owner(first); hi = owner(first + count - 1) + 1;
 }
 
-// Per-type constants and stage coefficients, then (where an output array is given) the layer costs, of the
-// configurations [p_lo, p_hi): a pass over a candidate range touches only the configurations that own its candidates.
+// Per-type constants and stage coefficients of the configurations [p_lo, p_hi) in integer (coef) and / or fp64 form (coeff);
+// `live`: also the classes' lists of configurations (a pass over the trees)
+static hap_status launch_type_consts(hap_problem *p, i64 *coef, double *coeff, cudaStream_t st, unsigned p_lo, unsigned p_hi, const LiveArgs *live = nullptr)
+{
+    const unsigned n_conf = p_hi - p_lo;
+    static const LiveArgs none{};
+    const unsigned per = 32 / (unsigned)p->T;                 // configurations of a block
+    type_const_kernel<<<(n_conf + per - 1) / per, kTcThreads, 0, st>>>(p->dc, p->d_tc, coef, coeff, p->d_range, p_lo, n_conf, live ? *live : none);
+    CUDA_TRY(p, cudaGetLastError());
+    return HAP_OK;
+}
+
+// ... and then (where an output array is given) the layer costs: a pass over a candidate range touches only the
+// configurations that own its candidates.
 static hap_status launch_layer_costs(hap_problem *p, i64 *c2, i64 *coef, double *c2f, double *coeff, bool quant, cudaStream_t st,
                                      i64 *lb_sum = nullptr, unsigned p_lo = 0, unsigned p_hi = ~0u)
 {
     if (p_hi > p->pconfs.size()) p_hi = (unsigned)p->pconfs.size();
     if (p_lo >= p_hi) return HAP_OK;
-    const unsigned n_conf = p_hi - p_lo;
-    const u64 nph = (u64)n_conf * HAP_MAX_TYPES;
-    const unsigned b1 = (unsigned)((nph + kLcThreads - 1) / kLcThreads);
-    if (quant) type_const_kernel<true><<<dim3(b1, 3), kLcThreads, 0, st>>>(p->dc, p->d_tc, coef, nullptr, p->d_range, p_lo, n_conf);
-    else type_const_kernel<false><<<dim3(b1, 3), kLcThreads, 0, st>>>(p->dc, p->d_tc, nullptr, coeff, p->d_range, p_lo, n_conf);
-    CUDA_TRY(p, cudaGetLastError());
-    if ((quant && c2) || (!quant && c2f)) {
-        hap_status s = launch_layer_kernel(p, c2, c2f, quant, st, lb_sum, nullptr, p_lo, n_conf, true);
-        if (s != HAP_OK) return s;
-    }
-    CUDA_TRY(p, cudaGetLastError());
+    hap_status s = launch_type_consts(p, quant ? coef : nullptr, quant ? nullptr : coeff, st, p_lo, p_hi);
+    if (s != HAP_OK) return s;
+    if ((quant && c2) || (!quant && c2f)) return launch_layer_kernel(p, c2, c2f, quant, st, lb_sum, nullptr, p_lo, p_hi - p_lo, true);
     return HAP_OK;
 }
 
 extern "C" hap_status hap_eval_layer_costs(hap_problem *p, int64_t *dev_c2, int64_t *dev_coef, void *stream)
 {
-    hap_status s = enter(p);
+    hap_status s = enter(p, (cudaStream_t)stream);
     if (s != HAP_OK) return s;
     if (!dev_c2 && !dev_coef) return HAP_OK;
-    return launch_layer_costs(p, (i64 *)dev_c2, (i64 *)dev_coef, nullptr, nullptr, true, (cudaStream_t)stream);
+    if ((s = launch_layer_costs(p, (i64 *)dev_c2, (i64 *)dev_coef, nullptr, nullptr, true, (cudaStream_t)stream)) != HAP_OK) return s;
+    return leave_async(p, (cudaStream_t)stream);
 }
 
 extern "C" hap_status hap_eval_layer_costs_f64(hap_problem *p, double *dev_c2, double *dev_coef, void *stream)
 {
-    hap_status s = enter(p);
+    hap_status s = enter(p, (cudaStream_t)stream);
     if (s != HAP_OK) return s;
     if (!dev_c2 && !dev_coef) return HAP_OK;
-    return launch_layer_costs(p, nullptr, nullptr, dev_c2, dev_coef, false, (cudaStream_t)stream);
+    if ((s = launch_layer_costs(p, nullptr, nullptr, dev_c2, dev_coef, false, (cudaStream_t)stream)) != HAP_OK) return s;
+    return leave_async(p, (cudaStream_t)stream);
 }
 
 // whether all candidates of the class lie outside the range the pass writes
@@ -1575,95 +1282,161 @@ static bool class_outside(const hap_problem *p, const hap_problem::PpClass &cl, 
     return c1 <= out.first || c0 >= out.first + out.count;
 }
 
-// plain integer passes over more than one candidate walk the class's prefix tree; tables, refinement, fp64, cell
-// counting and the one-candidate re-evaluation stay in pipeline_dp_kernel
-static bool pass_uses_trie(const hap_problem *p, const hap_problem::PpClass &cl, const DpOut &out, bool f64)
+// Plain passes walk the prefix trees of the classes that have one; tables, refinement, cell counting and the
+// one-candidate re-evaluation stay in pipeline_dp_kernel.  (The tree kernel writes partitions in 16-byte pieces.)
+static bool pass_uses_trees(const hap_problem *p, const DpOut &out)
 {
-    const bool refine = (p->opts.flags & (HAP_OPT_REFINE | HAP_OPT_EXACT)) != 0 && !out.count_only && !out.force_plain;
-    (void)f64;                                  // both value types walk the tree
-    return cl.trie.ok && !out.count_only && !refine && p->dc.tau_linear != 0 && !out.dp_table && !out.choice && out.count > 1;
+    const bool refine = (p->opts.flags & (HAP_OPT_REFINE | HAP_OPT_EXACT)) != 0 && !out.force_plain;
+    const bool aligned = ((reinterpret_cast<uintptr_t>(out.partition) | reinterpret_cast<uintptr_t>(out.recompute)) & 15) == 0;
+    return !p->image->cls.empty() && !out.count_only && !refine && !out.dp_table && !out.choice && !out.detail && !out.first_dev && aligned;
 }
 
-// Whether every class the pass touches walks its prefix tree: then the blocks of the tree kernel compute the layer
-// times of their configuration themselves (Eq. 2 from the profiled tables and the per-type constants) and the pass
-// neither writes nor reads the layer-cost array.
-static bool pass_fuses_layer_costs(const hap_problem *p, const DpOut &out, bool search)
+// The dynamic shared memory limit is a per-kernel, per-device attribute shared by every problem of the process: raised
+// (never lowered) before a launch that needs more.
+static cudaError_t raise_smem_limit(int device, const void *fn, size_t bytes)
 {
-    if (p->opts.flags & HAP_OPT_NO_FUSE) return false;
-    bool any = false;
-    for (const auto &cl : p->classes) {
-        if (!search && !out.first_dev && class_outside(p, cl, out)) continue;
-        if (!pass_uses_trie(p, cl, out, false)) return false;
-        any = true;
-    }
-    return any;
+    static std::mutex mu;
+    static std::map<std::pair<int, const void *>, size_t> limit;
+    std::lock_guard<std::mutex> lock(mu);
+    size_t &l = limit[{device, fn}];
+    if (bytes <= l) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) l = bytes;
+    return e;
 }
 
-// candidate decode of a class for this pass, then its stage bytes into the class's tree
-static hap_status launch_class_decode(hap_problem *p, const hap_problem::PpClass &cl)
+static int sm_count(int device)
 {
-    const hap_problem::Trie &tr = cl.trie;
-    const uint8_t *tab = p->d_maptab + cl.map_base;
-    const u64 nmap = p->pconfs[p->items[cl.item_lo].p].nmap;
-    maptab_kernel<<<(unsigned)((nmap + 3) / 4), 128, 0, cl.stream>>>(p->dc, p->items[cl.item_lo].p, nmap, p->d_maptab + cl.map_base);
-    CUDA_TRY(p, cudaGetLastError());
-    for (const auto &pd : tr.parts) {
-        const u32 n_g = pd.n_nodes + pd.n_cells + pd.nmap;
-        TrieRowMap rmap;
-        std::memcpy(rmap.mrow_of, pd.mrow_of, sizeof(rmap.mrow_of));
-        trie_gather_kernel<<<(n_g + 255) / 256, 256, 0, cl.stream>>>(tab, cl.PP, pd.n_nodes, pd.n_cells, pd.nmap, pd.m_lo, pd.d_first_leaf,
-                                                                      pd.d_depth, pd.d_gnode, rmap, pd.d_nodes, pd.d_cells, pd.d_leaves);
-        CUDA_TRY(p, cudaGetLastError());
+    static int n[64];                                       // (the same value whoever writes it)
+    int &v = n[device & 63];
+    if (!v && cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) { cudaGetLastError(); v = 148; }
+    return v;
+}
+
+// launch behind the kernel before it in the stream, as its programmatic dependent
+static cudaError_t launch_dependent(const void *fn, unsigned grid, unsigned threads, size_t smem, cudaStream_t st, void **args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelExC(&cfg, fn, args);
+}
+
+// One launch of the tree kernel: classes [c_lo, c_hi) of the image.
+struct TreeLaunch { int c_lo, c_hi; size_t smem; unsigned grid; u64 items; };
+
+// A pass runs the deep pipelines (long chains of small depths) and the others in launches of their own, deep ones first:
+// the blocks of each take the shared memory their own classes need.  A search is one launch where it may prune (its items
+// go in order of their bounds) or where everything starts at once.
+static std::vector<TreeLaunch> tree_launches(const hap_problem *p, bool search, bool prune, unsigned p_lo, unsigned p_hi)
+{
+    const auto &cls = p->image->cls;
+    std::vector<TreeLaunch> ls;
+    auto group = [&](int c_lo, int c_hi) {
+        TreeLaunch l{c_lo, c_hi, 0, 0, 0};
+        for (int c = c_lo; c < c_hi; ++c) {
+            const TreeClass &cl = cls[(size_t)c];
+            const unsigned a = std::max(p_lo, cl.p_lo), b = std::min(p_hi, cl.p_lo + cl.n_conf);
+            if (a >= b) continue;
+            const u64 cpi = prune ? 1 : cl.conf_per_item;
+            l.items += (b - a + cpi - 1) / cpi * cl.items_per_conf;
+            l.smem = std::max(l.smem, tree_smem_bytes(cl));
+        }
+        if (!l.items) return;
+        const unsigned per_sm = (unsigned)std::max<size_t>(1, std::min<size_t>(kTreeBlocksPerSm, (227 * 1024) / (l.smem + 1024 + 256)));
+        l.grid = (unsigned)std::min<u64>(l.items, std::min<u64>((u64)sm_count(p->device) * per_sm, kTreeSlots / 2));
+        ls.push_back(l);
+    };
+    if (search) {
+        group(0, (int)cls.size());
+        if (prune || ls.empty() || ls[0].items <= ls[0].grid) return ls;
+        ls.clear();
     }
+    int split = 0;
+    while (split < (int)cls.size() && cls[(size_t)split].PP >= 16) ++split;
+    if (split > 0) group(0, split);
+    if (split < (int)cls.size()) group(split, (int)cls.size());
+    return ls;
+}
+
+// A pass or a search over the prefix trees: per-type constants, (the layer-cost array where it is asked for,) records,
+// recurrence -- each the programmatic dependent of the one before.  Classes without a tree are left to launch_dp; c2 / c2f
+// then hold their layer costs.
+static hap_status launch_trees(hap_problem *p, const DpOut &out_in, bool search, bool f64, cudaStream_t st, bool final_reduce)
+{
+    DpOut out = out_in;
+    out.range_flag = p->d_range;
+    unsigned p_lo, p_hi;
+    configs_of_range(p, out.first, out.count, p_lo, p_hi);
+    const bool separate = (p->opts.flags & HAP_OPT_NO_FUSE) != 0;
+    hap_status s;
+    if (p->state_dirty) CUDA_TRY(p, cudaMemsetAsync(p->targs.state, 0, sizeof(TreeState), st));
+    p->state_dirty = true;
+    const bool prune = search && !f64 && out.prune;
+    const std::vector<TreeLaunch> ls = tree_launches(p, search, prune, p_lo, p_hi);
+    const bool ordered = prune && ls.size() == 1 && ls[0].items > ls[0].grid;      // (in one wave everything starts at once)
+    p->largs.n_hist = ordered ? kOrderBuckets : 0;
+    if ((s = launch_type_consts(p, p->d_coef, f64 ? p->d_coeff : nullptr, st, p_lo, p_hi, &p->largs)) != HAP_OK) return s;
+    const void *c2v = nullptr;
+    if (separate || !p->all_trees) {
+        if (f64) { if ((s = launch_layer_kernel(p, nullptr, p->d_c2f, false, st, nullptr, nullptr, p_lo, p_hi - p_lo, true)) != HAP_OK) return s; }
+        else if ((s = launch_layer_kernel(p, p->d_c2, nullptr, true, st, p->d_lb, nullptr, p_lo, p_hi - p_lo, true)) != HAP_OK) return s;
+        if (separate) c2v = f64 ? (const void *)p->d_c2f : (const void *)p->d_c2;
+    }
+    const bool nl = !p->dc.tau_linear;
+    const DeviceImage &im = *p->image;
+    TreeArgs ta = p->targs;
+    if (!ordered) ta.order = nullptr;
+    int is_search = search ? 1 : 0;
+    {
+        const void *fn = f64 ? (nl ? (const void *)tree_prep_kernel<true, true> : (const void *)tree_prep_kernel<true, false>)
+                             : (nl ? (const void *)tree_prep_kernel<false, true> : (const void *)tree_prep_kernel<false, false>);
+        CUDA_TRY(p, raise_smem_limit(p->device, fn, im.prep_smem));
+        const double *coeff = p->d_coeff;
+        void *args[] = {(void *)&p->dc, (void *)&ta, (void *)&p->d_tc, (void *)&p->d_coef, (void *)&coeff, (void *)&c2v, (void *)&out, (void *)&is_search};
+        const unsigned per_sm = (unsigned)std::max<size_t>(1, std::min<size_t>(kTreePrepBlocksPerSm, (227 * 1024) / (im.prep_smem + 2048)));
+        CUDA_TRY(p, launch_dependent(fn, std::min<unsigned>(p_hi - p_lo, (unsigned)sm_count(p->device) * per_sm), kTreePrepThreads, im.prep_smem, st, args));
+    }
+    ta.blocks_total = 0;
+    for (const auto &l : ls) ta.blocks_total += l.grid;
+    if (!final_reduce) ta.res_dev = nullptr;
+    ta.res_host = final_reduce ? p->host_result : nullptr;
+    const bool counting = (p->opts.flags & HAP_OPT_COUNT_SPLITS) && !f64 && !search;
+    // two row entries are held where there are at most two levels, else they are read by level
+    const int form = nl ? 2 : p->prof.R > 2 ? 1 : 0;
+    using Fn = void (*)(const TreeArgs, const DevConst, DpOut);
+    static const Fn fns[5][3] = {
+        {tree_dp_kernel<false, false, 2, false, false>, tree_dp_kernel<false, false, 4, false, false>, tree_dp_kernel<false, false, 4, true, false>},
+        {tree_dp_kernel<true, false, 2, false, false>, tree_dp_kernel<true, false, 4, false, false>, tree_dp_kernel<true, false, 4, true, false>},
+        {tree_dp_kernel<false, true, 2, false, false>, tree_dp_kernel<false, true, 4, false, false>, tree_dp_kernel<false, true, 4, true, false>},
+        {tree_dp_kernel<true, true, 2, false, false>, tree_dp_kernel<true, true, 4, false, false>, tree_dp_kernel<true, true, 4, true, false>},
+        {tree_dp_kernel<false, false, 2, false, true>, tree_dp_kernel<false, false, 4, false, true>, tree_dp_kernel<false, false, 4, true, true>}};
+    const void *fn = (const void *)fns[counting ? 4 : (f64 ? 2 : 0) + (search ? 1 : 0)][form];
+    int n = 0;
+    for (const auto &l : ls) {
+        ta.c_lo = l.c_lo; ta.c_hi = l.c_hi; ta.launch = n;
+        ta.slot_lo = n == 0 ? 0 : ls[0].grid;
+        CUDA_TRY(p, raise_smem_limit(p->device, fn, l.smem));
+        void *args[] = {(void *)&ta, (void *)&p->dc, (void *)&out};
+        CUDA_TRY(p, launch_dependent(fn, l.grid, kTreeThreads, l.smem, st, args));
+        ++n;
+    }
+    p->state_dirty = ls.empty();                             // the last block of the recurrence clears the counters
     return HAP_OK;
 }
 
-// The candidate decode reads nothing the layer-cost kernels write: it waits only for the start of the pass (ev_pre,
-// recorded before the layer-cost launches) and runs on the class streams beside the layer costs instead of between
-// them and the recurrence.  On the host it is issued after the layer-cost launches, so that those reach an idle GPU
-// without waiting for a dozen other launches to be queued.
-static hap_status launch_decode_early(hap_problem *p, const DpOut &out, bool search)
+// One launch of the general kernel per PP class (each has its own block shape); every block clips to the candidate range.
+// skip_trees: only the classes without a tree.
+static hap_status launch_dp(hap_problem *p, const DpOut &out, bool search, cudaStream_t st, bool f64 = false, bool skip_trees = false)
 {
-    (void)search;
-    bool any = false, all = true;
-    for (const auto &cl : p->classes) {
-        const bool uses = pass_uses_trie(p, cl, out, false);
-        any |= uses;
-        if (cl.trie.ok && !uses) all = false;
-    }
-    if (!any || !all || !p->n_gather_jobs || p->decode_jobs.n == 0) return HAP_OK;
-    // one decode launch and one gather launch for all classes and parts, on the first class's stream
-    cudaStream_t sx = p->classes[0].stream;
-    CUDA_TRY(p, cudaStreamWaitEvent(sx, p->ev_pre, 0));
-    const DecodeJobs &dj = p->decode_jobs;
-    maptab_all_kernel<<<dj.blk_lo[dj.n], 128, 0, sx>>>(p->dc, dj, p->d_maptab);
-    CUDA_TRY(p, cudaGetLastError());
-    trie_gather_all_kernel<<<p->gather_blocks, 256, 0, sx>>>(p->d_gather_jobs, p->n_gather_jobs, p->d_maptab);
-    CUDA_TRY(p, cudaGetLastError());
-    CUDA_TRY(p, cudaEventRecord(p->ev_dec, sx));
-    p->decoded_all = true;
-    for (const auto &cl : p->classes) if (cl.trie.ok) cl.tab_valid = true;
-    return HAP_OK;
-}
-
-// One launch per PP class (each has its own block shape); every block clips to the candidate range.
-static hap_status launch_dp(hap_problem *p, const DpOut &out, bool search, cudaStream_t st, bool f64 = false)
-{
-    // the dynamic shared memory limit is a per-kernel, per-device attribute shared by every problem of the
-    // process: raise it (never lower it) before a launch that needs more
-    static size_t smem_limit[64][12];
-    static std::mutex limit_mu;                 // both tables of raised limits, for problems used from several host threads
-    std::lock_guard<std::mutex> limit_lock(limit_mu);
-    const int dev = p->device & 63;
-    // fork: every PP class runs on its own stream so that the tail of one class overlaps the next; a merged
-    // candidate decode queued earlier in this pass joins first, so that the fork event covers it
-    const bool decoded_all = p->decoded_all;
-    p->decoded_all = false;
-    if (decoded_all) CUDA_TRY(p, cudaStreamWaitEvent(st, p->ev_dec, 0));
+    // fork: every PP class runs on its own stream so that the tail of one class overlaps the next
     CUDA_TRY(p, cudaEventRecord(p->ev_fork, st));
     // the class with the most work goes first; the others fill the SMs it leaves free and its tail
     std::vector<const hap_problem::PpClass *> order;
-    for (const auto &cl : p->classes) order.push_back(&cl);
+    for (const auto &cl : p->classes) if (!(skip_trees && cl.tree >= 0)) order.push_back(&cl);
     std::stable_sort(order.begin(), order.end(), [](const hap_problem::PpClass *a, const hap_problem::PpClass *b) {
         return (a->item_hi - a->item_lo) * (size_t)a->PP > (b->item_hi - b->item_lo) * (size_t)b->PP;
     });
@@ -1677,7 +1450,6 @@ static hap_status launch_dp(hap_problem *p, const DpOut &out, bool search, cudaS
         if (!search && !out.first_dev && class_outside(p, cl, out)) continue;     // (a range that starts at a device-side index: every class looks)
         const bool lin = p->dc.tau_linear != 0;
         const bool refine = (p->opts.flags & (HAP_OPT_REFINE | HAP_OPT_EXACT)) != 0 && !out.count_only && !out.force_plain;
-        const int variant = f64 ? 6 + (lin ? 1 : 0) : out.count_only ? 4 + (lin ? 1 : 0) : (refine ? 8 : 0) + (search ? 2 : 0) + (lin ? 1 : 0);
         const void *fn;
         if (f64) fn = lin ? (const void *)pipeline_dp_kernel<false, true, false, double> : (const void *)pipeline_dp_kernel<false, false, false, double>;
         else if (out.count_only) fn = lin ? (const void *)pipeline_dp_kernel<false, true, true> : (const void *)pipeline_dp_kernel<false, false, true>;
@@ -1685,49 +1457,12 @@ static hap_status launch_dp(hap_problem *p, const DpOut &out, bool search, cudaS
                                      : (lin ? (const void *)pipeline_dp_kernel<false, true, false, i64, true> : (const void *)pipeline_dp_kernel<false, false, false, i64, true>);
         else fn = search ? (lin ? (const void *)pipeline_dp_kernel<true, true> : (const void *)pipeline_dp_kernel<true, false>)
                          : (lin ? (const void *)pipeline_dp_kernel<false, true> : (const void *)pipeline_dp_kernel<false, false>);
-        if (cl.smem > smem_limit[dev][variant]) {
-            CUDA_TRY(p, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cl.smem));
-            smem_limit[dev][variant] = cl.smem;
-        }
+        CUDA_TRY(p, raise_smem_limit(p->device, fn, cl.smem));
         const unsigned blocks = (unsigned)(cl.item_hi - cl.item_lo);
         const uint8_t *tab = cl.has_tab ? p->d_maptab + cl.map_base : nullptr;
         DpOut o = out;
         o.exact = (p->opts.flags & HAP_OPT_EXACT) != 0 && !out.force_plain;
-        if (search) { o.partial_cost += cl.pslot_lo; o.partial_index += cl.pslot_lo; if (o.block_plan) o.block_plan += cl.pslot_lo; }
-        if (pass_uses_trie(p, cl, out, f64)) {
-            const hap_problem::Trie &tr = cl.trie;
-            // 64 registers per thread in both shapes (measured: more warps per SM beat more registers per thread)
-            const int tv = tr.threads > 512 ? 0 : 1;
-            if (search && f64) return fail(p, HAP_E_STATE, "the fp64 search reduces a cost array");
-            const bool counting = (p->opts.flags & HAP_OPT_COUNT_SPLITS) && !f64 && !search;
-            const void *tfn = f64 ? (tv == 0 ? (const void *)trie_dp_kernel<false, 1024, 1, double> : (const void *)trie_dp_kernel<false, 512, 2, double>)
-                            : search ? (tv == 0 ? (const void *)trie_dp_kernel<true, 1024, 1> : (const void *)trie_dp_kernel<true, 512, 2>)
-                            : counting ? (tv == 0 ? (const void *)trie_dp_kernel<false, 1024, 1, i64, true> : (const void *)trie_dp_kernel<false, 512, 2, i64, true>)
-                                       : (tv == 0 ? (const void *)trie_dp_kernel<false, 1024, 1> : (const void *)trie_dp_kernel<false, 512, 2>);
-            static size_t trie_limit[64][8];
-            const int vi = (f64 ? 4 : search ? 2 : counting ? 6 : 0) + tv;
-            if (tr.smem > trie_limit[dev][vi]) {
-                CUDA_TRY(p, cudaFuncSetAttribute(tfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tr.smem));
-                trie_limit[dev][vi] = tr.smem;
-            }
-            CUDA_TRY(p, cudaStreamWaitEvent(cl.stream, p->ev_fork, 0));
-            if (!decoded_all) {                     // not queued beside the layer costs by this pass
-                hap_status sd = launch_class_decode(p, cl);
-                cl.tab_valid = true;
-                if (sd != HAP_OK) return sd;
-            }
-            int n_parts = (int)tr.parts.size();
-            unsigned n_active = tr.n_conf * (unsigned)n_parts;
-            const u32 *plist = tr.d_plist;
-            const TrieMeta *metas = tr.d_metas;
-            void *c2v = f64 ? (void *)p->d_c2f : (void *)p->d_c2, *coefv = f64 ? (void *)p->d_coeff : (void *)p->d_coef;
-            void *targs[] = {(void *)&p->dc, (void *)&plist, (void *)&n_active, (void *)&c2v, (void *)&p->d_coef, (void *)&coefv, (void *)&metas, (void *)&n_parts, (void *)&o};
-            const unsigned tblocks = search ? (unsigned)cl.pslot_n : n_active;             // search: every partial slot of the class is written
-            CUDA_TRY(p, cudaLaunchKernel(tfn, dim3(tblocks), dim3(tr.threads), targs, tr.smem, cl.stream));
-            CUDA_TRY(p, cudaEventRecord(cl.done, cl.stream));
-            CUDA_TRY(p, cudaStreamWaitEvent(st, cl.done, 0));
-            continue;
-        }
+        if (search) { o.partial_cost += kTreeSlots + cl.item_lo; o.partial_index += kTreeSlots + cl.item_lo; }
         const WorkItem *its = p->d_items + cl.item_lo;
         int nw = cl.warps;
         unsigned used = cl.masks_used;
@@ -1735,9 +1470,7 @@ static hap_status launch_dp(hap_problem *p, const DpOut &out, bool search, cudaS
         void *cvarg = f64 ? (void *)p->d_coeff : (void *)p->d_coef;
         void *args[] = {(void *)&p->dc, (void *)&its, (void *)&c2arg, (void *)&p->d_coef, (void *)&cvarg, (void *)&tab, (void *)&o, (void *)&nw, (void *)&used};
         CUDA_TRY(p, cudaStreamWaitEvent(cl.stream, p->ev_fork, 0));
-        if (cl.has_tab && (out.count > 1 || !cl.tab_valid)) {        // (a single candidate reuses a table that some pass has filled)
-            // candidate decode (stage masks and link classes of every mapping of the class) is part of every pass,
-            // not a cached result of hap_enumerate; the one-candidate re-evaluation of a winner reuses the table
+        if (cl.has_tab && !cl.tab_valid) {        // stage masks and link classes of every mapping of the class
             const WorkItem &rep = p->items[cl.item_lo];
             const u64 nmap = p->pconfs[rep.p].nmap;
             maptab_kernel<<<(unsigned)((nmap + 3) / 4), 128, 0, cl.stream>>>(p->dc, rep.p, nmap, p->d_maptab + cl.map_base);
@@ -1745,14 +1478,51 @@ static hap_status launch_dp(hap_problem *p, const DpOut &out, bool search, cudaS
             cl.tab_valid = true;
         }
         CUDA_TRY(p, cudaLaunchKernel(fn, dim3(blocks), dim3(cl.warps * 32), args, cl.smem, cl.stream));
-        if (search && cl.pslot_n > blocks) {       // slots that only the class's tree kernel would write
-            const unsigned extra = (unsigned)(cl.pslot_n - blocks);
-            fill_partials_kernel<<<(extra + 255) / 256, 256, 0, cl.stream>>>(o.partial_cost + blocks, o.partial_index + blocks, extra);
-            CUDA_TRY(p, cudaGetLastError());
-        }
         CUDA_TRY(p, cudaEventRecord(cl.done, cl.stream));
         CUDA_TRY(p, cudaStreamWaitEvent(st, cl.done, 0));      // join
     }
+    return HAP_OK;
+}
+
+static hap_status ensure_f64_buffers(hap_problem *p, bool layer_costs)
+{
+    const size_t np = p->pconfs.size();
+    if (layer_costs && !p->d_c2f) CUDA_TRY(p, cached_malloc(p->device, (void **)&p->d_c2f, np * p->T * p->model.N * 2 * sizeof(double)));
+    if (!p->d_coeff) CUDA_TRY(p, cached_malloc(p->device, (void **)&p->d_coeff, np * p->T * HAP_NCOEF * sizeof(double)));
+    return HAP_OK;
+}
+
+// The recurrence of a pass: trees, the general kernel, or both.
+static hap_status run_pass(hap_problem *p, DpOut &out, bool f64, cudaStream_t st)
+{
+    hap_status s;
+    const bool trees = pass_uses_trees(p, out), general = !trees || !p->all_trees;
+    if (general && (s = ensure_general(p)) != HAP_OK) return s;
+    if (f64 && (s = ensure_f64_buffers(p, general || (p->opts.flags & HAP_OPT_NO_FUSE))) != HAP_OK) return s;
+    if (trees && (p->opts.flags & HAP_OPT_NO_FUSE) && !f64 && (s = ensure_general(p)) != HAP_OK) return s;
+    out.range_flag = p->d_range;
+    if (trees && !general) {
+        if ((s = launch_trees(p, out, false, f64, st, false)) != HAP_OK) return s;
+        p->timed = 2;
+        return HAP_OK;
+    }
+    out.counters = p->d_counters;
+    CUDA_TRY(p, cudaMemsetAsync(p->d_counters, 0, 8 * sizeof(u64), st));
+    CUDA_TRY(p, cudaEventRecord(p->ev[0], st));
+    if (!trees) {
+        unsigned p_lo, p_hi;
+        configs_of_range(p, out.first, out.count, p_lo, p_hi);
+        // the memory model stays on the integer byte coefficients in fp64 mode; times stay unrounded
+        if (f64) {
+            if ((s = launch_type_consts(p, p->d_coef, p->d_coeff, st, p_lo, p_hi)) != HAP_OK) return s;
+            if ((s = launch_layer_kernel(p, nullptr, p->d_c2f, false, st, nullptr, nullptr, p_lo, p_hi - p_lo, true)) != HAP_OK) return s;
+        } else if ((s = launch_layer_costs(p, p->d_c2, p->d_coef, nullptr, nullptr, true, st, nullptr, p_lo, p_hi)) != HAP_OK) return s;
+    }
+    CUDA_TRY(p, cudaEventRecord(p->ev[1], st));
+    if (trees && (s = launch_trees(p, out, false, f64, st, false)) != HAP_OK) return s;
+    if ((s = launch_dp(p, out, false, st, f64, trees)) != HAP_OK) return s;
+    CUDA_TRY(p, cudaEventRecord(p->ev[2], st));
+    p->timed = 1;
     return HAP_OK;
 }
 
@@ -1760,80 +1530,91 @@ extern "C" hap_status hap_pipeline_dp(hap_problem *p, uint64_t first, uint64_t c
                                       int64_t *dev_bottleneck, uint8_t *dev_partition, uint8_t *dev_recompute,
                                       int64_t *dev_dp_table, uint8_t *dev_choice, void *stream)
 {
-    hap_status s = enter(p);
+    cudaStream_t st = (cudaStream_t)stream;
+    hap_status s = enter(p, st);
     if (s != HAP_OK) return s;
     if ((s = check_range(p, first, count)) != HAP_OK) return s;
     if (count == 0) return HAP_OK;
-    cudaStream_t st = (cudaStream_t)stream;
-    CUDA_TRY(p, cudaMemsetAsync(p->d_counters, 0, 8 * sizeof(u64), st));
-    CUDA_TRY(p, cudaEventRecord(p->ev[0], st));
     DpOut out{};
-    out.counters = p->d_counters;
     out.cost = (i64 *)dev_cost; out.bottleneck = (i64 *)dev_bottleneck; out.partition = dev_partition;
     out.recompute = dev_recompute; out.dp_table = (i64 *)dev_dp_table; out.choice = dev_choice;
     out.first = first; out.count = count;
-    const bool fused = pass_fuses_layer_costs(p, out, false);
-    out.tcg = fused ? p->d_tc : nullptr; out.range_flag = p->d_range;
-    CUDA_TRY(p, cudaEventRecord(p->ev_pre, st));
-    unsigned p_lo, p_hi;
-    configs_of_range(p, first, count, p_lo, p_hi);
-    if ((s = launch_layer_costs(p, fused ? nullptr : p->d_c2, p->d_coef, nullptr, nullptr, true, st, nullptr, p_lo, p_hi)) != HAP_OK) return s;
-    CUDA_TRY(p, cudaEventRecord(p->ev[1], st));
-    if ((s = launch_decode_early(p, out, false)) != HAP_OK) return s;
-    if ((s = launch_dp(p, out, false, st)) != HAP_OK) return s;
-    CUDA_TRY(p, cudaEventRecord(p->ev[2], st));
-    p->timed = true;
-    return HAP_OK;
-}
-
-static hap_status ensure_f64_buffers(hap_problem *p)
-{
-    const size_t np = p->pconfs.size();
-    if (!p->d_c2f) CUDA_TRY(p, cached_malloc(p->device, (void **)&p->d_c2f, np * p->T * p->model.N * 2 * sizeof(double)));
-    if (!p->d_coeff) CUDA_TRY(p, cached_malloc(p->device, (void **)&p->d_coeff, np * p->T * HAP_NCOEF * sizeof(double)));
-    return HAP_OK;
+    if ((s = run_pass(p, out, false, st)) != HAP_OK) return s;
+    return leave_async(p, st);
 }
 
 extern "C" hap_status hap_pipeline_dp_f64(hap_problem *p, uint64_t first, uint64_t count, double *dev_cost,
                                           double *dev_bottleneck, uint8_t *dev_partition, uint8_t *dev_recompute,
                                           void *stream)
 {
-    hap_status s = enter(p);
+    cudaStream_t st = (cudaStream_t)stream;
+    hap_status s = enter(p, st);
     if (s != HAP_OK) return s;
     if ((s = check_range(p, first, count)) != HAP_OK) return s;
     if (count == 0) return HAP_OK;
     if (p->opts.flags & (HAP_OPT_REFINE | HAP_OPT_EXACT)) return fail(p, HAP_E_INVALID, "the refinement passes exist in integer mode only");
-    if ((s = ensure_f64_buffers(p)) != HAP_OK) return s;
-    cudaStream_t st = (cudaStream_t)stream;
-    CUDA_TRY(p, cudaMemsetAsync(p->d_counters, 0, 8 * sizeof(u64), st));
-    CUDA_TRY(p, cudaEventRecord(p->ev[0], st));
-    // the memory model stays on the integer byte coefficients; times stay unrounded
     DpOut out{};
-    out.counters = p->d_counters;
     out.cost = (i64 *)dev_cost; out.bottleneck = (i64 *)dev_bottleneck; out.partition = dev_partition;
     out.recompute = dev_recompute; out.first = first; out.count = count;
-    const bool fused = pass_fuses_layer_costs(p, out, false);
-    out.tcg = fused ? p->d_tc : nullptr; out.range_flag = p->d_range;
-    unsigned p_lo, p_hi;
-    configs_of_range(p, first, count, p_lo, p_hi);
-    if ((s = launch_layer_costs(p, nullptr, p->d_coef, nullptr, nullptr, true, st, nullptr, p_lo, p_hi)) != HAP_OK) return s;
-    if ((s = launch_layer_costs(p, nullptr, nullptr, fused ? nullptr : p->d_c2f, p->d_coeff, false, st, nullptr, p_lo, p_hi)) != HAP_OK) return s;
-    CUDA_TRY(p, cudaEventRecord(p->ev[1], st));
-    if ((s = launch_dp(p, out, false, st, true)) != HAP_OK) return s;
-    CUDA_TRY(p, cudaEventRecord(p->ev[2], st));
-    p->timed = true;
+    if ((s = run_pass(p, out, true, st)) != HAP_OK) return s;
+    return leave_async(p, st);
+}
+
+// The plan a tree search's last block left, with the configuration's degrees
+static void plan_of_result(const hap_problem *p, const TreeResult &r, hap_plan *host_out)
+{
+    const hap_pconf &pc = p->pconfs[r.pconf];
+    host_out->index = r.index;
+    host_out->PP = pc.PP; host_out->TP = pc.TP; host_out->CP = pc.CP; host_out->DP = pc.DP; host_out->EP = pc.EP;
+    host_out->TPE = pc.TPE; host_out->b = pc.b; host_out->M = pc.M; host_out->rc_mask = r.rc_mask;
+    std::memcpy(host_out->n, r.n, HAP_MAX_PP);
+    std::memcpy(host_out->r, r.r, HAP_MAX_PP);
+    std::memcpy(host_out->mask, r.mask, HAP_MAX_PP);
+}
+
+// Runs a search over the trees (every class has one) and waits for its result.
+static hap_status tree_search(hap_problem *p, uint64_t first, uint64_t count, bool f64, cudaStream_t st, TreeResult &res)
+{
+    hap_status s;
+    if (f64 && (s = ensure_f64_buffers(p, (p->opts.flags & HAP_OPT_NO_FUSE) != 0)) != HAP_OK) return s;
+    if ((p->opts.flags & HAP_OPT_NO_FUSE) && !f64 && (s = ensure_general(p)) != HAP_OK) return s;
+    if (!p->host_result) p->host_result = result_slot_get();
+    DpOut out{};
+    out.first = first; out.count = count; out.prune = f64 ? 0 : p->opts.prune;
+    if ((s = launch_trees(p, out, true, f64, st, true)) != HAP_OK) return s;
+    p->timed = 2;
+    if (!p->host_result) CUDA_TRY(p, cudaMemcpyAsync(&res, p->targs.res_dev, sizeof(res), cudaMemcpyDeviceToHost, st));
+    if ((s = leave_synced(p, st)) != HAP_OK) return s;
+    if (p->host_result) std::memcpy(&res, p->host_result, sizeof(res));
     return HAP_OK;
 }
 
 extern "C" hap_status hap_search_range_f64(hap_problem *p, uint64_t first, uint64_t count, hap_plan *host_out,
                                            double *host_T_iter, double *host_bottleneck, void *stream)
 {
-    hap_status s = enter(p);
+    cudaStream_t st = (cudaStream_t)stream;
+    hap_status s = enter(p, st);
     if (s != HAP_OK) return s;
     if (!host_out) return HAP_E_INVALID;
     if ((s = check_range(p, first, count)) != HAP_OK) return s;
     if (count == 0) return fail(p, HAP_E_RANGE, "empty candidate range");
-    cudaStream_t st = (cudaStream_t)stream;
+    if (p->opts.flags & (HAP_OPT_REFINE | HAP_OPT_EXACT)) return fail(p, HAP_E_INVALID, "the refinement passes exist in integer mode only");
+    if (p->all_trees) {
+        TreeResult r;
+        if ((s = tree_search(p, first, count, true, st, r)) != HAP_OK) return s;
+        std::memset(host_out, 0, sizeof(*host_out));
+        double v[5];
+        std::memcpy(&v[0], &r.cost, 8);
+        if (!(v[0] < 1.0e300)) return fail(p, HAP_E_INFEASIBLE, "no candidate satisfies the memory constraint");
+        std::memcpy(&v[1], &r.bott, 8); std::memcpy(&v[2], &r.T_pipe, 8); std::memcpy(&v[3], &r.T_sync, 8); std::memcpy(&v[4], &r.T_opt, 8);
+        plan_of_result(p, r, host_out);
+        host_out->T_iter = (int64_t)llrint(v[0]); host_out->bottleneck = (int64_t)llrint(v[1]);
+        host_out->T_pipe = (int64_t)llrint(v[2]); host_out->T_sync = (int64_t)llrint(v[3]); host_out->T_opt = (int64_t)llrint(v[4]);
+        if (host_T_iter) *host_T_iter = v[0];
+        if (host_bottleneck) *host_bottleneck = v[1];
+        return HAP_OK;
+    }
+    if ((s = ensure_general(p)) != HAP_OK || (s = ensure_f64_buffers(p, true)) != HAP_OK) return s;
     if (!p->d_fcost) CUDA_TRY(p, cached_malloc(p->device, (void **)&p->d_fcost, (size_t)p->n_cand * sizeof(i64)));
     if ((s = hap_pipeline_dp_f64(p, first, count, (double *)p->d_fcost, nullptr, nullptr, nullptr, stream)) != HAP_OK) return s;
     // non-negative doubles order like their bit patterns read as int64 (+inf is the largest), so the integer
@@ -1861,7 +1642,7 @@ extern "C" hap_status hap_search_range_f64(hap_problem *p, uint64_t first, uint6
     CUDA_TRY(p, cudaGetLastError());
     SingleOut h1;
     CUDA_TRY(p, cudaMemcpyAsync(&h1, d1, sizeof(h1), cudaMemcpyDeviceToHost, st));
-    CUDA_TRY(p, cudaStreamSynchronize(st));
+    if ((s = leave_synced(p, st)) != HAP_OK) return s;
     const hap_candidate &hc = h1.cand;
     const hap_pconf &pc = p->pconfs[hc.pconf];
     host_out->index = win;
@@ -1947,10 +1728,10 @@ static hap_status joint_setup(hap_problem *p)
 
 extern "C" hap_status hap_joint_bottleneck(hap_problem *p, int64_t *dev_out, void *stream)
 {
-    hap_status s = enter(p);
+    hap_status s = enter(p, (cudaStream_t)stream);
     if (s != HAP_OK) return s;
     if (!dev_out) return HAP_E_INVALID;
-    if ((s = joint_setup(p)) != HAP_OK) return s;
+    if ((s = joint_setup(p)) != HAP_OK || (s = ensure_general(p)) != HAP_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
     const size_t np = p->pconfs.size();
     CUDA_TRY(p, cudaMemsetAsync(dev_out, 0xff, np * p->opts.n_rc * sizeof(int64_t), st));     // -1: stages not homogeneous
@@ -1971,34 +1752,43 @@ extern "C" hap_status hap_joint_bottleneck(hap_problem *p, int64_t *dev_out, voi
         else joint_dp_kernel<false><<<grid, 256, jh.smem, st>>>(p->dc, jh.d_ids, n_ids, p->d_c2, p->d_coef, jh.jc, p->d_joint_scratch, (i64 *)dev_out);
         CUDA_TRY(p, cudaGetLastError());
     }
-    return HAP_OK;
+    return leave_async(p, st);
 }
 
 extern "C" hap_status hap_count_cells(hap_problem *p, uint64_t first, uint64_t count, uint64_t *host_cells, void *stream)
 {
-    hap_status s = enter(p);
+    hap_status s = enter(p, (cudaStream_t)stream);
     if (s != HAP_OK) return s;
     if (!host_cells) return HAP_E_INVALID;
     if ((s = check_range(p, first, count)) != HAP_OK) return s;
     *host_cells = 0;
     if (count == 0) return HAP_OK;
     cudaStream_t st = (cudaStream_t)stream;
+    if ((s = ensure_general(p)) != HAP_OK) return s;
     CUDA_TRY(p, cudaMemsetAsync(p->d_counters, 0, 8 * sizeof(u64), st));
     if ((s = launch_layer_costs(p, p->d_c2, p->d_coef, nullptr, nullptr, true, st)) != HAP_OK) return s;
     DpOut out{};
     out.counters = p->d_counters; out.first = first; out.count = count; out.count_only = 1;
     if ((s = launch_dp(p, out, false, st)) != HAP_OK) return s;
     CUDA_TRY(p, cudaMemcpyAsync(host_cells, p->d_counters + 4, sizeof(u64), cudaMemcpyDeviceToHost, st));
-    CUDA_TRY(p, cudaStreamSynchronize(st));
+    if ((s = leave_synced(p, st)) != HAP_OK) return s;
     return check_values(p);
 }
 
 extern "C" hap_status hap_get_timings(hap_problem *p, float *ms_layer_cost, float *ms_dp, uint64_t *cells)
 {
-    hap_status s = enter(p);
-    if (s != HAP_OK) return s;
-    if (!p->timed) return fail(p, HAP_E_STATE, "no hap_pipeline_dp or hap_search_* call to report on");
-    CUDA_TRY(p, cudaEventSynchronize(p->ev[2]));
+    if (!p) return HAP_E_INVALID;
+    if (!p->enumerated || !p->timed) return fail(p, HAP_E_STATE, "no hap_pipeline_dp or hap_search_* call to report on");
+    if (cudaSetDevice(p->device) != cudaSuccess) return fail(p, HAP_E_CUDA, "cudaSetDevice");
+    if (p->in_flight) CUDA_TRY(p, cudaEventSynchronize(p->ev_done));
+    if (p->timed == 2) {
+        TreeReport ts;
+        CUDA_TRY(p, cudaMemcpy(&ts, p->targs.report, sizeof(ts), cudaMemcpyDeviceToHost));
+        if (ms_layer_cost) *ms_layer_cost = (float)((double)(ts.stamp[1] - ts.stamp[0]) * 1e-6);
+        if (ms_dp) *ms_dp = (float)((double)(ts.stamp[2] - ts.stamp[1]) * 1e-6);
+        if (cells) *cells = ts.splits;
+        return check_values(p);
+    }
     if (ms_layer_cost) CUDA_TRY(p, cudaEventElapsedTime(ms_layer_cost, p->ev[0], p->ev[1]));
     if (ms_dp) CUDA_TRY(p, cudaEventElapsedTime(ms_dp, p->ev[1], p->ev[2]));
     if (cells) CUDA_TRY(p, cudaMemcpy(cells, p->d_counters + 4, sizeof(u64), cudaMemcpyDeviceToHost));
@@ -2008,7 +1798,7 @@ extern "C" hap_status hap_get_timings(hap_problem *p, float *ms_layer_cost, floa
 extern "C" hap_status hap_eval_appendix_b(hap_problem *p, uint64_t first, uint64_t count, const uint8_t *dev_partition,
                                           const uint8_t *dev_recompute, int64_t *dev_t_iter, int64_t *dev_detail, void *stream)
 {
-    hap_status s = enter(p);
+    hap_status s = enter(p, (cudaStream_t)stream);
     if (s != HAP_OK) return s;
     if ((s = check_range(p, first, count)) != HAP_OK) return s;
     if (count == 0) return HAP_OK;
@@ -2016,28 +1806,30 @@ extern "C" hap_status hap_eval_appendix_b(hap_problem *p, uint64_t first, uint64
     const uint64_t blocks = (count + 3) / 4;
     if (blocks > 0x7fffffffull) return fail(p, HAP_E_RANGE, "count too large for one launch");
     cudaStream_t st = (cudaStream_t)stream;
+    if ((s = ensure_general(p)) != HAP_OK) return s;
     if ((s = launch_layer_costs(p, p->d_c2, p->d_coef, nullptr, nullptr, true, st)) != HAP_OK) return s;
     appendix_b_kernel<<<(unsigned)blocks, 128, 0, st>>>(p->dc, first, count, p->d_c2, p->d_coef, dev_partition, dev_recompute,
                                                         (i64 *)dev_t_iter, (i64 *)dev_detail);
     CUDA_TRY(p, cudaGetLastError());
-    return HAP_OK;
+    return leave_async(p, st);
 }
 
 extern "C" hap_status hap_simulate_1f1b(hap_problem *p, uint64_t first, uint64_t count, const uint8_t *dev_partition,
                                         const uint8_t *dev_recompute, int64_t *dev_t_iter, int64_t *dev_detail, void *stream)
 {
-    hap_status s = enter(p);
+    hap_status s = enter(p, (cudaStream_t)stream);
     if (s != HAP_OK) return s;
     if ((s = check_range(p, first, count)) != HAP_OK) return s;
     if (count == 0) return HAP_OK;
     if (!dev_partition || !dev_recompute || !dev_t_iter) return HAP_E_INVALID;
     if (count > 0x7fffffffull) return fail(p, HAP_E_RANGE, "count too large for one launch");
     cudaStream_t st = (cudaStream_t)stream;
+    if ((s = ensure_general(p)) != HAP_OK) return s;
     if ((s = launch_layer_costs(p, p->d_c2, p->d_coef, nullptr, nullptr, true, st)) != HAP_OK) return s;
     simulate_1f1b_kernel<<<(unsigned)count, 32, 0, st>>>(p->dc, first, count, p->d_c2, p->d_coef, dev_partition, dev_recompute,
                                                          (i64 *)dev_t_iter, (i64 *)dev_detail);
     CUDA_TRY(p, cudaGetLastError());
-    return HAP_OK;
+    return leave_async(p, st);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -2076,7 +1868,7 @@ extern "C" hap_status hap_problem_save(hap_problem *p, void *host_buf, uint64_t 
     // the tables live on the device only (per-layer ones interleaved entry by entry): read them back in the caller's layout
     std::vector<double> dev(4 * n5 + 2 * n4), tab[4];
     CUDA_TRY(p, uploads_done(p));
-    CUDA_TRY(p, cudaMemcpy(dev.data(), p->d_tables, dev.size() * sizeof(double), cudaMemcpyDeviceToHost));
+    CUDA_TRY(p, cudaMemcpy(dev.data(), p->dc.tab4, dev.size() * sizeof(double), cudaMemcpyDeviceToHost));
     for (int t = 0; t < 4; ++t) { tab[t].resize(n5); for (size_t i = 0; i < n5; ++i) tab[t][i] = dev[4 * i + t]; }
     std::vector<double> tpre(dev.begin() + 4 * n5, dev.begin() + 4 * n5 + n4), tpost(dev.begin() + 4 * n5 + n4, dev.end());
     std::vector<double> fsize(p->dc.fsize, p->dc.fsize + pf.n_fsize), feff;
@@ -2193,19 +1985,12 @@ extern "C" hap_status hap_launches_per_pass(hap_problem *p, uint32_t *host_count
 {
     if (!p || !host_count) return HAP_E_INVALID;
     if (!p->enumerated) return fail(p, HAP_E_STATE, "hap_enumerate has not run");
-    const bool lin = p->dc.tau_linear != 0;
-    const bool refine = (p->opts.flags & (HAP_OPT_REFINE | HAP_OPT_EXACT)) != 0;
-    uint32_t n = 2 + 2;                                     // type constants, layer costs; argmin partial and final
-    bool all_trees = p->n_gather_jobs > 0;
-    for (const auto &cl : p->classes) if (cl.trie.ok && !(lin && !refine)) all_trees = false;
-    bool fused = !(p->opts.flags & HAP_OPT_NO_FUSE) && lin && !refine && !p->classes.empty();
-    for (const auto &cl : p->classes) if (!cl.trie.ok) fused = false;
-    if (fused) n -= 1;                                      // the tree blocks compute the layer costs themselves
-    if (all_trees) n += 2;                                  // one decode and one tree-gather launch for all classes
-    for (const auto &cl : p->classes) {
-        if (cl.trie.ok && lin && !refine) n += all_trees ? 1 : 1 + (uint32_t)cl.trie.parts.size() + 1;   // (decode, gather per part,) tree DP
-        else n += (cl.has_tab ? 1 : 0) + 1;                                            // decode table, one-warp-per-candidate DP
-    }
+    DpOut out{};
+    const bool trees = pass_uses_trees(p, out);
+    uint32_t n = 1 + 2;                                     // type constants; argmin partial and final
+    if (!trees || !p->all_trees || (p->opts.flags & HAP_OPT_NO_FUSE)) n += 1;              // layer-cost array
+    if (trees) n += 1 + (uint32_t)tree_launches(p, false, false, 0, (unsigned)p->pconfs.size()).size();     // records, recurrence
+    for (const auto &cl : p->classes) if (!trees || cl.tree < 0) n += 1;                    // one warp per candidate
     *host_count = n;
     return HAP_OK;
 }
@@ -2222,45 +2007,65 @@ static hap_status argmin_launch(hap_problem *p, const i64 *dev_cost, uint64_t co
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
     const i64 *pc = p->d_pcost; const u64 *pi = p->d_pindex; const u64 nb = blocks;
-    const PlanSlot *no_plans = nullptr; i64 *no_vals = nullptr; uint8_t *no_bytes = nullptr;
-    CUDA_TRY(p, cudaLaunchKernelEx(&cfg, argmin_final_kernel, pc, pi, nb, dev_out, init, no_plans, no_vals, no_bytes, no_bytes));
+    CUDA_TRY(p, cudaLaunchKernelEx(&cfg, argmin_final_kernel, pc, pi, nb, dev_out, init));
     return HAP_OK;
 }
 
 extern "C" hap_status hap_argmin(hap_problem *p, const int64_t *dev_cost, uint64_t count, int64_t *dev_out, void *stream)
 {
-    hap_status s = enter(p);
+    hap_status s = enter(p, (cudaStream_t)stream);
     if (s != HAP_OK) return s;
     if (!dev_cost || !dev_out || count == 0) return HAP_E_INVALID;
-    return argmin_launch(p, (const i64 *)dev_cost, count, (i64 *)dev_out, (cudaStream_t)stream, kInf);
+    if ((s = argmin_launch(p, (const i64 *)dev_cost, count, (i64 *)dev_out, (cudaStream_t)stream, kInf)) != HAP_OK) return s;
+    return leave_async(p, (cudaStream_t)stream);
+}
+
+static void search_stats(const hap_problem *p, hap_search_stats *st, u64 evaluated, u64 feasible, u64 pruned, float ms_lc, float ms_dp)
+{
+    if (!st) return;
+    std::memset(st, 0, sizeof(*st));
+    st->n_pconf = p->pconfs.size(); st->n_candidates = p->n_cand;
+    st->n_evaluated = evaluated; st->n_feasible = feasible; st->n_pruned = pruned;
+    st->ms_layer_cost = ms_lc; st->ms_dp = ms_dp; st->ms_total = ms_lc + ms_dp;
 }
 
 extern "C" hap_status hap_search_range(hap_problem *p, uint64_t first, uint64_t count, hap_plan *host_out,
                                        hap_search_stats *host_stats, void *stream)
 {
-    hap_status s = enter(p);
+    cudaStream_t st = (cudaStream_t)stream;
+    hap_status s = enter(p, st);
     if (s != HAP_OK) return s;
     if (!host_out) return HAP_E_INVALID;
     if ((s = check_range(p, first, count)) != HAP_OK) return s;
     if (count == 0) return fail(p, HAP_E_RANGE, "empty candidate range");
-    cudaStream_t st = (cudaStream_t)stream;
     std::memset(host_out, 0, sizeof(*host_out));
+    const bool refine_mode = (p->opts.flags & (HAP_OPT_REFINE | HAP_OPT_EXACT)) != 0;
+    DpOut out{};
+    out.first = first; out.count = count; out.prune = p->opts.prune;
+    if (p->all_trees && pass_uses_trees(p, out)) {
+        // three launches; the last block writes the plan of the winner to the host
+        TreeResult r;
+        if ((s = tree_search(p, first, count, false, st, r)) != HAP_OK) return s;
+        search_stats(p, host_stats, count - r.n_pruned, r.n_feasible, r.n_pruned, (float)((double)(r.stamp[1] - r.stamp[0]) * 1e-6),
+                     (float)((double)(r.stamp[2] - r.stamp[1]) * 1e-6));
+        if (r.range_flag) return fail(p, HAP_E_RANGE, "a layer time or stage coefficient exceeds the supported range (see hap.h)");
+        if (r.cost >= kInf) return fail(p, HAP_E_INFEASIBLE, "no candidate satisfies the memory constraint");
+        plan_of_result(p, r, host_out);
+        host_out->T_iter = r.cost; host_out->bottleneck = r.bott; host_out->T_pipe = r.T_pipe; host_out->T_sync = r.T_sync; host_out->T_opt = r.T_opt;
+        return HAP_OK;
+    }
+    if ((s = ensure_general(p)) != HAP_OK) return s;
     const u64 init_counters[8] = {0, 0, 0, (u64)kInf, 0, 0, 0, 0};           // [3] = incumbent starts at +INF
     CUDA_TRY(p, cudaMemcpyAsync(p->d_counters, init_counters, sizeof(init_counters), cudaMemcpyHostToDevice, st));
     CUDA_TRY(p, cudaEventRecord(p->ev[0], st));
-    DpOut out{};
     out.lb_sum = p->d_lb;
-    out.first = first; out.count = count; out.prune = p->opts.prune;
     out.partial_cost = p->d_pcost; out.partial_index = p->d_pindex; out.counters = p->d_counters;
-    out.incumbent = p->d_counters + 3;
-    const bool refine_mode = (p->opts.flags & (HAP_OPT_REFINE | HAP_OPT_EXACT)) != 0;
-    const bool fused = pass_fuses_layer_costs(p, out, true);
-    out.tcg = fused ? p->d_tc : nullptr; out.range_flag = p->d_range;
-    CUDA_TRY(p, cudaEventRecord(p->ev_pre, st));
+    out.incumbent = p->d_counters + 3; out.range_flag = p->d_range;
+    const bool trees = pass_uses_trees(p, out);               // (some classes have a tree, some do not)
     unsigned p_lo, p_hi;
     configs_of_range(p, first, count, p_lo, p_hi);
     if (refine_mode && count > 1) { p_lo = 0; p_hi = ~0u; }          // (the bounds kernel below reads every configuration's S)
-    if ((s = launch_layer_costs(p, fused ? nullptr : p->d_c2, p->d_coef, nullptr, nullptr, true, st, fused ? nullptr : p->d_lb, p_lo, p_hi)) != HAP_OK) return s;
+    if (!trees && (s = launch_layer_costs(p, p->d_c2, p->d_coef, nullptr, nullptr, true, st, p->d_lb, p_lo, p_hi)) != HAP_OK) return s;
     CUDA_TRY(p, cudaEventRecord(p->ev[1], st));
     if (refine_mode && count > 1) {
         // The refinement and the exact sweep cost one warp per candidate and up to dozens of passes each, so they run
@@ -2273,8 +2078,9 @@ extern "C" hap_status hap_search_range(hap_problem *p, uint64_t first, uint64_t 
         DpOut plain{};
         plain.bottleneck = p->d_cand_lb + first;         // the kernels index outputs by candidate - first: entry c of the array
         plain.first = first; plain.count = count; plain.force_plain = 1; plain.range_flag = p->d_range;
-        if ((s = launch_decode_early(p, plain, false)) != HAP_OK) return s;
-        if ((s = launch_dp(p, plain, false, st)) != HAP_OK) return s;
+        const bool plain_trees = pass_uses_trees(p, plain);
+        if (plain_trees && (s = launch_trees(p, plain, false, false, st, false)) != HAP_OK) return s;
+        if ((!plain_trees || !p->all_trees) && (s = launch_dp(p, plain, false, st, false, plain_trees)) != HAP_OK) return s;
         cand_bound_kernel<<<(unsigned)p->pconfs.size(), 128, 0, st>>>(p->dc, p->d_lb, p->d_cand_lb, first, count);
         CUDA_TRY(p, cudaGetLastError());
         if ((s = argmin_launch(p, p->d_cand_lb + first, count, p->d_best, st, kInf)) != HAP_OK) return s;
@@ -2287,57 +2093,42 @@ extern "C" hap_status hap_search_range(hap_problem *p, uint64_t first, uint64_t 
         CUDA_TRY(p, cudaGetLastError());
         out.cand_lb = p->d_cand_lb;
     }
-    // When every class of the search walks its prefix tree, each block also leaves the plan of its best candidate
-    // (partition, levels, the terms of Eq. 4) and the final reduction copies the winner's: nothing is evaluated twice.
-    bool plans = count > 1;
-    for (const auto &cl : p->classes) plans = plans && pass_uses_trie(p, cl, out, false);
-    SingleOut *d1 = (SingleOut *)p->d_single;
-    if (plans) {
-        if (!p->d_plans) CUDA_TRY(p, cached_malloc(p->device, (void **)&p->d_plans, p->n_pslots * sizeof(PlanSlot)));
-        out.block_plan = p->d_plans;
+    if (trees) {
+        const unsigned slots = kTreeSlots + (unsigned)p->items.size();      // (the tree kernel's idle slots and the items it takes over)
+        fill_partials_kernel<<<(slots + 255) / 256, 256, 0, st>>>(p->d_pcost, p->d_pindex, slots);
+        CUDA_TRY(p, cudaGetLastError());
+        if ((s = launch_trees(p, out, true, false, st, false)) != HAP_OK) return s;
     }
-    if ((s = launch_decode_early(p, out, true)) != HAP_OK) return s;
-    if ((s = launch_dp(p, out, true, st)) != HAP_OK) return s;
-    static_assert(offsetof(SingleOut, bott) == 8 && offsetof(SingleOut, detail) == 16, "the final reduction writes cost, bottleneck and the three terms in a row");
-    if (plans) argmin_final_kernel<<<1, 256, 0, st>>>(p->d_pcost, p->d_pindex, p->n_pslots, p->d_best, kInf, p->d_plans, &d1->cost, d1->part, d1->rec);
-    else argmin_final_kernel<<<1, 256, 0, st>>>(p->d_pcost, p->d_pindex, p->n_pslots, p->d_best, kInf);
+    if ((s = launch_dp(p, out, true, st, false, trees)) != HAP_OK) return s;
+    const size_t slot0 = trees ? 0 : kTreeSlots;
+    argmin_final_kernel<<<1, 256, 0, st>>>(p->d_pcost + slot0, p->d_pindex + slot0, kTreeSlots + p->items.size() - slot0, p->d_best, kInf);
     CUDA_TRY(p, cudaGetLastError());
     CUDA_TRY(p, cudaEventRecord(p->ev[2], st));
-    p->timed = true;
-    if (!plans) {
-        // the winner is evaluated once more alone, for its partition and recomputation levels; its index stays on the
-        // device (every class's kernel looks whether the index is its own), so the host waits only once
-        DpOut one{};
-        one.cost = &d1->cost; one.bottleneck = &d1->bott; one.detail = d1->detail; one.partition = d1->part;
-        one.recompute = d1->rec; one.first = 0; one.count = 1; one.first_dev = p->d_best + 1;
-        if (fused && (s = launch_layer_kernel(p, p->d_c2, nullptr, true, st, nullptr, p->d_best + 1, 0, 1, false)) != HAP_OK) return s;
-        if ((s = launch_dp(p, one, false, st)) != HAP_OK) return s;
-    }
+    p->timed = 1;
+    // the winner is evaluated once more alone, for its partition and recomputation levels; its index stays on the device
+    // (every class's kernel looks whether the index is its own), so the host waits only once
+    SingleOut *d1 = (SingleOut *)p->d_single;
+    DpOut one{};
+    one.cost = &d1->cost; one.bottleneck = &d1->bott; one.detail = d1->detail; one.partition = d1->part;
+    one.recompute = d1->rec; one.first = 0; one.count = 1; one.first_dev = p->d_best + 1;
+    if ((s = launch_dp(p, one, false, st)) != HAP_OK) return s;
     decode_kernel<<<1, 32, 0, st>>>(p->dc, 0, 1, &d1->cand, p->d_best + 1);
     CUDA_TRY(p, cudaGetLastError());
-    // range flag, counters, minimum and the re-evaluated winner sit in consecutive 256-byte slots at the end of the
-    // arena: one copy brings all four back
-    alignas(16) unsigned char tail[3 * 256 + sizeof(SingleOut)];
-    if ((unsigned char *)p->d_counters - (unsigned char *)p->d_range != 256 || (unsigned char *)p->d_best - (unsigned char *)p->d_range != 512 ||
-        (unsigned char *)p->d_single - (unsigned char *)p->d_range != 768)
-        return fail(p, HAP_E_STATE, "result slots are not adjacent");
-    CUDA_TRY(p, cudaMemcpyAsync(tail, p->d_range, sizeof(tail), cudaMemcpyDeviceToHost, st));
-    CUDA_TRY(p, cudaStreamSynchronize(st));
     i64 best[2];
     u64 counters[4], flag = 0;
     SingleOut h1;
-    std::memcpy(&flag, tail, sizeof(flag));
-    std::memcpy(counters, tail + 256, sizeof(counters));
-    std::memcpy(best, tail + 512, sizeof(best));
-    std::memcpy(&h1, tail + 768, sizeof(h1));
-    if (host_stats) {
-        std::memset(host_stats, 0, sizeof(*host_stats));
-        host_stats->n_pconf = p->pconfs.size(); host_stats->n_candidates = p->n_cand;
-        host_stats->n_evaluated = counters[0]; host_stats->n_feasible = counters[1]; host_stats->n_pruned = counters[2];
-        cudaEventElapsedTime(&host_stats->ms_layer_cost, p->ev[0], p->ev[1]);
-        cudaEventElapsedTime(&host_stats->ms_dp, p->ev[1], p->ev[2]);
-        host_stats->ms_total = host_stats->ms_layer_cost + host_stats->ms_dp;
-    }
+    TreeReport ts{};
+    CUDA_TRY(p, cudaMemcpyAsync(&flag, p->d_range, sizeof(flag), cudaMemcpyDeviceToHost, st));
+    CUDA_TRY(p, cudaMemcpyAsync(counters, p->d_counters, sizeof(counters), cudaMemcpyDeviceToHost, st));
+    CUDA_TRY(p, cudaMemcpyAsync(best, p->d_best, sizeof(best), cudaMemcpyDeviceToHost, st));
+    CUDA_TRY(p, cudaMemcpyAsync(&h1, d1, sizeof(h1), cudaMemcpyDeviceToHost, st));
+    if (trees) CUDA_TRY(p, cudaMemcpyAsync(&ts, p->targs.report, sizeof(ts), cudaMemcpyDeviceToHost, st));
+    if ((s = leave_synced(p, st)) != HAP_OK) return s;
+    float ms_lc = 0.0f, ms_dp = 0.0f;
+    cudaEventElapsedTime(&ms_lc, p->ev[0], p->ev[1]);
+    cudaEventElapsedTime(&ms_dp, p->ev[1], p->ev[2]);
+    const u64 pruned = counters[2] + ts.n_pruned;
+    search_stats(p, host_stats, count - pruned, counters[1] + ts.n_feasible, pruned, ms_lc, ms_dp);
     if (flag) return fail(p, HAP_E_RANGE, "a layer time or stage coefficient exceeds the supported range (see hap.h)");
     if (best[0] >= kInf) return fail(p, HAP_E_INFEASIBLE, "no candidate satisfies the memory constraint");
     const u64 win = (u64)best[1];

@@ -4,12 +4,12 @@
 //   type_const_kernel   per (configuration, type): constants of Eq. 2 / Eq. 3 and the 21 stage
 //                       coefficients, fp64 with one IEEE operation per operator (the translation
 //                       unit is compiled with --fmad=false), three independent roles per pair.
+//                       Ahead of a pass over the prefix trees it also lists the configurations that can be feasible.
 //   layer_cost_kernel   per (configuration, type, layer): Eq. 2 with imbalance scaling, rounding,
 //                       one block per configuration, one thread per layer.
 //   decode_kernel       candidate index -> stage type masks and boundary link classes;
-//   maptab_kernel       the same for every mapping of one PP class; maptab_all_kernel for all classes in one
-//                       launch (every pass).
-//   trie_dp_kernel      (hap_trie.cuh) the default dynamic program: all mappings of a configuration
+//   maptab_kernel       the same for every mapping of one PP class.
+//   tree_*_kernel       (hap_tree.cuh) the default dynamic program: all mappings of a configuration
 //                       together through the prefix tree of their stage sequences.
 //   pipeline_dp_kernel  the general form (DP tables on request, refinement / exact modes, classes
 //                       without a tree): one warp per candidate, stage rows and memory-threshold tables in shared
@@ -33,6 +33,9 @@ namespace hap {
 typedef long long i64;
 typedef unsigned long long u64;
 typedef unsigned int u32;
+
+struct TreeState;                     // counters of a pass over the prefix trees (hap_tree.cuh)
+struct TreeReport;
 
 // Self-checking build (-DHAP_CHECKED): what a memory checker would do from outside, done by the kernels themselves.
 // Indices and shared-memory addresses that a kernel forms from tables (tree records, row origins, threshold
@@ -89,13 +92,11 @@ struct WorkItem {
     u64 lo;
 };
 
-// What a block of a search leaves beside its (cost, index) minimum when it can: the plan of that candidate.
+// What a block of a tree search leaves beside its (cost, index) minimum: the plan of that candidate.
 struct __align__(16) PlanSlot {
     i64 bott, T_pipe, T_sync, T_opt;
     uint8_t n[HAP_MAX_PP], r[HAP_MAX_PP];     // layers and recomputation level of stages 1..PP (the rest is not written)
-    int PP, pad[3];
 };
-static_assert(HAP_MAX_PP == 32 && sizeof(PlanSlot) % 16 == 0, "the plan bytes move as 16-byte pieces");
 
 struct DpOut {
     i64 *cost, *bottleneck;
@@ -114,15 +115,11 @@ struct DpOut {
     int prune;                        // search mode: skip blocks whose lower bound exceeds the incumbent
     int exact;                        // refinement kernels: sweep the stage-cost limit for the optimum of sum + (M-1) max
     int count_only;                   // instrumentation: count the finite-cost cells of each candidate, run no recurrence
-    // layer costs computed by the DP blocks themselves (prefix-tree kernel): per (configuration, type) constants of
-    // Eq. 2; null: the blocks read the layer-cost array.  range_flag: set when a layer time leaves the supported range
-    const struct TypeConst *tcg;
-    u64 *range_flag;
+    u64 *range_flag;                  // set when a layer time leaves the supported range
     // search with the refinement / exact objective: per-candidate lower bounds on T_iter from a preceding plain pass,
     // indexed by the global candidate index (HAP_INF: the candidate has no feasible partition); a candidate whose
     // bound exceeds the incumbent is skipped
     const i64 *cand_lb;
-    PlanSlot *block_plan;             // search over the prefix trees: per block the plan of its best candidate (nullable)
     int force_plain;                  // run the plain min-max pass although the problem asks for a refinement mode
 };
 
@@ -235,7 +232,21 @@ __device__ __forceinline__ void store_pair(i64 *qi, double *qd, size_t at, doubl
     }
 }
 
-constexpr int kLcThreads = 128;
+constexpr int kTcThreads = 96;                        // a warp per role
+
+// What a pass over the prefix trees wants from its first kernel besides the constants: per class that walks a tree the list
+// of its configurations whose first stage fits some device at some level (the others go to a list of their own).
+struct LiveArgs {
+    TreeState *state;                 // null: nothing is wanted
+    TreeReport *report;               // takes the time the pass begins
+    u32 *live_list;                   // [n_pconf] class c's from entry p_lo[c] on
+    u32 *dead_list;                   // [n_pconf]
+    u64 *hist;                        // [n_hist] counters to clear
+    u32 n_hist;
+    int n_cls;
+    u32 p_lo[HAP_MAX_PP + 1], p_hi[HAP_MAX_PP + 1];
+    u32 first_min[HAP_MAX_PP + 1];    // shortest first stage by capacity type, a byte each (255: no first stage on it)
+};
 
 // Eq. 2 for one (configuration, device type, layer): forward and backward time of the layer from its table entries
 // ta = (t_dense fwd, bwd), tf = (t_ffn fwd, bwd) and the per-(configuration, type) constants tc (a TypeConst read as
@@ -271,34 +282,80 @@ __device__ __forceinline__ double div_by(double a, double b, double y)
 
 // Phase 1 (type_const_kernel): per (configuration, type) the constants of Eq. 2 / Eq. 3 (into a scratch array)
 // and the 21 stage coefficients.  The work of one (configuration, type) is a chain of about 40 fp64 divisions,
-// so it is cut into three independent roles (blockIdx.y: layer constants; p2p / activation / extra-memory
-// coefficients; weight / sync / optimizer coefficients), one thread per (configuration, type) and role.
+// so it is cut into three independent roles (layer constants; p2p / activation / extra-memory coefficients; weight /
+// sync / optimizer coefficients), one thread per (configuration, type) and one warp per role; the roles of the same
+// configurations share a block, which can then say at once which of them cannot place a first stage.
 // Phase 2 (layer_cost_kernel): one block per configuration, one thread per layer.
-template <bool QUANT>
 __device__ __forceinline__ bool put_coef(i64 *coef, double *coeff, size_t at, int q, double v)
 {
-    if (QUANT) coef[at + q] = __double2ll_rn(v);
-    else coeff[at + q] = v;
+    if (coef) coef[at + q] = __double2ll_rn(v);
+    if (coeff) coeff[at + q] = v;
     // time coefficients must stay below 2^40 ns (per-layer ones below 2^36), bytes below 2^50
     const double lim = (q <= HAP_SLAT || q == HAP_KXD) ? 1.0995e12 : (q < HAP_MW ? 6.8719e10 : 1.1259e15);
     return !(v < lim);
 }
 
-template <bool QUANT>
-__global__ void __launch_bounds__(kLcThreads)
-type_const_kernel(const DevConst dc, TypeConst *tcg, i64 *coef, double *coeff, u64 *range_flag, unsigned p_first, unsigned n_conf)
+__device__ void tree_stamp_begin(TreeReport *report);
+__device__ u32 *tree_state_live(TreeState *state);
+
+// Configurations whose first stage fits no device type at any level: nothing is feasible.  Decided from the byte
+// coefficients: the memory of a span is its numbers of dense and MoE layers times the per-kind bytes, and a shorter span
+// needs no more, so the shortest first stage of each capacity type decides.
+__device__ __forceinline__ bool first_stage_fits(const DevConst &dc, const hap_pconf &pc, const i64 *cfp, int t, int b, unsigned levels)
 {
-    // the layer-cost kernel behind this one may start its table reads now (programmatic dependent launch)
+    if (b == 255) return false;
+    const i64 extra = cfp[HAP_MPRE] + (pc.PP == 1 ? cfp[HAP_MPOST] : 0), mx = cfp[HAP_MX];
+    const i64 mstore = pc.M < pc.PP ? pc.M : pc.PP;
+    const i64 nm = moe_before(dc, b), nd = (i64)b - nm;
+    const i64 Wb = nd * cfp[HAP_MW] + nm * cfp[HAP_MW + 1] + extra + (nm ? mx : 0);
+    const i64 A = mstore * (nd * cfp[HAP_MA] + nm * cfp[HAP_MA + 1]);
+    bool fits = false;
+    for (int r = 0; r < dc.R; ++r) fits |= ((levels >> r) & 1u) && Wb + (((i64)dc.xi_q[r] * A) >> 10) <= dc.cap_eff[t];
+    return fits;
+}
+
+__device__ __forceinline__ void type_const_role(const DevConst &dc, TypeConst *tcg, i64 *coef, double *coeff, u64 *range_flag, u64 p, int h, int role);
+
+// coef / coeff: integer and / or fp64 form of the coefficients (nullable)
+__global__ void __launch_bounds__(kTcThreads)
+type_const_kernel(const DevConst dc, TypeConst *tcg, i64 *coef, double *coeff, u64 *range_flag, unsigned p_first, unsigned n_conf, const LiveArgs la)
+{
+    // the kernel behind this one may start what does not depend on the constants now (programmatic dependent launch)
     asm volatile("griddepcontrol.launch_dependents;");
+    const int role = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int per = 32 / dc.T, ql = lane / dc.T, h = lane - ql * dc.T;          // configurations of the block; this lane's
+    const unsigned pi = blockIdx.x * per + ql;
+    const u64 p = (u64)p_first + pi;                          // configurations [p_first, p_first + n_conf)
+    const bool on = ql < per && pi < n_conf && p < dc.n_pconf;
+    if (on) type_const_role(dc, tcg, coef, coeff, range_flag, p, h, role);
+    if (!la.state) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) tree_stamp_begin(la.report);
+    for (u32 b = blockIdx.x * kTcThreads + threadIdx.x; b < la.n_hist; b += gridDim.x * kTcThreads) la.hist[b] = 0;
+    __syncthreads();                                          // (the byte coefficients come from two roles)
+    if (role != 0) return;
+    // one lane per (configuration, capacity type); the first of a configuration's lanes puts it on its list
+    unsigned levels = 0;
+    for (int r = 0; r < dc.n_rc; ++r) levels |= dc.rc_masks[r];
+    int ci = 0;
+    while (ci < la.n_cls && !(p >= la.p_lo[ci] && p < la.p_hi[ci])) ++ci;
+    int fits = 0;
+    if (on && ci < la.n_cls)
+        fits = first_stage_fits(dc, dc.pconf[p], coef + (size_t)p * dc.T * HAP_NCOEF, h, (int)((la.first_min[ci] >> (8 * h)) & 255u), levels);
+    const bool live = ((__ballot_sync(0xffffffffu, fits) >> (ql * dc.T)) & ((1u << dc.T) - 1u)) != 0;
+    const bool listed = on && h == 0 && ci < la.n_cls;
+    const int list = !listed ? -1 : live ? ci : la.n_cls;
+    const unsigned same = __match_any_sync(0xffffffffu, list);
+    u32 at = 0;
+    if (listed && lane == __ffs(same) - 1) at = atomicAdd(tree_state_live(la.state) + list, (u32)__popc(same));
+    at = __shfl_sync(0xffffffffu, at, __ffs(same) - 1);
+    if (listed) (live ? la.live_list + la.p_lo[ci] : la.dead_list)[at + __popc(same & ((1u << lane) - 1u))] = (u32)p;
+}
+
+__device__ __forceinline__ void type_const_role(const DevConst &dc, TypeConst *tcg, i64 *coef, double *coeff, u64 *range_flag, u64 p, int h, int role)
+{
     const int T = dc.T;
-    const int role = blockIdx.y;
     const i64 H = dc.H;
-    const u64 gid = (u64)blockIdx.x * kLcThreads + threadIdx.x;
-    const u64 p = (u64)p_first + gid / HAP_MAX_TYPES;          // configurations [p_first, p_first + n_conf)
-    const int h = (int)(gid % HAP_MAX_TYPES);
-    if (gid / HAP_MAX_TYPES >= n_conf || p >= dc.n_pconf || h >= T) return;
-    const bool want_coef = (QUANT && coef) || (!QUANT && coeff);
-    if (role != 0 && !want_coef) return;
+    if (role != 0 && !coef && !coeff) return;
     const hap_pconf pc = dc.pconf[p];
     const int TP = pc.TP, CP = pc.CP, DP = pc.DP, EP = pc.EP, TPE = pc.TPE, EDP = pc.EDP, b = pc.b;
     const i64 G = pc.G;
@@ -341,27 +398,27 @@ type_const_kernel(const DevConst dc, TypeConst *tcg, i64 *coef, double *coeff, u
         tcg[p * T + h] = tc;
     } else if (role == 1) {
         const size_t i4 = (((size_t)h * dc.ntp + pc.itp) * dc.ncp + pc.icp) * dc.nmb + pc.ib;
-        bad |= put_coef<QUANT>(coef, coeff, at, HAP_KPRE, dc.tpre[i4]);
-        bad |= put_coef<QUANT>(coef, coeff, at, HAP_KPOST, dc.tpost[i4]);
+        bad |= put_coef(coef, coeff, at, HAP_KPRE, dc.tpre[i4]);
+        bad |= put_coef(coef, coeff, at, HAP_KPOST, dc.tpost[i4]);
         const double Dp = Dtp / (double)TP;
-        bad |= put_coef<QUANT>(coef, coeff, at, HAP_KP2P_INTRA, 2.0 * (dc.alpha[HAP_INTRA] + xfer_ns(dc, HAP_INTRA, Dp, dc.bw_intra[h])));
-        bad |= put_coef<QUANT>(coef, coeff, at, HAP_KP2P_INTER, 2.0 * (dc.alpha[HAP_INTER] + xfer_ns(dc, HAP_INTER, Dp, dc.bw_inter[h])));
+        bad |= put_coef(coef, coeff, at, HAP_KP2P_INTRA, 2.0 * (dc.alpha[HAP_INTRA] + xfer_ns(dc, HAP_INTRA, Dp, dc.bw_intra[h])));
+        bad |= put_coef(coef, coeff, at, HAP_KP2P_INTER, 2.0 * (dc.alpha[HAP_INTER] + xfer_ns(dc, HAP_INTER, Dp, dc.bw_inter[h])));
 #pragma unroll
         for (int h2 = 0; h2 < HAP_MAX_TYPES; ++h2) {
             const double bo = h2 < T ? dc.bw_inter[h2] : dc.bw_inter[h];
             const double bmin = dc.bw_inter[h] < bo ? dc.bw_inter[h] : bo;
-            bad |= put_coef<QUANT>(coef, coeff, at, HAP_KP2P_CROSS + h2, 2.0 * (dc.alpha[HAP_CROSS] + xfer_ns(dc, HAP_CROSS, Dp, bmin * dc.chi)));
+            bad |= put_coef(coef, coeff, at, HAP_KP2P_CROSS + h2, 2.0 * (dc.alpha[HAP_CROSS] + xfer_ns(dc, HAP_CROSS, Dp, bmin * dc.chi)));
         }
         const i64 wd = (i64)DP * CP;
         const double shd = 6.0 + 12.0 / (double)wd;
-        bad |= put_coef<QUANT>(coef, coeff, at, HAP_MA + HAP_DENSE, (thb * dc.act_coef[HAP_DENSE]) / (double)TP);
-        bad |= put_coef<QUANT>(coef, coeff, at, HAP_MA + HAP_MOE, (thb * dc.act_coef[HAP_MOE]) / (double)TP);
-        bad |= put_coef<QUANT>(coef, coeff, at, HAP_MX,
+        bad |= put_coef(coef, coeff, at, HAP_MA + HAP_DENSE, (thb * dc.act_coef[HAP_DENSE]) / (double)TP);
+        bad |= put_coef(coef, coeff, at, HAP_MA + HAP_MOE, (thb * dc.act_coef[HAP_MOE]) / (double)TP);
+        bad |= put_coef(coef, coeff, at, HAP_MX,
                                ((2.0 * ((thb * dc.beta) * (double)dc.k)) * (1.0 - 1.0 / (double)EP)) * dc.capf
                                + ((double)tok * (double)dc.E) * 4.0);
         const double mpre = (((double)dc.V * (double)H) / (double)TP) * shd;
-        bad |= put_coef<QUANT>(coef, coeff, at, HAP_MPRE, mpre);
-        bad |= put_coef<QUANT>(coef, coeff, at, HAP_MPOST, mpre);
+        bad |= put_coef(coef, coeff, at, HAP_MPRE, mpre);
+        bad |= put_coef(coef, coeff, at, HAP_MPOST, mpre);
         // dispatch + combine of one MoE layer (forward and backward, with the imbalance factor of Eq. 2) when the
         // expert-parallel group spans device types: Eq. 3's volumes over the cross-type link
         double kxd = 0.0;
@@ -373,7 +430,7 @@ type_const_kernel(const DevConst dc, TypeConst *tcg, i64 *coef, double *coeff, u
             const double fg = dc.alpha[HAP_CROSS] * (double)(EP - 1) + xfer_ns(dc, HAP_CROSS, Dag, bx);
             kxd = (4.0 * ((fa <= fg) ? fa : fg)) * (1.0 + dc.gamma * (dc.rho[pc.iep] - 1.0));
         }
-        bad |= put_coef<QUANT>(coef, coeff, at, HAP_KXD, kxd);
+        bad |= put_coef(coef, coeff, at, HAP_KXD, kxd);
     } else {
         const i64 wd = (i64)DP * CP;
         const double shd = 6.0 + 12.0 / (double)wd;
@@ -386,8 +443,8 @@ type_const_kernel(const DevConst dc, TypeConst *tcg, i64 *coef, double *coeff, u
         Pd[HAP_DENSE] = Pattn + Pffn_d;
         Pd[HAP_MOE] = Pattn + (i64)dc.n_shared * Pffn_e;
         const double PeT = (double)Pe / (double)TPE;
-        bad |= put_coef<QUANT>(coef, coeff, at, HAP_MW + HAP_DENSE, ((double)Pd[HAP_DENSE] / (double)TP) * shd);
-        bad |= put_coef<QUANT>(coef, coeff, at, HAP_MW + HAP_MOE,
+        bad |= put_coef(coef, coeff, at, HAP_MW + HAP_DENSE, ((double)Pd[HAP_DENSE] / (double)TP) * shd);
+        bad |= put_coef(coef, coeff, at, HAP_MW + HAP_MOE,
                                ((double)Pd[HAP_MOE] / (double)TP + (double)Prt) * shd + PeT * she);
         const int cG = link_class(lc, G);
         const double bwG = link_bw(lc, cG);
@@ -396,12 +453,12 @@ type_const_kernel(const DevConst dc, TypeConst *tcg, i64 *coef, double *coeff, u
         for (int kd = 0; kd < 2; ++kd) {
             const i64 Pdd = Pd[kd] + (kd == HAP_MOE ? Prt : 0);
             const double Pel = kd == HAP_MOE ? PeT : 0.0;
-            bad |= put_coef<QUANT>(coef, coeff, at, HAP_SBW + kd,
+            bad |= put_coef(coef, coeff, at, HAP_SBW + kd,
                                    dc.ovl_dp * (xfer_ns(dc, cG, (6.0 * ((double)Pdd / (double)TP)) * vfd, bwG) + xfer_ns(dc, cG, (6.0 * Pel) * vfe, bwG)));
-            bad |= put_coef<QUANT>(coef, coeff, at, HAP_OPT + kd,
+            bad |= put_coef(coef, coeff, at, HAP_OPT + kd,
                                    dc.copt[h] * ((double)Pdd / (double)((i64)TP * DP * CP) + Pel / (double)EDP));
         }
-        bad |= put_coef<QUANT>(coef, coeff, at, HAP_SLAT,
+        bad |= put_coef(coef, coeff, at, HAP_SLAT,
                                dc.ovl_dp * (dc.alpha[cG] * (2.0 * (double)(wd - 1) + 2.0 * (double)(EDP - 1))));
     }
     if (bad && range_flag) atomicOr(range_flag, 1ull);
@@ -508,7 +565,7 @@ struct StageMap {
     int ha, hb;     // sending / receiving device type of that boundary
 };
 
-__device__ __forceinline__ StageMap decode_stage(const DevConst &dc, const hap_pconf &pc, u64 map_idx, int lane)
+__host__ __device__ __forceinline__ StageMap decode_stage(const DevConst &dc, const hap_pconf &pc, u64 map_idx, int lane)
 {
     StageMap sm; sm.mask = 0; sm.cls = 0; sm.ha = 0; sm.hb = 0;
     const int PP = pc.PP, T = dc.T;
@@ -572,7 +629,11 @@ __device__ __forceinline__ StageMap decode_stage(const DevConst &dc, const hap_p
                     // pick-th set bit of avail
                     unsigned a = avail;
                     for (int t = 0; t < pick; ++t) a &= a - 1;
+#ifdef __CUDA_ARCH__
                     const int h = __ffs(a) - 1;
+#else
+                    const int h = __builtin_ffs((int)a) - 1;
+#endif
                     sigma[pos] = h;
                     avail &= ~(1u << h);
                 }
@@ -859,24 +920,6 @@ __device__ __forceinline__ void maptab_one(const DevConst &dc, u64 p_rep, u64 nm
 __global__ void maptab_kernel(const DevConst dc, u64 p_rep, u64 nmap, uint8_t *tab)
 {
     maptab_one(dc, p_rep, nmap, tab, ((u64)blockIdx.x * blockDim.x + threadIdx.x) >> 5, threadIdx.x & 31);
-}
-
-// The same for several PP classes in one launch (a pass decodes all classes that walk a prefix tree this way):
-// class q owns blocks [blk_lo[q], blk_lo[q+1]) of 128 threads, four mappings per block.
-struct DecodeJobs {
-    int n;
-    u32 blk_lo[HAP_MAX_PP + 2];
-    u32 p_rep[HAP_MAX_PP + 1];
-    u32 nmap[HAP_MAX_PP + 1];
-    u64 tab_off[HAP_MAX_PP + 1];            // byte offset of the class's table
-};
-
-__global__ void __launch_bounds__(128) maptab_all_kernel(const DevConst dc, const DecodeJobs jobs, uint8_t *tab_base)
-{
-    int q = 0;
-    while (q + 1 < jobs.n && blockIdx.x >= jobs.blk_lo[q + 1]) ++q;
-    const u64 w = ((u64)(blockIdx.x - jobs.blk_lo[q]) * blockDim.x + threadIdx.x) >> 5;
-    maptab_one(dc, jobs.p_rep[q], jobs.nmap[q], tab_base + jobs.tab_off[q], w, threadIdx.x & 31);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1918,8 +1961,7 @@ argmin_partial_kernel(const i64 *cost, u64 count, i64 *pcost, u64 *pindex, i64 i
 }
 
 __global__ void __launch_bounds__(256)
-argmin_final_kernel(const i64 *pcost, const u64 *pindex, u64 n, i64 *out2, i64 init, const PlanSlot *plans = nullptr,
-                    i64 *w_vals = nullptr, uint8_t *w_part = nullptr, uint8_t *w_rec = nullptr)
+argmin_final_kernel(const i64 *pcost, const u64 *pindex, u64 n, i64 *out2, i64 init)
 {
     // launched as a programmatic dependent of the first stage where it follows one directly: the partials are
     // complete and visible after this wait (a no-op in an ordinary launch)
@@ -1937,21 +1979,7 @@ argmin_final_kernel(const i64 *pcost, const u64 *pindex, u64 n, i64 *out2, i64 i
     if (threadIdx.x == 0) {
         for (int q = 1; q < 8; ++q) if (sc[q] < bc || (sc[q] == bc && si[q] < bi)) { bc = sc[q]; bi = si[q]; }
         out2[0] = bc; out2[1] = (i64)bi;
-        sc[0] = bc; si[0] = bi;
-        if (plans) w_vals[0] = init;             // (a winner whose plan is not found below shows as a cost that differs)
     }
-    if (!plans) return;
-    // the block that reported the minimum also left the candidate's plan: copy it beside the minimum
-    // (w_vals: cost, bottleneck, T_pipe, T_sync, T_opt)
-    __syncthreads();
-    bc = sc[0]; bi = si[0];
-    if (!(bc < init)) return;
-    for (u64 i = threadIdx.x; i < n; i += blockDim.x)
-        if (pindex[i] == bi && pcost[i] == bc) {
-            const PlanSlot ps = plans[i];
-            w_vals[0] = bc; w_vals[1] = ps.bott; w_vals[2] = ps.T_pipe; w_vals[3] = ps.T_sync; w_vals[4] = ps.T_opt;
-            for (int q = 0; q < HAP_MAX_PP; ++q) { w_part[q] = q < ps.PP ? ps.n[q] : 0; w_rec[q] = q < ps.PP ? ps.r[q] : 0; }
-        }
 }
 
 }  // namespace hap

@@ -1,0 +1,1136 @@
+// Prefix-tree form of the min-max pipeline recurrence (sm_100a).
+//
+// The DP row of stage d of a candidate depends only on the candidate's stages 1..d (their device
+// types, boundary links and load-balance windows), the configuration and the recomputation policy.
+// All mappings of a PP class therefore form a prefix tree whose nodes are distinct stage prefixes;
+// the tree, the band of reachable end layers of every node and the task list below depend on the
+// class alone and are laid out once on the host.
+//
+//   type_const_kernel  (hap_device.cuh) constants of Eq. 2 / Eq. 3, and which configurations can place a first stage.
+//   tree_prep_kernel   a block per such configuration: Eq. 2 for every (device type, layer), the prefix rows of the
+//                      stage time per type mask and level, the memory thresholds and the stage constants, written
+//                      as one record for the DP kernel.  The other configurations' candidates are infeasible: a
+//                      warp each writes their results.
+//   tree_dp_kernel     persistent blocks of four warps that take (configuration, group of tree parts) items from
+//                      a counter.  A warp owns a part of the tree -- some tens of mappings -- and walks it depth
+//                      by depth on its own: no block barrier inside an item.  A task is four consecutive end
+//                      layers of a node; a lane keeps their running minima and slides one window of the parent's
+//                      row over the stage lengths (tree_scan).  Then one lane per mapping evaluates the last stage,
+//                      walks the choices back and assembles Eq. 4.  A search leaves the plan of the best candidate;
+//                      the last block to finish reduces the blocks' minima and decodes the winner.
+//
+// Bounds and figures (B200; 1,024 devices, 128 layers, 2.4 million candidates; a pass of 438 us before this form, 400 us
+// with it; 256 devices with partitions, 549 us after 990 us).  The recurrence is bound by instruction issue (57 % of the
+// slots, 20 lanes of 32 active); its row entries never leave shared memory.  A deeper split into blocks that share a tree
+// needs a barrier per depth (31 of them at 32 stages); a warp of its own per part needs none.  Two end layers per
+// task and eight blocks an SM: 475 us; one: 536 us; eight parts an item instead of four: 405 us; the registers of five
+// blocks of four warps (96) spill nothing, those of eight do.
+//
+// Integer mode holds times (integer ns below 2^52) as doubles: every sum, difference and comparison is exact.
+#pragma once
+#include "hap_device.cuh"
+
+namespace hap {
+
+constexpr int kTreeWarps = 4;             // warps of a DP block
+constexpr int kTreeThreads = kTreeWarps * 32;
+constexpr int kTreeBlocksPerSm = 5;       // (100 registers a thread)
+constexpr int kTreeJ = 4;                 // end layers of a task
+constexpr int kTreePad = kTreeJ - 1;      // infinite entries in front of every row and behind the last one
+constexpr int kTreeKtab = 16 + HAP_MAX_TYPES * 6;    // stage constants: [0,16) pre-work by row group, then p2p [type][6]
+constexpr int kTreeMinfo = 8;             // doubles per row group: sync latency, sync bandwidth x 2, optimizer x 2, cross dispatch, post-work, pad
+
+// A task: up to four consecutive end layers j0..j0+cnt-1 of one node (a stage prefix of depth d < PP) and the stage lengths
+// a..b that reach the parent's row from any of them.
+//   x = slot of prev[j0 - a] in the previous depth's buffer | slot of j0's value in this depth's << 16
+//   y = j0 | a << 8 | b << 16 | (cnt - 1) << 24 | first of its row << 26 | last of the depth << 27
+//   z = stage constant index | row group of the stage's types << 8 | capacity type << 16
+//   w = unused
+typedef uint4 TreeTask;
+
+// A contiguous range of a class's mappings with the tree of their prefixes.
+struct TreePart {
+    const TreeTask *tasks;                  // grouped by depth
+    const u32 *path;                        // [PP][nmap] stage d of mapping m: origin of its node among the choices (choice of
+                                            // end layer 0, + 256), 20 bits; d = PP: slot of prev[N - a] of the last stage;
+                                            // | stage constant index << 20 | row group << 26 | capacity type << 30
+    const u32 *leaf;                        // [nmap] lengths of the last stage that reach the parent's row: a | b << 8;
+                                            // a > b: the windows cannot add up to N
+    u32 nmap, m_lo;                         // mappings [m_lo, m_lo + nmap) of the class
+    u32 task_lo[HAP_MAX_PP + 1];            // tasks of depth d: [task_lo[d], task_lo[d+1]), d = 1..PP-1
+    u32 cell_lo[HAP_MAX_PP + 1];            // choices of depth d start here
+};
+
+// A PP class that walks its tree.
+struct TreeClass {
+    const TreePart *parts;
+    u64 rec_off;                            // byte offset of the class's records
+    u32 p_lo, n_conf;                       // its configurations are contiguous
+    u32 rec_bytes;                          // one configuration's record
+    u32 o_minfo, o_rows, o_thr, o_thr_nf;   // offsets in a record
+    u32 buf_cells[2], ch_bytes;             // a warp's row buffers (even / odd depths, in values) and choices
+    int PP, n_parts, n_mrows;
+    int items_per_conf;                     // an item is a group of the configuration's parts ...
+    int conf_per_item;                      // ... or one part each of several configurations (classes of one part)
+    uint8_t mrow_of[16], mask_of_row[16];   // type mask <-> row group
+    uint8_t first_min[HAP_MAX_TYPES];       // per capacity type: shortest first stage (255: no first stage on it)
+    uint8_t wmax[HAP_MAX_PP + 1];           // longest stage of depth d
+    uint8_t tmask[HAP_MAX_PP + 1];          // capacity types that occur at depth d
+    uint8_t jlo[HAP_MAX_PP + 1], jhi[HAP_MAX_PP + 1], kmin[HAP_MAX_PP + 1], kmax[HAP_MAX_PP + 1];
+    uint8_t flat[HAP_MAX_PP + 1];           // depth d sees spans of one layer kind only: its thresholds are lengths (one word
+                                            // per type, a byte per level); else a byte per (type, level, end layer) at nf_off[d]
+    uint8_t all_flat;
+    u32 nf_off[HAP_MAX_PP + 1], nf_w[HAP_MAX_PP + 1];
+};
+
+// Head of a configuration's record.
+struct __align__(16) TreeHead {
+    u64 offset;                             // first candidate of the configuration
+    i64 m1;                                 // micro-batches - 1
+    i64 lb;                                 // lower bound on T_iter of its candidates (searches)
+    u32 p;
+    u32 dead_policies;                      // by position in rc_order: no mapping can be feasible
+    u64 pad[4];
+};
+static_assert(sizeof(TreeHead) == 64, "the stage constants start behind it");
+constexpr u32 kTreeOffKtab = sizeof(TreeHead);
+constexpr u32 kTreeOffMinfo = kTreeOffKtab + kTreeKtab * 8;
+
+// What a search brings back, written by the last block (device memory and, if mapped, the host's copy).
+struct TreeResult {
+    u64 range_flag, n_feasible, n_pruned;
+    i64 cost; u64 index;
+    i64 bott, T_pipe, T_sync, T_opt;
+    u32 pconf, rc_mask;
+    u64 stamp[3];                           // global timer: pass begins, recurrence begins, all done
+    uint8_t n[HAP_MAX_PP], r[HAP_MAX_PP], mask[HAP_MAX_PP];
+};
+
+// Device words a pass counts in.  All zero between passes: the last block of a pass leaves them so.
+struct TreeState {
+    u32 live[HAP_MAX_PP + 2];               // configurations on each class's list; behind the last class, on the dead list
+    u32 ticket[2];                          // next item of each DP launch
+    u32 blocks_done, prep_done;
+    u64 n_feasible, n_pruned, splits;
+    u64 incumbent;                          // of a pruning search: ~(smallest T_iter so far)
+};
+
+// A pruning search hands its configurations out by their lower bounds, smallest first: buckets of 1/64 octave between 2^20
+// and 2^40 ns.
+constexpr int kOrderSub = 6, kOrderLow = 20, kOrderBuckets = 20 << kOrderSub;
+__device__ __forceinline__ int order_bucket(i64 lb)
+{
+    if (lb < (1ll << kOrderLow)) return 0;
+    const int e = 63 - __clzll(lb);
+    const int b = ((e - kOrderLow) << kOrderSub) + (int)((lb >> (e - kOrderSub)) & ((1 << kOrderSub) - 1));
+    return b < kOrderBuckets ? b : kOrderBuckets - 1;
+}
+// smallest bound of bucket b
+__device__ __forceinline__ i64 order_edge(int b)
+{
+    return b == 0 ? 0 : (i64)((1 << kOrderSub) + (b & ((1 << kOrderSub) - 1))) << ((b >> kOrderSub) + kOrderLow - kOrderSub);
+}
+
+// What the last block keeps of a pass.
+struct TreeReport {
+    u64 n_feasible, n_pruned, splits;
+    u64 stamp[3];                           // global timer: pass begins, recurrence begins, all done
+};
+
+__device__ __forceinline__ u64 global_timer()
+{
+    u64 t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
+__device__ u32 *tree_state_live(TreeState *state) { return state->live; }
+__device__ void tree_stamp_begin(TreeReport *report) { report->stamp[0] = global_timer(); }
+
+struct TreeArgs {
+    int N, T, R, n_rc, RW;
+    int eta_q, kind_uniform, kind0;
+    unsigned rc_masks[HAP_MAX_RC_MASKS], rc_sup[HAP_MAX_RC_MASKS];
+    int rc_order[HAP_MAX_RC_MASKS];
+    double tau[HAP_MAX_RC];                 // repeated forward fraction per level (rows that are not combined by level)
+    u64 kindbits[4];
+    const TreeClass *cls;
+    int n_cls;
+    u32 p_lo[HAP_MAX_PP + 1];               // first configuration of each class (its list starts there)
+    u32 nmap[HAP_MAX_PP + 1];               // mappings of its configurations
+    const u32 *live_list, *dead_list;
+    int c_lo, c_hi;                         // classes of this launch
+    int launch;                             // which ticket counter; blocks that must be done before the last one reduces
+    u32 blocks_total;
+    u32 slot_lo;                            // first per-block slot of this launch
+    u64 *hist;                              // pruning searches of more than one wave of items: configurations | items << 32 per bucket
+    uint4 *order_key, *order;               // by list position: class | bucket << 8, list entry, place in the bucket, items before it
+                                            // by order: first item, class | bucket << 8, list entry, -
+    unsigned char *rec;
+    TreeState *state;
+    TreeReport *report;
+    TreeResult *res_dev, *res_host;
+    const u64 *range_flag;
+    PlanSlot *slots;                        // [blocks_total] per-block plan
+    i64 *slot_cost; u64 *slot_index;        // [blocks_total]
+};
+
+// shared-memory accesses by 32-bit address (the scans walk rows with plain address decrements)
+__device__ __forceinline__ u32 smem_u32(const void *p) { return (u32)__cvta_generic_to_shared(p); }
+#ifdef HAP_CHECKED
+__device__ __forceinline__ bool smem_addr_ok(u32 a, u32 bytes)
+{
+    // the dynamic part lies behind the static variables of the kernel: nothing is addressable past its end
+    extern __shared__ __align__(16) unsigned char dyn_smem_base[];
+    u32 dyn;
+    asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
+    return HAP_CHECK_OK(0, a % bytes == 0 && a + bytes <= smem_u32(dyn_smem_base) + dyn);
+}
+#else
+__device__ __forceinline__ bool smem_addr_ok(u32, u32) { return true; }
+#endif
+__device__ __forceinline__ double lds_f64(u32 a)
+{
+    if (!smem_addr_ok(a, 8)) return 0.0;
+    double v;
+    asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ u32 lds_u32(u32 a)
+{
+    if (!smem_addr_ok(a, 4)) return 0;
+    u32 v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ int lds_u8(u32 a)
+{
+    if (!smem_addr_ok(a, 1)) return 0;
+    u32 v;
+    asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(a));
+    return (int)v;
+}
+__device__ __forceinline__ void sts_f64(u32 a, double v)
+{
+    if (!smem_addr_ok(a, 8)) return;
+    asm volatile("st.shared.f64 [%0], %1;" :: "r"(a), "d"(v) : "memory");
+}
+__device__ __forceinline__ void sts_u8(u32 a, u32 v)
+{
+    if (!smem_addr_ok(a, 1)) return;
+    asm volatile("st.shared.u8 [%0], %1;" :: "r"(a), "r"(v) : "memory");
+}
+
+template <typename T> struct IsF64 { static constexpr bool value = false; };
+template <> struct IsF64<double> { static constexpr bool value = true; };
+
+constexpr double kTreeInf = 4611686018427387904.0;        // 2^62, the integer INF: above every finite value
+constexpr double kTreeBound = 2305843009213693952.0;      // 2^61: every finite value is below
+
+// ------------------------------------------------------------------------------------------------------------------
+// per-configuration records
+// ------------------------------------------------------------------------------------------------------------------
+
+// the candidates of a configuration none of whose first stages fits any device, results of a pass: by one warp
+template <bool F64>
+__device__ __forceinline__ void tree_fill_dead(const DpOut &out, u64 c0, u64 c1, int lane)
+{
+    const u64 a = c0 > out.first ? c0 : out.first, b = c1 < out.first + out.count ? c1 : out.first + out.count;
+    if (a >= b) return;
+    const i64 inf = F64 ? 0x7ff0000000000000ll : kInf;
+    const u64 n = b - a, o = a - out.first;
+    for (u64 q = lane; q < n; q += 32) {
+        if (out.cost) out.cost[o + q] = inf;
+        if (out.bottleneck) out.bottleneck[o + q] = inf;
+    }
+    const uint4 z = make_uint4(0, 0, 0, 0);
+    static_assert(HAP_MAX_PP == 32, "two 16-byte pieces per candidate");
+    if (out.partition) for (u64 q = lane; q < 2 * n; q += 32) reinterpret_cast<uint4 *>(out.partition + o * HAP_MAX_PP)[q] = z;
+    if (out.recompute) for (u64 q = lane; q < 2 * n; q += 32) reinterpret_cast<uint4 *>(out.recompute + o * HAP_MAX_PP)[q] = z;
+}
+
+// Persistent blocks over the configurations on the classes' lists: entry i of a class's list becomes its record i.  What
+// bounds a configuration is a chain of dependent steps (constants, layer costs, scans), hidden by the resident blocks.
+constexpr int kTreePrepThreads = 128;
+constexpr int kTreePrepBlocksPerSm = 9;
+template <bool F64, bool NL>
+__global__ void __launch_bounds__(kTreePrepThreads, kTreePrepBlocksPerSm)
+tree_prep_kernel(const DevConst dc, const TreeArgs ta, const TypeConst *__restrict__ tcg, const i64 *__restrict__ coef,
+                 const double *__restrict__ coeff, const void *__restrict__ c2v, DpOut out, int search)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ TreeClass cl;
+    __shared__ u32 s_first[HAP_MAX_PP + 3];         // entries of the lists before class c; dead ones behind the last class
+    __shared__ i64 s_lb;
+    const int tid = threadIdx.x, nthreads = kTreePrepThreads, lane = tid & 31, wib = tid >> 5;
+    constexpr int nwarps = kTreePrepThreads / 32;
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (tid < 32) {
+        // exclusive sums of the list lengths
+        const u32 n = tid <= ta.n_cls ? __ldcg(&ta.state->live[tid]) : 0u;
+        u32 v = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const u32 t = __shfl_up_sync(0xffffffffu, v, o); if (lane >= o) v += t; }
+        if (tid <= ta.n_cls) s_first[tid] = v - n;
+    }
+    if (tid == 0) s_lb = 0;
+    __syncthreads();
+    unsigned all_levels = 0;
+    for (int q = 0; q < dc.n_rc; ++q) all_levels |= dc.rc_masks[q];
+    const int N = dc.N, T = dc.T, R = dc.R, n1 = N + 1;
+    const u32 n_live = s_first[ta.n_cls];
+    int loaded = -1;
+  for (u32 item = blockIdx.x; item < n_live; item += gridDim.x) {
+    int ci = 0;
+    while (item >= s_first[ci + 1]) ++ci;
+    const u32 s_slot = item - s_first[ci];
+    const u32 p = __ldcg(ta.live_list + ta.p_lo[ci] + s_slot);
+    if (ci != loaded) {
+        static_assert(sizeof(TreeClass) % 4 == 0, "copied in words");
+        const u32 *src = reinterpret_cast<const u32 *>(ta.cls + ci);
+        u32 *dst = reinterpret_cast<u32 *>(&cl);
+        for (int q = tid; q < (int)(sizeof(TreeClass) / 4); q += nthreads) dst[q] = src[q];
+        loaded = ci;
+        __syncthreads();
+    }
+    const hap_pconf pc = dc.pconf[p];
+    const int PP = pc.PP;
+    const i64 *cfp = coef + (size_t)p * T * HAP_NCOEF;                                        // integer coefficients (bytes)
+    auto cv = [&](int h, int q) -> double {                                                  // time coefficients
+        const size_t at = ((size_t)p * T + h) * HAP_NCOEF + q;
+        return F64 ? coeff[at] : (double)coef[at];
+    };
+
+    double2 *sC = reinterpret_cast<double2 *>(smem_raw);                                      // [T][N] forward, backward
+    uint8_t *sThr = reinterpret_cast<uint8_t *>(sC + (size_t)T * N);                          // flat words, then the other depths' bytes
+    const u32 thr_bytes = cl.rec_bytes - cl.o_thr;
+    i64 *sW = reinterpret_cast<i64 *>(sThr + (thr_bytes + 15) / 16 * 16);                     // byte prefixes (mixed kinds only)
+    i64 *sA = sW + n1;
+    uint8_t *sK = reinterpret_cast<uint8_t *>(sA + n1);
+
+    // ---- Eq. 2 for every (device type, layer), with the arithmetic of layer_cost_kernel -------------------------
+    if (c2v) {                                                                                // a preceding launch left them
+        for (int q = tid; q < T * N; q += nthreads) {
+            if (F64) sC[q] = reinterpret_cast<const double2 *>(c2v)[(size_t)p * T * N + q];
+            else { const longlong2 v = reinterpret_cast<const longlong2 *>(c2v)[(size_t)p * T * N + q]; sC[q] = make_double2((double)v.x, (double)v.y); }
+        }
+    } else {
+        const size_t row = ((size_t)pc.itp * dc.ncp + pc.icp) * dc.nmb + pc.ib;              // the same table row for every type
+        const size_t stride_h = (size_t)dc.ntp * dc.ncp * dc.nmb * N * 2;                     // 16-byte pairs between device types
+        const double2 *tab = reinterpret_cast<const double2 *>(dc.tab4) + row * N * 2;
+        const TypeConst *tcp = tcg + (size_t)p * T;
+        bool bad = false;
+        for (int q = tid; q < T * N; q += nthreads) {
+            const int h = q / N, l = q - h * N;
+            const bool dense = layer_kind(dc, l) == HAP_DENSE;
+            const double2 *tp = tab + (size_t)h * stride_h + (size_t)l * 2;
+            const double2 tb = __ldg(tp);
+            const double2 tf = dense ? make_double2(0.0, 0.0) : __ldg(tp + 1);
+            double cf, cb;
+            layer_cost_pair(reinterpret_cast<const double2 *>(tcp + h), tb, tf, dense, dc.kappa, cf, cb);
+            bad |= !(cf < 6.8719e10) | !(cb < 6.8719e10);                                     // 2^36 ns per layer
+            sC[q] = F64 ? make_double2(cf, cb) : make_double2((double)__double2ll_rn(cf), (double)__double2ll_rn(cb));
+        }
+        if (bad) atomicOr(out.range_flag, 1ull);
+    }
+    if (!cl.all_flat) {
+        for (int l = tid; l <= N; l += nthreads) sK[l] = (uint8_t)moe_before(dc, l);
+        for (int l = tid; l <= N; l += nthreads) {                                            // byte prefixes from the counts of layers per kind
+            const i64 nm = moe_before(dc, l), nd = (i64)l - nm;
+            sW[l] = nd * cfp[HAP_MW] + nm * cfp[HAP_MW + 1];
+            sA[l] = nd * cfp[HAP_MA] + nm * cfp[HAP_MA + 1];
+        }
+    }
+    __syncthreads();
+    unsigned char *rec = ta.rec + cl.rec_off + (u64)s_slot * cl.rec_bytes;
+
+    // ---- prefix rows of the stage time: per row group the slowest member type of every layer, one warp per group ---
+    double *rows = reinterpret_cast<double *>(rec + cl.o_rows);
+    for (int mr = wib; mr < cl.n_mrows; mr += nwarps) {
+        const int mk = cl.mask_of_row[mr];
+        double runC = 0.0, runF = 0.0;
+        for (int base = 0; base < N; base += 32) {
+            const int l = base + lane;
+            double vC = 0.0, vF = 0.0;                                                        // fwd + bwd, fwd
+            if (l < N) {
+                double F = 0.0, B = 0.0;
+                for (int h = 0; h < T; ++h)
+                    if (mk >> h & 1) { const double2 q = sC[(size_t)h * N + l]; F = q.x > F ? q.x : F; B = q.y > B ? q.y : B; }
+                vC = F + B; vF = F;
+            }
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const double tC = __shfl_up_sync(0xffffffffu, vC, o), tF = __shfl_up_sync(0xffffffffu, vF, o);
+                if (lane >= o) { vC += tC; vF += tF; }
+            }
+            vC += runC; vF += runF;
+            if (l < N) {
+                if (NL) { rows[(size_t)(mr * 2) * n1 + l + 1] = vC; rows[(size_t)(mr * 2 + 1) * n1 + l + 1] = vF; }
+                else for (int r = 0; r < R; ++r) rows[(size_t)(mr * R + r) * n1 + l + 1] = vC + (double)(dc.tau_q[r] >> 10) * vF;
+            }
+            runC = __shfl_sync(0xffffffffu, vC, 31); runF = __shfl_sync(0xffffffffu, vF, 31);
+        }
+        const int RW = NL ? 2 : R;
+        if (lane < RW) rows[(size_t)(mr * RW + lane) * n1] = 0.0;
+    }
+    // ---- lower bound on the summed stage time: the cheapest type's time of every layer (pruning searches) ----------
+    if (search && !F64) {
+        i64 lmin = 0;
+        for (int l = tid; l < N; l += nthreads) {
+            double m = 0.0;
+            for (int h = 0; h < T; ++h) { const double2 q = sC[(size_t)h * N + l]; const double v = q.x + q.y; m = (h == 0 || v < m) ? v : m; }
+            lmin += (i64)m;
+        }
+        lmin = warp_sum_i64(lmin);
+        if (lane == 0 && lmin) atomicAdd(reinterpret_cast<unsigned long long *>(&s_lb), (unsigned long long)lmin);
+    }
+    // ---- memory thresholds -------------------------------------------------------------------------------------------
+    {
+        const i64 mx = cfp[HAP_MX], mpre = cfp[HAP_MPRE], mpost = cfp[HAP_MPOST];
+        // Depths whose spans are of one kind: the longest length that fits, a byte per level in one word per (depth, type)
+        const i64 mwk = cfp[HAP_MW + layer_kind(dc, N - 1)], mak = cfp[HAP_MA + layer_kind(dc, N - 1)];
+        const i64 mxk = layer_kind(dc, N - 1) == HAP_MOE ? mx : 0;
+        const int len_cap = N - dc.kind_uniform_from;
+        u32 *w4 = reinterpret_cast<u32 *>(sThr);
+        for (int q = tid; q < PP * T; q += nthreads) {
+            const int t = q % T, d = q / T + 1;
+            u32 word = 0;
+            if (cl.flat[d] && ((cl.tmask[d] >> t) & 1u)) {
+                const i64 base = (d == 1 ? mpre : 0) + (d == PP ? mpost : 0) + mxk, cap = dc.cap_eff[t];
+                const int inflight = PP - d + 1;
+                const i64 ma = (i64)(pc.M < inflight ? pc.M : inflight) * mak;
+                for (int r = 0; r < R; ++r) {
+                    if (!((all_levels >> r) & 1u)) continue;
+                    const i64 xi = dc.xi_q[r];
+                    // longest length n with n mwk + base + floor(xi n ma / 1024) <= cap: the quotient, then exact steps from there
+                    const int most = cl.wmax[d] < len_cap ? cl.wmax[d] : len_cap;
+                    auto fits = [&](int n) { return (i64)n * mwk + base + ((xi * ((i64)n * ma)) >> 10) <= cap; };
+                    const float guess = (float)(cap - base) / ((float)mwk + (float)xi * (float)ma * 9.765625e-4f);
+                    int lo = guess < 0.0f ? 0 : guess > (float)most ? most : (int)guess;             // (a zero divisor: most, or NaN: 0)
+                    while (lo < most && fits(lo + 1)) ++lo;
+                    while (lo > 0 && !fits(lo)) --lo;
+                    word |= (u32)lo << (8 * r);
+                }
+            }
+            w4[q] = word;
+        }
+        if (!cl.all_flat) {
+            // other depths: per (type, level, end layer) the longest span ending there that fits; feasibility is monotone in
+            // the span, so a thread sweeps a segment of end layers with a split pointer that only moves forward
+            uint8_t *nf = sThr + (cl.o_thr_nf - cl.o_thr);
+            constexpr int kSeg = 8;
+            for (int d = 1; d <= PP; ++d) {
+                if (cl.flat[d]) continue;
+                const int w = (int)cl.nf_w[d], nseg = (w + kSeg - 1) / kSeg;
+                for (int e = tid; e < T * R * nseg; e += nthreads) {
+                    const int seg = e % nseg, q = e / nseg, r = q % R, t = q / R;
+                    uint8_t *row = nf + cl.nf_off[d] + (size_t)q * w - cl.jlo[d];
+                    const int j0 = cl.jlo[d] + seg * kSeg;
+                    int j1 = j0 + kSeg - 1; if (j1 > cl.jhi[d]) j1 = cl.jhi[d];
+                    const bool want = ((all_levels >> r) & 1u) && ((cl.tmask[d] >> t) & 1u);
+                    const i64 extra = (d == 1 ? mpre : 0) + (d == PP ? mpost : 0);
+                    const int inflight = PP - d + 1;
+                    const i64 mstore = pc.M < inflight ? pc.M : inflight, cap = dc.cap_eff[t], xi = dc.xi_q[r];
+                    int k = cl.kmin[d];
+                    for (int j = j0; j <= j1; ++j) {
+                        if (!want) { row[j] = 0; continue; }
+                        if (k < j - (int)cl.wmax[d]) k = j - (int)cl.wmax[d];
+                        const int kcap = (int)cl.kmax[d] < j - 1 ? (int)cl.kmax[d] : j - 1;      // no cell looks at a split beyond this
+                        while (k <= kcap && !span_fits(sW, sA, sK, extra, mx, mstore, cap, xi, k, j)) ++k;
+                        row[j] = (uint8_t)(k <= kcap ? j - k : 0);
+                    }
+                }
+            }
+        }
+    }
+    // ---- stage constants ---------------------------------------------------------------------------------------------
+    {
+        double *ktab = reinterpret_cast<double *>(rec + kTreeOffKtab), *mi = reinterpret_cast<double *>(rec + cl.o_minfo);
+        for (int q = tid; q < cl.n_mrows * kTreeMinfo; q += nthreads) {
+            const int mr = q / kTreeMinfo, e = q % kTreeMinfo, mk = cl.mask_of_row[mr];
+            // the slowest member of a stage of several types
+            const int col = e == 0 ? HAP_SLAT : e <= 2 ? HAP_SBW + e - 1 : e <= 4 ? HAP_OPT + e - 3 : e == 5 ? HAP_KXD : HAP_KPOST;
+            double v = 0.0, pre = 0.0;
+            for (int h = 0; h < T; ++h)
+                if (mk >> h & 1) { const double x = cv(h, col); v = x > v ? x : v; const double y = cv(h, HAP_KPRE); pre = y > pre ? y : pre; }
+            if (e == 5 && !(dc.het_dispatch && (mk & (mk - 1)) != 0)) v = 0.0;
+            mi[q] = v;
+            if (e == 7) ktab[mr] = pre;
+        }
+        for (int q = tid; q < T * 6; q += nthreads) ktab[16 + q] = cv(q / 6, HAP_KP2P_INTRA + q % 6);   // intra, inter, cross[0..3]
+    }
+    __syncthreads();
+    // ---- policies that cannot be feasible: the longest stages that fit do not add up to N ------------------------------
+    {
+        const uint4 *src = reinterpret_cast<const uint4 *>(sThr);
+        uint4 *dst = reinterpret_cast<uint4 *>(rec + cl.o_thr);
+        for (int q = tid; q < (int)(thr_bytes / 16); q += nthreads) dst[q] = src[q];
+    }
+    if (wib == 0) {
+        u32 dead = 0;
+        for (int pos = 0; pos < dc.n_rc; ++pos) {
+            const unsigned mask = dc.rc_masks[dc.rc_order[pos]];
+            int most = 0;
+            if (lane < PP) {
+                const int d = lane + 1;
+                if (!cl.flat[d]) most = cl.wmax[d];
+                else
+                    for (int t = 0; t < T; ++t) {
+                        const u32 w = reinterpret_cast<const u32 *>(sThr)[lane * T + t];
+                        for (int r = 0; r < R; ++r) if ((mask >> r) & 1u) { const int v = (int)((w >> (8 * r)) & 255u); most = v > most ? v : most; }
+                    }
+            }
+            const int none = __any_sync(0xffffffffu, lane < PP && most == 0);
+            most = __reduce_add_sync(0xffffffffu, most);
+            if (none || most < N) dead |= 1u << pos;
+        }
+        if (lane == 0) {
+            TreeHead h{};
+            h.offset = pc.offset; h.m1 = (i64)pc.M - 1; h.p = p; h.dead_policies = dead;
+            h.lb = s_lb + h.m1 * ((s_lb + PP - 1) / PP);
+            *reinterpret_cast<TreeHead *>(rec) = h;
+            s_lb = 0;
+            if (search && out.prune) {
+                // candidates are counted as pruned until a part is evaluated
+                const u64 c1 = pc.offset + pc.nmap * (u64)dc.n_rc, a = pc.offset > out.first ? pc.offset : out.first;
+                const u64 b = c1 < out.first + out.count ? c1 : out.first + out.count;
+                if (a < b) atomicAdd(&ta.state->n_pruned, b - a);
+                if (ta.order) {
+                    const int bk = order_bucket(h.lb);
+                    const u64 before = atomicAdd(ta.hist + bk, (u64)cl.items_per_conf << 32 | 1ull);
+                    __stcg(ta.order_key + item, make_uint4((u32)ci | (u32)bk << 8, s_slot, (u32)before, (u32)(before >> 32)));
+                }
+            }
+        }
+    }
+    __syncthreads();                                    // the shared arrays are free for the next configuration
+  }
+    if (search) {
+        if (!ta.order) return;
+        // the last block turns the buckets into the order
+        __shared__ u64 s_sum[nwarps];
+        __shared__ int s_last;
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) s_last = atomicAdd(&ta.state->prep_done, 1u) + 1u == gridDim.x;
+        __syncthreads();
+        if (!s_last) return;
+        __threadfence();
+        constexpr int kPer = kOrderBuckets / kTreePrepThreads;
+        static_assert(kPer * kTreePrepThreads == kOrderBuckets, "a whole number of buckets per thread");
+        u64 n[kPer], sum = 0;
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) { n[q] = __ldcg(ta.hist + tid * kPer + q); sum += n[q]; }
+        u64 v = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const u64 t = __shfl_up_sync(0xffffffffu, v, o); if (lane >= o) v += t; }
+        if (lane == 31) s_sum[wib] = v;
+        __syncthreads();
+        v -= sum;
+        for (int q = 0; q < wib; ++q) v += s_sum[q];
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) { __stcg(ta.hist + tid * kPer + q, v); v += n[q]; }
+        if (tid == kTreePrepThreads - 1) __stcg(ta.order + n_live, make_uint4((u32)(v >> 32), 0, 0, 0));
+        __syncthreads();
+        for (u32 i = (u32)tid; i < n_live; i += nthreads) {
+            const uint4 k = __ldcg(ta.order_key + i);
+            const u64 base = __ldcg(ta.hist + (k.x >> 8));
+            const u32 at = (u32)base + k.z;
+            if (HAP_CHECK_OK(4, at < n_live)) __stcg(ta.order + at, make_uint4((u32)(base >> 32) + k.w, k.x, k.y, 0));
+        }
+        return;
+    }
+    const u32 n_dead = __ldcg(&ta.state->live[ta.n_cls]);
+    // a warp per configuration; one with many candidates is shared by sixteen
+    constexpr u32 kSlices = 16;
+    constexpr u64 kMany = 1024;
+    for (u32 w = blockIdx.x * nwarps + wib; w < n_dead; w += gridDim.x * nwarps) {
+        const hap_pconf *pc = dc.pconf + __ldcg(ta.dead_list + w);
+        if (pc->nmap * (u64)dc.n_rc <= kMany) tree_fill_dead<F64>(out, pc->offset, pc->offset + pc->nmap * (u64)dc.n_rc, lane);
+    }
+    u64 most = 0;
+    for (int c = 0; c < ta.n_cls; ++c) { const u64 n = ta.nmap[c] * (u64)dc.n_rc; most = n > most ? n : most; }
+    if (most <= kMany) return;
+    for (u32 q = blockIdx.x * nwarps + wib; q < n_dead * kSlices; q += gridDim.x * nwarps) {
+        const hap_pconf *pc = dc.pconf + __ldcg(ta.dead_list + q / kSlices);
+        const u64 c0 = pc->offset, n = pc->nmap * (u64)dc.n_rc;
+        if (n > kMany) tree_fill_dead<F64>(out, c0 + n * (q % kSlices) / kSlices, c0 + n * (q % kSlices + 1) / kSlices, lane);
+    }
+}
+
+// ------------------------------------------------------------------------------------------------------------------
+// recurrence
+// ------------------------------------------------------------------------------------------------------------------
+
+// Levels of a policy at one (depth, capacity type): level of a stage of n layers = number of the bounds below n, longest
+// stage that fits at all = nx.  A level that is not allowed or never the lowest that fits has the bound of the one before it.
+struct TreeLevels { int b0, b1, b2, nx; };
+
+__device__ __forceinline__ TreeLevels tree_levels(int R, unsigned rc_mask, u32 len4)
+{
+    TreeLevels lv;
+    int run = -1;                                   // (level 0 not allowed: every length is above it)
+    auto step = [&](int r) { if ((rc_mask >> r) & 1u) { const int l = (int)((len4 >> (8 * r)) & 255u); run = l > run ? l : run; } return run; };
+    lv.b0 = step(0);
+    lv.b1 = R > 1 ? step(1) : run;
+    lv.b2 = R > 2 ? step(2) : run;
+    lv.nx = R > 3 ? step(3) : run;
+    return lv;
+}
+
+// Stage cost over layers (k, j] with the stage constant, from the row entries of j and k.
+//   combined rows (one per level): row[j] - row[k] + K; integer mode adds K to row[j] first, exact in any order
+//   NL: rows C (fwd + bwd) and F (fwd): C[j] - C[k] + floor(tau (F[j] - F[k])) + K; the product of an integer below 2^36 N
+//       and tau = tau_q / 1024 is exact in a double (the host checks N tau_q < 2^17), adding 2^52 rounding down floors it
+template <bool F64, bool NL>
+__device__ __forceinline__ double tree_span(double Cj, double Ck, double Fj, double Fk, double K, double tau)
+{
+    double c = Cj - Ck;
+    if (NL) {
+        const double t = (Fj - Fk) * tau;
+        if (F64) c = c + t;
+        else c = c + (__dadd_rd(t, 4503599627370496.0) - 4503599627370496.0);
+    }
+    return F64 ? c + K : c;
+}
+
+constexpr int kNever = 1 << 20;
+__device__ __forceinline__ int tree_bound(const TreeLevels &lv, int r) { return r == 0 ? lv.b0 : r == 1 ? lv.b1 : r == 2 ? lv.b2 : lv.nx; }
+
+// J consecutive end layers at once: DP[j] = min over stage lengths n in [a, b] of max(prev[j - n], cost), longest stage
+// (smallest split) on ties.  The lane holds a window of J entries of prev and of the row, prev[j0 + i - n], that moves by
+// one entry per length: two loads serve J splits, and the J minima are independent chains.  Entries of prev outside the
+// parent's row are infinite (padding), so nothing is clipped per split; lengths run level by level, the bounds in lv.
+// What bounds it is instruction issue: eight instructions per split (one subtraction, two comparisons and five selects of
+// 64-bit values), five more per length for the window.
+//   a_prev: address of prev[j0 - a]; a_row0: address of entry 0 of the row group's first row, `stride` bytes per row
+template <int J, int RK, bool F64, bool NL, bool COUNT>
+__device__ __forceinline__ void tree_scan(const TreeArgs &ta, u32 a_prev, u32 a_row0, u32 stride, int j0, int cnt, int a, int b, const TreeLevels &lv,
+                                          double K, double (&best)[J], int (&arg)[J], u32 &splits)
+{
+#pragma unroll
+    for (int i = 0; i < J; ++i) { best[i] = kTreeBound; arg[i] = 0; }
+    const int end = b < lv.nx ? b : lv.nx;
+    if (a > end) return;
+    int n = a, r = RK == 2 && !NL ? (int)(a > lv.b0) : (a > lv.b0) + (a > lv.b1) + (a > lv.b2);
+    int change = RK == 2 && !NL ? (r == 0 ? lv.b0 + 1 : kNever) : tree_bound(lv, r) + 1;     // first length of the next level
+    u32 a_row = a_row0 + (NL ? 0u : (u32)r * stride);
+    double tau = NL ? ta.tau[r] : 0.0;
+    double C[J], F[J], p[J], q[J], f[J];
+    u32 pa = a_prev, k0 = 8u * (u32)(j0 - a);                     // cell 0's entries: prev, and offset in a row
+    {
+        const u32 aj = a_row + 8u * (u32)j0;
+#pragma unroll
+        for (int i = 0; i < J; ++i) {
+            C[i] = lds_f64(aj + 8u * i);                          // (entries past the last layer are other words of the record)
+            if (!F64) C[i] += K;
+            F[i] = NL ? lds_f64(aj + 8u * i + stride) : 0.0;
+            p[i] = lds_f64(pa + 8u * i);
+            q[i] = lds_f64(a_row + k0 + 8u * i);
+            f[i] = NL ? lds_f64(a_row + k0 + 8u * i + stride) : 0.0;
+        }
+    }
+    while (true) {
+        double last[J];
+#pragma unroll
+        for (int s = 0; s < J; ++s) {
+            if (s == 0 || n + s <= end) {
+                if (n + s == change) {                            // the next level's row: the whole window is read anew
+                    do { ++r; } while (RK != 2 && n + s > tree_bound(lv, r));
+                    change = RK == 2 ? kNever : tree_bound(lv, r) + 1;
+                    if (NL) tau = ta.tau[r];
+                    else {
+                        a_row = a_row0 + (u32)r * stride;
+                        const u32 aj = a_row + 8u * (u32)j0;
+#pragma unroll
+                        for (int i = 0; i < J; ++i) {
+                            C[i] = lds_f64(aj + 8u * i);
+                            if (!F64) C[i] += K;
+                            q[(i - s) & (J - 1)] = lds_f64(a_row + k0 + 8u * i - 8u * s);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < J; ++i) {
+                    const int w = (i - s) & (J - 1);
+                    const double c = tree_span<F64, NL>(C[i], q[w], F[i], f[w], K, tau);
+                    const double v = p[w] > c ? p[w] : c;
+                    if (v <= best[i]) { best[i] = v; arg[i] = n + s; }
+                    last[i] = c;
+                    if (COUNT) splits += i < cnt ? 1u : 0u;
+                }
+                // the entry that leaves the window is that of cell J-1; the next one lies below cell 0's
+                const int w = (J - 1 - s) & (J - 1);
+                p[w] = lds_f64(pa - 8u * (s + 1));
+                q[w] = lds_f64(a_row + k0 - 8u * (s + 1));
+                if (NL) f[w] = lds_f64(a_row + k0 + stride - 8u * (s + 1));
+            }
+        }
+        n += J; pa -= 8u * J; k0 -= 8u * J;
+        if (n > end) break;
+        // costs grow with the length (the host sends policies whose higher levels repeat less forward work to the general
+        // kernel): once they exceed all the minima, longer stages cannot win
+        bool over = true;
+#pragma unroll
+        for (int i = 0; i < J; ++i) over = over && last[i] > best[i];
+        if (over) break;
+    }
+}
+
+template <bool SEARCH, bool F64, int RK, bool NL, bool COUNT>
+__global__ void __launch_bounds__(kTreeThreads, kTreeBlocksPerSm)
+tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ u32 s_item, s_unit, s_total[HAP_MAX_PP + 2];
+    __shared__ uint4 s_entry;
+    __shared__ double s_zero[2 * kTreePad + 1];             // the row before the first stage: 0 at layer 0
+    __shared__ i64 s_cost[kTreeWarps];
+    __shared__ u64 s_index[kTreeWarps];
+    __shared__ int s_last;
+    const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
+    const int N = ta.N, T = ta.T, R = ta.R, n1 = N + 1, n_rc = ta.n_rc, RW = NL ? 2 : R;
+    const i64 inf_bits = F64 ? 0x7ff0000000000000ll : kInf;
+    const double dInfOut = F64 ? __longlong_as_double(0x7ff0000000000000ll) : kTreeInf;
+
+    i64 best_cost = inf_bits;               // (non-negative doubles order like their bit patterns)
+    u64 best_index = ~0ull;
+    u32 n_feas = 0, splits = 0;
+    u64 plan_n[2][HAP_MAX_PP / 8], plan_r[2][HAP_MAX_PP / 8];    // the plan at hand and the plan of the thread's best candidate
+    i64 plan_val[2][4];
+    u32 plan_cur = 0;
+
+    // A second launch of the same pass starts once every block of the first is running, i.e. past the first one's wait for
+    // the records; it waits for the first launch itself only at its end.
+    if (ta.launch == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    const bool ordered = SEARCH && !F64 && ta.order != nullptr;
+    if (tid == 0) {
+        if (blockIdx.x == 0 && ta.launch == 0) ta.report->stamp[1] = global_timer();
+        for (int q = 0; q < 2 * kTreePad + 1; ++q) s_zero[q] = q == kTreePad ? 0.0 : kTreeInf;
+        u32 t = 0;                          // items before class c (in order of the bounds: configurations)
+        for (int c = ta.c_lo; c < ta.c_hi; ++c) {
+            s_total[c - ta.c_lo] = t;
+            const u32 live = __ldcg(&ta.state->live[c]), cpi = (u32)ta.cls[c].conf_per_item;
+            t += ordered ? live : (live + cpi - 1) / cpi * (u32)ta.cls[c].items_per_conf;
+        }
+        s_total[ta.c_hi - ta.c_lo] = t;
+        s_item = blockIdx.x;
+    }
+    __syncthreads();
+    const u32 a_zero = smem_u32(s_zero), n_total = s_total[ta.c_hi - ta.c_lo];
+    // in order of the bounds: the configuration an item belongs to, by one warp; none left where the bucket of the next one
+    // lies above the incumbent, like those of all that follow
+    auto locate = [&](u32 item) {
+        u32 lo = 0, hi = n_total + 1;       // order[lo].x <= item; order[hi].x > item, or hi is past the last one
+        while (hi - lo > 1) {
+            const u32 step = (hi - lo + 31) / 32, at = lo + (u32)lane * step;
+            const u32 n = __popc(__ballot_sync(0xffffffffu, at < hi && __ldcg(&ta.order[at].x) <= item));
+            lo += (n - 1) * step;
+            hi = lo + step < hi ? lo + step : hi;
+        }
+        const uint4 en = __ldcg(ta.order + lo);
+        if (lane == 0) {
+            const bool none = lo >= n_total || (u64)order_edge((int)(en.y >> 8)) > ~*reinterpret_cast<volatile const u64 *>(&ta.state->incumbent);
+            s_item = none ? ~0u : item;
+            s_entry = en;
+        }
+    };
+    if (ordered) {
+        __syncthreads();
+        if (wib == 0) locate(blockIdx.x);
+        __syncthreads();
+    }
+
+    while (true) {
+        const u32 item = s_item;
+        if (item >= (ordered ? ~0u : n_total)) break;
+        u32 next_item = 0;
+        if (tid == 0) next_item = atomicAdd(&ta.state->ticket[ta.launch], 1u) + gridDim.x;
+        int ci = ta.c_lo;
+        if (ordered) ci = (int)(s_entry.y & 255u);
+        else while (item >= s_total[ci + 1 - ta.c_lo]) ++ci;
+        const TreeClass *cl = ta.cls + ci;
+        const u32 local = ordered ? item - s_entry.x : item - s_total[ci - ta.c_lo], ipc = (u32)cl->items_per_conf, cpi = ordered ? 1u : (u32)cl->conf_per_item;
+        const u32 live = __ldcg(&ta.state->live[ci]);
+        const u32 conf0 = ordered ? s_entry.z : local / ipc * cpi, sub = local % ipc;
+        const u32 n_confs = conf0 + cpi <= live ? cpi : live - conf0;
+        const u32 n_parts = (u32)cl->n_parts, part0 = n_parts * sub / ipc, part1 = n_parts * (sub + 1) / ipc;
+        const u32 rec_bytes = cl->rec_bytes;
+        const int PP = cl->PP;
+        // records of the item's configurations into shared memory
+        {
+            const unsigned char *src = ta.rec + cl->rec_off + (u64)conf0 * rec_bytes;
+            const u32 total = n_confs * rec_bytes, dst = smem_u32(smem_raw);
+            for (u32 q = (u32)tid * 16u; q < total; q += kTreeThreads * 16u)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + q), "l"(src + q) : "memory");
+            if (tid == 0) s_unit = 0;
+            asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+        const u32 slice_bytes = (cl->buf_cells[0] + cl->buf_cells[1]) * 8u + cl->ch_bytes;
+        const u32 a_slice = smem_u32(smem_raw) + cpi * rec_bytes + (u32)wib * slice_bytes;
+        const u32 a_buf[2] = {a_slice, a_slice + cl->buf_cells[0] * 8u};
+        const u32 a_ch = a_buf[1] + cl->buf_cells[1] * 8u;
+        const u32 o_thr = cl->o_thr, o_nf = cl->o_thr_nf, o_rows = cl->o_rows, o_minfo = cl->o_minfo;
+        const bool all_flat = cl->all_flat != 0;
+        const bool packed = ta.kind_uniform && cl->n_mrows <= 4;       // sync and optimizer terms from the longest stage per row group
+        const u32 units = n_confs * (part1 - part0), row_stride = (u32)n1 * 8u, row_group = (u32)RW * row_stride;
+
+        while (true) {
+            u32 u = 0;
+            if (lane == 0) u = atomicAdd(&s_unit, 1u);
+            u = __shfl_sync(0xffffffffu, u, 0);
+            if (u >= units) break;
+            const u32 conf = u / (part1 - part0);
+            const TreePart *pt = cl->parts + part0 + u % (part1 - part0);
+            const unsigned char *rec = smem_raw + conf * rec_bytes;
+            const TreeHead *hd = reinterpret_cast<const TreeHead *>(rec);
+            const u32 a_rec = smem_u32(rec);
+            const u32 nmap = pt->nmap;
+            const u64 c_lo = hd->offset + (u64)pt->m_lo * (u64)n_rc, c_hi = c_lo + (u64)nmap * (u64)n_rc;
+            const u64 w_lo = out.first, w_hi = out.first + out.count;
+            if (c_hi <= w_lo || c_lo >= w_hi) continue;
+            const bool whole = c_lo >= w_lo && c_hi <= w_hi;
+            if (SEARCH && out.prune) {
+                // a part whose configuration's lower bound exceeds the incumbent cannot hold the minimum (strict); one lane
+                // reads the moving incumbent and the warp follows it as a whole
+                int skip = 0;
+                if (lane == 0) skip = (u64)hd->lb > ~*reinterpret_cast<volatile const u64 *>(&ta.state->incumbent);
+                skip = __shfl_sync(0xffffffffu, skip, 0);
+                if (skip) continue;
+                if (lane == 0) atomicAdd(&ta.state->n_pruned, 0ull - ((c_hi < w_hi ? c_hi : w_hi) - (c_lo > w_lo ? c_lo : w_lo)));
+            }
+            unsigned without_plan = 0;          // positions in rc_order under which no mapping was feasible
+            const TreeTask *tasks = pt->tasks;
+
+            for (int pos = 0; pos < n_rc; ++pos) {
+                const int rc_idx = ta.rc_order[pos];
+                const unsigned rc_mask = ta.rc_masks[rc_idx];
+                bool dead = ((hd->dead_policies >> pos) & 1u) || (ta.rc_sup[pos] & without_plan) != 0;
+                // levels at a depth whose spans mix layer kinds: per end layer
+                auto nf_levels = [&](int d, int capt, int j) {
+                    const u32 w = cl->nf_w[d], a = a_rec + o_nf + cl->nf_off[d] + (u32)(capt * R) * w + (u32)(j - (int)cl->jlo[d]);
+                    u32 len4 = 0;
+                    for (int r = 0; r < R; ++r) len4 |= (u32)lds_u8(a + (u32)r * w) << (8 * r);
+                    return tree_levels(R, rc_mask, len4);
+                };
+
+                // ---- rows of the tree, depth by depth ------------------------------------------------------
+                if (!dead && PP > 1) {
+                    u32 e_end = pt->task_lo[2];
+                    u32 e = (u32)lane;
+                    TreeTask nxt = make_uint4(0, 0, 0, 0);
+                    if (e < e_end) nxt = __ldg(tasks + e);
+                    for (int d = 1; d < PP; ++d) {
+                        const u32 cell0 = pt->cell_lo[d];
+                        const u32 next_end = d + 1 < PP ? pt->task_lo[d + 2] : e_end;
+                        const bool flat = all_flat || cl->flat[d];
+                        const u32 a_cur = a_buf[d & 1];
+                        const u32 a_prv = d == 1 ? a_zero : a_buf[(d & 1) ^ 1];
+                        bool alive = false;
+                        while (e < e_end) {
+                            const TreeTask t = nxt;
+                            e += 32u;
+                            if (e < e_end) nxt = __ldg(tasks + e);
+                            const int j0 = (int)(t.y & 255u), a = (int)(t.y >> 8) & 255, b = (int)(t.y >> 16) & 255, cnt = ((int)(t.y >> 24) & 3) + 1;
+                            const u32 kidx = t.z & 255u, mrow = (t.z >> 8) & 255u;
+                            const int capt = (int)(t.z >> 16);
+                            const double K = lds_f64(a_rec + kTreeOffKtab + 8u * kidx);
+                            const u32 a_row0 = a_rec + o_rows + mrow * row_group, slot = t.x >> 16;
+                            const u32 a_prev = a_prv + 8u * (t.x & 0xffffu), a_out = a_cur + 8u * slot, a_cho = a_ch + cell0 + slot;
+                            constexpr int J = NL && kTreeJ > 2 ? kTreeJ / 2 : kTreeJ;
+                            if (flat) {
+                                const TreeLevels lv = tree_levels(R, rc_mask, lds_u32(a_rec + o_thr + 4u * (u32)((d - 1) * T + capt)));
+#pragma unroll
+                                for (int h = 0; h < kTreeJ; h += J) {
+                                    if (h && h >= cnt) break;
+                                    double best[J];
+                                    int arg[J];
+                                    tree_scan<J, RK, F64, NL, COUNT>(ta, a_prev + 8u * h, a_row0, row_stride, j0 + h, cnt - h, a, b, lv, K, best, arg, splits);
+#pragma unroll
+                                    for (int i = 0; i < J; ++i)
+                                        if (h + i < cnt) {
+                                            if (HAP_CHECK_OK(1, slot + h + i < cl->buf_cells[d & 1])) sts_f64(a_out + 8u * (h + i), arg[i] ? best[i] : kTreeInf);
+                                            if (HAP_CHECK_OK(2, cell0 + slot + h + i < cl->ch_bytes)) sts_u8(a_cho + h + i, (u32)arg[i]);
+                                            alive |= arg[i] != 0;
+                                        }
+                                }
+                            } else {
+                                for (int i = 0; i < cnt; ++i) {                     // thresholds by end layer
+                                    double best[1];
+                                    int arg[1];
+                                    const TreeLevels lv = nf_levels(d, capt, j0 + i);
+                                    tree_scan<1, RK, F64, NL, COUNT>(ta, a_prev + 8u * i, a_row0, row_stride, j0 + i, 1, a, b, lv, K, best, arg, splits);
+                                    if (HAP_CHECK_OK(1, slot + i < cl->buf_cells[d & 1])) sts_f64(a_out + 8u * i, arg[0] ? best[0] : kTreeInf);
+                                    if (HAP_CHECK_OK(2, cell0 + slot + i < cl->ch_bytes)) sts_u8(a_cho + i, (u32)arg[0]);
+                                    alive |= arg[0] != 0;
+                                }
+                            }
+                            if (t.y & (1u << 26)) {                                 // the row's padding
+#pragma unroll
+                                for (int i = 1; i <= kTreePad; ++i) sts_f64(a_out - 8u * i, kTreeInf);
+                            }
+                            if (t.y & (1u << 27)) {
+#pragma unroll
+                                for (int i = 0; i < kTreePad; ++i) sts_f64(a_out + 8u * (cnt + i), kTreeInf);
+                            }
+                        }
+                        // the first record of the next depth is requested before this depth is closed
+                        e = e_end + (u32)lane;
+                        e_end = next_end;
+                        if (d + 1 < PP && e < e_end) nxt = __ldg(tasks + e);
+                        __syncwarp();
+                        if (!__any_sync(0xffffffffu, alive)) { dead = true; break; }      // no cell of this depth is finite: nothing below is
+                    }
+                }
+                // ---- one lane per mapping: cell (PP, N), walk back, Eq. 4 ----------------------------------------
+                bool any_plan = false;
+                const u32 a_last = PP == 1 ? a_zero : a_buf[(PP - 1) & 1];
+                for (u32 m = (u32)lane; m < nmap; m += 32u) {
+                    const u64 c = c_lo + (u64)m * (u64)n_rc + (u64)rc_idx;
+                    if (c < w_lo || c >= w_hi) continue;
+                    const u64 o = c - w_lo;
+                    if (!HAP_CHECK_OK(3, o < out.count)) continue;
+                    double bott = kTreeInf;
+                    int n = 0;
+                    const u32 *path = pt->path + m;
+                    u32 pw = 0;
+                    if (!dead) {
+                        pw = __ldg(path + (size_t)(PP - 1) * nmap);
+                        const u32 lf = __ldg(pt->leaf + m);
+                        const int a = (int)(lf & 255u), b = (int)(lf >> 8) & 255;
+                        const u32 kidx = (pw >> 20) & 63u, mrow = (pw >> 26) & 15u;
+                        const int capt = (int)(pw >> 30);
+                        if (a <= b) {
+                            const double K = lds_f64(a_rec + kTreeOffKtab + 8u * kidx) + lds_f64(a_rec + o_minfo + (mrow * kTreeMinfo + 6) * 8u);
+                            const TreeLevels lv = all_flat || cl->flat[PP] ? tree_levels(R, rc_mask, lds_u32(a_rec + o_thr + 4u * (u32)((PP - 1) * T + capt)))
+                                                                           : nf_levels(PP, capt, N);
+                            double best[1];
+                            int arg[1];
+                            tree_scan<1, RK, F64, NL, COUNT>(ta, a_last + 8u * (pw & 0xfffffu), a_rec + o_rows + mrow * row_group, row_stride, N, 1, a, b, lv, K,
+                                                             best, arg, splits);
+                            bott = best[0]; n = arg[0];
+                        }
+                    }
+                    if (n == 0) {
+                        if (!SEARCH) {
+                            if (out.cost) out.cost[o] = inf_bits;
+                            if (out.bottleneck) out.bottleneck[o] = inf_bits;
+                            const uint4 z = make_uint4(0, 0, 0, 0);
+                            if (out.partition) { uint4 *d = reinterpret_cast<uint4 *>(out.partition + o * HAP_MAX_PP); d[0] = z; d[1] = z; }
+                            if (out.recompute) { uint4 *d = reinterpret_cast<uint4 *>(out.recompute + o * HAP_MAX_PP); d[0] = z; d[1] = z; }
+                        }
+                        continue;
+                    }
+                    double sum = 0.0, t_sync = 0.0, t_opt = 0.0, het = 0.0;
+                    u32 most = 0;                                                  // per row group the longest stage, a byte each (packed)
+                    u64 acc_n = 0, acc_r = 0;
+                    const bool want_plan = SEARCH ? true : (out.partition != nullptr || out.recompute != nullptr);
+                    int b = N;
+                    for (int d = PP; d >= 1; --d) {
+                        const u32 pn = d > 1 ? __ldg(path + (size_t)(d - 2) * nmap) : 0u;       // the stage before: asked for early
+                        const int kidx = (int)(pw >> 20) & 63, capt = (int)(pw >> 30);
+                        const u32 mrow = (pw >> 26) & 15u;
+                        if (!HAP_CHECK_OK(5, n >= 1 && n <= b && b <= N)) break;
+                        double K = lds_f64(a_rec + kTreeOffKtab + 8u * (u32)kidx);
+                        const u32 a_mi = a_rec + o_minfo + mrow * (kTreeMinfo * 8u);
+                        if (d == PP) K += lds_f64(a_mi + 48u);
+                        // lowest allowed level whose longest stage holds n layers
+                        const TreeLevels lv = all_flat || cl->flat[d] ? tree_levels(R, rc_mask, lds_u32(a_rec + o_thr + 4u * (u32)((d - 1) * T + capt)))
+                                                                      : nf_levels(d, capt, b);
+                        const int r = RK == 2 && !NL ? (int)(n > lv.b0) : (n > lv.b0) + (n > lv.b1) + (n > lv.b2);
+                        const u32 a_row = a_rec + o_rows + mrow * row_group + (NL ? 0u : (u32)r * row_stride);
+                        double cst = lds_f64(a_row + 8u * (u32)b) - lds_f64(a_row + 8u * (u32)(b - n));
+                        if (NL) {
+                            const double t = (lds_f64(a_row + 8u * (u32)(n1 + b)) - lds_f64(a_row + 8u * (u32)(n1 + b - n))) * ta.tau[r];
+                            cst += F64 ? t : __dadd_rd(t, 4503599627370496.0) - 4503599627370496.0;
+                        }
+                        cst += K;
+                        sum += cst;
+                        int n_moe = n;
+                        if (packed) {                                          // sync and optimizer terms follow below
+                            most = __vmaxu4(most, (u32)n << (8u * mrow));
+                            n_moe = ta.kind0 == HAP_MOE ? n : 0;
+                        } else {
+                            n_moe = moe_before(dc, b) - moe_before(dc, b - n);
+                            const double dm = (double)n_moe, dd = (double)(n - n_moe);
+                            const double sy = lds_f64(a_mi) + dd * lds_f64(a_mi + 8u) + dm * lds_f64(a_mi + 16u);
+                            const double op = dd * lds_f64(a_mi + 24u) + dm * lds_f64(a_mi + 32u);
+                            t_sync = sy > t_sync ? sy : t_sync; t_opt = op > t_opt ? op : t_opt;
+                        }
+                        if (ta.eta_q > 0) {                                    // Pruning 3: cross-type transfer into the stage; dispatch of a mixed-type stage
+                            if (d > 1 && (kidx - 16) % 6 >= 2) het += lds_f64(a_rec + kTreeOffKtab + 8u * (u32)kidx);
+                            het += (double)n_moe * lds_f64(a_mi + 40u);
+                        }
+                        if (want_plan) {
+                            // layers and levels of eight stages in a word, stage d in byte (d - 1) & 7
+                            acc_n = (acc_n << 8) | (u64)(u32)n; acc_r = (acc_r << 8) | (u64)(u32)r;
+                            if (((d - 1) & 7) == 0) {
+                                const int w = (d - 1) >> 3;
+                                if (SEARCH) { plan_n[plan_cur][w] = acc_n; plan_r[plan_cur][w] = acc_r; }
+                                else {
+                                    if (out.partition) reinterpret_cast<u64 *>(out.partition + o * HAP_MAX_PP)[w] = acc_n;
+                                    if (out.recompute) reinterpret_cast<u64 *>(out.recompute + o * HAP_MAX_PP)[w] = acc_r;
+                                }
+                                acc_n = 0; acc_r = 0;
+                            }
+                        }
+                        b -= n;
+                        pw = pn;
+                        if (d > 1) {
+                            const u32 at = (pw & 0xfffffu) + (u32)b - 256u;
+                            if (!HAP_CHECK_OK(2, at < cl->ch_bytes)) break;
+                            n = lds_u8(a_ch + at);
+                        }
+                    }
+                    if (packed)
+                        for (int g = 0; g < cl->n_mrows; ++g) {                // the terms grow with the stage: the longest one of a row group counts
+                            const u32 len = (most >> (8 * g)) & 255u;
+                            const u32 a_mi = a_rec + o_minfo + (u32)(g * kTreeMinfo) * 8u;
+                            const double dn = (double)len;
+                            const double sy = lds_f64(a_mi) + dn * lds_f64(a_mi + 8u + 8u * (u32)ta.kind0), op = dn * lds_f64(a_mi + 24u + 8u * (u32)ta.kind0);
+                            if (len) { t_sync = sy > t_sync ? sy : t_sync; t_opt = op > t_opt ? op : t_opt; }
+                        }
+                    const double mxc = bott;                                   // the largest stage cost is the cell's value
+                    i64 T_iter, T_pipe;                                        // (bit patterns in fp64 mode)
+                    bool keep = true;
+                    if (F64) {
+                        const double tp = sum + (double)hd->m1 * mxc;
+                        if (ta.eta_q > 0 && het * (double)PP * 1024.0 > (double)ta.eta_q * sum) keep = false;
+                        T_pipe = __double_as_longlong(keep ? tp : dInfOut);
+                        T_iter = __double_as_longlong(keep ? tp + t_sync + t_opt : dInfOut);
+                    } else {
+                        const i64 s = (i64)sum;
+                        T_pipe = s + hd->m1 * (i64)mxc;
+                        T_iter = T_pipe + (i64)t_sync + (i64)t_opt;
+                        if (ta.eta_q > 0 && (i64)het * (i64)PP * 1024 > (i64)ta.eta_q * s) { keep = false; T_iter = kInf; T_pipe = kInf; }   // Pruning 3
+                    }
+                    const i64 bott_bits = F64 ? __double_as_longlong(bott) : (i64)bott;
+                    if (SEARCH) {
+                        if (keep) { n_feas++; any_plan = true; }
+                        if (T_iter < best_cost || (T_iter == best_cost && c < best_index)) {
+                            best_cost = T_iter; best_index = c;
+                            plan_val[plan_cur][0] = bott_bits; plan_val[plan_cur][1] = T_pipe;
+                            plan_val[plan_cur][2] = F64 ? __double_as_longlong(t_sync) : (i64)t_sync;
+                            plan_val[plan_cur][3] = F64 ? __double_as_longlong(t_opt) : (i64)t_opt;
+                            plan_cur ^= 1u;                                    // the place just filled is kept, the other one is written next
+                        }
+                    } else {
+                        any_plan = true;
+                        if (out.cost) out.cost[o] = T_iter;
+                        if (out.bottleneck) out.bottleneck[o] = bott_bits;
+                        for (int w = keep ? (PP + 7) >> 3 : 0; w < HAP_MAX_PP / 8; ++w) {
+                            if (out.partition) reinterpret_cast<u64 *>(out.partition + o * HAP_MAX_PP)[w] = 0;
+                            if (out.recompute) reinterpret_cast<u64 *>(out.recompute + o * HAP_MAX_PP)[w] = 0;
+                        }
+                    }
+                }
+                // (also keeps the next policy from overwriting rows and choices that other lanes still read)
+                const int plan = __any_sync(0xffffffffu, any_plan);
+                // a policy under which none of the part's mappings has a feasible partition settles its subsets
+                if (!plan && whole && ta.eta_q <= 0) without_plan |= 1u << pos;
+                __syncwarp();
+            }
+            if (SEARCH && out.prune) {
+                // the incumbent moves on after every part
+                i64 bc = best_cost;
+#pragma unroll
+                for (int s = 16; s > 0; s >>= 1) { const i64 v = __shfl_xor_sync(0xffffffffu, bc, s); bc = v < bc ? v : bc; }
+                if (lane == 0 && bc < inf_bits) atomicMax(&ta.state->incumbent, ~(u64)bc);
+            }
+        }
+        __syncthreads();                        // every warp is done with the item's records
+        if (ordered) { if (wib == 0) locate(__shfl_sync(0xffffffffu, next_item, 0)); }
+        else if (tid == 0) s_item = next_item;
+        __syncthreads();
+    }
+
+    if (COUNT) {
+        const u64 s = (u64)warp_sum_i64((i64)splits);
+        if (lane == 0 && s) atomicAdd(&ta.state->splits, s);
+    }
+    if (SEARCH) {
+        const u64 nf = (u64)warp_sum_i64((i64)n_feas);
+        if (lane == 0 && nf) atomicAdd(&ta.state->n_feasible, nf);
+        i64 bc = best_cost; u64 bi = best_index;
+        warp_argmin(bc, bi);
+        if (lane == 0) { s_cost[wib] = bc; s_index[wib] = bi; }
+        __syncthreads();
+        bc = s_cost[0]; bi = s_index[0];
+        for (int q = 1; q < kTreeWarps; ++q) if (s_cost[q] < bc || (s_cost[q] == bc && s_index[q] < bi)) { bc = s_cost[q]; bi = s_index[q]; }
+        const u32 slot = ta.slot_lo + blockIdx.x;
+        if (tid == 0) { ta.slot_cost[slot] = bc; ta.slot_index[slot] = bi; }
+        if (bc < inf_bits && best_index == bi) {
+            // the thread that evaluated the block's best candidate leaves its plan
+            PlanSlot *ps = ta.slots + slot;
+            const u32 kp = plan_cur ^ 1u;
+            ps->bott = plan_val[kp][0]; ps->T_pipe = plan_val[kp][1]; ps->T_sync = plan_val[kp][2]; ps->T_opt = plan_val[kp][3];
+            for (int w = 0; w < HAP_MAX_PP / 8; ++w) {                       // (words of later stages are whatever the thread's memory held)
+                reinterpret_cast<u64 *>(ps->n)[w] = plan_n[kp][w];
+                reinterpret_cast<u64 *>(ps->r)[w] = plan_r[kp][w];
+            }
+        }
+    }
+    // ---- the last block of the pass -------------------------------------------------------------------------------------
+    if (ta.launch != 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(&ta.state->blocks_done, 1u) + 1u == ta.blocks_total;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    if (tid == 0) {
+        ta.report->n_feasible = __ldcg(&ta.state->n_feasible); ta.report->n_pruned = __ldcg(&ta.state->n_pruned);
+        ta.report->splits = __ldcg(&ta.state->splits);
+        ta.report->stamp[2] = global_timer();
+    }
+    __syncthreads();
+    static_assert(sizeof(TreeState) % 4 == 0, "cleared in words");
+    for (int q = tid; q < (int)(sizeof(TreeState) / 4); q += kTreeThreads) reinterpret_cast<u32 *>(ta.state)[q] = 0;
+    if (!SEARCH || !ta.res_dev) return;
+    i64 bc = inf_bits; u64 bi = ~0ull; u32 at = 0;
+    for (u32 q = (u32)tid; q < ta.blocks_total; q += kTreeThreads) {
+        const i64 v = __ldcg(ta.slot_cost + q); const u64 ix = __ldcg(ta.slot_index + q);
+        if (v < bc || (v == bc && ix < bi)) { bc = v; bi = ix; at = q; }
+    }
+    const u64 mine = bi;
+    const i64 mine_c = bc;
+    warp_argmin(bc, bi);
+    if (lane == 0) { s_cost[wib] = bc; s_index[wib] = bi; }
+    __syncthreads();
+    bc = s_cost[0]; bi = s_index[0];
+    for (int q = 1; q < kTreeWarps; ++q) if (s_cost[q] < bc || (s_cost[q] == bc && s_index[q] < bi)) { bc = s_cost[q]; bi = s_index[q]; }
+    // the winner's slot: (cost, index) pairs are distinct unless nothing is feasible
+    if (bc < inf_bits && mine == bi && mine_c == bc) s_item = at;
+    __syncthreads();
+    if (wib != 0) return;
+    TreeResult *rs = ta.res_dev, *rh = ta.res_host;
+    for (int copy = 0; copy < 2; ++copy) {
+        TreeResult *w = copy == 0 ? rs : rh;
+        if (!w) continue;
+        if (lane == 0) {
+            w->range_flag = __ldcg(ta.range_flag);
+            w->n_feasible = __ldcg(&ta.report->n_feasible); w->n_pruned = __ldcg(&ta.report->n_pruned);
+            w->cost = bc; w->index = bi;
+            for (int q = 0; q < 3; ++q) w->stamp[q] = __ldcg(&ta.report->stamp[q]);
+        }
+        if (!(bc < inf_bits)) continue;
+        const u64 p = find_pconf(dc, bi);
+        const hap_pconf pc = dc.pconf[p];
+        const u64 loc = bi - pc.offset, map_idx = loc / (u64)n_rc;
+        const StageMap sm = decode_stage(dc, pc, map_idx, lane);
+        const PlanSlot *ps = ta.slots + s_item;
+        if (lane == 0) {
+            w->pconf = (u32)p; w->rc_mask = ta.rc_masks[loc - map_idx * (u64)n_rc];
+            w->bott = __ldcg(&ps->bott); w->T_pipe = __ldcg(&ps->T_pipe); w->T_sync = __ldcg(&ps->T_sync); w->T_opt = __ldcg(&ps->T_opt);
+        }
+        w->mask[lane] = lane < pc.PP ? (uint8_t)sm.mask : 0;
+        w->n[lane] = lane < pc.PP ? __ldcg(ps->n + lane) : 0;
+        w->r[lane] = lane < pc.PP ? __ldcg(ps->r + lane) : 0;
+    }
+    __threadfence_system();
+}
+
+}  // namespace hap

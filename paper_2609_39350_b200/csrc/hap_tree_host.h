@@ -1,0 +1,425 @@
+// Host side of the prefix trees: the mappings of a PP class, their windows and bands, the tree's split into parts and the
+// task lists that tree_dp_kernel walks.  Everything here depends on the cluster, the stage count, the layer kinds and
+// the window only, never on the profiled tables.
+#pragma once
+#include "hap_tree.cuh"
+
+#include <algorithm>
+#include <cstring>
+#include <vector>
+
+namespace hap {
+
+struct TreePartHost {
+    TreePart meta{};                        // pointers are filled in at the upload
+    std::vector<TreeTask> tasks;
+    std::vector<u32> path, leaf;
+};
+
+struct TreeClassHost {
+    bool ok = false;                        // false: the class runs one warp per candidate
+    unsigned masks_used = 0xffffffffu;      // type masks that occur (the general kernel builds rows for those only)
+    TreeClass cls{};
+    std::vector<TreePartHost> parts;
+};
+
+struct TreeInputs {
+    const DevConst *dc;                     // N, T, m, node_size, P, cap_eff, kind_uniform_from, delta_q, uniform, R, tau_linear
+    hap_pconf rep;                          // any configuration of the class
+    size_t n_conf;
+    bool want_tree;
+};
+
+constexpr u64 kTreeMaxMappings = 1u << 18;
+constexpr size_t kTreeSliceBytes = 9216;  // a warp's rows and choices: what lets five blocks of four warps share an SM
+
+class TreeBuilder {
+public:
+    explicit TreeBuilder(const TreeInputs &in) : in_(in), dc_(*in.dc), N_(in.dc->N), PP_(in.rep.PP), T_(in.dc->T) {}
+
+    void build(TreeClassHost &out)
+    {
+        nmap_ = in_.rep.nmap;
+        if (nmap_ == 0 || nmap_ > kTreeMaxMappings) return;
+        decode();
+        out.masks_used = 0;
+        for (size_t q = 0; q < mask_.size(); ++q) out.masks_used |= 1u << mask_[q];
+        if (!in_.want_tree || !windows()) return;
+        out.ok = class_fields(out.cls) && split(out);
+    }
+
+private:
+    struct Node { u32 parent, rowoff; uint8_t mask, link, nmin, nmax; int bl, bh; };
+    struct Part { u64 m0, m1; std::vector<std::vector<Node>> lv; std::vector<u32> leaf_node; };
+
+    // the class's mappings in enumeration order (decode_stage unranks single ones; here they follow one another)
+    void decode()
+    {
+        mask_.resize((size_t)nmap_ * PP_); link_.resize((size_t)nmap_ * PP_);
+        if (in_.rep.mode != HAP_MAP_MULTISET) {
+            for (u64 m = 0; m < nmap_; ++m)
+                for (int s = 0; s < PP_; ++s) {
+                    const StageMap sm = decode_stage(dc_, in_.rep, m, s);
+                    mask_[(size_t)m * PP_ + s] = (uint8_t)sm.mask;
+                    link_[(size_t)m * PP_ + s] = (uint8_t)(s > 0 ? (sm.cls | (sm.ha << 2) | (sm.hb << 4)) : 0);
+                }
+            return;
+        }
+        const i64 G = in_.rep.G;
+        std::vector<uint8_t> seq;
+        std::vector<uint8_t> same[HAP_MAX_TYPES];               // link class into the q-th stage of a type from the one before it
+        for (int h = 0; h < T_; ++h) {
+            const int cnt = (int)(dc_.m[h] / G);
+            for (int q = 0; q < cnt; ++q) {
+                seq.push_back((uint8_t)h);
+                const i64 first = (i64)q * G;
+                same[h].push_back((first - 1) / dc_.node_size[h] == first / dc_.node_size[h] ? HAP_INTRA : HAP_INTER);
+            }
+        }
+        u64 m = 0;
+        do {
+            int used[HAP_MAX_TYPES] = {0, 0, 0, 0};
+            for (int s = 0; s < PP_; ++s) {
+                const int h = seq[s], q = used[h]++;
+                mask_[(size_t)m * PP_ + s] = (uint8_t)(1 << h);
+                const int cls = s == 0 ? 0 : seq[s - 1] != h ? HAP_CROSS : same[h][q];
+                link_[(size_t)m * PP_ + s] = (uint8_t)(s > 0 ? (cls | (seq[s - 1] << 2) | (h << 4)) : 0);
+            }
+            ++m;
+        } while (m < nmap_ && std::next_permutation(seq.begin(), seq.end()));
+    }
+
+    // load-balance window of every stage and band of reachable end layers, by the formulas of pipeline_dp_kernel
+    bool windows()
+    {
+        nmin_.resize(mask_.size()); nmax_.resize(mask_.size()); bl_.resize(mask_.size()); bh_.resize(mask_.size()); dead_.assign((size_t)nmap_, 0);
+        i64 Pmin[1 << HAP_MAX_TYPES] = {0};
+        for (int mk = 1; mk < (1 << T_); ++mk) {
+            bool seen = false, capseen = false;
+            i64 cap = 0;
+            for (int h = 0; h < T_; ++h)
+                if (mk >> h & 1) {
+                    if (!seen || dc_.P[h] < Pmin[mk]) Pmin[mk] = dc_.P[h];
+                    if (!capseen || dc_.cap_eff[h] < cap) { cap = dc_.cap_eff[h]; capt_[mk] = h; }
+                    seen = capseen = true;
+                }
+        }
+        // the window of a stage depends on its type mask and on the mapping's summed compute power only
+        i64 win_Ps = -1;
+        int win_lo[1 << HAP_MAX_TYPES], win_hi[1 << HAP_MAX_TYPES];
+        std::vector<int> lo(PP_), hi(PP_);
+        for (u64 m = 0; m < nmap_; ++m) {
+            const size_t at = (size_t)m * PP_;
+            i64 Ps = 0;
+            for (int s = 0; s < PP_; ++s) {
+                const int mk = mask_[at + s];
+                if (mk < 1 || mk >= (1 << T_)) return false;
+                Ps += Pmin[mk];
+            }
+            if (!dc_.uniform && dc_.delta_q >= 0 && Ps != win_Ps) {
+                const i64 den = 1024 * Ps;
+                for (int mk = 1; mk < (1 << T_); ++mk) {
+                    i64 a = ((i64)(1024 - dc_.delta_q) * Pmin[mk] * N_) / den;
+                    i64 b = ((i64)(1024 + dc_.delta_q) * Pmin[mk] * N_ + den - 1) / den;
+                    if (a < 1) a = 1;
+                    if (b > N_ - PP_ + 1) b = N_ - PP_ + 1;
+                    win_lo[mk] = (int)a; win_hi[mk] = (int)b;
+                }
+                win_Ps = Ps;
+            }
+            int tmin = 0, tmax = 0;
+            for (int s = 0; s < PP_; ++s) {
+                lo[s] = 1; hi[s] = N_ - PP_ + 1;
+                if (dc_.uniform) { lo[s] = N_ / PP_; hi[s] = (N_ + PP_ - 1) / PP_; }
+                else if (dc_.delta_q >= 0) { lo[s] = win_lo[mask_[at + s]]; hi[s] = win_hi[mask_[at + s]]; }
+                if (lo[s] < 0 || lo[s] > 255 || hi[s] < 0 || hi[s] > 255) return false;
+                tmin += lo[s]; tmax += hi[s];
+            }
+            int smin = 0, smax = 0;
+            for (int s = 0; s < PP_; ++s) {
+                smin += lo[s]; smax += hi[s];
+                int a = std::max(smin, s + 1), b = std::min(smax, N_ - PP_ + s + 1);
+                a = std::max(a, N_ - (tmax - smax)); b = std::min(b, N_ - (tmin - smin));
+                if (a > b) dead_[m] = 1;
+                nmin_[at + s] = (uint8_t)lo[s]; nmax_[at + s] = (uint8_t)hi[s];
+                bl_[at + s] = (uint8_t)std::max(0, std::min(255, a)); bh_[at + s] = (uint8_t)std::max(0, std::min(255, b));
+            }
+        }
+        return true;
+    }
+
+    // distinct stage prefixes of mappings [m0, m1); a node's band is the union over the mappings below it, which only adds
+    // cells that hold their plain recurrence value
+    void nodes(u64 m0, u64 m1, Part &pt) const
+    {
+        pt.m0 = m0; pt.m1 = m1;
+        pt.lv.assign(PP_ + 1, {});
+        pt.leaf_node.assign((size_t)(m1 - m0), 0);
+        std::vector<u32> path(PP_ + 1, 0);
+        std::vector<size_t> key(PP_ + 1, 0);                    // position of the stage the path's node was made from
+        bool have = false;
+        for (u64 m = m0; m < m1; ++m) {
+            if (dead_[m]) continue;
+            const size_t at = (size_t)m * PP_;
+            int d0 = 1;
+            if (have)
+                for (; d0 < PP_; ++d0) {
+                    const size_t a = key[d0], b = at + d0 - 1;
+                    if (mask_[a] != mask_[b] || link_[a] != link_[b] || nmin_[a] != nmin_[b] || nmax_[a] != nmax_[b]) break;
+                }
+            for (int d = d0; d < PP_; ++d) {
+                const size_t b = at + d - 1;
+                path[d] = (u32)pt.lv[d].size(); key[d] = b;
+                pt.lv[d].push_back(Node{d > 1 ? path[d - 1] : 0, 0, mask_[b], link_[b], nmin_[b], nmax_[b], 1 << 20, -1});
+            }
+            have = true;
+            for (int d = 1; d < PP_; ++d) {
+                Node &nd = pt.lv[d][path[d]];
+                nd.bl = std::min(nd.bl, (int)bl_[at + d - 1]); nd.bh = std::max(nd.bh, (int)bh_[at + d - 1]);
+            }
+            pt.leaf_node[(size_t)(m - m0)] = PP_ > 1 ? path[PP_ - 1] : 0;
+        }
+        // nodes of a depth by the width of their band, then of their window (widest first): the lanes of a warp get runs of
+        // similar length
+        for (int d = 1; d < PP_; ++d) {
+            std::vector<u32> ord(pt.lv[d].size()), newidx(pt.lv[d].size());
+            for (size_t i = 0; i < ord.size(); ++i) ord[i] = (u32)i;
+            std::stable_sort(ord.begin(), ord.end(), [&](u32 a, u32 b) {
+                const Node &x = pt.lv[d][a], &y = pt.lv[d][b];
+                const int wx = x.bh - x.bl, wy = y.bh - y.bl;
+                return wx != wy ? wx > wy : (int)x.nmax - (int)x.nmin > (int)y.nmax - (int)y.nmin; });
+            std::vector<Node> sorted(pt.lv[d].size());
+            for (size_t i = 0; i < ord.size(); ++i) { sorted[i] = pt.lv[d][ord[i]]; newidx[ord[i]] = (u32)i; }
+            pt.lv[d].swap(sorted);
+            if (d + 1 < PP_) for (auto &ch : pt.lv[d + 1]) ch.parent = newidx[ch.parent];
+            else for (u64 m = m0; m < m1; ++m) if (!dead_[m]) pt.leaf_node[(size_t)(m - m0)] = newidx[pt.leaf_node[(size_t)(m - m0)]];
+            u32 c = 0;
+            for (auto &nd : pt.lv[d]) { c += kTreePad; nd.rowoff = c; c += (u32)(nd.bh - nd.bl + 1); }
+        }
+    }
+
+    int kidx(int d, uint8_t mask, uint8_t link, const TreeClass &cl) const
+    {
+        const int cls = link & 3, ha = (link >> 2) & 3, hb = (link >> 4) & 3;
+        return d == 1 ? cl.mrow_of[mask] : 16 + hb * 6 + (cls == HAP_CROSS ? 2 + ha : cls);
+    }
+
+    // row groups, windows, thresholds and the layout of a configuration's record
+    bool class_fields(TreeClass &cl)
+    {
+        const int R = dc_.R;
+        cl.PP = PP_;
+        std::memset(cl.mrow_of, 255, sizeof(cl.mrow_of));
+        unsigned used = 0;
+        for (size_t q = 0; q < mask_.size(); ++q) used |= 1u << mask_[q];
+        for (int mk = 1; mk < (1 << T_); ++mk)
+            if ((used >> mk) & 1u) { cl.mrow_of[mk] = (uint8_t)cl.n_mrows; cl.mask_of_row[cl.n_mrows] = (uint8_t)mk; cl.n_mrows++; }
+        Part all;
+        nodes(0, nmap_, all);
+        std::memset(cl.first_min, 255, sizeof(cl.first_min));
+        for (int d = 1; d <= PP_; ++d) { cl.jlo[d] = 255; cl.jhi[d] = 0; cl.kmin[d] = 255; cl.kmax[d] = 0; }
+        auto see_split = [&](int d, int j, const Node &nd, int pbl, int pbh) {
+            const int klo = std::max(j - (int)nd.nmax, pbl), khi = std::min(j - (int)nd.nmin, pbh);
+            if (klo > khi) return;
+            cl.kmin[d] = (uint8_t)std::min<int>(cl.kmin[d], klo); cl.kmax[d] = (uint8_t)std::max<int>(cl.kmax[d], khi);
+        };
+        for (int d = 1; d < PP_; ++d)
+            for (const Node &nd : all.lv[d]) {
+                const int t = capt_[nd.mask];
+                cl.jlo[d] = (uint8_t)std::min<int>(cl.jlo[d], nd.bl); cl.jhi[d] = (uint8_t)std::max<int>(cl.jhi[d], nd.bh);
+                cl.wmax[d] = std::max(cl.wmax[d], nd.nmax);
+                cl.tmask[d] |= (uint8_t)(1u << t);
+                if (d == 1) cl.first_min[t] = (uint8_t)std::min<int>(cl.first_min[t], nd.bl);
+                const int pbl = d > 1 ? all.lv[d - 1][nd.parent].bl : 0, pbh = d > 1 ? all.lv[d - 1][nd.parent].bh : 0;
+                for (int j = nd.bl; j <= nd.bh; ++j) see_split(d, j, nd, pbl, pbh);
+            }
+        cl.jlo[PP_] = cl.jhi[PP_] = (uint8_t)N_;
+        for (u64 m = 0; m < nmap_; ++m) {
+            if (dead_[m]) continue;
+            const size_t at = (size_t)m * PP_ + PP_ - 1;
+            const int t = capt_[mask_[at]];
+            cl.wmax[PP_] = std::max(cl.wmax[PP_], nmax_[at]);
+            cl.tmask[PP_] |= (uint8_t)(1u << t);
+            if (PP_ == 1) cl.first_min[t] = (uint8_t)N_;
+            Node lf{};
+            lf.nmin = nmin_[at]; lf.nmax = nmax_[at];
+            const int pbl = PP_ > 1 ? all.lv[PP_ - 1][all.leaf_node[(size_t)m]].bl : 0, pbh = PP_ > 1 ? all.lv[PP_ - 1][all.leaf_node[(size_t)m]].bh : 0;
+            see_split(PP_, N_, lf, pbl, pbh);
+        }
+        // A depth whose cells only look at splits behind the last change of layer kind sees spans of one kind only: their
+        // memory depends on the length alone.  All depths of a model whose layers are all of one kind; every depth but the
+        // first few of a model with a dense prefix.
+        u32 nf = 0;
+        cl.all_flat = 1;
+        for (int d = 1; d <= PP_; ++d) {
+            cl.flat[d] = (cl.kmin[d] > cl.kmax[d] || (int)cl.kmin[d] >= dc_.kind_uniform_from) ? 1 : 0;
+            if (cl.flat[d]) continue;
+            cl.all_flat = 0;
+            cl.nf_off[d] = nf; cl.nf_w[d] = (u32)(cl.jhi[d] - cl.jlo[d] + 1);
+            nf += (u32)(T_ * R) * cl.nf_w[d];
+        }
+        auto up16 = [](u32 v) { return (v + 15) / 16 * 16; };
+        const int RW = dc_.tau_linear ? R : 2;
+        cl.o_minfo = kTreeOffMinfo;
+        cl.o_rows = up16(cl.o_minfo + (u32)(cl.n_mrows * kTreeMinfo * 8));
+        cl.o_thr = up16(cl.o_rows + (u32)(cl.n_mrows * RW * (N_ + 1) * 8));
+        cl.o_thr_nf = cl.o_thr + up16((u32)(PP_ * T_ * 4));
+        cl.rec_bytes = up16(cl.o_thr_nf + nf);
+        return true;
+    }
+
+    // warp instructions of a part, roughly: what the split is chosen by
+    void cost(const Part &pt, double &total, size_t &slice) const
+    {
+        u32 cells[2] = {0, 0}, ch = 0;
+        total = 0;
+        for (int d = 1; d < PP_; ++d) {
+            u32 n_tasks = 0, c = kTreePad;
+            int w = 1;
+            for (const Node &nd : pt.lv[d]) {
+                const int b = nd.bh - nd.bl + 1;
+                n_tasks += (u32)((b + kTreeJ - 1) / kTreeJ); c += (u32)b + kTreePad;
+                w = std::max(w, (int)nd.nmax - (int)nd.nmin + 1);
+            }
+            cells[d & 1] = std::max(cells[d & 1], c); ch += c;
+            total += (double)((n_tasks + 31) / 32) * (150.0 + 42.0 * std::min(w, d == 1 ? kTreeJ : w));
+        }
+        total += (double)((pt.m1 - pt.m0 + 31) / 32) * (150.0 + 50.0 * PP_);
+        slice = ((size_t)((cells[0] + 1) / 2 * 2) + (cells[1] + 1) / 2 * 2) * 8 + (ch + 15) / 16 * 16;
+    }
+
+    bool split(TreeClassHost &out)
+    {
+        // Parts over contiguous ranges of mappings: the few nodes near the root that two parts share are computed by both, so
+        // smaller parts cost little; more parts shorten the longest chain, fewer fill the lanes of a warp better.  Score =
+        // work of the class spread over the chip + the chain of one part.
+        TreeClass &cl = out.cls;
+        int best_np = 0;
+        double best = 0;
+        size_t best_slice = 0;
+        for (u64 np : {1, 2, 3, 4, 6, 8, 12, 16, 20, 24, 28, 32, 40, 48, 56, 64, 80, 96, 128, 192, 256, 384, 512, 768, 1024, 2048, 4096, 8192}) {
+            if (np > nmap_) break;
+            std::vector<Part> parts((size_t)np);
+            for (u64 q = 0; q < np; ++q) nodes(nmap_ * q / np, nmap_ * (q + 1) / np, parts[(size_t)q]);
+            double work = 0, longest = 0;
+            size_t slice = 0;
+            for (const Part &pt : parts) {
+                double c; size_t s;
+                cost(pt, c, s);
+                work += c; longest = std::max(longest, c); slice = std::max(slice, s);
+            }
+            const double score = work * (double)in_.n_conf / 380.0 + 4.0 * longest;
+            const bool fits = slice <= kTreeSliceBytes, best_fits = best_np && best_slice <= kTreeSliceBytes;
+            if (!best_np || (fits && (!best_fits || score < best)) || (!fits && !best_fits && slice < best_slice)) {
+                best_np = (int)np; best = score; best_slice = slice;
+            }
+            if (best_slice <= kTreeSliceBytes && best_np != (int)np && score > 1.5 * best) break;
+        }
+        cl.n_parts = best_np;
+        out.parts.resize((size_t)best_np);
+        for (int q = 0; q < best_np; ++q) {
+            Part pt;
+            nodes(nmap_ * q / best_np, nmap_ * (q + 1) / best_np, pt);
+            if (!emit(pt, cl, out.parts[(size_t)q])) return false;
+        }
+        return true;
+    }
+
+    bool emit(const Part &pt, TreeClass &cl, TreePartHost &ph) const
+    {
+        TreePart &tp = ph.meta;
+        const u32 nmap = (u32)(pt.m1 - pt.m0);
+        tp.nmap = nmap; tp.m_lo = (u32)pt.m0;
+        u32 cells = 0, buf[2] = {0, 0};
+        std::vector<u32> cell_lo(PP_ + 1, 0);
+        for (int d = 1; d < PP_; ++d) {
+            tp.task_lo[d] = (u32)ph.tasks.size();
+            tp.cell_lo[d] = cells;
+            u32 c = kTreePad;
+            for (size_t ni = 0; ni < pt.lv[d].size(); ++ni) {
+                const Node &nd = pt.lv[d][ni];
+                const Node *pn = d > 1 ? &pt.lv[d - 1][nd.parent] : nullptr;
+                // slot of the parent's entry 0 (before the first stage: one row of layer 0 behind its padding)
+                const int pbl = pn ? pn->bl : 0, pbh = pn ? pn->bh : 0, porg = pn ? (int)pn->rowoff - pn->bl : kTreePad;
+                for (int j = nd.bl; j <= nd.bh; j += kTreeJ) {
+                    const int cnt = std::min(kTreeJ, nd.bh - j + 1);
+                    const int a = std::max((int)nd.nmin, j - pbh);
+                    int b = std::min((int)nd.nmax, j + cnt - 1 - pbl);
+                    if (a > b) b = a - 1;
+                    // (no length reaches the parent's row: the origin below only has to be a slot of it)
+                    const int src = a > b ? porg + pbl : porg + j - a, dst = (int)nd.rowoff + j - nd.bl;
+                    if (src < 0 || src > 65535 || dst > 65535) return false;
+                    TreeTask t;
+                    t.x = (u32)src | ((u32)dst << 16);
+                    t.y = (u32)j | ((u32)a << 8) | ((u32)b << 16) | ((u32)(cnt - 1) << 24) | (j == nd.bl ? 1u << 26 : 0u) |
+                          (ni + 1 == pt.lv[d].size() && j + kTreeJ > nd.bh ? 1u << 27 : 0u);
+                    t.z = (u32)kidx(d, nd.mask, nd.link, cl) | ((u32)cl.mrow_of[nd.mask] << 8) | ((u32)capt_[nd.mask] << 16);
+                    t.w = 0;
+                    ph.tasks.push_back(t);
+                }
+                c += (u32)(nd.bh - nd.bl + 1) + kTreePad;
+            }
+            buf[d & 1] = std::max(buf[d & 1], c);
+            cells += c;
+        }
+        for (int d = PP_; d <= HAP_MAX_PP; ++d) { tp.task_lo[d] = (u32)ph.tasks.size(); tp.cell_lo[d] = cells; }
+        if (cells >= (1u << 19)) return false;
+        for (int q = 0; q < 2; ++q) cl.buf_cells[q] = std::max(cl.buf_cells[q], (buf[q] + 1) / 2 * 2);
+        cl.ch_bytes = std::max(cl.ch_bytes, (cells + 15) / 16 * 16);
+        ph.path.assign((size_t)nmap * PP_, 0);
+        ph.leaf.assign(nmap, 1u);                               // a = 1 > b = 0
+        for (u32 m = 0; m < nmap; ++m) {
+            if (dead_[pt.m0 + m]) continue;
+            const size_t at = (size_t)(pt.m0 + m) * PP_;
+            u32 nd = PP_ > 1 ? pt.leaf_node[m] : 0;
+            // lengths of the last stage that reach the parent's row
+            const int pbl = PP_ > 1 ? pt.lv[PP_ - 1][nd].bl : 0, pbh = PP_ > 1 ? pt.lv[PP_ - 1][nd].bh : 0;
+            const int a = std::max((int)nmin_[at + PP_ - 1], N_ - pbh), b = std::min((int)nmax_[at + PP_ - 1], N_ - pbl);
+            if (a > b) continue;
+            ph.leaf[m] = (u32)a | ((u32)b << 8);
+            for (int d = PP_; d >= 1; --d) {
+                int org = PP_ > 1 ? 0 : kTreePad;
+                if (d == PP_) { if (PP_ > 1) { const Node &p = pt.lv[PP_ - 1][nd]; org = (int)p.rowoff - p.bl + N_ - a; } }
+                else { const Node &p = pt.lv[d][nd]; org = (int)tp.cell_lo[d] + (int)p.rowoff - p.bl + 256; nd = p.parent; }
+                ph.path[(size_t)(d - 1) * nmap + m] = (u32)org | ((u32)kidx(d, mask_[at + d - 1], link_[at + d - 1], cl) << 20) |
+                                                      ((u32)cl.mrow_of[mask_[at + d - 1]] << 26) | ((u32)capt_[mask_[at + d - 1]] << 30);
+            }
+        }
+        return true;
+    }
+
+    const TreeInputs &in_;
+    const DevConst &dc_;
+    const int N_, PP_, T_;
+    u64 nmap_ = 0;
+    std::vector<uint8_t> mask_, link_, nmin_, nmax_, bl_, bh_, dead_;
+    int capt_[1 << HAP_MAX_TYPES] = {0};
+};
+
+// How the parts of a class are handed out: an item is a group of a configuration's parts, or all parts of several
+// configurations (classes of few parts); its parts fill the warps of a block a whole number of times.
+inline void tree_items(TreeClass &cl)
+{
+    cl.items_per_conf = 1; cl.conf_per_item = 1;
+    const size_t units = (size_t)cl.n_conf * cl.n_parts, all_warps = (size_t)148 * kTreeBlocksPerSm * kTreeWarps;
+    if (cl.n_parts > kTreeWarps) cl.items_per_conf = (cl.n_parts + kTreeWarps - 1) / kTreeWarps;
+    else if (units > all_warps && cl.n_parts < kTreeWarps) {
+        // as many configurations as fill the warps, where their records fit
+        const u32 slice = (cl.buf_cells[0] + cl.buf_cells[1]) * 8 + cl.ch_bytes;
+        const u32 budget = 220 * 1024 / kTreeBlocksPerSm;
+        const u32 room = budget > kTreeWarps * slice ? budget - kTreeWarps * slice : 0;
+        cl.conf_per_item = std::max<int>(1, std::min<int>(kTreeWarps / cl.n_parts, (int)(room / cl.rec_bytes)));
+    }
+}
+
+inline size_t tree_smem_bytes(const TreeClass &cl)
+{
+    return (size_t)cl.conf_per_item * cl.rec_bytes + kTreeWarps * ((size_t)(cl.buf_cells[0] + cl.buf_cells[1]) * 8 + cl.ch_bytes) + 64;
+}
+
+inline size_t tree_prep_smem_bytes(const TreeClass &cl, int N, int T)
+{
+    return (size_t)T * N * 16 + (cl.rec_bytes - cl.o_thr + 15) / 16 * 16 + (size_t)(N + 1) * 17 + 32;
+}
+
+}  // namespace hap

@@ -1,0 +1,61 @@
+"""The tree kernel at the edges of its tasks and parts, against the oracle."""
+import os
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from gen import problems  # noqa: E402
+from oracle import Oracle, INF  # noqa: E402
+
+NTHREADS = max(1, len(os.sched_getaffinity(0)))
+
+# nodes per type, layers (rows end 0..3 layers into a task of four), levels (repeated fraction), policies, layer kinds
+CASES = [
+    ((1, 1), 4, (0, 1024), (3,), "uniform"),
+    ((2, 2), 9, (0, 1024), (1, 3), "dense_first"),
+    ((2, 1, 1), 18, (0, 307, 1024), (1, 3, 7), "dense_first"),         # levels that are not combined into rows
+    ((2, 1, 1), 23, (0, 1024, 2048), (7, 5, 4), "mixed"),
+    ((1, 1, 1, 1), 16, (0, 1024, 2048, 3072), (15, 9, 6, 1), "uniform"),
+    ((4, 2, 2), 25, (0, 200, 700, 1000), (15, 3), "dense_first"),
+]
+
+
+@pytest.mark.parametrize("nodes,N,tau,policies,kinds", CASES)
+def test_tree_tasks_and_levels(nodes, N, tau, policies, kinds):
+    import paper_2609_39350_b200 as hap
+    pb = problems.random_small(40 + N, N=N, T=len(nodes), nodes_per_type=nodes, node_size=2, window=N % 2 == 1, first_dense=kinds == "dense_first")
+    if kinds == "mixed":
+        pb.kind[3] = 0
+    R = len(tau)
+    pb.tau_q = np.array(tau, np.int32)
+    pb.xi_q = np.array([1024, 512, 200, 64][:R - 1] + [64], np.int32)
+    pb.rc_masks = np.array(policies, np.uint32)
+    o = Oracle(pb)
+    n, best, index, costs, _ = o.search_pconfs(0, 1, threads=NTHREADS, want_costs=True)
+    hp = hap.hap_problem_create(pb)
+    hap.hap_enumerate(hp)
+    out = hap.hap_pipeline_dp(hp, 0, hp.n_cand, partition=True)
+    torch.cuda.synchronize()
+    got = out["cost"].cpu().numpy()
+    bad = np.nonzero(got != costs)[0]
+    assert n == hp.n_cand and bad.size == 0, bad[:8]
+    part, rec = out["partition"].cpu().numpy(), out["recompute"].cpu().numpy()
+    for idx in np.random.default_rng(N).integers(0, o.n_cand, 60).tolist():
+        plan, _, _ = o.eval_index(idx)
+        if plan["T_iter"] < INF:
+            assert part[idx, :plan["PP"]].tolist() == plan["n"] and rec[idx, :plan["PP"]].tolist() == plan["r"], idx
+    hap.hap_problem_destroy(hp)
+    for prune in (0, 1):                       # in the order of the lists, in the order of the bounds
+        hp = hap.hap_problem_create(pb, prune=prune)
+        hap.hap_enumerate(hp)
+        if best < INF:
+            plan, st = hap.hap_search_best(hp)
+            assert (plan["index"], plan["T_iter"]) == (index, best)
+            assert st["n_evaluated"] + st["n_pruned"] == hp.n_cand
+        else:
+            with pytest.raises(hap.HapError):
+                hap.hap_search_best(hp)
+        hap.hap_problem_destroy(hp)
