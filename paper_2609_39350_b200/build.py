@@ -9,7 +9,8 @@ LIB = os.path.join(_DIR, "libhap.so")
 LIB_CHECKED = os.path.join(_DIR, "libhap_checked.so")      # the same sources with -DHAP_CHECKED (self-checking kernels)
 SOURCES = [os.path.join(_DIR, "csrc", "hap_api.cu")]
 HEADERS = [os.path.join(_DIR, "csrc", "hap_device.cuh"), os.path.join(_DIR, "csrc", "hap_tree.cuh"),
-           os.path.join(_DIR, "csrc", "hap_tree_host.h"), os.path.join(os.path.dirname(_DIR), "include", "hap.h")]
+           os.path.join(_DIR, "csrc", "hap_tree_host.h"), os.path.join(_DIR, "csrc", "hap_joint.cuh"),
+           os.path.join(os.path.dirname(_DIR), "include", "hap.h")]
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "--fmad=false", "-std=c++17",
               "-shared", "-Xcompiler", "-fPIC"]

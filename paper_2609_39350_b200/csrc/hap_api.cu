@@ -4,6 +4,7 @@
 #include "hap_device.cuh"
 #include "hap_tree.cuh"
 #include "hap_tree_host.h"
+#include "hap_joint.cuh"
 
 #include <algorithm>
 #include <cstdarg>
@@ -114,6 +115,9 @@ struct hap_problem {
     std::vector<JointHost> joint;
     i64 *d_joint_scratch = nullptr;
     int joint_grid = 0;
+    // ... in the form of a search over reachable end layers: by 64-bit words per state
+    struct ReachHost { std::vector<JointReach> classes; std::vector<unsigned> ids; unsigned char *d = nullptr; size_t o_ids = 0, smem = 0; };
+    ReachHost reach[2];
     bool joint_ready = false;
     TreeResult *host_result = nullptr;     // page-locked, mapped: the last block of a search writes the plan here
     int timed = 0;                         // 1: events around the last pass, 2: the tree kernels' own time stamps
@@ -459,6 +463,7 @@ static void release_device(hap_problem *p)
     if (p->in_flight) { cudaEventSynchronize(p->ev_done); p->in_flight = false; }
     cached_free(p->d_tables); cached_free(p->d_arena); cached_free(p->d_gen_arena);
     cached_free(p->d_joint_scratch);
+    for (auto &r : p->reach) cached_free(r.d);
     for (auto &j : p->joint) { cached_free(j.d_ids); cached_free(j.d_arrays); }
     cached_free(p->d_c2f); cached_free(p->d_coeff); cached_free(p->d_fcost); cached_free(p->d_cand_lb);
     for (auto &e : p->ev) if (e) cudaEventDestroy(e);
@@ -1660,6 +1665,75 @@ extern "C" hap_status hap_search_range_f64(hap_problem *p, uint64_t first, uint6
     return HAP_OK;
 }
 
+// The class's states as entries of joint_reach_kernel; false: its bits, masks or layer kinds do not fit that form.
+static bool joint_reach_class(const hap_problem *p, int PP, int64_t G, const JointClass &jc, const std::vector<int> &lvl_off,
+                              const std::vector<int> &st_idx, const std::vector<int> &slot, JointReach &jr, std::vector<unsigned> &ent)
+{
+    const int T = p->T, N = p->model.N;
+    jr = JointReach{};
+    jr.PP = PP; jr.lmax = jc.lmax; jr.nwin = 1;
+    if (jc.lmax > 0xffff) return false;
+    i64 Ps = 0;
+    for (int h = 0; h < T; ++h) Ps += (p->m[h] / G) * p->dc.P[h];
+    for (int h = 0; h < T; ++h) {
+        // the window of dp_prologue_thr
+        int lo = 1, hi = N - PP + 1;
+        if (p->dc.delta_q >= 0) {
+            const i64 den = 1024 * Ps, Ph = p->dc.P[h];
+            const i64 a = ((i64)(1024 - p->dc.delta_q) * Ph * N) / den, b = ((i64)(1024 + p->dc.delta_q) * Ph * N + den - 1) / den;
+            lo = a < 1 ? 1 : (int)a; hi = b > N - PP + 1 ? N - PP + 1 : (int)b;
+        }
+        if (p->dc.uniform) { lo = N / PP; hi = (N + PP - 1) / PP; }
+        jr.nmin[h] = lo; jr.nmax[h] = hi; jr.cnt[h] = jc.cnt[h];
+        if (lo < 1) return false;
+        if (jc.cnt[h] == 0) continue;
+        jr.nwin = std::max(jr.nwin, hi - lo + 1);
+        // behind the first stage every span is of one layer kind
+        if (PP > 1 && lo < p->dc.kind_uniform_from) return false;
+    }
+    int words = 1;
+    for (int i = 0; i <= PP; ++i) {
+        const int l0 = lvl_off[i], l1 = lvl_off[i + 1];
+        jr.n_states[i] = (unsigned)(l1 - l0);
+        int base = 1 << 20, top = -1;
+        std::vector<uint8_t> out((size_t)(l1 - l0), 0);
+        std::vector<int> u((size_t)(l1 - l0) * HAP_MAX_TYPES, 0);
+        for (int q = l0; q < l1; ++q) {
+            int smin = 0, smax = 0, rmin = 0, rmax = 0;
+            for (int h = 0; h < T; ++h) {
+                const int n = (st_idx[q] / jc.stride[h]) % (jc.cnt[h] + 1), left = jc.cnt[h] - n;
+                u[(size_t)(q - l0) * HAP_MAX_TYPES + h] = n;
+                smin += n * jr.nmin[h]; smax += n * jr.nmax[h]; rmin += left * jr.nmin[h]; rmax += left * jr.nmax[h];
+            }
+            const int bl = std::max(smin, N - rmax), bh = std::min(smax, N - rmin);
+            if (bl > bh) { out[(size_t)(q - l0)] = 1; continue; }
+            base = std::min(base, bl); top = std::max(top, bh);
+        }
+        jr.base[i] = top < 0 ? (i ? jr.base[i - 1] : 0) : base;
+        if (i >= 1 && i < PP && top >= 0) words = std::max(words, (top - base + 64) / 64);
+        jr.ent_off[i] = (unsigned)ent.size();
+        if (i == 1)
+            for (int h = 0; h < T; ++h) jr.first[h] = jc.cnt[h] > 0 ? (unsigned)slot[jc.stride[h]] : 0u;
+        if (i == PP - 1)
+            for (int h = 0; h < T; ++h) jr.fin[h] = jc.cnt[h] > 0 ? slot[jc.S - 1 - jc.stride[h]] : 0;
+        if (i < 2 || i >= PP) continue;
+        for (int t = 0; t < T; ++t)
+            for (int q = l0; q < l1; ++q) {
+                const int ut = u[(size_t)(q - l0) * HAP_MAX_TYPES + t];
+                unsigned e = (unsigned)t << 16;
+                if (ut > 0 && !out[(size_t)(q - l0)]) {
+                    const i64 first = (i64)(ut - 1) * G;
+                    const int same = (first - 1) / p->dc.node_size[t] == first / p->dc.node_size[t] ? 0 : 1;
+                    e |= (unsigned)slot[st_idx[q] - jc.stride[t]] | (unsigned)same << 18 | 1u << 19;
+                }
+                ent.push_back(e);
+            }
+    }
+    if (words > 2) return false;
+    jr.words = words;
+    return reach_smem(N, T, p->prof.R, p->dc.tau_linear ? p->prof.R : 2, PP, jc.lmax, jr.nwin, words).total <= 110 * 1024;
+}
+
 static hap_status joint_setup(hap_problem *p)
 {
     if (p->joint_ready) return HAP_OK;
@@ -1667,6 +1741,8 @@ static hap_status joint_setup(hap_problem *p)
     size_t lmax_all = 0;
     std::vector<int> pps;
     for (const auto &r : p->pconfs) if (std::find(pps.begin(), pps.end(), r.PP) == pps.end()) pps.push_back(r.PP);
+    std::sort(pps.begin(), pps.end(), std::greater<int>());      // the longest configurations start first
+    std::vector<unsigned> ent[2];
     for (int PP : pps) {
         const int64_t G = p->W / PP;
         bool homog = true;
@@ -1695,6 +1771,20 @@ static hap_status joint_setup(hap_problem *p)
         std::vector<int> fill(lvl_off.begin(), lvl_off.end() - 1);
         for (int ui = 0; ui < S; ++ui) { slot[ui] = fill[level[ui]] - lvl_off[level[ui]]; st_idx[fill[level[ui]]++] = ui; }
         jc.lmax = lmax;
+        JointReach jr;
+        std::vector<unsigned> en;
+        if (joint_reach_class(p, PP, G, jc, lvl_off, st_idx, slot, jr, en)) {
+            const int w = jr.words - 1;
+            hap_problem::ReachHost &rh = p->reach[w];
+            for (int i = 0; i <= HAP_MAX_PP; ++i) jr.ent_off[i] += (unsigned)ent[w].size();
+            jr.id_lo = (unsigned)rh.ids.size();
+            for (size_t pi = 0; pi < p->pconfs.size(); ++pi) if (p->pconfs[pi].PP == PP) rh.ids.push_back((unsigned)pi);
+            jr.n_ids = (unsigned)rh.ids.size() - jr.id_lo;
+            rh.smem = std::max<size_t>(rh.smem, reach_smem(N, T, p->prof.R, p->dc.tau_linear ? p->prof.R : 2, PP, lmax, jr.nwin, jr.words).total);
+            rh.classes.push_back(jr);
+            ent[w].insert(ent[w].end(), en.begin(), en.end());
+            continue;
+        }
         lmax_all = std::max(lmax_all, (size_t)lmax);
         std::vector<int> arrays;
         arrays.insert(arrays.end(), lvl_off.begin(), lvl_off.end());
@@ -1717,6 +1807,21 @@ static hap_status joint_setup(hap_problem *p)
         if (jh.smem > 227 * 1024) return fail(p, HAP_E_RANGE, "shared memory need of the joint recurrence exceeds the SM");
         p->joint.push_back(jh);
     }
+    for (int w = 0; w < 2; ++w) {
+        // classes | ids | entries
+        hap_problem::ReachHost &rh = p->reach[w];
+        if (rh.classes.empty()) continue;
+        auto up = [](size_t v) { return (v + 255) / 256 * 256; };
+        rh.o_ids = up(rh.classes.size() * sizeof(JointReach));
+        const size_t o_ent = rh.o_ids + up(rh.ids.size() * sizeof(unsigned)), total = o_ent + up(ent[w].size() * sizeof(unsigned));
+        CUDA_TRY(p, cached_malloc(p->device, (void **)&rh.d, total));
+        for (auto &c : rh.classes) c.ent = reinterpret_cast<const unsigned *>(rh.d + o_ent);
+        std::vector<unsigned char> img(total, 0);
+        std::memcpy(img.data(), rh.classes.data(), rh.classes.size() * sizeof(JointReach));
+        std::memcpy(img.data() + rh.o_ids, rh.ids.data(), rh.ids.size() * sizeof(unsigned));
+        if (!ent[w].empty()) std::memcpy(img.data() + o_ent, ent[w].data(), ent[w].size() * sizeof(unsigned));
+        CUDA_TRY(p, cudaMemcpy(rh.d, img.data(), total, cudaMemcpyHostToDevice));
+    }
     p->joint_grid = 2 * 148;
     if (lmax_all) {
         const size_t bytes = (size_t)p->joint_grid * 2 * lmax_all * T * (N + 1) * sizeof(i64);
@@ -1736,15 +1841,21 @@ extern "C" hap_status hap_joint_bottleneck(hap_problem *p, int64_t *dev_out, voi
     const size_t np = p->pconfs.size();
     CUDA_TRY(p, cudaMemsetAsync(dev_out, 0xff, np * p->opts.n_rc * sizeof(int64_t), st));     // -1: stages not homogeneous
     if ((s = launch_layer_costs(p, p->d_c2, p->d_coef, nullptr, nullptr, true, st)) != HAP_OK) return s;
-    static size_t smem_limit[64][2];
-    const int dev = p->device & 63;
     const bool lin = p->dc.tau_linear != 0;
+    for (int w = 0; w < 2; ++w) {
+        const hap_problem::ReachHost &rh = p->reach[w];
+        if (rh.classes.empty()) continue;
+        using Fn = void (*)(const DevConst, const JointReach *, int, const unsigned *, const i64 *, const i64 *, i64 *);
+        static const Fn fns[2][2] = {{joint_reach_kernel<false, 1>, joint_reach_kernel<false, 2>}, {joint_reach_kernel<true, 1>, joint_reach_kernel<true, 2>}};
+        const Fn fn = fns[lin][w];
+        CUDA_TRY(p, raise_smem_limit(p->device, (const void *)fn, rh.smem));
+        fn<<<(unsigned)rh.ids.size(), kReachThreads, rh.smem, st>>>(p->dc, reinterpret_cast<const JointReach *>(rh.d), (int)rh.classes.size(),
+                                                                    reinterpret_cast<const unsigned *>(rh.d + rh.o_ids), p->d_c2, p->d_coef, (i64 *)dev_out);
+        CUDA_TRY(p, cudaGetLastError());
+    }
     for (const auto &jh : p->joint) {
         const void *fn = lin ? (const void *)joint_dp_kernel<true> : (const void *)joint_dp_kernel<false>;
-        if (jh.smem > smem_limit[dev][lin]) {
-            CUDA_TRY(p, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)jh.smem));
-            smem_limit[dev][lin] = jh.smem;
-        }
+        CUDA_TRY(p, raise_smem_limit(p->device, fn, jh.smem));
         const unsigned n_ids = (unsigned)jh.ids.size();
         const unsigned grid = std::min<unsigned>(n_ids, (unsigned)p->joint_grid);
         // scratch slices are sized for the widest class

@@ -1,0 +1,43 @@
+"""The joint recurrence at the edges of its bit words (64 and 128 end layers a level; beyond them the form with a value per
+end layer), with a dense first layer and with levels that are not combined into rows, against the oracle."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from gen import problems  # noqa: E402
+from oracle import Oracle  # noqa: E402
+
+
+@pytest.mark.parametrize("nodes,N,window,tau,dense_first", [
+    ((2, 2), 8, True, (0, 1024), False),           # as many layers as stages
+    ((2, 2), 67, False, (0, 1024), False),         # 64 end layers at four stages: one word, the last bit of it
+    ((2, 2), 68, False, (0, 1024), False),         # 65: two words
+    ((2, 2), 75, False, (0, 1024), False),
+    ((2, 2), 67, True, (0, 307, 1024), True),
+    ((2, 1, 1), 130, False, (0, 1024), True),      # value form
+    ((1, 1, 1, 1), 21, True, (0, 1024, 2048), False),
+    ((4,), 33, True, (0, 500), False),             # one type
+])
+def test_joint_bottleneck_words(nodes, N, window, tau, dense_first):
+    import paper_2609_39350_b200 as hap
+    pb = problems.random_small(7 * N, N=N, T=len(nodes), nodes_per_type=nodes, node_size=2, window=window, first_dense=dense_first)
+    pb.cap_eff[:] = pb.cap_eff * max(1, N // 8)    # (some policies fit, some do not)
+    pb.tau_q = np.array(tau, np.int32)
+    pb.xi_q = np.array([1024, 512, 64][-len(tau):], np.int32)
+    pb.rc_masks = np.array([(1 << len(tau)) - 1, 1], np.uint32)
+    o = Oracle(pb)
+    hp = hap.hap_problem_create(pb)
+    hap.hap_enumerate(hp)
+    got = hap.hap_joint_bottleneck(hp).cpu().numpy()
+    seen = 0
+    for p in np.random.default_rng(N).permutation(o.n_pconf).tolist():
+        for rc in range(2):
+            if got[p, rc] == -1 or seen >= 60:
+                continue
+            c2, _, coef, _ = o.layer_costs(p)
+            assert got[p, rc] == o.joint_bottleneck(p, int(pb.rc_masks[rc]), c2, coef), (p, rc)
+            seen += 1
+    assert seen > 0
+    hap.hap_problem_destroy(hp)
