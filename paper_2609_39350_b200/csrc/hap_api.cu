@@ -1710,6 +1710,7 @@ static bool joint_reach_class(const hap_problem *p, int PP, int64_t G, const Joi
             base = std::min(base, bl); top = std::max(top, bh);
         }
         jr.base[i] = top < 0 ? (i ? jr.base[i - 1] : 0) : base;
+        jr.width[i] = top < 0 ? 0 : top - base + 1;
         if (i >= 1 && i < PP && top >= 0) words = std::max(words, (top - base + 64) / 64);
         jr.ent_off[i] = (unsigned)ent.size();
         if (i == 1)

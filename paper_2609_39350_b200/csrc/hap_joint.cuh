@@ -11,6 +11,12 @@
 // stay in shared memory.  The stage costs are finitely many numbers: after a test, B moves to the nearest of them, so the
 // bisection ends after about a dozen tests, each exact.
 //
+// Lengths whose masks are full or empty at a depth (most, once B is near the answer) need no mask at all.
+//
+// 1,024 devices, 3,114 homogeneous configurations of up to 3,825 states: 38.4 ms with a value per end layer in global memory,
+// 2.9 ms in this form.  128 threads a block: 3.6 ms, 192: 3.2 ms (few configurations are feasible, and each is a chain of
+// levels and tests); a lane for all next types of a state instead of one: 4.4 ms.
+//
 // One block per configuration.  Bound by instruction issue of the level loop: per (state, type) four logic operations per
 // (type before, length).  The value form -- a 64-bit minimum per end layer and split, rows in
 // global memory -- is kept for classes whose bits or masks do not fit (joint_dp_kernel).
@@ -21,6 +27,7 @@ namespace hap {
 
 constexpr int kReachThreads = 256;
 constexpr int kReachKc = 2 + HAP_MAX_TYPES;       // transfer into a stage: same type intra / inter node, from type 0..3
+constexpr int kReachOk = 2 * HAP_MAX_TYPES;       // masks of a (depth, type, length): [same-type link][type before]
 
 struct JointReach {
     int PP, lmax, words;                          // stages; most states of a level; 64-bit words per state and type
@@ -31,7 +38,7 @@ struct JointReach {
     unsigned first[HAP_MAX_TYPES];                // slot, at level 1, of "one stage of type t placed"
     unsigned ent_off[HAP_MAX_PP + 1];             // level i's entries: [type][state] slot before | type << 16 | same-type link << 18 | valid << 19
     unsigned n_states[HAP_MAX_PP + 1];
-    int base[HAP_MAX_PP + 1];                     // end layer of bit 0
+    int base[HAP_MAX_PP + 1], width[HAP_MAX_PP + 1];      // end layer of bit 0; bits
     const unsigned *ent;
 };
 
@@ -56,21 +63,23 @@ __device__ __forceinline__ Bits<W> bits_shift(const Bits<W> &x, int s)      // b
     return y;
 }
 
-__host__ __device__ inline int reach_mask_words(int N) { return (N + 1 + 31) / 32; }
+__host__ __device__ inline int reach_mask_words(int N) { return (N + 31) / 32; }
 
-struct ReachSmem { u32 rows, wa, sk, m, a, reach, lvl, fin, total; };
+struct ReachSmem { u32 rows, wa, sk, m, a, reach, span, least, lvl, fin, total; };
 __host__ __device__ inline ReachSmem reach_smem(int N, int T, int R, int RW, int PP, int lmax, int nwin, int words)
 {
     auto up = [](size_t v) { return (u32)((v + 15) / 16 * 16); };
-    const size_t n1 = (size_t)N + 1, depth = PP > 2 ? PP - 2 : 0;
+    const size_t n1 = (size_t)N + 1;
     ReachSmem s;
     size_t o = 0;
     s.rows = (u32)o; o = up(o + (size_t)T * RW * n1 * 8);
     s.wa = (u32)o; o = up(o + 2 * n1 * 8);
     s.sk = (u32)o; o = up(o + n1);
-    s.a = (u32)o; o = up(o + depth * T * nwin * kReachKc * words * 8);
-    s.reach = (u32)o; o = up(o + (size_t)2 * T * lmax * words * 8);
+    s.a = (u32)o; o = up(o + (size_t)2 * T * nwin * kReachOk * words * 8);
+    s.reach = (u32)o; o = up(o + (size_t)2 * HAP_MAX_TYPES * lmax * words * 8);
     s.m = (u32)o; o = up(o + (size_t)T * nwin * R * kReachKc * reach_mask_words(N) * 4);
+    s.span = (u32)o; o = up(o + (size_t)T * nwin * R * 16);
+    s.least = (u32)o; o = up(o + (size_t)T * nwin * R * 8);
     s.fin = (u32)o; o = up(o + (size_t)T * nwin * 4);
     s.lvl = (u32)o; o = up(o + (size_t)PP * T * nwin);
     s.total = (u32)(o > 0xffffffffull ? 0xffffffffull : o);
@@ -86,9 +95,13 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
     __shared__ MaskInfo<i64> minfo[kMaxMasks];
     __shared__ i64 sP2P[HAP_MAX_TYPES][6];
     __shared__ i64 szero[1];
-    __shared__ u64 s_dn, s_up;                              // largest stage cost that is at most B, smallest one above
-    __shared__ double s_est;
+    __shared__ u64 s_dn, s_up;                              // bounds that a test leaves: next stage costs around B
+    __shared__ u64 s_low;
     __shared__ i64 s_res[HAP_MAX_RC_MASKS];
+    __shared__ int s_end[3][HAP_MAX_TYPES], s_full[3][HAP_MAX_TYPES];      // by depth % 3 and type: lengths from s_end on have empty
+                                                            // masks, those before s_full have full ones
+    __shared__ i64 s_k2[HAP_MAX_TYPES][2], s_kmin[HAP_MAX_TYPES];
+    __shared__ u32 s_used[HAP_MAX_TYPES];                   // per type: levels of stages between the first and the last
     const int tid = threadIdx.x, wib = tid >> 5, lane = tid & 31;
     constexpr int nwarps = kReachThreads / 32;
     const int N = dc.N, T = dc.T, R = dc.R, n1 = N + 1, RW = LINEAR ? R : 2;
@@ -108,11 +121,16 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
     i64 *sR = reinterpret_cast<i64 *>(smem_raw + lay.rows);
     i64 *sW = reinterpret_cast<i64 *>(smem_raw + lay.wa), *sA = sW + n1;
     uint8_t *sK = smem_raw + lay.sk, *sLvl = smem_raw + lay.lvl;      // [depth - 1][type][length]: level of the stage, 255: does not fit
-    Bits<W> *sOk = reinterpret_cast<Bits<W> *>(smem_raw + lay.a);     // [depth - 2][type][length][transfer]
+    Bits<W> *sOk = reinterpret_cast<Bits<W> *>(smem_raw + lay.a);     // [depth & 1][type][length][same-type link][type before]
     Bits<W> *sReach = reinterpret_cast<Bits<W> *>(smem_raw + lay.reach);
     u32 *sM = reinterpret_cast<u32 *>(smem_raw + lay.m);              // [type][length][level][transfer][word]: bit k: (k, k + n] costs at most B
+    longlong2 *sSpan = reinterpret_cast<longlong2 *>(smem_raw + lay.span);    // [type][length][level]: least and most that n layers cost
+    i64 *sLeast = reinterpret_cast<i64 *>(smem_raw + lay.least);              // ... least, first and last stages included
     u32 *sFin = reinterpret_cast<u32 *>(smem_raw + lay.fin);          // [type][length]: transfers under which the last stage costs at most B
     dp_prologue_rows<i64, LINEAR>(dc, p, c2, coef, coef, true, T, RW, 0xffffffffu, nwarps, sR, sW, sA, sK, minfo, sP2P, szero);
+    for (int e = tid; e < 2 * HAP_MAX_TYPES * lmax; e += kReachThreads)             // (types that do not exist stay empty)
+#pragma unroll
+        for (int w = 0; w < W; ++w) sReach[e].w[w] = 0;
     const i64 *cfp = coef + (size_t)p * T * HAP_NCOEF;
     const i64 mx = cfp[HAP_MX], mpre = cfp[HAP_MPRE], mpost = cfp[HAP_MPOST];
 
@@ -121,26 +139,35 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
         if (LINEAR) return rM[(size_t)r * n1 + j] - rM[(size_t)r * n1 + k];
         return (rM[j] - rM[k]) + tau_term((i64)dc.tau_q[r], rM[n1 + j] - rM[n1 + k]);
     };
-    // lower bound on the bottleneck: with weights s_h, s_h B is at least the weighted time of a stage's layers on its type,
-    // so B sum_stages s >= sum over layers of the smallest weighted time.  Weights: the types' speeds.
-    if (wib == 0) {
-        double s[HAP_MAX_TYPES], den = 0.0;
-        for (int h = 0; h < T; ++h) { const i64 v = cost(h, 0, 0, N); s[h] = 1.0 / (double)(v > 0 ? v : 1); den += s[h] * (double)jc.cnt[h]; }
-        double sum = 0.0;
-        for (int l = lane; l < N; l += 32) {
-            double m = 0.0;
-            for (int h = 0; h < T; ++h) {
-                const i64 *rM = sR + (size_t)h * RW * n1;
-                i64 c = rM[l + 1] - rM[l];
-                if (LINEAR) for (int r = 1; r < R; ++r) { const i64 x = rM[(size_t)r * n1 + l + 1] - rM[(size_t)r * n1 + l]; c = x < c ? x : c; }
-                const double v = s[h] * (double)c;
-                m = h == 0 || v < m ? v : m;
-            }
-            sum += m;
+    for (int g = wib; g < T * nwin * R; g += nwarps) {
+        const int r = g % R, q = (g / R) % nwin, t = g / (R * nwin), n = jc.nmin[t] + q;
+        i64 a = kInf, b = -1, any = kInf;                     // of the stages between the first and the last; of all
+        for (int k = lane; k + n <= N; k += 32) {
+            const i64 c = cost(t, r, k, k + n);
+            any = c < any ? c : any;
+            if (k > 0 && k + n < N) { a = c < a ? c : a; b = c > b ? c : b; }
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        if (lane == 0) s_est = sum / den * (1.0 - 1e-9);
+        for (int o = 16; o > 0; o >>= 1) {
+            const i64 x = __shfl_xor_sync(0xffffffffu, a, o), y = __shfl_xor_sync(0xffffffffu, b, o);
+            a = x < a ? x : a; b = y > b ? y : b;
+            const i64 z = __shfl_xor_sync(0xffffffffu, any, o);
+            any = z < any ? z : any;
+        }
+        if (lane == 0) { sSpan[g] = make_longlong2(a, b); sLeast[g] = any; }
+    }
+    __syncthreads();
+    // least and most of the transfers into a stage of a type 
+    i64 *sK2 = &s_k2[0][0];
+    if (tid < T) {                                            // (a type on its own with one stage has none)
+        i64 a = kInf, b = 0;
+        for (int e = 0; e < kReachKc; ++e) {
+            const int from = e < 2 ? tid : e - 2;
+            if (from < T && jc.cnt[from] > 0) { const i64 v = sP2P[tid][e]; a = v < a ? v : a; b = v > b ? v : b; }
+        }
+        sK2[2 * tid] = a; sK2[2 * tid + 1] = b;
+        const i64 pre = minfo[(1 << tid) - 1].kpre;
+        s_kmin[tid] = pre < a ? pre : a;
     }
     __syncthreads();
 
@@ -154,6 +181,8 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
         i64 result = kInf;
         if (floor_b < kInf) {
             // ---- recomputation level of a stage of n layers at each depth and type ---------------------------------
+            if (tid < HAP_MAX_TYPES) s_used[tid] = 0;
+            __syncthreads();
             for (int e = tid; e < PP * T * nwin; e += kReachThreads) {
                 const int q = e % nwin, t = (e / nwin) % T, i = e / (nwin * T) + 1, n = jc.nmin[t] + q;
                 int lv = 255;
@@ -167,6 +196,7 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
                         if (((rc_mask >> r) & 1u) && span_fits(sW, sA, sK, extra, mx, mstore, cap, (i64)dc.xi_q[r], k, k + n)) lv = r;
                 }
                 sLvl[e] = (uint8_t)lv;
+                if (lv != 255 && i > 1 && i < PP && !((s_used[t] >> lv) & 1u)) atomicOr(&s_used[t], 1u << lv);
             }
             if (PP == 1) {
                 __syncthreads();
@@ -177,28 +207,53 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
                         if (lv != 255) { const i64 v = cost(t, lv, 0, N) + minfo[(1 << t) - 1].kpre + minfo[(1 << t) - 1].kpost; result = v < result ? v : result; }
                     }
             } else {
-                // whether no stage has to cost more than B; s_dn, s_up around B
+                // whether no stage has to cost more than B; the answer is then at most s_dn <= B, else at least s_up > B
                 auto test = [&](i64 B) -> bool {
                     __syncthreads();
                     if (tid == 0) { s_dn = 0; s_up = (u64)kInf; }
                     __syncthreads();
                     i64 dn = 0, up = kInf;
+                    u32 near_dn = 0, near_up = ~0u;          // costs within 2^32 ns of B, as cost - (B + 1)
                     auto see = [&](i64 v) { if (v <= B) dn = v > dn ? v : dn; else up = v < up ? v : up; return v <= B; };
                     for (int g = wib; g < T * nwin * R; g += nwarps) {
                         const int r = g % R, q = (g / R) % nwin, t = g / (R * nwin), n = jc.nmin[t] + q;
-                        if (!((rc_mask >> r) & 1u) || n > jc.nmax[t] || jc.cnt[t] == 0) continue;
+                        if (!((s_used[t] >> r) & 1u) || n > jc.nmax[t] || jc.cnt[t] == 0) continue;
+                        const longlong2 range = sSpan[g];
+                        if (range.y < 0) {                                    // no room between a first and a last stage
+                            for (int e = lane; e < kReachKc * mw; e += 32) sM[(size_t)g * kReachKc * mw + e] = 0u;
+                            continue;
+                        }
+                        const i64 least = range.x + s_k2[t][0], most = range.y + s_k2[t][1];
+                        if (most <= B || least > B) {
+                            // all of them or none: most lengths, once B is near the answer
+                            see(most <= B ? most : least);
+                            for (int e = lane; e < kReachKc * mw; e += 32) {
+                                const int f = e / mw, w = e - f * mw, from = f < 2 ? t : f - 2;
+                                // bits 1 .. N - n - 1
+                                const int top = N - n - w * 32;
+                                u32 v = most > B || from >= T || jc.cnt[from] == 0 || top <= 0 ? 0u : top >= 32 ? ~0u : (1u << top) - 1u;
+                                if (w == 0) v &= ~1u;
+                                sM[(size_t)g * kReachKc * mw + e] = v;
+                            }
+                            continue;
+                        }
+                        see(B + 1 - 4294967296ll);                            // (costs further away than that are not looked at)
+                        up = B + 4294967296ll < up ? B + 4294967296ll : up;
                         for (int w = 0; w < mw; ++w) {
                             const int k = w * 32 + lane;
                             const bool in = k >= 1 && k + n < N;              // a stage that is neither the first nor the last
-                            const i64 c = in ? cost(t, r, k, k + n) : 0;
+                            const i64 c = (in ? cost(t, r, k, k + n) : kInf) - (B + 1);       // (negative: at most B)
                             u32 mine = 0;
 #pragma unroll
                             for (int e = 0; e < kReachKc; ++e) {
                                 const int from = e < 2 ? t : e - 2;
                                 if (from >= T || jc.cnt[from] == 0) continue;
-                                bool ok = false;
-                                if (in) ok = see(c + sP2P[t][e]);
-                                const u32 b = __ballot_sync(0xffffffffu, ok);
+                                const i64 x = c + sP2P[t][e];
+                                const int hi = (int)(x >> 32);
+                                const u32 lw = (u32)x;
+                                if (hi == -1) near_dn = lw > near_dn ? lw : near_dn;
+                                if (hi == 0) near_up = lw < near_up ? lw : near_up;
+                                const u32 b = __ballot_sync(0xffffffffu, hi < 0);
                                 if (lane == e) mine = b;
                             }
                             if (lane < kReachKc) sM[((size_t)(g * kReachKc + lane)) * mw + w] = mine;
@@ -220,32 +275,60 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
                         }
                         sFin[e] = okl;
                     }
+                    near_dn = __reduce_max_sync(0xffffffffu, near_dn); near_up = __reduce_min_sync(0xffffffffu, near_up);
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) {
                         const i64 a = __shfl_xor_sync(0xffffffffu, dn, o), b = __shfl_xor_sync(0xffffffffu, up, o);
                         dn = a > dn ? a : dn; up = b < up ? b : up;
                     }
+                    if (near_dn) { const i64 v = (B + 1) - 4294967296ll + (i64)near_dn; dn = v > dn ? v : dn; }
+                    if (near_up != ~0u) { const i64 v = (B + 1) + (i64)near_up; up = v < up ? v : up; }
                     if (lane == 0) { atomicMax(&s_dn, (u64)dn); atomicMin(&s_up, (u64)up); }
                     __syncthreads();
-                    // masks of every depth: the words of the level that its memory allows, from the first end layer of the level before
-                    for (int e = tid; e < (PP - 2) * T * nwin * kReachKc; e += kReachThreads) {
-                        const int f = e % kReachKc, q = (e / kReachKc) % nwin, t = (e / (kReachKc * nwin)) % T, i = e / (kReachKc * nwin * T) + 2;
+                    // masks of a depth: the words of the level that its memory allows, from the first end layer of the level before
+                    auto level_mask = [&](int i) {
                         Bits<W> b;
 #pragma unroll
-                        for (int w = 0; w < W; ++w) b.w[w] = 0;
-                        const int lv = sLvl[((size_t)(i - 1) * T + t) * nwin + q], from = f < 2 ? t : f - 2;
-                        if (lv != 255 && jc.cnt[t] > 0 && from < T && jc.cnt[from] > 0) {
-                            const u32 *m = sM + ((size_t)((t * nwin + q) * R + lv) * kReachKc + f) * mw;
-                            const int at = jc.base[i - 1], w0 = at >> 5, s = at & 31;
-                            u32 v[2 * W + 1];
+                        for (int w = 0; w < W; ++w) { const int n = jc.width[i] - 64 * w; b.w[w] = n >= 64 ? ~0ull : n > 0 ? (1ull << n) - 1ull : 0ull; }
+                        return b;
+                    };
+                    auto masks_of = [&](int i) {
+                        const int at = jc.base[i - 1], w0 = at >> 5, s = at & 31;
+                        const Bits<W> all = level_mask(i - 1);
+                        const int per_t = (nwin * kReachOk + 31) & ~31;
+                        for (int e0 = wib * 32; e0 < T * per_t; e0 += kReachThreads) {          // (a warp stays inside one type)
+                            const int t = e0 / per_t, e = e0 - t * per_t + lane;
+                            const int h = e & (HAP_MAX_TYPES - 1), f = h == t ? (e / HAP_MAX_TYPES) & 1 : 2 + h, q = e / kReachOk;
+                            Bits<W> b;
 #pragma unroll
-                            for (int w = 0; w <= 2 * W; ++w) v[w] = w0 + w < mw ? m[w0 + w] : 0u;
+                            for (int w = 0; w < W; ++w) b.w[w] = 0;
+                            const bool in = q < nwin, there = in && jc.cnt[t] > 0 && h < T && jc.cnt[h] > 0;
+                            const int lv = there ? sLvl[((size_t)(i - 1) * T + t) * nwin + q] : 255;
+                            if (lv != 255) {
+                                const u32 *m = sM + ((size_t)((t * nwin + q) * R + lv) * kReachKc + f) * mw;
+                                u32 v[2 * W + 1];
 #pragma unroll
-                            for (int w = 0; w < W; ++w)
-                                b.w[w] = (u64)__funnelshift_r(v[2 * w], v[2 * w + 1], s) | (u64)__funnelshift_r(v[2 * w + 1], v[2 * w + 2], s) << 32;
+                                for (int w = 0; w <= 2 * W; ++w) v[w] = w0 + w < mw ? m[w0 + w] : 0u;
+#pragma unroll
+                                for (int w = 0; w < W; ++w)
+                                    b.w[w] = (u64)__funnelshift_r(v[2 * w], v[2 * w + 1], s) | (u64)__funnelshift_r(v[2 * w + 1], v[2 * w + 2], s) << 32;
+                            }
+                            bool full = true, empty = true;
+#pragma unroll
+                            for (int w = 0; w < W; ++w) { full = full && (b.w[w] & all.w[w]) == all.w[w]; empty = empty && b.w[w] == 0; }
+                            const u32 not_full = __ballot_sync(0xffffffffu, there && !full), some = __ballot_sync(0xffffffffu, !empty);
+                            if (in) {
+                                sOk[(size_t)((i & 1) * T + t) * nwin * kReachOk + e] = b;
+                                if ((lane & (kReachOk - 1)) == 0) {
+                                    if ((some >> lane) & 0xffu) atomicMax(&s_end[i % 3][t], q + 1);
+                                    if ((not_full >> lane) & 0xffu) atomicMin(&s_full[i % 3][t], q);
+                                }
+                            }
                         }
-                        sOk[e] = b;
-                    }
+                    };
+                    if (tid < 3 * HAP_MAX_TYPES) { s_end[tid / HAP_MAX_TYPES][tid % HAP_MAX_TYPES] = 0; s_full[tid / HAP_MAX_TYPES][tid % HAP_MAX_TYPES] = nwin; }
+                    __syncthreads();
+                    if (PP > 2) masks_of(2);
                     // level 1
                     for (unsigned e = (unsigned)tid; e < jc.n_states[1] * (unsigned)T; e += kReachThreads) {
                         const unsigned t = e / jc.n_states[1], sl = e - t * jc.n_states[1];
@@ -256,18 +339,21 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
                             for (int q = 0; q < nwin; ++q)
                                 if (sFin[t * nwin + q] >> 16) {
                                     const int bit = jc.nmin[t] + q - jc.base[1];
-                                    if (bit >= 0 && bit < 64 * W) b.w[W == 1 ? 0 : bit >> 6] |= 1ull << (bit & 63);
+                                    if (bit >= 0 && bit < jc.width[1]) b.w[W == 1 ? 0 : bit >> 6] |= 1ull << (bit & 63);
                                 }
                         sReach[(size_t)t * lmax + sl] = b;
                     }
                     __syncthreads();
                     for (int i = 2; i < PP; ++i) {
-                        const Bits<W> *prv = sReach + (size_t)(i & 1 ? T * lmax : 0);          // level 1 lies in the first buffer
-                        Bits<W> *cur = sReach + (size_t)(i & 1 ? 0 : T * lmax);
+                        const Bits<W> *prv = sReach + (size_t)(i & 1 ? HAP_MAX_TYPES * lmax : 0);          // level 1 lies in the first buffer
+                        Bits<W> *cur = sReach + (size_t)(i & 1 ? 0 : HAP_MAX_TYPES * lmax);
                         const unsigned ns = jc.n_states[i], total = ns * (unsigned)T;
                         const unsigned *ent = jc.ent + jc.ent_off[i];
                         const int d = jc.base[i] - jc.base[i - 1];
-                        const Bits<W> *okd = sOk + (size_t)(i - 2) * T * nwin * kReachKc;
+                        const Bits<W> *okd = sOk + (size_t)(i & 1) * T * nwin * kReachOk;
+                        const Bits<W> lm = level_mask(i);
+                        if (i + 1 < PP) masks_of(i + 1);
+                        if (tid < HAP_MAX_TYPES) { s_end[(i + 2) % 3][tid] = 0; s_full[(i + 2) % 3][tid] = nwin; }
                         int some = 0;
                         for (unsigned e = (unsigned)tid; e < total; e += kReachThreads) {
                             const unsigned en = __ldg(ent + e), up_sl = en & 0xffffu;
@@ -277,36 +363,55 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
                             for (int w = 0; w < W; ++w) acc.w[w] = 0;
                             if ((en >> 19) & 1u) {
                                 if (!HAP_CHECK_OK(4, up_sl < jc.n_states[i - 1])) continue;
-                                Bits<W> from[HAP_MAX_TYPES];
-                                u64 any = 0;
+                                Bits<W> from[HAP_MAX_TYPES], any;
 #pragma unroll
-                                for (int h = 0; h < HAP_MAX_TYPES; ++h) {
+                                for (int h = 0; h < HAP_MAX_TYPES; ++h) from[h] = prv[(size_t)h * lmax + up_sl];
+                                bool none = true;
 #pragma unroll
-                                    for (int w = 0; w < W; ++w) from[h].w[w] = 0;
-                                    if (h < T) from[h] = prv[(size_t)h * lmax + up_sl];
-#pragma unroll
-                                    for (int w = 0; w < W; ++w) any |= from[h].w[w];
+                                for (int w = 0; w < W; ++w) {
+                                    any.w[w] = from[0].w[w] | from[1].w[w] | from[2].w[w] | from[3].w[w];
+                                    none = none && any.w[w] == 0;
                                 }
-                                if (any) {
-                                    const Bits<W> *ok = okd + (size_t)t * nwin * kReachKc;
-                                    const int lo = jc.nmin[t] - d, nl = jc.nmax[t] - jc.nmin[t] + 1;
-                                    for (int q = 0; q < nl; ++q, ok += kReachKc) {
+                                if (!none) {
+                                    // lengths are gathered by Horner's rule: the ones that move a bit down from the shortest on,
+                                    // the others from the longest on, one position a step
+                                    const Bits<W> *ok = okd + (size_t)t * nwin * kReachOk + cls * HAP_MAX_TYPES;
+                                    const int lo = jc.nmin[t] - d, nl = s_end[i % 3][t], nf = s_full[i % 3][t], q0 = lo < 0 ? -lo : 0;
+                                    auto gather = [&](int q) {
+                                        const Bits<W> *o = ok + q * kReachOk;
                                         Bits<W> x;
 #pragma unroll
-                                        for (int w = 0; w < W; ++w) x.w[w] = 0;
+                                        for (int w = 0; w < W; ++w)
+                                            x.w[w] = (from[0].w[w] & o[0].w[w]) | (from[1].w[w] & o[1].w[w]) | (from[2].w[w] & o[2].w[w]) | (from[3].w[w] & o[3].w[w]);
+                                        return x;
+                                    };
+                                    auto step_up = [&](const Bits<W> &x) {
+                                        if (W > 1) acc.w[W - 1] = acc.w[W - 1] << 1 | acc.w[0] >> 63 | x.w[W - 1];
+                                        acc.w[0] = acc.w[0] << 1 | x.w[0];
+                                    };
+                                    int q = nl - 1;
+                                    for (; q >= q0 && q >= nf; --q) step_up(gather(q));
+                                    for (; q >= q0; --q) step_up(any);
+                                    if (lo > 0) acc = bits_shift<W>(acc, lo);
+                                    if (q0 > 0) {
+                                        Bits<W> down;
 #pragma unroll
-                                        for (int h = 0; h < HAP_MAX_TYPES; ++h)
-                                            if (h < T) {
-                                                const Bits<W> m = ok[h == t ? cls : 2 + h];
+                                        for (int w = 0; w < W; ++w) down.w[w] = 0;
+                                        for (q = 0; q < q0; ++q) {
+                                            if (q < nl) {
+                                                const Bits<W> x = q < nf ? any : gather(q);
 #pragma unroll
-                                                for (int w = 0; w < W; ++w) x.w[w] |= from[h].w[w] & m.w[w];
+                                                for (int w = 0; w < W; ++w) down.w[w] |= x.w[w];
                                             }
-                                        x = bits_shift<W>(x, lo + q);
+                                            if (W > 1) down.w[0] = down.w[0] >> 1 | down.w[W - 1] << 63;
+                                            else down.w[0] >>= 1;
+                                            if (W > 1) down.w[W - 1] >>= 1;
+                                        }
 #pragma unroll
-                                        for (int w = 0; w < W; ++w) acc.w[w] |= x.w[w];
+                                        for (int w = 0; w < W; ++w) acc.w[w] |= down.w[w];
                                     }
 #pragma unroll
-                                    for (int w = 0; w < W; ++w) some |= acc.w[w] != 0;
+                                    for (int w = 0; w < W; ++w) { acc.w[w] &= lm.w[w]; some |= acc.w[w] != 0; }
                                 }
                             }
                             cur[(size_t)t * lmax + (e - (unsigned)t * ns)] = acc;
@@ -314,7 +419,7 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
                         if (!__syncthreads_or(some)) return false;
                     }
                     // last stage
-                    const Bits<W> *prv = sReach + (size_t)(PP & 1 ? T * lmax : 0);
+                    const Bits<W> *prv = sReach + (size_t)(PP & 1 ? HAP_MAX_TYPES * lmax : 0);
                     int done = 0;
                     for (int e = tid; e < T * nwin * T; e += kReachThreads) {
                         const int h = e % T, q = (e / T) % nwin, t = e / (T * nwin), n = jc.nmin[t] + q, bit = N - n - jc.base[PP - 1];
@@ -328,9 +433,27 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
                     }
                     return __syncthreads_or(done) != 0;
                 };
-                // between lo (no smaller stage cost can do) and hi (does): the next test lies above the lower bound by a
-                // sixteenth first, then halfway
+                // lower bound: every type's longest stages that cost at most B somewhere have to add up to N
+                if (tid == 0) s_low = (u64)kInf;
                 __syncthreads();
+                for (int e = tid; e < T * nwin * R; e += kReachThreads) {
+                    const int r = e % R, t = e / (R * nwin);
+                    if (!((rc_mask >> r) & 1u) || jc.cnt[t] == 0 || sLeast[e] >= kInf) continue;
+                    const i64 B = sLeast[e] + s_kmin[t];
+                    int room = 0;
+                    for (int h = 0; h < T; ++h) {
+                        int most = 0;
+                        for (int q = 0; jc.cnt[h] > 0 && q <= jc.nmax[h] - jc.nmin[h]; ++q)
+                            for (int x = 0; x < R; ++x)
+                                if (((rc_mask >> x) & 1u) && sLeast[(h * nwin + q) * R + x] + s_kmin[h] <= B) most = jc.nmin[h] + q;
+                        room += most * jc.cnt[h];
+                    }
+                    if (room >= N) atomicMin(&s_low, (u64)B);
+                }
+                __syncthreads();
+                const i64 low = (i64)s_low;
+                // between lo (no smaller stage cost can do) and hi (does): the next test lies a little above the lower bound
+                // first, then halfway
                 i64 lo = floor_b, hi;
                 bool ok = true;
                 if (floor_b > 0) ok = !test(floor_b);                // the larger choice of levels did not help: same answer
@@ -339,9 +462,8 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
                     if (floor_b > 0) lo = (i64)s_up;
                     if (test(kInf - 1)) {
                         hi = (i64)s_dn;
-                        const i64 est = (i64)s_est;
-                        if (est > lo) lo = est;
-                        i64 step = lo / 16;
+                        if (low > lo) lo = low;
+                        i64 step = lo / 64;
                         bool gallop = true;
                         while (lo < hi) {
                             i64 B = lo + (hi - lo) / 2;
