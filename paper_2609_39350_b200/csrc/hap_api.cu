@@ -1052,9 +1052,12 @@ extern "C" hap_status hap_enumerate(hap_problem *p, uint64_t *n_pconf, uint64_t 
             const size_t o_report = o; o = up(o + sizeof(TreeReport));
             const size_t o_live = o; o = up(o + np * sizeof(u32));
             const size_t o_dead = o; o = up(o + np * sizeof(u32));
-            const size_t o_hist = o; o = up(o + (p->opts.prune ? kOrderBuckets * sizeof(u64) : 0));
-            const size_t o_key = o; o = up(o + (p->opts.prune ? np * sizeof(uint4) : 0));
-            const size_t o_order = o; o = up(o + (p->opts.prune ? (np + 1) * sizeof(uint4) : 0));
+            const bool refining = (p->opts.flags & (HAP_OPT_REFINE | HAP_OPT_EXACT)) != 0 && !im.cls.empty(), ordering = p->opts.prune || refining;
+            const u64 n_surv = std::min<u64>(kMaxSurvivors, p->n_cand);
+            const size_t o_hist = o; o = up(o + (ordering ? kOrderBuckets * sizeof(u64) : 0));
+            const size_t o_key = o; o = up(o + (ordering ? np * sizeof(uint4) : 0));
+            const size_t o_order = o; o = up(o + (ordering ? (np + 1) * sizeof(uint4) : 0));
+            const size_t o_surv = o; o = up(o + (refining ? n_surv * sizeof(Survivor) : 0));
             const size_t o_res = o; o = up(o + sizeof(TreeResult));
             CUDA_TRY(p, cached_malloc(p->device, (void **)&p->d_arena, o));
             unsigned char *base = p->d_arena;
@@ -1071,6 +1074,7 @@ extern "C" hap_status hap_enumerate(hap_problem *p, uint64_t *n_pconf, uint64_t 
             ta.live_list = reinterpret_cast<const u32 *>(base + o_live); ta.dead_list = reinterpret_cast<const u32 *>(base + o_dead);
             ta.hist = reinterpret_cast<u64 *>(base + o_hist);
             ta.order_key = reinterpret_cast<uint4 *>(base + o_key); ta.order = reinterpret_cast<uint4 *>(base + o_order);
+            ta.surv = reinterpret_cast<Survivor *>(base + o_surv); ta.max_surv = n_surv;
             LiveArgs &la = p->largs;
             la.hist = ta.hist; la.n_hist = 0;
             la.state = ta.state; la.report = ta.report;
@@ -1370,7 +1374,7 @@ static std::vector<TreeLaunch> tree_launches(const hap_problem *p, bool search, 
 // A pass or a search over the prefix trees: per-type constants, (the layer-cost array where it is asked for,) records,
 // recurrence -- each the programmatic dependent of the one before.  Classes without a tree are left to launch_dp; c2 / c2f
 // then hold their layer costs.
-static hap_status launch_trees(hap_problem *p, const DpOut &out_in, bool search, bool f64, cudaStream_t st, bool final_reduce)
+static hap_status launch_trees(hap_problem *p, const DpOut &out_in, bool search, bool f64, cudaStream_t st, bool final_reduce, bool refine = false)
 {
     DpOut out = out_in;
     out.range_flag = p->d_range;
@@ -1380,6 +1384,7 @@ static hap_status launch_trees(hap_problem *p, const DpOut &out_in, bool search,
     hap_status s;
     if (p->state_dirty) CUDA_TRY(p, cudaMemsetAsync(p->targs.state, 0, sizeof(TreeState), st));
     p->state_dirty = true;
+    if (refine) out.prune = 1;
     const bool prune = search && !f64 && out.prune;
     const std::vector<TreeLaunch> ls = tree_launches(p, search, prune, p_lo, p_hi);
     const bool ordered = prune && ls.size() == 1 && ls[0].items > ls[0].grid;      // (in one wave everything starts at once)
@@ -1413,13 +1418,15 @@ static hap_status launch_trees(hap_problem *p, const DpOut &out_in, bool search,
     // two row entries are held where there are at most two levels, else they are read by level
     const int form = nl ? 2 : p->prof.R > 2 ? 1 : 0;
     using Fn = void (*)(const TreeArgs, const DevConst, DpOut);
-    static const Fn fns[5][3] = {
-        {tree_dp_kernel<false, false, 2, false, false>, tree_dp_kernel<false, false, 4, false, false>, tree_dp_kernel<false, false, 4, true, false>},
-        {tree_dp_kernel<true, false, 2, false, false>, tree_dp_kernel<true, false, 4, false, false>, tree_dp_kernel<true, false, 4, true, false>},
-        {tree_dp_kernel<false, true, 2, false, false>, tree_dp_kernel<false, true, 4, false, false>, tree_dp_kernel<false, true, 4, true, false>},
-        {tree_dp_kernel<true, true, 2, false, false>, tree_dp_kernel<true, true, 4, false, false>, tree_dp_kernel<true, true, 4, true, false>},
-        {tree_dp_kernel<false, false, 2, false, true>, tree_dp_kernel<false, false, 4, false, true>, tree_dp_kernel<false, false, 4, true, true>}};
-    const void *fn = (const void *)fns[counting ? 4 : (f64 ? 2 : 0) + (search ? 1 : 0)][form];
+    constexpr int kP = kTreePass, kS = kTreeSearch, kL = kTreeList;
+    static const Fn fns[6][3] = {
+        {tree_dp_kernel<kP, false, 2, false, false>, tree_dp_kernel<kP, false, 4, false, false>, tree_dp_kernel<kP, false, 4, true, false>},
+        {tree_dp_kernel<kS, false, 2, false, false>, tree_dp_kernel<kS, false, 4, false, false>, tree_dp_kernel<kS, false, 4, true, false>},
+        {tree_dp_kernel<kP, true, 2, false, false>, tree_dp_kernel<kP, true, 4, false, false>, tree_dp_kernel<kP, true, 4, true, false>},
+        {tree_dp_kernel<kS, true, 2, false, false>, tree_dp_kernel<kS, true, 4, false, false>, tree_dp_kernel<kS, true, 4, true, false>},
+        {tree_dp_kernel<kP, false, 2, false, true>, tree_dp_kernel<kP, false, 4, false, true>, tree_dp_kernel<kP, false, 4, true, true>},
+        {tree_dp_kernel<kL, false, 2, false, false>, tree_dp_kernel<kL, false, 4, false, false>, tree_dp_kernel<kL, false, 4, true, false>}};
+    const void *fn = (const void *)fns[refine ? 5 : counting ? 4 : (f64 ? 2 : 0) + (search ? 1 : 0)][form];
     int n = 0;
     for (const auto &l : ls) {
         ta.c_lo = l.c_lo; ta.c_hi = l.c_hi; ta.launch = n;
@@ -1428,6 +1435,17 @@ static hap_status launch_trees(hap_problem *p, const DpOut &out_in, bool search,
         void *args[] = {(void *)&ta, (void *)&p->dc, (void *)&out};
         CUDA_TRY(p, launch_dependent(fn, l.grid, kTreeThreads, l.smem, st, args));
         ++n;
+    }
+    if (refine) {
+        // two blocks an SM: the candidates left are few
+        int exact = (p->opts.flags & HAP_OPT_EXACT) != 0, max_pp = 1;
+        for (const auto &cl : im.cls) max_pp = std::max(max_pp, cl.PP);
+        const size_t smem = refine_smem_bytes(p->model.N, max_pp);
+        ta.blocks_total = 2u * (unsigned)sm_count(p->device);
+        const void *rf = nl ? (const void *)tree_refine_kernel<true> : (const void *)tree_refine_kernel<false>;
+        CUDA_TRY(p, raise_smem_limit(p->device, rf, smem));
+        void *args[] = {(void *)&ta, (void *)&p->dc, (void *)&exact, (void *)&max_pp};
+        CUDA_TRY(p, launch_dependent(rf, ta.blocks_total, kRefineWarps * 32, smem, st, args));
     }
     p->state_dirty = ls.empty();                             // the last block of the recurrence clears the counters
     return HAP_OK;
@@ -1578,7 +1596,7 @@ static void plan_of_result(const hap_problem *p, const TreeResult &r, hap_plan *
 }
 
 // Runs a search over the trees (every class has one) and waits for its result.
-static hap_status tree_search(hap_problem *p, uint64_t first, uint64_t count, bool f64, cudaStream_t st, TreeResult &res)
+static hap_status tree_search(hap_problem *p, uint64_t first, uint64_t count, bool f64, cudaStream_t st, TreeResult &res, bool refine = false)
 {
     hap_status s;
     if (f64 && (s = ensure_f64_buffers(p, (p->opts.flags & HAP_OPT_NO_FUSE) != 0)) != HAP_OK) return s;
@@ -1586,7 +1604,7 @@ static hap_status tree_search(hap_problem *p, uint64_t first, uint64_t count, bo
     if (!p->host_result) p->host_result = result_slot_get();
     DpOut out{};
     out.first = first; out.count = count; out.prune = f64 ? 0 : p->opts.prune;
-    if ((s = launch_trees(p, out, true, f64, st, true)) != HAP_OK) return s;
+    if ((s = launch_trees(p, out, true, f64, st, true, refine)) != HAP_OK) return s;
     p->timed = 2;
     if (!p->host_result) CUDA_TRY(p, cudaMemcpyAsync(&res, p->targs.res_dev, sizeof(res), cudaMemcpyDeviceToHost, st));
     if ((s = leave_synced(p, st)) != HAP_OK) return s;
@@ -2154,10 +2172,18 @@ extern "C" hap_status hap_search_range(hap_problem *p, uint64_t first, uint64_t 
     const bool refine_mode = (p->opts.flags & (HAP_OPT_REFINE | HAP_OPT_EXACT)) != 0;
     DpOut out{};
     out.first = first; out.count = count; out.prune = p->opts.prune;
-    if (p->all_trees && pass_uses_trees(p, out)) {
-        // three launches; the last block writes the plan of the winner to the host
-        TreeResult r;
-        if ((s = tree_search(p, first, count, false, st, r)) != HAP_OK) return s;
+    // A refinement objective costs a warp per candidate and up to dozens of recurrences each: the trees list the candidates
+    // whose lower bound does not exceed the smallest plain T_iter, and those are refined.  (Where that does not decide the
+    // search -- every refined T_iter above the plain one, or too long a list -- the general form below does.)
+    DpOut as_plain = out;
+    as_plain.force_plain = 1;
+    TreeResult r;
+    r.again = 1;
+    if (p->all_trees && pass_uses_trees(p, as_plain)) {
+        // the last block writes the plan of the winner to the host
+        if ((s = tree_search(p, first, count, false, st, r, refine_mode)) != HAP_OK) return s;
+    }
+    if (!r.again) {
         search_stats(p, host_stats, count - r.n_pruned, r.n_feasible, r.n_pruned, (float)((double)(r.stamp[1] - r.stamp[0]) * 1e-6),
                      (float)((double)(r.stamp[2] - r.stamp[1]) * 1e-6));
         if (r.range_flag) return fail(p, HAP_E_RANGE, "a layer time or stage coefficient exceeds the supported range (see hap.h)");

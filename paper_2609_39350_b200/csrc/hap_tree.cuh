@@ -90,7 +90,8 @@ struct __align__(16) TreeHead {
     i64 lb;                                 // lower bound on T_iter of its candidates (searches)
     u32 p;
     u32 dead_policies;                      // by position in rc_order: no mapping can be feasible
-    u64 pad[4];
+    i64 S;                                  // lower bound on the summed stage time (searches)
+    u64 pad[3];
 };
 static_assert(sizeof(TreeHead) == 64, "the stage constants start behind it");
 constexpr u32 kTreeOffKtab = sizeof(TreeHead);
@@ -98,7 +99,7 @@ constexpr u32 kTreeOffMinfo = kTreeOffKtab + kTreeKtab * 8;
 
 // What a search brings back, written by the last block (device memory and, if mapped, the host's copy).
 struct TreeResult {
-    u64 range_flag, n_feasible, n_pruned;
+    u64 range_flag, n_feasible, n_pruned, again;      // again: the listed candidates do not decide the search
     i64 cost; u64 index;
     i64 bott, T_pipe, T_sync, T_opt;
     u32 pconf, rc_mask;
@@ -113,7 +114,14 @@ struct TreeState {
     u32 blocks_done, prep_done;
     u64 n_feasible, n_pruned, splits;
     u64 incumbent;                          // of a pruning search: ~(smallest T_iter so far)
+    // searches with a refinement objective: entries of the survivor list, candidates with a feasible partition, refined
+    // ones, feasible ones of those, ~(smallest refined T_iter so far)
+    u64 n_surv, n_finite, n_refined, n_refined_ok, refined;
 };
+
+// A candidate whose lower bound on T_iter did not exceed the smallest plain T_iter when its part was evaluated.
+struct __align__(16) Survivor { u64 c; i64 lb, bott; u32 ci, slot; };
+constexpr u64 kMaxSurvivors = 1u << 17;
 
 // A pruning search hands its configurations out by their lower bounds, smallest first: buckets of 1/64 octave between 2^20
 // and 2^40 ns.
@@ -173,6 +181,8 @@ struct TreeArgs {
     const u64 *range_flag;
     PlanSlot *slots;                        // [blocks_total] per-block plan
     i64 *slot_cost; u64 *slot_index;        // [blocks_total]
+    Survivor *surv;                         // [max_surv]
+    u64 max_surv;
 };
 
 // shared-memory accesses by 32-bit address (the scans walk rows with plain address decrements)
@@ -488,6 +498,7 @@ tree_prep_kernel(const DevConst dc, const TreeArgs ta, const TypeConst *__restri
         if (lane == 0) {
             TreeHead h{};
             h.offset = pc.offset; h.m1 = (i64)pc.M - 1; h.p = p; h.dead_policies = dead;
+            h.S = s_lb;
             h.lb = s_lb + h.m1 * ((s_lb + PP - 1) / PP);
             *reinterpret_cast<TreeHead *>(rec) = h;
             s_lb = 0;
@@ -595,6 +606,8 @@ __device__ __forceinline__ double tree_span(double Cj, double Ck, double Fj, dou
     return F64 ? c + K : c;
 }
 
+// what tree_dp_kernel leaves: results of every candidate, the best candidate, or the candidates that a refinement may make best
+constexpr int kTreePass = 0, kTreeSearch = 1, kTreeList = 2;
 constexpr int kNever = 1 << 20;
 __device__ __forceinline__ int tree_bound(const TreeLevels &lv, int r) { return r == 0 ? lv.b0 : r == 1 ? lv.b1 : r == 2 ? lv.b2 : lv.nx; }
 
@@ -678,10 +691,70 @@ __device__ __forceinline__ void tree_scan(const TreeArgs &ta, u32 a_prev, u32 a_
     }
 }
 
-template <bool SEARCH, bool F64, int RK, bool NL, bool COUNT>
+// The last block of a pass (all of its threads): leaves the report and, for a search, the winner; clears the counters.
+template <int THREADS, bool SEARCH, bool F64>
+__device__ __forceinline__ void tree_finish(const TreeArgs &ta, const DevConst &dc, u64 n_feasible, u64 n_pruned, u64 again, i64 *s_cost, u64 *s_index, u32 *s_item)
+{
+    const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
+    const i64 inf_bits = F64 ? 0x7ff0000000000000ll : kInf;
+    const int n_rc = ta.n_rc;
+    if (tid == 0) {
+        ta.report->n_feasible = n_feasible; ta.report->n_pruned = n_pruned;
+        ta.report->splits = __ldcg(&ta.state->splits);
+        ta.report->stamp[2] = global_timer();
+    }
+    __syncthreads();
+    static_assert(sizeof(TreeState) % 4 == 0, "cleared in words");
+    for (int q = tid; q < (int)(sizeof(TreeState) / 4); q += THREADS) reinterpret_cast<u32 *>(ta.state)[q] = 0;
+    if (!SEARCH || !ta.res_dev) return;
+    i64 bc = inf_bits; u64 bi = ~0ull; u32 at = 0;
+    for (u32 q = (u32)tid; q < ta.blocks_total; q += THREADS) {
+        const i64 v = __ldcg(ta.slot_cost + q); const u64 ix = __ldcg(ta.slot_index + q);
+        if (v < bc || (v == bc && ix < bi)) { bc = v; bi = ix; at = q; }
+    }
+    const u64 mine = bi;
+    const i64 mine_c = bc;
+    warp_argmin(bc, bi);
+    if (lane == 0) { s_cost[wib] = bc; s_index[wib] = bi; }
+    __syncthreads();
+    bc = s_cost[0]; bi = s_index[0];
+    for (int q = 1; q < THREADS / 32; ++q) if (s_cost[q] < bc || (s_cost[q] == bc && s_index[q] < bi)) { bc = s_cost[q]; bi = s_index[q]; }
+    // the winner's slot: (cost, index) pairs are distinct unless nothing is feasible
+    if (bc < inf_bits && mine == bi && mine_c == bc) *s_item = at;
+    __syncthreads();
+    if (wib != 0) return;
+    TreeResult *rs = ta.res_dev, *rh = ta.res_host;
+    for (int copy = 0; copy < 2; ++copy) {
+        TreeResult *w = copy == 0 ? rs : rh;
+        if (!w) continue;
+        if (lane == 0) {
+            w->range_flag = __ldcg(ta.range_flag);
+            w->n_feasible = __ldcg(&ta.report->n_feasible); w->n_pruned = __ldcg(&ta.report->n_pruned);
+            w->cost = bc; w->index = bi; w->again = again;
+            for (int q = 0; q < 3; ++q) w->stamp[q] = __ldcg(&ta.report->stamp[q]);
+        }
+        if (!(bc < inf_bits)) continue;
+        const u64 p = find_pconf(dc, bi);
+        const hap_pconf pc = dc.pconf[p];
+        const u64 loc = bi - pc.offset, map_idx = loc / (u64)n_rc;
+        const StageMap sm = decode_stage(dc, pc, map_idx, lane);
+        const PlanSlot *ps = ta.slots + *s_item;
+        if (lane == 0) {
+            w->pconf = (u32)p; w->rc_mask = ta.rc_masks[loc - map_idx * (u64)n_rc];
+            w->bott = __ldcg(&ps->bott); w->T_pipe = __ldcg(&ps->T_pipe); w->T_sync = __ldcg(&ps->T_sync); w->T_opt = __ldcg(&ps->T_opt);
+        }
+        w->mask[lane] = lane < pc.PP ? (uint8_t)sm.mask : 0;
+        w->n[lane] = lane < pc.PP ? __ldcg(ps->n + lane) : 0;
+        w->r[lane] = lane < pc.PP ? __ldcg(ps->r + lane) : 0;
+    }
+    __threadfence_system();
+}
+
+template <int MODE, bool F64, int RK, bool NL, bool COUNT>
 __global__ void __launch_bounds__(kTreeThreads, kTreeBlocksPerSm)
 tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
 {
+    constexpr bool SEARCH = MODE != kTreePass, LIST = MODE == kTreeList;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ u32 s_item, s_unit, s_total[HAP_MAX_PP + 2];
     __shared__ uint4 s_entry;
@@ -888,12 +961,11 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
                 // ---- one lane per mapping: cell (PP, N), walk back, Eq. 4 ----------------------------------------
                 bool any_plan = false;
                 const u32 a_last = PP == 1 ? a_zero : a_buf[(PP - 1) & 1];
-                for (u32 m = (u32)lane; m < nmap; m += 32u) {
+                auto leaf = [&](u32 m, double &bott) {
                     const u64 c = c_lo + (u64)m * (u64)n_rc + (u64)rc_idx;
-                    if (c < w_lo || c >= w_hi) continue;
+                    if (c < w_lo || c >= w_hi) return;
                     const u64 o = c - w_lo;
-                    if (!HAP_CHECK_OK(3, o < out.count)) continue;
-                    double bott = kTreeInf;
+                    if (!HAP_CHECK_OK(3, o < out.count)) return;
                     int n = 0;
                     const u32 *path = pt->path + m;
                     u32 pw = 0;
@@ -915,6 +987,7 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
                         }
                     }
                     if (n == 0) {
+                        bott = kTreeInf;
                         if (!SEARCH) {
                             if (out.cost) out.cost[o] = inf_bits;
                             if (out.bottleneck) out.bottleneck[o] = inf_bits;
@@ -922,12 +995,12 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
                             if (out.partition) { uint4 *d = reinterpret_cast<uint4 *>(out.partition + o * HAP_MAX_PP); d[0] = z; d[1] = z; }
                             if (out.recompute) { uint4 *d = reinterpret_cast<uint4 *>(out.recompute + o * HAP_MAX_PP); d[0] = z; d[1] = z; }
                         }
-                        continue;
+                        return;
                     }
                     double sum = 0.0, t_sync = 0.0, t_opt = 0.0, het = 0.0;
                     u32 most = 0;                                                  // per row group the longest stage, a byte each (packed)
                     u64 acc_n = 0, acc_r = 0;
-                    const bool want_plan = SEARCH ? true : (out.partition != nullptr || out.recompute != nullptr);
+                    const bool want_plan = LIST ? false : SEARCH ? true : (out.partition != nullptr || out.recompute != nullptr);
                     int b = N;
                     for (int d = PP; d >= 1; --d) {
                         const u32 pn = d > 1 ? __ldg(path + (size_t)(d - 2) * nmap) : 0u;       // the stage before: asked for early
@@ -1009,7 +1082,8 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
                     }
                     const i64 bott_bits = F64 ? __double_as_longlong(bott) : (i64)bott;
                     if (SEARCH) {
-                        if (keep) { n_feas++; any_plan = true; }
+                        if (LIST) { n_feas++; any_plan = true; }               // (a refined partition may pass Pruning 3 where this one does not)
+                        else if (keep) { n_feas++; any_plan = true; }
                         if (T_iter < best_cost || (T_iter == best_cost && c < best_index)) {
                             best_cost = T_iter; best_index = c;
                             plan_val[plan_cur][0] = bott_bits; plan_val[plan_cur][1] = T_pipe;
@@ -1026,14 +1100,41 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
                             if (out.recompute) reinterpret_cast<u64 *>(out.recompute + o * HAP_MAX_PP)[w] = 0;
                         }
                     }
-                }
+                };
+                if (LIST) {
+                    for (u32 m0 = 0; m0 < nmap; m0 += 32u) {
+                        const u32 m = m0 + (u32)lane;
+                        double bott = kTreeInf;
+                        if (m < nmap) leaf(m, bott);
+                        __syncwarp();
+                        if (!__any_sync(0xffffffffu, bott < kTreeBound)) continue;
+                        // the incumbent moves first, then the candidates that it leaves are listed
+                        i64 v = best_cost;
+#pragma unroll
+                        for (int s = 16; s > 0; s >>= 1) { const i64 x = __shfl_xor_sync(0xffffffffu, v, s); v = x < v ? x : v; }
+                        if (lane == 0) { const u64 was = ~atomicMax(&ta.state->incumbent, v < inf_bits ? ~(u64)v : 0ull); v = was < (u64)v ? (i64)was : v; }
+                        v = shfl_i64(v, 0);
+                        const i64 lb = bott < kTreeBound ? hd->S + hd->m1 * (i64)bott : kInf;
+                        const bool keep = bott < kTreeBound && lb <= v;
+                        const u32 kept = __ballot_sync(0xffffffffu, keep);
+                        u64 at = 0;
+                        if (lane == 0 && kept) at = atomicAdd(&ta.state->n_surv, (u64)__popc(kept));
+                        at = (u64)shfl_i64((i64)at, 0) + (u64)__popc(kept & ((1u << lane) - 1u));
+                        if (keep && at < ta.max_surv) {
+                            Survivor sv;
+                            sv.c = c_lo + (u64)m * (u64)n_rc + (u64)rc_idx; sv.lb = lb; sv.bott = (i64)bott; sv.ci = (u32)ci; sv.slot = conf0 + conf;
+                            ta.surv[at] = sv;
+                        }
+                    }
+                } else
+                    for (u32 m = (u32)lane; m < nmap; m += 32u) { double bott = kTreeInf; leaf(m, bott); }
                 // (also keeps the next policy from overwriting rows and choices that other lanes still read)
                 const int plan = __any_sync(0xffffffffu, any_plan);
                 // a policy under which none of the part's mappings has a feasible partition settles its subsets
                 if (!plan && whole && ta.eta_q <= 0) without_plan |= 1u << pos;
                 __syncwarp();
             }
-            if (SEARCH && out.prune) {
+            if (SEARCH && !LIST && out.prune) {
                 // the incumbent moves on after every part
                 i64 bc = best_cost;
 #pragma unroll
@@ -1050,6 +1151,11 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
     if (COUNT) {
         const u64 s = (u64)warp_sum_i64((i64)splits);
         if (lane == 0 && s) atomicAdd(&ta.state->splits, s);
+    }
+    if (LIST) {
+        const u64 nf = (u64)warp_sum_i64((i64)n_feas);
+        if (lane == 0 && nf) atomicAdd(&ta.state->n_finite, nf);
+        return;                             // the refinement follows
     }
     if (SEARCH) {
         const u64 nf = (u64)warp_sum_i64((i64)n_feas);
@@ -1081,56 +1187,255 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    if (tid == 0) {
-        ta.report->n_feasible = __ldcg(&ta.state->n_feasible); ta.report->n_pruned = __ldcg(&ta.state->n_pruned);
-        ta.report->splits = __ldcg(&ta.state->splits);
-        ta.report->stamp[2] = global_timer();
-    }
-    __syncthreads();
-    static_assert(sizeof(TreeState) % 4 == 0, "cleared in words");
-    for (int q = tid; q < (int)(sizeof(TreeState) / 4); q += kTreeThreads) reinterpret_cast<u32 *>(ta.state)[q] = 0;
-    if (!SEARCH || !ta.res_dev) return;
-    i64 bc = inf_bits; u64 bi = ~0ull; u32 at = 0;
-    for (u32 q = (u32)tid; q < ta.blocks_total; q += kTreeThreads) {
-        const i64 v = __ldcg(ta.slot_cost + q); const u64 ix = __ldcg(ta.slot_index + q);
-        if (v < bc || (v == bc && ix < bi)) { bc = v; bi = ix; at = q; }
-    }
-    const u64 mine = bi;
-    const i64 mine_c = bc;
-    warp_argmin(bc, bi);
-    if (lane == 0) { s_cost[wib] = bc; s_index[wib] = bi; }
-    __syncthreads();
-    bc = s_cost[0]; bi = s_index[0];
-    for (int q = 1; q < kTreeWarps; ++q) if (s_cost[q] < bc || (s_cost[q] == bc && s_index[q] < bi)) { bc = s_cost[q]; bi = s_index[q]; }
-    // the winner's slot: (cost, index) pairs are distinct unless nothing is feasible
-    if (bc < inf_bits && mine == bi && mine_c == bc) s_item = at;
-    __syncthreads();
-    if (wib != 0) return;
-    TreeResult *rs = ta.res_dev, *rh = ta.res_host;
-    for (int copy = 0; copy < 2; ++copy) {
-        TreeResult *w = copy == 0 ? rs : rh;
-        if (!w) continue;
-        if (lane == 0) {
-            w->range_flag = __ldcg(ta.range_flag);
-            w->n_feasible = __ldcg(&ta.report->n_feasible); w->n_pruned = __ldcg(&ta.report->n_pruned);
-            w->cost = bc; w->index = bi;
-            for (int q = 0; q < 3; ++q) w->stamp[q] = __ldcg(&ta.report->stamp[q]);
-        }
-        if (!(bc < inf_bits)) continue;
-        const u64 p = find_pconf(dc, bi);
-        const hap_pconf pc = dc.pconf[p];
-        const u64 loc = bi - pc.offset, map_idx = loc / (u64)n_rc;
+    tree_finish<kTreeThreads, SEARCH, F64>(ta, dc, __ldcg(&ta.state->n_feasible), __ldcg(&ta.state->n_pruned), 0, s_cost, s_index, &s_item);
+}
+
+// ------------------------------------------------------------------------------------------------------------------
+// refinement objectives
+// ------------------------------------------------------------------------------------------------------------------
+
+// A warp per listed candidate: among its partitions without a stage above the bottleneck the one of the smallest sum, or (exact)
+// the one of the smallest sum + (M - 1) max of all, by an additive recurrence over the candidate's bands whose limit on the
+// stage cost is swept over the costs that occur.  Lanes run over the end layers.  Few candidates get here -- 169 of 1.35
+// million at 256 devices -- so a chain of recurrences bounds it: the unlimited one comes first, because its sum tells
+// whether the candidate can still beat the best one so far, and the sweep stops where it cannot any more.  An exact search
+// of those 1.35 million: 1,316 us when a plain pass over all of them was followed by a warp per candidate of every block
+// that held one left, 305 us in this form.
+constexpr int kRefineWarps = 4;
+inline size_t refine_smem_bytes(int N, int max_pp) { return (size_t)kRefineWarps * ((size_t)2 * (N + 1) * 8 + ((size_t)max_pp * (N + 1) + 15) / 16 * 16); }
+
+template <bool NL>
+__global__ void __launch_bounds__(kRefineWarps * 32)
+tree_refine_kernel(const TreeArgs ta, const DevConst dc, int exact, int max_pp)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ i64 s_cost[kRefineWarps];
+    __shared__ u64 s_index[kRefineWarps];
+    __shared__ u32 s_item;
+    __shared__ int s_last;
+    const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
+    const int N = ta.N, R = ta.R, n1 = N + 1, n_rc = ta.n_rc, RW = NL ? 2 : R;
+    double *rows = reinterpret_cast<double *>(smem_raw) + (size_t)wib * 2 * n1;
+    uint8_t *ch = smem_raw + (size_t)kRefineWarps * 2 * n1 * 8 + (size_t)wib * (((size_t)max_pp * n1 + 15) / 16 * 16);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const u64 listed = __ldcg(&ta.state->n_surv), n = listed < ta.max_surv ? listed : ta.max_surv;
+    const u64 plain = ~__ldcg(&ta.state->incumbent);
+    i64 best_cost = kInf, best_bott = 0, best_pipe = 0, best_sync = 0, best_opt = 0;
+    u64 best_index = ~0ull, n_refined = 0, n_ok = 0;
+    int best_n = 0, best_r = 0;
+
+    while (true) {
+        u32 at = 0;
+        if (lane == 0) at = atomicAdd(&ta.state->ticket[1], 1u);
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (at >= n) break;
+        u64 bar = 0;                                        // nothing above it can win (one lane reads, the warp follows)
+        if (lane == 0) { bar = ~*reinterpret_cast<volatile const u64 *>(&ta.state->refined); bar = plain < bar ? plain : bar; }
+        bar = (u64)shfl_i64((i64)bar, 0);
+        if ((u64)__ldcg(&ta.surv[at].lb) > bar) continue;
+        const u64 c = __ldcg(&ta.surv[at].c);
+        const double bott = (double)__ldcg(&ta.surv[at].bott);
+        const TreeClass *cl = ta.cls + __ldcg(&ta.surv[at].ci);
+        const unsigned char *rec = ta.rec + cl->rec_off + (u64)__ldcg(&ta.surv[at].slot) * cl->rec_bytes;
+        const TreeHead *hd = reinterpret_cast<const TreeHead *>(rec);
+        const hap_pconf pc = dc.pconf[hd->p];
+        const int PP = pc.PP;
+        const i64 M1 = hd->m1;
+        const u64 loc = c - pc.offset, map_idx = loc / (u64)n_rc;
+        const unsigned rc_mask = ta.rc_masks[loc - map_idx * (u64)n_rc];
+        const double *ktab = reinterpret_cast<const double *>(rec + kTreeOffKtab), *minfo = reinterpret_cast<const double *>(rec + cl->o_minfo);
+        const double *row0 = reinterpret_cast<const double *>(rec + cl->o_rows);
+
+        // ---- this lane's stage: row group, capacity type, constant, window, band (the formulas of pipeline_dp_kernel) -----
+        int mrow = 0, capt = 0, nmin = 0, nmax = 0, bl = 0, bh = 0, kidx = 0;
+        double K = 0.0;
+        i64 Pmin = 0;
         const StageMap sm = decode_stage(dc, pc, map_idx, lane);
-        const PlanSlot *ps = ta.slots + s_item;
-        if (lane == 0) {
-            w->pconf = (u32)p; w->rc_mask = ta.rc_masks[loc - map_idx * (u64)n_rc];
-            w->bott = __ldcg(&ps->bott); w->T_pipe = __ldcg(&ps->T_pipe); w->T_sync = __ldcg(&ps->T_sync); w->T_opt = __ldcg(&ps->T_opt);
+        if (lane < PP) {
+            bool seen = false;
+            i64 cap = 0;
+            for (int h = 0; h < dc.T; ++h)
+                if (sm.mask >> h & 1) {
+                    if (!seen || dc.P[h] < Pmin) Pmin = dc.P[h];
+                    if (!seen || dc.cap_eff[h] < cap) { cap = dc.cap_eff[h]; capt = h; }
+                    seen = true;
+                }
+            mrow = cl->mrow_of[sm.mask];
+            kidx = lane == 0 ? mrow : 16 + sm.hb * 6 + (sm.cls == HAP_CROSS ? 2 + sm.ha : sm.cls);
+            K = ktab[kidx] + (lane == PP - 1 ? minfo[mrow * kTreeMinfo + 6] : 0.0);
         }
-        w->mask[lane] = lane < pc.PP ? (uint8_t)sm.mask : 0;
-        w->n[lane] = lane < pc.PP ? __ldcg(ps->n + lane) : 0;
-        w->r[lane] = lane < pc.PP ? __ldcg(ps->r + lane) : 0;
+        {
+            const i64 Ps = warp_sum_i64(Pmin);
+            if (lane < PP) {
+                nmin = 1; nmax = N - PP + 1;
+                if (dc.uniform) { nmin = N / PP; nmax = (N + PP - 1) / PP; }
+                else if (dc.delta_q >= 0) {
+                    const i64 den = 1024 * Ps;
+                    const i64 lo = ((i64)(1024 - dc.delta_q) * Pmin * N) / den, hi = ((i64)(1024 + dc.delta_q) * Pmin * N + den - 1) / den;
+                    nmin = lo < 1 ? 1 : (int)lo; nmax = hi > N - PP + 1 ? N - PP + 1 : (int)hi;
+                }
+            }
+            int smin = nmin, smax = nmax;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int a = __shfl_up_sync(0xffffffffu, smin, o), b = __shfl_up_sync(0xffffffffu, smax, o);
+                if (lane >= o) { smin += a; smax += b; }
+            }
+            const int tmin = __shfl_sync(0xffffffffu, smin, PP - 1), tmax = __shfl_sync(0xffffffffu, smax, PP - 1), i = lane + 1;
+            bl = smin > i ? smin : i; bh = smax < N - PP + i ? smax : N - PP + i;
+            const int rl = N - (tmax - smax), rh = N - (tmin - smin);
+            bl = bl > rl ? bl : rl; bh = bh < rh ? bh : rh;
+        }
+        auto levels = [&](int d, int ct, int j) {
+            u32 len4 = 0;
+            if (cl->flat[d]) len4 = __ldg(reinterpret_cast<const u32 *>(rec + cl->o_thr) + (d - 1) * dc.T + ct);
+            else if (HAP_CHECK_OK(6, j >= (int)cl->jlo[d] && j <= (int)cl->jhi[d]))
+                for (int r = 0; r < R; ++r) len4 |= (u32)__ldg(rec + cl->o_thr_nf + cl->nf_off[d] + (u32)(ct * R + r) * cl->nf_w[d] + (u32)(j - (int)cl->jlo[d])) << (8 * r);
+            return tree_levels(R, rc_mask, len4);
+        };
+        auto span = [&](int mr, int r, int k, int j, double kk) {
+            if (!HAP_CHECK_OK(5, k >= 0 && k <= j && j <= N && r < R)) return kk;
+            const double *row = row0 + (size_t)(mr * RW + (NL ? 0 : r)) * n1;
+            return tree_span<false, NL>(__ldg(row + j), __ldg(row + k), NL ? __ldg(row + n1 + j) : 0.0, NL ? __ldg(row + n1 + k) : 0.0, 0.0, NL ? ta.tau[r] : 0.0) + kk;
+        };
+        auto level_of = [&](const TreeLevels &lv, int len) { return (len > lv.b0) + (len > lv.b1) + (len > lv.b2); };
+        // cost of this lane's stage over (a, b]
+        auto stage_of_lane = [&](int a, int b) -> double {
+            if (lane >= PP) return 0.0;
+            return span(mrow, level_of(levels(lane + 1, capt, b), b - a), a, b, K);
+        };
+        // one recurrence under a limit on the stage cost: false if no partition respects it; else the sum, the largest stage
+        // cost of the chosen partition, this lane's span, and in nxt the smallest stage cost above the limit
+        auto pass = [&](double limit, double &psum, double &pmax, double &nxt, int &pa, int &pb) -> bool {
+            int pbl = 0, pbh = 0;
+            double skipped = kTreeInf;
+            for (int i = 1; i <= PP; ++i) {
+                const int mr = __shfl_sync(0xffffffffu, mrow, i - 1), ct = __shfl_sync(0xffffffffu, capt, i - 1);
+                const int lo_n = __shfl_sync(0xffffffffu, nmin, i - 1), hi_n = __shfl_sync(0xffffffffu, nmax, i - 1);
+                const int lo_j = __shfl_sync(0xffffffffu, bl, i - 1), hi_j = __shfl_sync(0xffffffffu, bh, i - 1);
+                const double kk = __shfl_sync(0xffffffffu, K, i - 1);
+                const double *prev = rows + (size_t)(i & 1) * n1;
+                double *cur = rows + (size_t)((i - 1) & 1) * n1;
+                for (int j = lo_j + lane; j <= hi_j; j += 32) {
+                    double best = kTreeInf;
+                    int arg = 255;
+                    const TreeLevels lv = levels(i, ct, j);
+                    int a = lo_n > j - pbh ? lo_n : j - pbh, b = hi_n < j - pbl ? hi_n : j - pbl;
+                    if (b > lv.nx) b = lv.nx;
+                    for (int len = a; len <= b; ++len) {
+                        const double cst = span(mr, level_of(lv, len), j - len, j, kk);
+                        if (cst > limit) { skipped = cst < skipped ? cst : skipped; continue; }
+                        const double v = (i == 1 ? 0.0 : prev[j - len]) + cst;
+                        if (v <= best && v < kTreeBound) { best = v; arg = j - len; }
+                    }
+                    cur[j] = best;
+                    if (HAP_CHECK_OK(2, i <= max_pp)) ch[(size_t)(i - 1) * n1 + j] = (uint8_t)arg;
+                }
+                __syncwarp();
+                pbl = lo_j; pbh = hi_j;
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) { const double t = __shfl_xor_sync(0xffffffffu, skipped, o); skipped = t < skipped ? t : skipped; }
+            nxt = skipped;
+            psum = rows[(size_t)((PP - 1) & 1) * n1 + N];
+            pa = 0; pb = 0;
+            if (!(psum < kTreeBound)) { __syncwarp(); return false; }
+            int j = N;
+            for (int i = PP; i >= 1; --i) {
+                const int k = ch[(size_t)(i - 1) * n1 + j];
+                if (lane == i - 1) { pa = k; pb = j; }
+                if (!HAP_CHECK_OK(5, k < j)) break;
+                j = k;
+            }
+            double m = stage_of_lane(pa, pb);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) { const double t = __shfl_xor_sync(0xffffffffu, m, o); m = t > m ? t : m; }
+            pmax = m;
+            __syncwarp();
+            return true;
+        };
+        auto value = [&](double sum, double most) { return (i64)sum + M1 * (i64)most; };
+        int a_me = 0, b_me = 0, ua = 0, ub = 0;
+        double bs, bm, nx, us = 0.0, um = 0.0, unx;
+        if (exact) {
+            if (!pass(kTreeBound, us, um, unx, ua, ub)) continue;
+            // the sum without a limit and the smallest maximum (whether Pruning 3 drops it, only its partition tells)
+            if (ta.eta_q <= 0 && (u64)value(us, bott) > bar) { n_refined++; n_ok++; continue; }
+        }
+        n_refined++;
+        if (!pass(bott, bs, bm, nx, a_me, b_me)) continue;  // (always feasible: the min-max partition respects the limit)
+        if (exact) {
+            // the first limit that reaches the smallest value wins
+            i64 best = value(bs, bm);
+            double t = nx;
+            while (t < kTreeBound && value(us, t) < best && (ta.eta_q > 0 || (u64)value(us, t) <= bar)) {
+                double cs, cm, cn;
+                int ca, cb;
+                if (pass(t, cs, cm, cn, ca, cb) && value(cs, cm) < best) { best = value(cs, cm); a_me = ca; b_me = cb; }
+                t = cn;
+            }
+            if (value(us, um) < best) { a_me = ua; b_me = ub; }
+        }
+        // ---- Eq. 4 --------------------------------------------------------------------------------------------------
+        const int len = b_me - a_me;
+        int my_r = 0;
+        double cst = 0.0, sy = 0.0, op = 0.0, het = 0.0;
+        if (lane < PP) {
+            my_r = level_of(levels(lane + 1, capt, b_me), len);
+            cst = span(mrow, my_r, a_me, b_me, K);
+            const int n_moe = moe_before(dc, b_me) - moe_before(dc, a_me);
+            const double dm = (double)n_moe, dd = (double)(len - n_moe);
+            const double *mi = minfo + mrow * kTreeMinfo;
+            sy = mi[0] + dd * mi[1] + dm * mi[2];
+            op = dd * mi[3] + dm * mi[4];
+            if (ta.eta_q > 0) {
+                if (lane > 0 && (kidx - 16) % 6 >= 2) het += ktab[kidx];
+                het += dm * mi[5];
+            }
+        }
+        double sum = cst, mxc = cst;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const double t1 = __shfl_xor_sync(0xffffffffu, mxc, o), t2 = __shfl_xor_sync(0xffffffffu, sy, o), t3 = __shfl_xor_sync(0xffffffffu, op, o);
+            sum += __shfl_xor_sync(0xffffffffu, sum, o); het += __shfl_xor_sync(0xffffffffu, het, o);
+            mxc = t1 > mxc ? t1 : mxc; sy = t2 > sy ? t2 : sy; op = t3 > op ? t3 : op;
+        }
+        const i64 T_pipe = value(sum, mxc);
+        i64 T_iter = T_pipe + (i64)sy + (i64)op;
+        if (ta.eta_q > 0 && (i64)het * (i64)PP * 1024 > (i64)ta.eta_q * (i64)sum) T_iter = kInf;        // Pruning 3
+        if (T_iter < kInf) n_ok++;
+        if (T_iter < best_cost || (T_iter == best_cost && T_iter < kInf && c < best_index)) {
+            best_cost = T_iter; best_index = c; best_bott = (i64)bott; best_pipe = T_pipe; best_sync = (i64)sy; best_opt = (i64)op;
+            best_n = len; best_r = my_r;
+            if (lane == 0) atomicMax(&ta.state->refined, ~(u64)T_iter);
+        }
     }
-    __threadfence_system();
+
+    if (lane == 0) {
+        s_cost[wib] = best_cost; s_index[wib] = best_index;
+        if (n_refined) { atomicAdd(&ta.state->n_refined, n_refined); atomicAdd(&ta.state->n_refined_ok, n_ok); }
+    }
+    __syncthreads();
+    int win = 0;
+    for (int q = 1; q < kRefineWarps; ++q) if (s_cost[q] < s_cost[win] || (s_cost[q] == s_cost[win] && s_index[q] < s_index[win])) win = q;
+    if (wib == win) {
+        PlanSlot *ps = ta.slots + blockIdx.x;
+        if (lane == 0) {
+            ta.slot_cost[blockIdx.x] = best_cost; ta.slot_index[blockIdx.x] = best_index;
+            ps->bott = best_bott; ps->T_pipe = best_pipe; ps->T_sync = best_sync; ps->T_opt = best_opt;
+        }
+        ps->n[lane] = (uint8_t)best_n; ps->r[lane] = (uint8_t)best_r;
+    }
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(&ta.state->blocks_done, 1u) + 1u == gridDim.x;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    // candidates were dropped against the smallest plain T_iter: that decides the search unless every refined one is above it
+    const u64 refined = ~__ldcg(&ta.state->refined), finite = __ldcg(&ta.state->n_finite), done = __ldcg(&ta.state->n_refined);
+    const u64 again = listed > ta.max_surv || (finite > 0 && refined > plain) ? 1 : 0;
+    tree_finish<kRefineWarps * 32, true, false>(ta, dc, __ldcg(&ta.state->n_refined_ok), __ldcg(&ta.state->n_pruned) + finite - done, again, s_cost, s_index, &s_item);
 }
 
 }  // namespace hap

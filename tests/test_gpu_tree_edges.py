@@ -59,3 +59,29 @@ def test_tree_tasks_and_levels(nodes, N, tau, policies, kinds):
             with pytest.raises(hap.HapError):
                 hap.hap_search_best(hp)
         hap.hap_problem_destroy(hp)
+
+
+@pytest.mark.parametrize("objective", ["refine", "exact"])
+@pytest.mark.parametrize("nodes,N,tau,policies,kinds", CASES)
+def test_refined_search_over_listed_candidates(nodes, N, tau, policies, kinds, objective):
+    """The search that refines only listed candidates finds what refining every candidate finds."""
+    import paper_2609_39350_b200 as hap
+    pb = problems.random_small(90 + N, N=N, T=len(nodes), nodes_per_type=nodes, node_size=2, window=N % 2 == 0, first_dense=kinds == "dense_first")
+    R = len(tau)
+    pb.tau_q = np.array(tau, np.int32)
+    pb.xi_q = np.array([1024, 512, 200, 64][:R - 1] + [64], np.int32)
+    pb.rc_masks = np.array(policies, np.uint32)
+    pb.eta_q = 1024 if N % 3 == 0 else 0
+    o = Oracle(pb)
+    _, best, index, _, _ = (o.search_pconfs_refined if objective == "refine" else o.search_pconfs_exact)(0, 1, threads=NTHREADS)
+    hp = hap.hap_problem_create(pb, flags=hap.OPT_REFINE if objective == "refine" else hap.OPT_EXACT)
+    hap.hap_enumerate(hp)
+    if best < INF:
+        plan, st = hap.hap_search_best(hp)
+        assert (plan["index"], plan["T_iter"]) == (index, best)
+        want = (o.eval_index_refined if objective == "refine" else o.eval_index_exact)(index)
+        assert plan["n"] == want["n"] and plan["r"] == want["r"] and st["n_evaluated"] + st["n_pruned"] == hp.n_cand
+    else:
+        with pytest.raises(hap.HapError):
+            hap.hap_search_best(hp)
+    hap.hap_problem_destroy(hp)
