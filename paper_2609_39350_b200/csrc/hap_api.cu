@@ -380,7 +380,14 @@ static void cached_free(void *ptr)
     if (it == mc.live.end()) { cudaFree(ptr); return; }
     const CachedBlock b = it->second;
     mc.live.erase(it);
-    if (mc.idle.size() >= kCacheBlocks || mc.idle_bytes + b.bytes > kCacheBytes) { cudaFree(ptr); return; }
+    if (b.bytes > kCacheBytes) { cudaFree(ptr); return; }
+    // full: the block that has been idle longest goes (sizes that are no longer asked for would otherwise keep every new size
+    // out, and each problem of that size would pay for an allocation and a release: 0.8 ms instead of 0.2)
+    while (mc.idle.size() >= kCacheBlocks || mc.idle_bytes + b.bytes > kCacheBytes) {
+        cudaFree(mc.idle.front().ptr);
+        mc.idle_bytes -= mc.idle.front().bytes;
+        mc.idle.erase(mc.idle.begin());
+    }
     mc.idle.push_back(b);
     mc.idle_bytes += b.bytes;
 }
@@ -1240,14 +1247,27 @@ static void configs_of_range(const hap_problem *p, u64 first, u64 count, unsigne
     lo = owner(first); hi = owner(first + count - 1) + 1;
 }
 
+static int sm_count(int device)
+{
+    static int n[64];                                       // (the same value whoever writes it)
+    int &v = n[device & 63];
+    if (!v && cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) { cudaGetLastError(); v = 148; }
+    return v;
+}
+
 // Per-type constants and stage coefficients of the configurations [p_lo, p_hi) in integer (coef) and / or fp64 form (coeff);
 // `live`: also the classes' lists of configurations (a pass over the trees)
 static hap_status launch_type_consts(hap_problem *p, i64 *coef, double *coeff, cudaStream_t st, unsigned p_lo, unsigned p_hi, const LiveArgs *live = nullptr)
 {
     const unsigned n_conf = p_hi - p_lo;
-    static const LiveArgs none{};
-    const unsigned per = 32 / (unsigned)p->T;                 // configurations of a block
-    type_const_kernel<<<(n_conf + per - 1) / per, kTcThreads, 0, st>>>(p->dc, p->d_tc, coef, coeff, p->d_range, p_lo, n_conf, live ? *live : none);
+    if (live) {
+        const unsigned per = 32 / (unsigned)p->T;             // configurations of a block
+        type_const_kernel<<<(n_conf + per - 1) / per, kTcThreads, 0, st>>>(p->dc, p->d_tc, coef, coeff, p->d_range, p_lo, n_conf, *live);
+    } else {
+        const unsigned blocks = (unsigned)(((u64)n_conf * HAP_MAX_TYPES + kTcPlainThreads - 1) / kTcPlainThreads);
+        if (coeff) type_const_plain_kernel<false><<<dim3(blocks, 3), kTcPlainThreads, 0, st>>>(p->dc, p->d_tc, coef, coeff, p->d_range, p_lo, n_conf);
+        else type_const_plain_kernel<true><<<dim3(blocks, 3), kTcPlainThreads, 0, st>>>(p->dc, p->d_tc, coef, nullptr, p->d_range, p_lo, n_conf);
+    }
     CUDA_TRY(p, cudaGetLastError());
     return HAP_OK;
 }
@@ -1259,9 +1279,24 @@ static hap_status launch_layer_costs(hap_problem *p, i64 *c2, i64 *coef, double 
 {
     if (p_hi > p->pconfs.size()) p_hi = (unsigned)p->pconfs.size();
     if (p_lo >= p_hi) return HAP_OK;
-    hap_status s = launch_type_consts(p, quant ? coef : nullptr, quant ? nullptr : coeff, st, p_lo, p_hi);
-    if (s != HAP_OK) return s;
-    if ((quant && c2) || (!quant && c2f)) return launch_layer_kernel(p, c2, c2f, quant, st, lb_sum, nullptr, p_lo, p_hi - p_lo, true);
+    if (!(quant ? c2 != nullptr : c2f != nullptr)) return launch_type_consts(p, quant ? coef : nullptr, quant ? nullptr : coeff, st, p_lo, p_hi);
+    const unsigned n_conf = p_hi - p_lo, per = 32 / (unsigned)p->T;
+    // one launch up to three blocks an SM, all of them running at once: the chain of constants is then followed by the writes
+    // without a second launch (12.3 -> 10.2 us at 2,392 configurations of three types); beyond, the constants of later blocks
+    // delay the writes (1,024 devices, 7,783 configurations: 20.5 us in two launches, 26.8 us in one)
+    if ((n_conf + per - 1) / per > 3 * (unsigned)sm_count(p->device)) {
+        hap_status s = launch_type_consts(p, quant ? coef : nullptr, quant ? nullptr : coeff, st, p_lo, p_hi);
+        if (s != HAP_OK) return s;
+        return launch_layer_kernel(p, c2, c2f, quant, st, lb_sum, nullptr, p_lo, n_conf, true);
+    }
+    const int kind = !p->dc.kind_uniform ? 2 : (p->kind[0] == HAP_MOE ? 1 : 0);      // layer kinds: all dense, all MoE, mixed
+    using Fn = void (*)(const DevConst, i64 *, double *, i64 *, double *, i64 *, u64 *, unsigned, unsigned);
+    static const Fn fns[3][3] = {{cost_kernel<false, 0, false>, cost_kernel<true, 0, false>, cost_kernel<true, 0, true>},
+                                 {cost_kernel<false, 1, false>, cost_kernel<true, 1, false>, cost_kernel<true, 1, true>},
+                                 {cost_kernel<false, 2, false>, cost_kernel<true, 2, false>, cost_kernel<true, 2, true>}};
+    fns[kind][!quant ? 0 : lb_sum ? 2 : 1]<<<(n_conf + per - 1) / per, kCostThreads, 0, st>>>(
+        p->dc, c2, c2f, quant ? coef : nullptr, quant ? nullptr : coeff, lb_sum, p->d_range, p_lo, n_conf);
+    CUDA_TRY(p, cudaGetLastError());
     return HAP_OK;
 }
 
@@ -1314,13 +1349,6 @@ static cudaError_t raise_smem_limit(int device, const void *fn, size_t bytes)
     return e;
 }
 
-static int sm_count(int device)
-{
-    static int n[64];                                       // (the same value whoever writes it)
-    int &v = n[device & 63];
-    if (!v && cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) { cudaGetLastError(); v = 148; }
-    return v;
-}
 
 // launch behind the kernel before it in the stream, as its programmatic dependent
 static cudaError_t launch_dependent(const void *fn, unsigned grid, unsigned threads, size_t smem, cudaStream_t st, void **args)
@@ -1748,7 +1776,9 @@ static bool joint_reach_class(const hap_problem *p, int PP, int64_t G, const Joi
                 ent.push_back(e);
             }
     }
-    if (words > 2) return false;
+    // few cells: the value form's chain (a level each) is shorter than a dozen tests of it (32 devices, 19 layers: 244 us
+    // against 418 us; 48 devices, 29 layers: 185 against 332; the line lies between those and 16 stages at 1,024 devices)
+    if (words > 2 || (i64)jc.S * T * N < 16384) return false;
     jr.words = words;
     return reach_smem(N, T, p->prof.R, p->dc.tau_linear ? p->prof.R : 2, PP, jc.lmax, jr.nwin, words).total <= 110 * 1024;
 }
@@ -1925,6 +1955,22 @@ extern "C" hap_status hap_get_timings(hap_problem *p, float *ms_layer_cost, floa
     return check_values(p);
 }
 
+// The layer costs of the configurations that own the given plans, then the kernel that evaluates them as their programmatic
+// dependent.
+static hap_status launch_plan_eval(hap_problem *p, const void *fn, unsigned blocks, unsigned threads, u64 first, u64 count, const uint8_t *part,
+                                   const uint8_t *rec, int64_t *t_iter, int64_t *detail, cudaStream_t st)
+{
+    unsigned p_lo, p_hi;
+    configs_of_range(p, first, count, p_lo, p_hi);
+    hap_status s;
+    if ((s = launch_layer_costs(p, p->d_c2, p->d_coef, nullptr, nullptr, true, st, nullptr, p_lo, p_hi)) != HAP_OK) return s;
+    const i64 *c2 = p->d_c2, *coef = p->d_coef;
+    void *args[] = {(void *)&p->dc, (void *)&first, (void *)&count, (void *)&c2, (void *)&coef, (void *)&part, (void *)&rec, (void *)&t_iter, (void *)&detail,
+                    (void *)&p_lo, (void *)&p_hi};
+    CUDA_TRY(p, launch_dependent(fn, blocks, threads, 0, st, args));
+    return HAP_OK;
+}
+
 extern "C" hap_status hap_eval_appendix_b(hap_problem *p, uint64_t first, uint64_t count, const uint8_t *dev_partition,
                                           const uint8_t *dev_recompute, int64_t *dev_t_iter, int64_t *dev_detail, void *stream)
 {
@@ -1937,10 +1983,7 @@ extern "C" hap_status hap_eval_appendix_b(hap_problem *p, uint64_t first, uint64
     if (blocks > 0x7fffffffull) return fail(p, HAP_E_RANGE, "count too large for one launch");
     cudaStream_t st = (cudaStream_t)stream;
     if ((s = ensure_general(p)) != HAP_OK) return s;
-    if ((s = launch_layer_costs(p, p->d_c2, p->d_coef, nullptr, nullptr, true, st)) != HAP_OK) return s;
-    appendix_b_kernel<<<(unsigned)blocks, 128, 0, st>>>(p->dc, first, count, p->d_c2, p->d_coef, dev_partition, dev_recompute,
-                                                        (i64 *)dev_t_iter, (i64 *)dev_detail);
-    CUDA_TRY(p, cudaGetLastError());
+    if ((s = launch_plan_eval(p, (const void *)appendix_b_kernel, (unsigned)blocks, 128, first, count, dev_partition, dev_recompute, dev_t_iter, dev_detail, st)) != HAP_OK) return s;
     return leave_async(p, st);
 }
 
@@ -1955,10 +1998,7 @@ extern "C" hap_status hap_simulate_1f1b(hap_problem *p, uint64_t first, uint64_t
     if (count > 0x7fffffffull) return fail(p, HAP_E_RANGE, "count too large for one launch");
     cudaStream_t st = (cudaStream_t)stream;
     if ((s = ensure_general(p)) != HAP_OK) return s;
-    if ((s = launch_layer_costs(p, p->d_c2, p->d_coef, nullptr, nullptr, true, st)) != HAP_OK) return s;
-    simulate_1f1b_kernel<<<(unsigned)count, 32, 0, st>>>(p->dc, first, count, p->d_c2, p->d_coef, dev_partition, dev_recompute,
-                                                         (i64 *)dev_t_iter, (i64 *)dev_detail);
-    CUDA_TRY(p, cudaGetLastError());
+    if ((s = launch_plan_eval(p, (const void *)simulate_1f1b_kernel, (unsigned)count, 32, first, count, dev_partition, dev_recompute, dev_t_iter, dev_detail, st)) != HAP_OK) return s;
     return leave_async(p, st);
 }
 

@@ -314,7 +314,7 @@ __device__ __forceinline__ bool first_stage_fits(const DevConst &dc, const hap_p
     return fits;
 }
 
-__device__ __forceinline__ void type_const_role(const DevConst &dc, TypeConst *tcg, i64 *coef, double *coeff, u64 *range_flag, u64 p, int h, int role);
+__device__ __forceinline__ void type_const_role(const DevConst &dc, TypeConst *tc_out, i64 *coef, double *coeff, u64 *range_flag, u64 p, int h, int role);
 
 // coef / coeff: integer and / or fp64 form of the coefficients (nullable)
 __global__ void __launch_bounds__(kTcThreads)
@@ -327,7 +327,7 @@ type_const_kernel(const DevConst dc, TypeConst *tcg, i64 *coef, double *coeff, u
     const unsigned pi = blockIdx.x * per + ql;
     const u64 p = (u64)p_first + pi;                          // configurations [p_first, p_first + n_conf)
     const bool on = ql < per && pi < n_conf && p < dc.n_pconf;
-    if (on) type_const_role(dc, tcg, coef, coeff, range_flag, p, h, role);
+    if (on) type_const_role(dc, tcg + p * dc.T + h, coef, coeff, range_flag, p, h, role);
     if (!la.state) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) tree_stamp_begin(la.report);
     for (u32 b = blockIdx.x * kTcThreads + threadIdx.x; b < la.n_hist; b += gridDim.x * kTcThreads) la.hist[b] = 0;
@@ -351,7 +351,20 @@ type_const_kernel(const DevConst dc, TypeConst *tcg, i64 *coef, double *coeff, u
     if (listed) (live ? la.live_list + la.p_lo[ci] : la.dead_list)[at + __popc(same & ((1u << lane) - 1u))] = (u32)p;
 }
 
-__device__ __forceinline__ void type_const_role(const DevConst &dc, TypeConst *tcg, i64 *coef, double *coeff, u64 *range_flag, u64 p, int h, int role)
+// ... without the lists: a grid row per role
+constexpr int kTcPlainThreads = 128;
+template <bool INTEGER>
+__global__ void __launch_bounds__(kTcPlainThreads)
+type_const_plain_kernel(const DevConst dc, TypeConst *tcg, i64 *coef, double *coeff, u64 *range_flag, unsigned p_first, unsigned n_conf)
+{
+    asm volatile("griddepcontrol.launch_dependents;");
+    const unsigned gid = blockIdx.x * kTcPlainThreads + threadIdx.x, pi = gid / HAP_MAX_TYPES;
+    const int h = (int)(gid % HAP_MAX_TYPES);
+    const u64 p = (u64)p_first + pi;
+    if (pi < n_conf && p < dc.n_pconf && h < dc.T) type_const_role(dc, tcg + p * dc.T + h, coef, INTEGER ? nullptr : coeff, range_flag, p, h, (int)blockIdx.y);
+}
+
+__device__ __forceinline__ void type_const_role(const DevConst &dc, TypeConst *tc_out, i64 *coef, double *coeff, u64 *range_flag, u64 p, int h, int role)
 {
     const int T = dc.T;
     const i64 H = dc.H;
@@ -395,7 +408,7 @@ __device__ __forceinline__ void type_const_role(const DevConst &dc, TypeConst *t
         tc.rden = 1.0 / tc.den;
         tc.row = (pc.itp * dc.ncp + pc.icp) * dc.nmb + pc.ib;
         tc.pad = 0;
-        tcg[p * T + h] = tc;
+        *tc_out = tc;
     } else if (role == 1) {
         const size_t i4 = (((size_t)h * dc.ntp + pc.itp) * dc.ncp + pc.icp) * dc.nmb + pc.ib;
         bad |= put_coef(coef, coeff, at, HAP_KPRE, dc.tpre[i4]);
@@ -556,6 +569,76 @@ layer_cost_kernel(const DevConst dc, const TypeConst *__restrict__ tcg, i64 *__r
     }
 }
 
+// The constants and the layer costs of `per` = 32 / T configurations per block: three warps compute the constants (a warp per
+// role) into shared memory and the coefficients, then all warps write the layer costs, a thread per (configuration, layer)
+// for every type.  Written bytes bound it (16 per configuration, type and layer): blocks that compute constants run beside
+// blocks that write, where two launches in a row left the memory idle for the first.  1,024 devices (7,783
+// configurations, 48 MB) do better in two launches, see launch_layer_costs.
+constexpr int kCostThreads = 256;
+template <bool QUANT, int KIND, bool WANT_LB>
+__global__ void __launch_bounds__(kCostThreads)
+cost_kernel(const DevConst dc, i64 *__restrict__ c2, double *__restrict__ c2f, i64 *coef, double *coeff, i64 *__restrict__ lb_sum,
+            u64 *range_flag, unsigned p_first, unsigned n_conf)
+{
+    __shared__ TypeConst tcs[32];
+    __shared__ size_t s_row[32];
+    __shared__ u64 s_lb[32];
+    // what follows may start its part that does not need the costs
+    asm volatile("griddepcontrol.launch_dependents;");
+    const int N = dc.N, T = dc.T, per = 32 / T, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned p0 = p_first + blockIdx.x * per;
+    const int here = (int)(p_first + n_conf - p0 < (unsigned)per ? p_first + n_conf - p0 : (unsigned)per);
+    if (warp < 3) {
+        const int q = lane / T, h = lane - q * T;
+        if (q < here) type_const_role(dc, &tcs[lane], coef, coeff, range_flag, p0 + q, h, warp);
+    } else if (warp == 3 && lane < here) {
+        const hap_pconf *pcf = dc.pconf + p0 + lane;
+        s_row[lane] = ((size_t)pcf->itp * dc.ncp + pcf->icp) * dc.nmb + pcf->ib;               // the same table row for every type
+        s_lb[lane] = 0;
+    }
+    __syncthreads();
+    const size_t stride_h = (size_t)dc.ntp * dc.ncp * dc.nmb * N * 2;                            // double2 pairs between device types
+    const double kappa = dc.kappa;
+    bool bad = false;                                                                          // a value left the supported range
+    for (int e = threadIdx.x; e < here * N; e += kCostThreads) {
+        const int q = e / N, l = e - q * N;
+        const bool dense = KIND == 0 || (KIND == 2 && layer_kind(dc, l) == HAP_DENSE);
+        const double2 *tp = reinterpret_cast<const double2 *>(dc.tab4) + (s_row[q] * N + l) * 2;
+        double2 ta[HAP_MAX_TYPES], tf[HAP_MAX_TYPES];
+#pragma unroll
+        for (int h = 0; h < HAP_MAX_TYPES; ++h)
+            if (h < T) {
+                ta[h] = __ldg(tp);
+                tf[h] = dense ? make_double2(0.0, 0.0) : __ldg(tp + 1);
+                tp += stride_h;
+            }
+        const size_t at = ((size_t)(p0 + q) * T * N + l) * 2;
+        i64 lmin = 0;
+#pragma unroll
+        for (int h = 0; h < HAP_MAX_TYPES; ++h)
+            if (h < T) {
+                double cf, cb;
+                layer_cost_pair(reinterpret_cast<const double2 *>(&tcs[q * T + h]), ta[h], tf[h], dense, kappa, cf, cb);
+                bad |= !(cf < 6.8719e10) | !(cb < 6.8719e10);                                     // 2^36 ns per layer
+                if (QUANT) {
+                    longlong2 v; v.x = __double2ll_rn(cf); v.y = __double2ll_rn(cb);
+                    *reinterpret_cast<longlong2 *>(c2 + at + (size_t)h * N * 2) = v;
+                    if (WANT_LB) { const i64 x = v.x + v.y; lmin = (h == 0 || x < lmin) ? x : lmin; }
+                } else {
+                    double2 v; v.x = cf; v.y = cb;
+                    *reinterpret_cast<double2 *>(c2f + at + (size_t)h * N * 2) = v;
+                }
+            }
+        // every layer runs on some device type: the sum over layers of the cheapest type's time bounds the summed stage time
+        if (QUANT && WANT_LB) atomicAdd(&s_lb[q], (u64)lmin);
+    }
+    if (bad && range_flag) atomicOr(range_flag, 1ull);
+    if (QUANT && WANT_LB) {
+        __syncthreads();
+        if ((int)threadIdx.x < here) lb_sum[p0 + threadIdx.x] = (i64)s_lb[threadIdx.x];
+    }
+}
+
 // ------------------------------------------------------------------------------------------
 // candidate decode: every lane of the warp calls this; lane s < PP receives stage s
 // ------------------------------------------------------------------------------------------
@@ -676,6 +759,16 @@ __device__ __forceinline__ u64 find_pconf(const DevConst &dc, u64 c)
     return lo;
 }
 
+// ... among configurations [lo, hi)
+__device__ __forceinline__ u64 find_pconf_from(const DevConst &dc, u64 c, u64 lo, u64 hi)
+{
+    while (hi - lo > 1) {
+        const u64 mid = (lo + hi) >> 1;
+        if (dc.pconf[mid].offset <= c) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
 __global__ void decode_kernel(const DevConst dc, u64 first, u64 count, hap_candidate *out, const i64 *first_dev)
 {
     const u64 w = ((u64)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -703,33 +796,55 @@ __global__ void decode_kernel(const DevConst dc, u64 first, u64 count, hap_candi
     o->link[lane] = (lane < pc.PP && lane > 0) ? (uint8_t)(sm.cls | (sm.ha << 2) | (sm.hb << 4)) : 0;
 }
 
-// Terms of one stage of a GIVEN plan (layers [a, b) at recomputation level r on the stage's device types): t_f, the
+// Terms of the stages of a GIVEN plan (lane s: layers [a, b) at recomputation level r on the device types of stage s + 1): t_f, the
 // forward time of its layers (slowest member type per layer); the stage cost c = t_f + t_b with t_b the backward
 // time, the recomputed forward work and the stage constant (pre / post-processing, the transfer into the stage);
-// the stage's gradient-synchronisation and optimizer times.  `stage` is 0-based.
-__device__ __forceinline__ void plan_stage_terms(const DevConst &dc, u64 p, int PP, const StageMap &sm, int stage, int a, int b, int r,
-                                                 const i64 *__restrict__ c2, const i64 *__restrict__ coef,
+// the stage's gradient-synchronisation and optimizer times.  The whole warp calls it: lanes run over the layers, whose loads are
+// then independent, and a stage is the difference of two prefix sums in pre[N + 1] (a lane that walks its own
+// layers waits for memory once per layer: 11.4 us instead of 6.3 for 32 layers on up to eight stages).
+__device__ __forceinline__ void plan_stage_terms(const DevConst &dc, u64 p, int PP, const StageMap &sm, int lane, int a, int b, int r,
+                                                 const i64 *__restrict__ c2, const i64 *__restrict__ coef, longlong2 *pre, uint8_t *owner,
                                                  i64 &tf, i64 &cst, i64 &sy, i64 &op)
 {
     const int N = dc.N, T = dc.T;
     const i64 *c2p = c2 + (size_t)p * T * N * 2;
     const i64 *cfp = coef + (size_t)p * T * HAP_NCOEF;
-    i64 tb = 0;
-    tf = 0;
-    for (int l = a; l < b; ++l) {
+    const bool on = lane < PP;
+    if (on) for (int l = a; l < b; ++l) owner[l] = (uint8_t)lane;
+    if (lane == 0) pre[0] = make_longlong2(0, 0);
+    __syncwarp();
+    i64 runF = 0, runB = 0;
+    for (int base = 0; base < N; base += 32) {
+        const int l = base + lane, mask = __shfl_sync(0xffffffffu, sm.mask, l < N ? owner[l] : 0);
         i64 F = 0, B = 0;
-        for (int h = 0; h < T; ++h)
-            if (sm.mask >> h & 1) {
-                const i64 qx = c2p[((size_t)h * N + l) * 2], qy = c2p[((size_t)h * N + l) * 2 + 1];
-                F = qx > F ? qx : F;
-                B = qy > B ? qy : B;
-            }
-        tf += F; tb += B;
+        if (l < N) {
+#pragma unroll
+            for (int h = 0; h < HAP_MAX_TYPES; ++h)
+                if (h < T && (mask >> h & 1)) {
+                    const longlong2 q = *reinterpret_cast<const longlong2 *>(c2p + ((size_t)h * N + l) * 2);
+                    F = q.x > F ? q.x : F;
+                    B = q.y > B ? q.y : B;
+                }
+        }
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const i64 x = __shfl_up_sync(0xffffffffu, F, o), y = __shfl_up_sync(0xffffffffu, B, o);
+            if (lane >= o) { F += x; B += y; }
+        }
+        F += runF; B += runB;
+        if (l < N) pre[l + 1] = make_longlong2(F, B);
+        runF = shfl_i64(F, 31); runB = shfl_i64(B, 31);
     }
+    __syncwarp();
+    tf = cst = sy = op = 0;
+    if (!on) return;
+    tf = pre[b].x - pre[a].x;
+    i64 tb = pre[b].y - pre[a].y;
     // coefficients of a stage of several types: the slowest member's
     i64 kpre = 0, kpost = 0, slat = 0, sbw[2] = {0, 0}, opt[2] = {0, 0};
-    for (int h = 0; h < T; ++h)
-        if (sm.mask >> h & 1) {
+#pragma unroll
+    for (int h = 0; h < HAP_MAX_TYPES; ++h)
+        if (h < T && (sm.mask >> h & 1)) {
             const i64 *row = cfp + h * HAP_NCOEF;
             kpre = row[HAP_KPRE] > kpre ? row[HAP_KPRE] : kpre;
             kpost = row[HAP_KPOST] > kpost ? row[HAP_KPOST] : kpost;
@@ -740,9 +855,9 @@ __device__ __forceinline__ void plan_stage_terms(const DevConst &dc, u64 p, int 
             }
         }
     tb += ((i64)dc.tau_q[r] * tf) >> 10;              // forward work repeated in the backward pass
-    if (stage == 0) tb += kpre;
-    if (stage == PP - 1) tb += kpost;
-    if (stage > 0) tb += cfp[sm.hb * HAP_NCOEF + (sm.cls == HAP_CROSS ? HAP_KP2P_CROSS + sm.ha : HAP_KP2P_INTRA + sm.cls)];
+    if (lane == 0) tb += kpre;
+    if (lane == PP - 1) tb += kpost;
+    if (lane > 0) tb += cfp[sm.hb * HAP_NCOEF + (sm.cls == HAP_CROSS ? HAP_KP2P_CROSS + sm.ha : HAP_KP2P_INTRA + sm.cls)];
     cst = tf + tb;
     const i64 n_moe = (i64)(moe_before(dc, b) - moe_before(dc, a)), n_dense = (i64)(b - a) - n_moe;
     sy = slat + n_dense * sbw[0] + n_moe * sbw[1];
@@ -759,13 +874,16 @@ __device__ __forceinline__ void plan_stage_terms(const DevConst &dc, u64 p, int 
 // ------------------------------------------------------------------------------------------
 __global__ void appendix_b_kernel(const DevConst dc, u64 first, u64 count, const i64 *__restrict__ c2,
                                   const i64 *__restrict__ coef, const uint8_t *__restrict__ partition,
-                                  const uint8_t *__restrict__ recompute, i64 *t_iter, i64 *detail)
+                                  const uint8_t *__restrict__ recompute, i64 *t_iter, i64 *detail, unsigned p_lo, unsigned p_hi)
 {
+    // (launched behind the layer costs: everything up to the wait overlaps them)
+    __shared__ longlong2 s_pre[4][HAP_MAX_LAYERS + 1];
+    __shared__ uint8_t s_owner[4][HAP_MAX_LAYERS + 1];
     const u64 w = ((u64)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     if (w >= count) return;
     const u64 c = first + w;
-    const u64 p = find_pconf(dc, c);
+    const u64 p = find_pconf_from(dc, c, p_lo, p_hi);
     const hap_pconf pc = dc.pconf[p];
     const int PP = pc.PP, N = dc.N;
     const u64 map_idx = (c - pc.offset) / (u64)dc.n_rc;
@@ -785,8 +903,9 @@ __global__ void appendix_b_kernel(const DevConst dc, u64 first, u64 count, const
         }
         return;
     }
-    i64 tf = 0, cst = 0, sy = 0, op = 0;
-    if (on) plan_stage_terms(dc, p, PP, sm, lane, b_me - n_me, b_me, r_me, c2, coef, tf, cst, sy, op);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    i64 tf, cst, sy, op;
+    plan_stage_terms(dc, p, PP, sm, lane, b_me - n_me, b_me, r_me, c2, coef, s_pre[wib], s_owner[wib], tf, cst, sy, op);
     const i64 edge = warp_sum_i64(cst), cmax = warp_max_i64(cst);
     const i64 t_sync = warp_max_i64(sy), t_opt = warp_max_i64(op);
     const unsigned at_max = __ballot_sync(0xffffffffu, on && cst == cmax);
@@ -820,14 +939,16 @@ constexpr int kSimRing = 64;
 
 __global__ void __launch_bounds__(32)
 simulate_1f1b_kernel(const DevConst dc, u64 first, u64 count, const i64 *__restrict__ c2, const i64 *__restrict__ coef,
-                     const uint8_t *__restrict__ partition, const uint8_t *__restrict__ recompute, i64 *t_iter, i64 *detail)
+                     const uint8_t *__restrict__ partition, const uint8_t *__restrict__ recompute, i64 *t_iter, i64 *detail, unsigned p_lo, unsigned p_hi)
 {
+    __shared__ longlong2 s_pre[HAP_MAX_LAYERS + 1];
+    __shared__ uint8_t s_owner[HAP_MAX_LAYERS + 1];
     __shared__ i64 ringF[HAP_MAX_PP][kSimRing], ringB[HAP_MAX_PP][kSimRing];
     const u64 w = blockIdx.x;
     const int lane = threadIdx.x;
     if (w >= count) return;
     const u64 c = first + w;
-    const u64 p = find_pconf(dc, c);
+    const u64 p = find_pconf_from(dc, c, p_lo, p_hi);
     const hap_pconf pc = dc.pconf[p];
     const int PP = pc.PP, N = dc.N, M = pc.M;
     const u64 map_idx = (c - pc.offset) / (u64)dc.n_rc;
@@ -847,8 +968,9 @@ simulate_1f1b_kernel(const DevConst dc, u64 first, u64 count, const i64 *__restr
         }
         return;
     }
-    i64 tf = 0, cst = 0, sy = 0, op = 0;
-    if (on) plan_stage_terms(dc, p, PP, sm, lane, b_me - n_me, b_me, r_me, c2, coef, tf, cst, sy, op);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    i64 tf, cst, sy, op;
+    plan_stage_terms(dc, p, PP, sm, lane, b_me - n_me, b_me, r_me, c2, coef, s_pre, s_owner, tf, cst, sy, op);
     const i64 tb = cst - tf;
     const i64 csum = warp_sum_i64(cst), cmax = warp_max_i64(cst);
     const i64 t_sync = warp_max_i64(sy), t_opt = warp_max_i64(op);
@@ -860,38 +982,35 @@ simulate_1f1b_kernel(const DevConst dc, u64 first, u64 count, const i64 *__restr
     // 2 (M + PP), which bounds the rounds
     const int max_rounds = 4 * (M + PP) + 16;
     bool stuck = true;
+    // A round is a chain of one shuffle, a maximum and an addition: the end times that either kind of pass would wait for are
+    // read beside the shuffle, and whether all stages are done is asked every eighth round (a finished stage does nothing).
+    const int from = lane > 0 ? lane - 1 : 0, to = lane + 1 < PP ? lane + 1 : lane;
     for (int round = 0; round < max_rounds; ++round) {
-        const int nf_prev = __shfl_up_sync(0xffffffffu, nf, 1), nb_next = __shfl_down_sync(0xffffffffu, nb, 1);
         const bool active = on && nb < M;
-        if (!__any_sync(0xffffffffu, active)) { stuck = false; break; }
+        if ((round & 7) == 0 && !__any_sync(0xffffffffu, active)) { stuck = false; break; }
+        const int nf_prev = __shfl_up_sync(0xffffffffu, nf, 1), nb_next = __shfl_down_sync(0xffffffffu, nb, 1);
+        const i64 in_f = ringF[from][nf & (kSimRing - 1)];
+        // (the last stage's own forward pass of the micro-batch came just before its backward pass)
+        const i64 in_b = lane == PP - 1 ? t_free : ringB[to][nb & (kSimRing - 1)];
+#ifdef HAP_CHECKED
         {   // a stage is never a whole ring of passes ahead of the neighbour that consumes them
             const int nf_next = __shfl_down_sync(0xffffffffu, nf, 1), nb_prev = __shfl_up_sync(0xffffffffu, nb, 1);
             (void)HAP_CHECK_OK(9, !(on && lane + 1 < PP) || nf - nf_next < kSimRing);
             (void)HAP_CHECK_OK(9, !(on && lane > 0) || nb - nb_prev < kSimRing);
-            (void)nf_next; (void)nb_prev;
         }
-        if (active) {
-            const bool fwd = nf < M && (nf < warm || nf - nb == warm);       // the stage's next pass in its fixed order
-            bool ready;
-            i64 dep = 0;
-            if (fwd) {
-                ready = lane == 0 || nf_prev > nf;
-                if (ready && lane > 0) dep = ringF[lane - 1][nf & (kSimRing - 1)];
-            } else if (lane == PP - 1) {
-                ready = true;                                                 // its own forward pass of the micro-batch came just before
-                dep = ringF[lane][nb & (kSimRing - 1)];
-            } else {
-                ready = nb_next > nb;
-                if (ready) dep = ringB[lane + 1][nb & (kSimRing - 1)];
-            }
-            if (ready) {
-                const i64 start = t_free > dep ? t_free : dep;
-                if (fwd) { t_free = start + tf; ringF[lane][nf & (kSimRing - 1)] = t_free; ++nf; }
-                else { t_free = start + tb; ringB[lane][nb & (kSimRing - 1)] = t_free; ++nb; }
-            }
+#endif
+        const bool fwd = nf < M && (nf < warm || nf - nb == warm);           // the stage's next pass in its fixed order
+        const bool ready = active && (fwd ? lane == 0 || nf_prev > nf : lane == PP - 1 || nb_next > nb);
+        const i64 dep = fwd ? (lane > 0 ? in_f : 0) : in_b;
+        __syncwarp();                                                        // (the rings have been read)
+        if (ready) {
+            t_free = (t_free > dep ? t_free : dep) + (fwd ? tf : tb);
+            if (fwd) { ringF[lane][nf & (kSimRing - 1)] = t_free; ++nf; }
+            else { ringB[lane][nb & (kSimRing - 1)] = t_free; ++nb; }
         }
         __syncwarp();
     }
+    if (stuck && !__any_sync(0xffffffffu, on && nb < M)) stuck = false;
     const i64 end = warp_max_i64(on ? t_free : 0);
     if (lane == 0) {
         const i64 sim = stuck ? kInf : end;

@@ -11,14 +11,13 @@ from oracle import Oracle  # noqa: E402
 
 
 @pytest.mark.parametrize("nodes,N,window,tau,dense_first", [
-    ((2, 2), 8, True, (0, 1024), False),           # as many layers as stages
-    ((2, 2), 67, False, (0, 1024), False),         # 64 end layers at four stages: one word, the last bit of it
-    ((2, 2), 68, False, (0, 1024), False),         # 65: two words
-    ((2, 2), 75, False, (0, 1024), False),
-    ((2, 2), 67, True, (0, 307, 1024), True),
-    ((2, 1, 1), 130, False, (0, 1024), True),      # value form
-    ((1, 1, 1, 1), 21, True, (0, 1024, 2048), False),
-    ((4,), 33, True, (0, 500), False),             # one type
+    ((2, 2), 8, True, (0, 1024), False),              # as many layers as stages; few states: a value per end layer
+    ((1, 1, 1, 1), 71, False, (0, 1024), False),      # 64 end layers at eight stages: one word, the last bit of it
+    ((1, 1, 1, 1), 72, False, (0, 1024), False),      # 65: two words
+    ((2, 2, 2, 2), 48, True, (0, 307, 1024), True),
+    ((2, 1, 1), 130, False, (0, 1024), True),
+    ((1, 1, 1, 1), 150, False, (0, 1024), False),     # more than two words
+    ((2, 2, 2, 2), 33, True, (0, 500), False),
 ])
 def test_joint_bottleneck_words(nodes, N, window, tau, dense_first):
     import paper_2609_39350_b200 as hap
@@ -34,7 +33,7 @@ def test_joint_bottleneck_words(nodes, N, window, tau, dense_first):
     seen = 0
     for p in np.random.default_rng(N).permutation(o.n_pconf).tolist():
         for rc in range(2):
-            if got[p, rc] == -1 or seen >= 60:
+            if got[p, rc] == -1 or seen >= 60 or (seen >= 40 and o.pconfs[p]["PP"] < 8):
                 continue
             c2, _, coef, _ = o.layer_costs(p)
             assert got[p, rc] == o.joint_bottleneck(p, int(pb.rc_masks[rc]), c2, coef), (p, rc)

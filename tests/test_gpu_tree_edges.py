@@ -19,7 +19,7 @@ CASES = [
     ((2, 1, 1), 18, (0, 307, 1024), (1, 3, 7), "dense_first"),         # levels that are not combined into rows
     ((2, 1, 1), 23, (0, 1024, 2048), (7, 5, 4), "mixed"),
     ((1, 1, 1, 1), 16, (0, 1024, 2048, 3072), (15, 9, 6, 1), "uniform"),
-    ((4, 2, 2), 25, (0, 200, 700, 1000), (15, 3), "dense_first"),
+    ((3, 1), 25, (0, 200, 700, 1000), (15, 3), "dense_first"),
 ]
 
 
