@@ -125,9 +125,10 @@ struct hap_problem {
     cudaEvent_t ev_upload = nullptr;       // the upload of the tables
     bool upload_pending = false;           // no completed call has waited for that upload yet
     cudaEvent_t ev_fork = nullptr;         // general kernel: classes run on their own streams between this event and their `done` events
-    cudaEvent_t ev_done = nullptr;         // end of the last asynchronous call
-    bool in_flight = false;                // that call has not been waited for
+    bool in_flight = false;                // an asynchronous call has not been waited for
     cudaStream_t last_stream = nullptr;    // the stream it went to
+    bool upload_waited = false;            // a call on upload_stream has waited for the upload: later ones on it are behind it
+    cudaStream_t upload_stream = nullptr;
     std::string err;
 };
 
@@ -467,14 +468,14 @@ static void release_device(hap_problem *p)
 {
     // nothing of this problem may still be running when its memory goes back to the cache
     if (p->upload_pending) { cudaEventSynchronize(p->ev_upload); p->upload_pending = false; }
-    if (p->in_flight) { cudaEventSynchronize(p->ev_done); p->in_flight = false; }
+    if (p->in_flight) { cudaDeviceSynchronize(); p->in_flight = false; }
     cached_free(p->d_tables); cached_free(p->d_arena); cached_free(p->d_gen_arena);
     cached_free(p->d_joint_scratch);
     for (auto &r : p->reach) cached_free(r.d);
     for (auto &j : p->joint) { cached_free(j.d_ids); cached_free(j.d_arrays); }
     cached_free(p->d_c2f); cached_free(p->d_coeff); cached_free(p->d_fcost); cached_free(p->d_cand_lb);
     for (auto &e : p->ev) if (e) cudaEventDestroy(e);
-    pooled_event_put(p->device, p->ev_fork); pooled_event_put(p->device, p->ev_done); pooled_event_put(p->device, p->ev_upload);
+    pooled_event_put(p->device, p->ev_fork); pooled_event_put(p->device, p->ev_upload);
     for (auto &cl : p->classes) pooled_event_put(p->device, cl.done);              // the class streams belong to the pool
     result_slot_put(p->host_result);
 }
@@ -632,7 +633,6 @@ extern "C" hap_status hap_problem_create(const hap_model *mo, const hap_cluster 
         if (e == cudaErrorInvalidValue) { cudaGetLastError(); return HAP_E_INVALID; }
         if (e != cudaSuccess) return HAP_E_CUDA;
     }
-    if (!(p->ev_done = pooled_event(p->device))) return HAP_E_CUDA;
 
     DevConst &dc = p->dc;
     std::memset(&dc, 0, sizeof(dc));
@@ -1127,15 +1127,27 @@ static hap_status enter(hap_problem *p, cudaStream_t st)
     if (!p) return HAP_E_INVALID;
     if (!p->enumerated) return fail(p, HAP_E_STATE, "hap_enumerate has not run");
     if (cudaSetDevice(p->device) != cudaSuccess) return fail(p, HAP_E_CUDA, "cudaSetDevice");
-    if (p->upload_pending) CUDA_TRY(p, cudaStreamWaitEvent(st, p->ev_upload, 0));
-    if (p->in_flight && st != p->last_stream) CUDA_TRY(p, cudaStreamWaitEvent(st, p->ev_done, 0));
+    if (p->upload_pending && !(p->upload_waited && st == p->upload_stream)) {
+        if (p->upload_waited && cudaEventQuery(p->ev_upload) == cudaSuccess) p->upload_pending = false;
+        else {
+            if (p->upload_waited) cudaGetLastError();          // (not ready)
+            CUDA_TRY(p, cudaStreamWaitEvent(st, p->ev_upload, 0));
+            p->upload_waited = true; p->upload_stream = st;
+        }
+    }
+    if (p->in_flight && st != p->last_stream) {
+        // the calls of a problem share its scratch memory.  An event per call would order them, too, but costs each call a
+        // microsecond of its stream; a change of streams is rare (and cannot wait inside a capture)
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        CUDA_TRY(p, cudaStreamIsCapturing(st, &cap));
+        if (cap == cudaStreamCaptureStatusNone) { CUDA_TRY(p, cudaDeviceSynchronize()); p->in_flight = false; }
+    }
     return HAP_OK;
 }
 
 // ... and ends here: the work it queued on `st` is in flight
 static hap_status leave_async(hap_problem *p, cudaStream_t st)
 {
-    CUDA_TRY(p, cudaEventRecord(p->ev_done, st));
     p->in_flight = true;
     p->last_stream = st;
     return HAP_OK;
@@ -1940,7 +1952,7 @@ extern "C" hap_status hap_get_timings(hap_problem *p, float *ms_layer_cost, floa
     if (!p) return HAP_E_INVALID;
     if (!p->enumerated || !p->timed) return fail(p, HAP_E_STATE, "no hap_pipeline_dp or hap_search_* call to report on");
     if (cudaSetDevice(p->device) != cudaSuccess) return fail(p, HAP_E_CUDA, "cudaSetDevice");
-    if (p->in_flight) CUDA_TRY(p, cudaEventSynchronize(p->ev_done));
+    if (p->in_flight) { CUDA_TRY(p, cudaDeviceSynchronize()); p->in_flight = false; }
     if (p->timed == 2) {
         TreeReport ts;
         CUDA_TRY(p, cudaMemcpy(&ts, p->targs.report, sizeof(ts), cudaMemcpyDeviceToHost));
