@@ -2,6 +2,7 @@
 from __future__ import annotations
 
 import ctypes as C
+import operator
 import weakref
 import os
 from typing import Optional
@@ -187,16 +188,27 @@ def _field_address(memo: dict, pb, name: str, dtype, keep: list) -> int:
     return memo[name][2]
 
 
-def hap_problem_create(pb, prune: int = 0, flags: int = 0) -> HapProblem:
-    """Marshals a plain-data problem (see gen.problems.Problem) into the C descriptors."""
-    L = load_library()
+_FIELDS = ("N", "S", "H", "E", "k", "n_shared", "F_dense", "F_exp", "nq", "nkv", "V", "GB", "beta", "kind", "P", "C", "node_size", "bw_intra",
+           "node_type", "node_bw_inter", "tp_list", "cp_list", "mb_list", "ep_list", "xi_q", "tau_q", "tdf", "tdb", "tff", "tfb", "tpre",
+           "tpost", "eta", "croute", "alpha", "rho", "act_coef", "copt", "kappa", "chi", "gamma", "ovl_tp", "ovl_cp", "ovl_dp", "capf",
+           "cap_eff", "fsize", "feff", "pp_list", "tpe_list", "tp_max", "delta_q", "map_cap", "rc_masks", "uniform", "het_coll", "eta_q")
+_MISSING = object()
+
+
+def _descriptors(pb):
+    """The C descriptors of a problem (their arrays' owners beside them).  Filling them costs 16 us, an eighth of a small
+    replan, so they are remembered beside the problem object for as long as each of its fields holds the same object;
+    the library reads the arrays' contents anew on every call."""
+    memo = _address_memo(pb)
+    own = getattr(pb, "__dict__", None)
+    now = [own.get(n, _MISSING) for n in _FIELDS] if own is not None else None
+    hit = memo.get("")
+    if hit is not None and now is not None and all(map(operator.is_, now, hit[0])):
+        return hit[1]
     keep = []
 
-    # addresses of the problem's arrays, remembered per problem object and field for as long as the field holds the
-    # same array object (looking an address up costs more than everything else here); kept beside the object, not in
-    # it, so that copies of the problem start empty
-    memo = _address_memo(pb)
-
+    # addresses of the problem's arrays, remembered per field for as long as the field holds the same array object; kept
+    # beside the object, not in it, so that copies of the problem start empty
     def arr(name, dtype):
         return _field_address(memo, pb, name, dtype, keep)
 
@@ -232,10 +244,25 @@ def hap_problem_create(pb, prune: int = 0, flags: int = 0) -> HapProblem:
     so.tp_max, so.delta_q, so.map_cap = int(pb.tp_max), int(pb.delta_q), int(pb.map_cap)
     so.n_rc = len(pb.rc_masks)
     so.rc_masks = arr("rc_masks", np.uint32)
-    so.prune = int(prune)
-    so.flags = (int(flags) | (OPT_UNIFORM if int(getattr(pb, "uniform", 0)) else 0)
-                | (OPT_HETERO_DISPATCH if int(getattr(pb, "het_coll", 0)) else 0))
+    so.flags = (OPT_UNIFORM if int(getattr(pb, "uniform", 0)) else 0) | (OPT_HETERO_DISPATCH if int(getattr(pb, "het_coll", 0)) else 0)
     so.eta_q = int(getattr(pb, "eta_q", 0))
+    got = (mo, cl, pf, so, keep)
+    # not remembered: a field that the class provides (a property may change without the object's own fields changing) and
+    # one whose contents were converted or copied here
+    held = {id(a) for a in keep}
+    if now is not None and all((v is _MISSING and not hasattr(type(pb), n)) or isinstance(v, (int, float, np.generic)) or id(v) in held
+                               for n, v in zip(_FIELDS, now)):
+        memo[""] = (now, got)
+    return got
+
+
+def hap_problem_create(pb, prune: int = 0, flags: int = 0) -> HapProblem:
+    """Marshals a plain-data problem (see gen.problems.Problem) into the C descriptors."""
+    L = load_library()
+    mo, cl, pf, base, keep = _descriptors(pb)      # (`keep` holds the arrays until the call has read them)
+    so = _Opts.from_buffer_copy(base)
+    so.prune = int(prune)
+    so.flags = int(flags) | base.flags
     out = C.c_void_p(0)
     st = L.hap_problem_create(C.byref(mo), C.byref(cl), C.byref(pf), C.byref(so), C.byref(out))
     if st != 0:
@@ -331,14 +358,13 @@ def hap_search_range_f64(hp: HapProblem, first: int, count: int, stream=None):
 
 def _plan_dict(pl: _Plan) -> dict:
     PP = pl.PP
-    return dict(index=int(pl.index), **{n: int(getattr(pl, n)) for n in ("PP", "TP", "CP", "DP", "EP", "TPE", "b", "M")},
-                rc_mask=int(pl.rc_mask), n=[int(x) for x in pl.n[:PP]], mask=[int(x) for x in pl.mask[:PP]],
-                r=[int(x) for x in pl.r[:PP]], T_iter=int(pl.T_iter), bottleneck=int(pl.bottleneck),
-                T_pipe=int(pl.T_pipe), T_sync=int(pl.T_sync), T_opt=int(pl.T_opt))
+    return dict(index=pl.index, PP=PP, TP=pl.TP, CP=pl.CP, DP=pl.DP, EP=pl.EP, TPE=pl.TPE, b=pl.b, M=pl.M, rc_mask=pl.rc_mask,
+                n=pl.n[:PP], mask=pl.mask[:PP], r=pl.r[:PP], T_iter=pl.T_iter, bottleneck=pl.bottleneck, T_pipe=pl.T_pipe,
+                T_sync=pl.T_sync, T_opt=pl.T_opt)
 
 
 def _stats_dict(st: _Stats) -> dict:
-    return {n: (float(getattr(st, n)) if n.startswith("ms_") else int(getattr(st, n))) for n, _ in _Stats._fields_}
+    return {n: getattr(st, n) for n, _ in _Stats._fields_}          # (ctypes hands out Python ints and floats)
 
 
 def hap_search_range(hp: HapProblem, first: int, count: int, stream=None):
