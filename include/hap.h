@@ -212,7 +212,7 @@ typedef struct {
     uint64_t n_evaluated;   /* candidates whose dynamic program ran */
     uint64_t n_pruned;      /* candidates skipped by the lower bound */
     uint64_t n_feasible;    /* evaluated candidates with a finite cost */
-    float ms_layer_cost, ms_dp, ms_total;   /* CUDA-event times of the phases on `stream` */
+    float ms_layer_cost, ms_dp, ms_total;   /* device times of the phases on `stream` (time stamps of the kernels, or events) */
 } hap_search_stats;
 
 typedef struct hap_problem hap_problem;
@@ -339,7 +339,7 @@ hap_status hap_joint_bottleneck(hap_problem *, int64_t *dev_out, void *stream);
  * the range, independent of what the dynamic-program kernel skips or shares.  Synchronises `stream`. */
 hap_status hap_count_cells(hap_problem *, uint64_t first, uint64_t count, uint64_t *host_cells, void *stream);
 
-/* Measurement aid: CUDA-event durations (ms) of the layer-cost kernel and of the dynamic-program
+/* Measurement aid: device durations (ms) of the layer-cost kernel and of the dynamic-program
  * kernel of the most recent hap_pipeline_dp / hap_search_* call, and -- for a problem created with
  * HAP_OPT_COUNT_SPLITS, 0 otherwise -- the number of splits (k, j pairs inside the window and the memory limit) that
  * a hap_pipeline_dp launch evaluated, counted after its early exits: the work executed, as opposed to
@@ -399,9 +399,9 @@ hap_status hap_problem_dims(const hap_problem *, int32_t *host_N, int32_t *host_
 hap_status hap_self_check(uint64_t *host_sites);
 
 /* Measurement aid: the number of kernels one hap_pipeline_dp call over the whole candidate space followed by
- * one hap_argmin call launches (the two layer-cost kernels, the candidate decode and the tree gather - one launch
- * each for all PP classes when every class walks its prefix tree, else per class -, the dynamic program per PP
- * class, the two reduction kernels).  Host value, no device work. */
+ * one hap_argmin call launches (when every PP class walks its prefix tree: the per-type constants, the records, the
+ * dynamic program of the deep and of the other classes; else also the layer costs and the dynamic program per class on
+ * the general kernel; the two reduction kernels).  Host value, no device work. */
 hap_status hap_launches_per_pass(hap_problem *, uint32_t *host_count);
 
 const char *hap_status_str(hap_status);

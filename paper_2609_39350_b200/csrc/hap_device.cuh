@@ -95,6 +95,7 @@ struct WorkItem {
 // What a block of a tree search leaves beside its (cost, index) minimum: the plan of that candidate.
 struct __align__(16) PlanSlot {
     i64 bott, T_pipe, T_sync, T_opt;
+    u64 p;                                    // configuration
     uint8_t n[HAP_MAX_PP], r[HAP_MAX_PP];     // layers and recomputation level of stages 1..PP (the rest is not written)
 };
 

@@ -723,22 +723,20 @@ __device__ __forceinline__ void tree_finish(const TreeArgs &ta, const DevConst &
     if (bc < inf_bits && mine == bi && mine_c == bc) *s_item = at;
     __syncthreads();
     if (wib != 0) return;
-    TreeResult *rs = ta.res_dev, *rh = ta.res_host;
-    for (int copy = 0; copy < 2; ++copy) {
-        TreeResult *w = copy == 0 ? rs : rh;
-        if (!w) continue;
-        if (lane == 0) {
-            w->range_flag = __ldcg(ta.range_flag);
-            w->n_feasible = __ldcg(&ta.report->n_feasible); w->n_pruned = __ldcg(&ta.report->n_pruned);
-            w->cost = bc; w->index = bi; w->again = again;
-            for (int q = 0; q < 3; ++q) w->stamp[q] = __ldcg(&ta.report->stamp[q]);
-        }
-        if (!(bc < inf_bits)) continue;
-        const u64 p = find_pconf(dc, bi);
+    // (the slot names the winner's configuration: a search for it in the table is a chain of a dozen loads, 6 us)
+    TreeResult *w = ta.res_host ? ta.res_host : ta.res_dev;
+    if (lane == 0) {
+        w->range_flag = __ldcg(ta.range_flag);
+        w->n_feasible = n_feasible; w->n_pruned = n_pruned;
+        w->cost = bc; w->index = bi; w->again = again;
+        for (int q = 0; q < 3; ++q) w->stamp[q] = __ldcg(&ta.report->stamp[q]);
+    }
+    if (bc < inf_bits) {
+        const PlanSlot *ps = ta.slots + *s_item;
+        const u64 p = __ldcg(&ps->p);
         const hap_pconf pc = dc.pconf[p];
         const u64 loc = bi - pc.offset, map_idx = loc / (u64)n_rc;
         const StageMap sm = decode_stage(dc, pc, map_idx, lane);
-        const PlanSlot *ps = ta.slots + *s_item;
         if (lane == 0) {
             w->pconf = (u32)p; w->rc_mask = ta.rc_masks[loc - map_idx * (u64)n_rc];
             w->bott = __ldcg(&ps->bott); w->T_pipe = __ldcg(&ps->T_pipe); w->T_sync = __ldcg(&ps->T_sync); w->T_opt = __ldcg(&ps->T_opt);
@@ -771,7 +769,7 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
     u64 best_index = ~0ull;
     u32 n_feas = 0, splits = 0;
     u64 plan_n[2][HAP_MAX_PP / 8], plan_r[2][HAP_MAX_PP / 8];    // the plan at hand and the plan of the thread's best candidate
-    i64 plan_val[2][4];
+    i64 plan_val[2][5];
     u32 plan_cur = 0;
 
     // A second launch of the same pass starts once every block of the first is running, i.e. past the first one's wait for
@@ -1089,6 +1087,7 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
                             plan_val[plan_cur][0] = bott_bits; plan_val[plan_cur][1] = T_pipe;
                             plan_val[plan_cur][2] = F64 ? __double_as_longlong(t_sync) : (i64)t_sync;
                             plan_val[plan_cur][3] = F64 ? __double_as_longlong(t_opt) : (i64)t_opt;
+                            plan_val[plan_cur][4] = (i64)hd->p;
                             plan_cur ^= 1u;                                    // the place just filled is kept, the other one is written next
                         }
                     } else {
@@ -1173,6 +1172,7 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
             PlanSlot *ps = ta.slots + slot;
             const u32 kp = plan_cur ^ 1u;
             ps->bott = plan_val[kp][0]; ps->T_pipe = plan_val[kp][1]; ps->T_sync = plan_val[kp][2]; ps->T_opt = plan_val[kp][3];
+            ps->p = (u64)plan_val[kp][4];
             for (int w = 0; w < HAP_MAX_PP / 8; ++w) {                       // (words of later stages are whatever the thread's memory held)
                 reinterpret_cast<u64 *>(ps->n)[w] = plan_n[kp][w];
                 reinterpret_cast<u64 *>(ps->r)[w] = plan_r[kp][w];
@@ -1221,7 +1221,7 @@ tree_refine_kernel(const TreeArgs ta, const DevConst dc, int exact, int max_pp)
     const u64 listed = __ldcg(&ta.state->n_surv), n = listed < ta.max_surv ? listed : ta.max_surv;
     const u64 plain = ~__ldcg(&ta.state->incumbent);
     i64 best_cost = kInf, best_bott = 0, best_pipe = 0, best_sync = 0, best_opt = 0;
-    u64 best_index = ~0ull, n_refined = 0, n_ok = 0;
+    u64 best_index = ~0ull, best_p = 0, n_refined = 0, n_ok = 0;
     int best_n = 0, best_r = 0;
 
     while (true) {
@@ -1406,7 +1406,7 @@ tree_refine_kernel(const TreeArgs ta, const DevConst dc, int exact, int max_pp)
         if (T_iter < kInf) n_ok++;
         if (T_iter < best_cost || (T_iter == best_cost && T_iter < kInf && c < best_index)) {
             best_cost = T_iter; best_index = c; best_bott = (i64)bott; best_pipe = T_pipe; best_sync = (i64)sy; best_opt = (i64)op;
-            best_n = len; best_r = my_r;
+            best_n = len; best_r = my_r; best_p = hd->p;
             if (lane == 0) atomicMax(&ta.state->refined, ~(u64)T_iter);
         }
     }
@@ -1422,7 +1422,7 @@ tree_refine_kernel(const TreeArgs ta, const DevConst dc, int exact, int max_pp)
         PlanSlot *ps = ta.slots + blockIdx.x;
         if (lane == 0) {
             ta.slot_cost[blockIdx.x] = best_cost; ta.slot_index[blockIdx.x] = best_index;
-            ps->bott = best_bott; ps->T_pipe = best_pipe; ps->T_sync = best_sync; ps->T_opt = best_opt;
+            ps->bott = best_bott; ps->T_pipe = best_pipe; ps->T_sync = best_sync; ps->T_opt = best_opt; ps->p = best_p;
         }
         ps->n[lane] = (uint8_t)best_n; ps->r[lane] = (uint8_t)best_r;
     }
