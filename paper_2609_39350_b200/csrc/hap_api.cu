@@ -714,6 +714,14 @@ static uint64_t sequences_sat(const int *cnt, int T, uint64_t sat)
 
 template <class V> static void key_put(std::string &k, const V &v) { k.append(reinterpret_cast<const char *>(&v), sizeof(v)); }
 
+static int sm_count(int device)
+{
+    static int n[64];                                       // (the same value whoever writes it)
+    int &v = n[device & 63];
+    if (!v && cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) { cudaGetLastError(); v = 148; }
+    return v;
+}
+
 // ---- per-process cache of the classes' prefix trees (host side) ------------------------------------------
 namespace {
 struct TreeCache { std::mutex mu; std::map<std::string, std::shared_ptr<const TreeClassHost>> map; };
@@ -724,11 +732,11 @@ constexpr size_t kTreeCacheEntries = 256;
 // everything the mappings, the windows, the bands, the task lists and the split into parts depend on
 static std::string tree_cache_key(const hap_problem *p, const hap_problem::PpClass &cl, bool want_tree)
 {
-    std::string k("hap-tree-2");
+    std::string k("hap-tree-3");
     const hap_pconf &rep = p->pconfs[p->items[cl.item_lo].p];
     const size_t n_conf = p->items[cl.item_hi - 1].p - p->items[cl.item_lo].p + 1;
     const int32_t head[] = {p->model.N, p->T, p->prof.R, cl.PP, rep.G, rep.mode, p->opts.delta_q, (int32_t)(p->opts.flags & HAP_OPT_UNIFORM),
-                            p->dc.kind_uniform, p->dc.kind_uniform_from, (int32_t)n_conf, p->dc.tau_linear, (int32_t)want_tree};
+                            p->dc.kind_uniform, p->dc.kind_uniform_from, (int32_t)n_conf, p->dc.tau_linear, (int32_t)want_tree, sm_count(p->device)};
     key_put(k, head);
     key_put(k, rep.nmap);
     for (int h = 0; h < p->T; ++h) { key_put(k, p->P[h]); key_put(k, p->cap_eff[h]); key_put(k, p->dc.m[h]); key_put(k, p->dc.node_size[h]); }
@@ -748,13 +756,13 @@ static std::shared_ptr<const TreeClassHost> tree_of_class(const hap_problem *p, 
     TreeInputs in{};
     in.dc = &p->dc; in.rep = p->pconfs[p->items[cl.item_lo].p];
     in.n_conf = p->items[cl.item_hi - 1].p - p->items[cl.item_lo].p + 1;
+    in.n_sm = sm_count(p->device);
     in.want_tree = want_tree;
     TreeBuilder(in).build(*th);
     if (th->ok) {
         th->cls.n_conf = (u32)in.n_conf;
-        tree_items(th->cls);
         // (a record or a part that does not leave room for one block on an SM: the class runs one warp per candidate)
-        th->ok = tree_smem_bytes(th->cls) <= 200 * 1024 && tree_prep_smem_bytes(th->cls, p->model.N, p->T) <= 200 * 1024;
+        th->ok = tree_smem_bytes(th->cls) <= kTreeSmemMost && tree_prep_smem_bytes(th->cls, p->model.N, p->T) <= kTreeSmemMost;
     }
     std::lock_guard<std::mutex> lock(tc.mu);
     if (tc.map.size() >= kTreeCacheEntries) tc.map.clear();
@@ -853,6 +861,7 @@ static hap_status image_for(hap_problem *p, const std::string &ekey)
         im->cls.push_back(c);
         trees.push_back(th);
     }
+    tree_policy_items(im->cls, trees, sm_count(p->device), p->opts.n_rc);
     const size_t o_cls = o;
     o = up(o + trees.size() * sizeof(TreeClass));
     std::vector<size_t> o_parts;
@@ -1046,6 +1055,7 @@ extern "C" hap_status hap_enumerate(hap_problem *p, uint64_t *n_pconf, uint64_t 
         {
             auto up = [](size_t v) { return (v + 255) / 256 * 256; };
             size_t o = 0;
+            const bool refining = (p->opts.flags & (HAP_OPT_REFINE | HAP_OPT_EXACT)) != 0 && !im.cls.empty(), ordering = p->opts.prune || refining;
             const size_t o_coef = o; o = up(o + np * T * HAP_NCOEF * sizeof(i64));
             const size_t o_tc = o; o = up(o + np * T * sizeof(TypeConst));
             const size_t o_lb = o; o = up(o + np * sizeof(i64));
@@ -1059,7 +1069,6 @@ extern "C" hap_status hap_enumerate(hap_problem *p, uint64_t *n_pconf, uint64_t 
             const size_t o_report = o; o = up(o + sizeof(TreeReport));
             const size_t o_live = o; o = up(o + np * sizeof(u32));
             const size_t o_dead = o; o = up(o + np * sizeof(u32));
-            const bool refining = (p->opts.flags & (HAP_OPT_REFINE | HAP_OPT_EXACT)) != 0 && !im.cls.empty(), ordering = p->opts.prune || refining;
             const u64 n_surv = std::min<u64>(kMaxSurvivors, p->n_cand);
             const size_t o_hist = o; o = up(o + (ordering ? kOrderBuckets * sizeof(u64) : 0));
             const size_t o_key = o; o = up(o + (ordering ? np * sizeof(uint4) : 0));
@@ -1259,14 +1268,6 @@ static void configs_of_range(const hap_problem *p, u64 first, u64 count, unsigne
     lo = owner(first); hi = owner(first + count - 1) + 1;
 }
 
-static int sm_count(int device)
-{
-    static int n[64];                                       // (the same value whoever writes it)
-    int &v = n[device & 63];
-    if (!v && cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) { cudaGetLastError(); v = 148; }
-    return v;
-}
-
 // Per-type constants and stage coefficients of the configurations [p_lo, p_hi) in integer (coef) and / or fp64 form (coeff);
 // `live`: also the classes' lists of configurations (a pass over the trees)
 static hap_status launch_type_consts(hap_problem *p, i64 *coef, double *coeff, cudaStream_t st, unsigned p_lo, unsigned p_hi, const LiveArgs *live = nullptr)
@@ -1390,12 +1391,11 @@ static std::vector<TreeLaunch> tree_launches(const hap_problem *p, bool search, 
             const TreeClass &cl = cls[(size_t)c];
             const unsigned a = std::max(p_lo, cl.p_lo), b = std::min(p_hi, cl.p_lo + cl.n_conf);
             if (a >= b) continue;
-            const u64 cpi = prune ? 1 : cl.conf_per_item;
-            l.items += (b - a + cpi - 1) / cpi * cl.items_per_conf;
+            l.items += (u64)(b - a) * cl.items_per_conf * (prune ? 1 : cl.policy_items);
             l.smem = std::max(l.smem, tree_smem_bytes(cl));
         }
         if (!l.items) return;
-        const unsigned per_sm = (unsigned)std::max<size_t>(1, std::min<size_t>(kTreeBlocksPerSm, (227 * 1024) / (l.smem + 1024 + 256)));
+        const unsigned per_sm = (unsigned)std::max<size_t>(1, std::min<size_t>(kTreeBlocksPerSm, kSmemPerSm / (l.smem + kTreeSmemStatic)));
         l.grid = (unsigned)std::min<u64>(l.items, std::min<u64>((u64)sm_count(p->device) * per_sm, kTreeSlots / 2));
         ls.push_back(l);
     };
@@ -1440,13 +1440,15 @@ static hap_status launch_trees(hap_problem *p, const DpOut &out_in, bool search,
     const DeviceImage &im = *p->image;
     TreeArgs ta = p->targs;
     if (!ordered) ta.order = nullptr;
+    ta.by_policy = !prune;
     int is_search = search ? 1 : 0;
+    TreeInput in{p->d_tc, p->d_coef, p->d_coeff, c2v, {}};
+    for (int r = 0; r < p->prof.R; ++r) in.tau[r] = (double)(p->tau_q[r] >> 10);
     {
         const void *fn = f64 ? (nl ? (const void *)tree_prep_kernel<true, true> : (const void *)tree_prep_kernel<true, false>)
                              : (nl ? (const void *)tree_prep_kernel<false, true> : (const void *)tree_prep_kernel<false, false>);
         CUDA_TRY(p, raise_smem_limit(p->device, fn, im.prep_smem));
-        const double *coeff = p->d_coeff;
-        void *args[] = {(void *)&p->dc, (void *)&ta, (void *)&p->d_tc, (void *)&p->d_coef, (void *)&coeff, (void *)&c2v, (void *)&out, (void *)&is_search};
+        void *args[] = {(void *)&p->dc, (void *)&ta, (void *)&in, (void *)&out, (void *)&is_search};
         const unsigned per_sm = (unsigned)std::max<size_t>(1, std::min<size_t>(kTreePrepBlocksPerSm, (227 * 1024) / (im.prep_smem + 2048)));
         CUDA_TRY(p, launch_dependent(fn, std::min<unsigned>(p_hi - p_lo, (unsigned)sm_count(p->device) * per_sm), kTreePrepThreads, im.prep_smem, st, args));
     }

@@ -7,24 +7,29 @@
 // class alone and are laid out once on the host.
 //
 //   type_const_kernel  (hap_device.cuh) constants of Eq. 2 / Eq. 3, and which configurations can place a first stage.
-//   tree_prep_kernel   a block per such configuration: Eq. 2 for every (device type, layer), the prefix rows of the
+//   tree_prep_kernel   a block per such configuration at a time: Eq. 2 for every (device type, layer), the prefix rows of the
 //                      stage time per type mask and level, the memory thresholds and the stage constants, written
 //                      as one record for the DP kernel.  The other configurations' candidates are infeasible: a
 //                      warp each writes their results.
-//   tree_dp_kernel     persistent blocks of four warps that take (configuration, group of tree parts) items from
-//                      a counter.  A warp owns a part of the tree -- some tens of mappings -- and walks it depth
-//                      by depth on its own: no block barrier inside an item.  A task is four consecutive end
-//                      layers of a node; a lane keeps their running minima and slides one window of the parent's
-//                      row over the stage lengths (tree_scan).  Then one lane per mapping evaluates the last stage,
-//                      walks the choices back and assembles Eq. 4.  A search leaves the plan of the best candidate;
-//                      the last block to finish reduces the blocks' minima and decodes the winner.
+//   tree_dp_kernel     persistent blocks of four warps that take (configuration, up to four of its tree's parts) items
+//                      from a counter; in a pass an item of a class with long chains is one policy's.  A warp owns a
+//                      part of the tree -- a few to some tens of mappings -- and walks it depth by depth on its own:
+//                      no block barrier inside an item.  A task is four consecutive end layers of a node; a lane keeps
+//                      their running minima and slides one window of the parent's row over the stage lengths
+//                      (tree_scan).  Then one lane per mapping evaluates the last stage, walks the choices back and
+//                      assembles Eq. 4.  A search leaves the plan of the best candidate; the last block to finish
+//                      reduces the blocks' minima and decodes the winner.
 //
-// Bounds and figures (B200; 1,024 devices, 128 layers, 2.4 million candidates; a pass of 438 us before this form, 400 us
-// with it; 256 devices with partitions, 549 us after 990 us).  The recurrence is bound by instruction issue (57 % of the
-// slots, 20 lanes of 32 active); its row entries never leave shared memory.  A deeper split into blocks that share a tree
-// needs a barrier per depth (31 of them at 32 stages); a warp of its own per part needs none.  Two end layers per
-// task and eight blocks an SM: 475 us; one: 536 us; eight parts an item instead of four: 405 us; the registers of five
-// blocks of four warps (96) spill nothing, those of eight do.
+// Bounds and figures (B200).  1,024 devices, 96 layers, 2.4 million candidates: a pass takes 389 us (435 with a block per
+// configuration and a barrier per depth); the same devices where no stage size is homogeneous, 374 thousand candidates in
+// classes of 24 mappings: 244 us (274 in that form, 371 while one to three of a block's warps had a part); 256 devices
+// with partitions 474 us (985).  The recurrence is bound by instruction issue and by the chain of a part: a warp issues an
+// instruction every six to seven cycles, 15 to 20 of 32 lanes active; its row entries never leave shared memory.  A deeper
+// split into blocks that share a tree needs a barrier per depth (31 of them at 32 stages); a warp of its own per part needs
+// none.  Measured earlier in this form: two end layers per task and eight blocks an SM 475 us, one end layer 536, eight parts an
+// item instead of four 405.  Four blocks an SM, without the few spilled registers that five (96 a thread) cost, were no faster.
+// Records computed by the items themselves instead of tree_prep_kernel: 270 us instead of 284 in classes of few mappings,
+// but 513 instead of 475 at 256 devices, because the recurrence then has fewer registers; not kept.
 //
 // Integer mode holds times (integer ns below 2^52) as doubles: every sum, difference and comparison is exact.
 #pragma once
@@ -34,7 +39,7 @@ namespace hap {
 
 constexpr int kTreeWarps = 4;             // warps of a DP block
 constexpr int kTreeThreads = kTreeWarps * 32;
-constexpr int kTreeBlocksPerSm = 5;       // (100 registers a thread)
+constexpr int kTreeBlocksPerSm = 5;       // (96 registers a thread)
 constexpr int kTreeJ = 4;                 // end layers of a task
 constexpr int kTreePad = kTreeJ - 1;      // infinite entries in front of every row and behind the last one
 constexpr int kTreeKtab = 16 + HAP_MAX_TYPES * 6;    // stage constants: [0,16) pre-work by row group, then p2p [type][6]
@@ -67,11 +72,11 @@ struct TreeClass {
     u64 rec_off;                            // byte offset of the class's records
     u32 p_lo, n_conf;                       // its configurations are contiguous
     u32 rec_bytes;                          // one configuration's record
-    u32 o_minfo, o_rows, o_thr, o_thr_nf;   // offsets in a record
+    u32 o_rows, o_thr_nf;                   // offsets in a record
     u32 buf_cells[2], ch_bytes;             // a warp's row buffers (even / odd depths, in values) and choices
     int PP, n_parts, n_mrows;
-    int items_per_conf;                     // an item is a group of the configuration's parts ...
-    int conf_per_item;                      // ... or one part each of several configurations (classes of one part)
+    int items_per_conf;                     // an item is a group of the configuration's parts (at most a part a warp) ...
+    int policy_items;                       // ... under all policies (1) or, in passes, under one (then: the number of policies)
     uint8_t mrow_of[16], mask_of_row[16];   // type mask <-> row group
     uint8_t first_min[HAP_MAX_TYPES];       // per capacity type: shortest first stage (255: no first stage on it)
     uint8_t wmax[HAP_MAX_PP + 1];           // longest stage of depth d
@@ -95,7 +100,8 @@ struct __align__(16) TreeHead {
 };
 static_assert(sizeof(TreeHead) == 64, "the stage constants start behind it");
 constexpr u32 kTreeOffKtab = sizeof(TreeHead);
-constexpr u32 kTreeOffMinfo = kTreeOffKtab + kTreeKtab * 8;
+constexpr u32 kTreeOffThr = kTreeOffKtab + kTreeKtab * 8;                  // [depth - 1][HAP_MAX_TYPES] words
+constexpr u32 kTreeOffMinfo = kTreeOffThr + HAP_MAX_PP * HAP_MAX_TYPES * 4;
 
 // What a search brings back, written by the last block (device memory and, if mapped, the host's copy).
 struct TreeResult {
@@ -168,6 +174,7 @@ struct TreeArgs {
     u32 nmap[HAP_MAX_PP + 1];               // mappings of its configurations
     const u32 *live_list, *dead_list;
     int c_lo, c_hi;                         // classes of this launch
+    int by_policy;                          // classes may have items of one policy (not where candidates are counted as pruned)
     int launch;                             // which ticket counter; blocks that must be done before the last one reduces
     u32 blocks_total;
     u32 slot_lo;                            // first per-block slot of this launch
@@ -259,14 +266,245 @@ __device__ __forceinline__ void tree_fill_dead(const DpOut &out, u64 c0, u64 c1,
     if (out.recompute) for (u64 q = lane; q < 2 * n; q += 32) reinterpret_cast<uint4 *>(out.recompute + o * HAP_MAX_PP)[q] = z;
 }
 
+// What a record is computed from: constants of Eq. 2 and stage coefficients per (configuration, type), or the layer costs
+// themselves where a launch before left them (c2v).
+struct TreeInput {
+    const TypeConst *tcg;
+    const i64 *coef;
+    const double *coeff;
+    const void *c2v;
+    double tau[HAP_MAX_RC];                 // whole repeated forward passes per level (rows that are combined by level)
+};
+constexpr int kTreePrepThreads = 128;
+static_assert(kTreePrepThreads == kTreeThreads, "a block of either kernel computes a record");
+
+// One configuration's record in shared memory, by a whole block of kTreePrepThreads threads; `scratch`: shared memory behind it.
+// lb_sum (searches that prune; shared memory): the summed layer times at the cheapest type, 0 on entry.
+// A chain of dependent steps bounds it, so what needs no layer costs (thresholds, stage constants) stands in front of the first
+// barrier beside Eq. 2, and the blocks of 32 layers of a row are scanned side by side.
+template <bool F64, bool NL>
+__device__ __forceinline__ void tree_record(const DevConst &dc, const TreeClass &cl, u32 p, const hap_pconf &pc, const TreeInput &in,
+                                            u64 *range_flag, unsigned char *rec, unsigned char *scratch, i64 *lb_sum)
+{
+    constexpr int nthreads = kTreePrepThreads, nwarps = kTreePrepThreads / 32;
+    const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
+    const int N = dc.N, T = dc.T, R = dc.R, n1 = N + 1, PP = pc.PP;
+    unsigned all_levels = 0;
+    for (int q = 0; q < dc.n_rc; ++q) all_levels |= dc.rc_masks[q];
+    const i64 *cfp = in.coef + (size_t)p * T * HAP_NCOEF;                                     // integer coefficients (bytes)
+    auto cv = [&](int h, int q) -> double {                                                  // time coefficients
+        const size_t at = ((size_t)p * T + h) * HAP_NCOEF + q;
+        return F64 ? in.coeff[at] : (double)in.coef[at];
+    };
+
+    double2 *sC = reinterpret_cast<double2 *>(scratch);                                       // [T][N] forward, backward
+    u32 *w4 = reinterpret_cast<u32 *>(rec + kTreeOffThr);
+    i64 *sW = reinterpret_cast<i64 *>(sC + (size_t)T * N);
+    i64 *sA = sW + n1;                                                                        // byte prefixes (mixed kinds only)
+    uint8_t *sK = reinterpret_cast<uint8_t *>(sA + n1);
+    const i64 mx = cfp[HAP_MX], mpre = cfp[HAP_MPRE], mpost = cfp[HAP_MPOST];
+
+    // ---- Eq. 2 for every (device type, layer), with the arithmetic of layer_cost_kernel -------------------------
+    if (in.c2v) {                                                                             // a preceding launch left them
+        for (int q = tid; q < T * N; q += nthreads) {
+            if (F64) sC[q] = reinterpret_cast<const double2 *>(in.c2v)[(size_t)p * T * N + q];
+            else { const longlong2 v = reinterpret_cast<const longlong2 *>(in.c2v)[(size_t)p * T * N + q]; sC[q] = make_double2((double)v.x, (double)v.y); }
+        }
+    } else {
+        const size_t row = ((size_t)pc.itp * dc.ncp + pc.icp) * dc.nmb + pc.ib;              // the same table row for every type
+        const size_t stride_h = (size_t)dc.ntp * dc.ncp * dc.nmb * N * 2;                     // 16-byte pairs between device types
+        const double2 *tab = reinterpret_cast<const double2 *>(dc.tab4) + row * N * 2;
+        const TypeConst *tcp = in.tcg + (size_t)p * T;
+        bool bad = false;
+        int h = tid / N, l = tid - h * N;
+        for (int q = tid; q < T * N; q += nthreads) {
+            const bool dense = layer_kind(dc, l) == HAP_DENSE;
+            const double2 *tp = tab + (size_t)h * stride_h + (size_t)l * 2;
+            const double2 tb = __ldg(tp);
+            const double2 tf = dense ? make_double2(0.0, 0.0) : __ldg(tp + 1);
+            double cf, cb;
+            layer_cost_pair(reinterpret_cast<const double2 *>(tcp + h), tb, tf, dense, dc.kappa, cf, cb);
+            bad |= !(cf < 6.8719e10) | !(cb < 6.8719e10);                                     // 2^36 ns per layer
+            sC[q] = F64 ? make_double2(cf, cb) : make_double2(rint(cf), rint(cb));
+            for (l += nthreads; l >= N && h < T; l -= N) ++h;
+        }
+        if (bad) atomicOr(range_flag, 1ull);
+    }
+    if (!cl.all_flat) {
+        for (int l = tid; l <= N; l += nthreads) sK[l] = (uint8_t)moe_before(dc, l);
+        for (int l = tid; l <= N; l += nthreads) {                                            // byte prefixes from the counts of layers per kind
+            const i64 nm = moe_before(dc, l), nd = (i64)l - nm;
+            sW[l] = nd * cfp[HAP_MW] + nm * cfp[HAP_MW + 1];
+            sA[l] = nd * cfp[HAP_MA] + nm * cfp[HAP_MA + 1];
+        }
+    }
+    // ---- stage constants ---------------------------------------------------------------------------------------------
+    {
+        double *ktab = reinterpret_cast<double *>(rec + kTreeOffKtab), *mi = reinterpret_cast<double *>(rec + kTreeOffMinfo);
+        for (int q = tid; q < cl.n_mrows * kTreeMinfo; q += nthreads) {
+            const int mr = q / kTreeMinfo, e = q % kTreeMinfo, mk = cl.mask_of_row[mr];
+            // the slowest member of a stage of several types (column 7: pre-work, a stage constant)
+            const int col = e == 0 ? HAP_SLAT : e <= 2 ? HAP_SBW + e - 1 : e <= 4 ? HAP_OPT + e - 3 : e == 5 ? HAP_KXD : e == 6 ? HAP_KPOST : HAP_KPRE;
+            double v = 0.0;
+#pragma unroll
+            for (int h = 0; h < HAP_MAX_TYPES; ++h)
+                if (mk >> h & 1) { const double x = cv(h, col); v = x > v ? x : v; }
+            if (e == 5 && !(dc.het_dispatch && (mk & (mk - 1)) != 0)) v = 0.0;
+            if (e == 7) ktab[mr] = v;
+            else mi[q] = v;
+        }
+        for (int q = tid; q < T * 6; q += nthreads) ktab[16 + q] = cv(q / 6, HAP_KP2P_INTRA + q % 6);   // intra, inter, cross[0..3]
+    }
+    // ---- memory thresholds of the depths whose spans are of one kind: the longest length that fits, a byte per level in one word
+    // per (depth, type) -------------------------------------------------------------------------------------------------
+    {
+        const int last = layer_kind(dc, N - 1), len_cap = N - dc.kind_uniform_from;
+        const i64 mwk = cfp[HAP_MW + last], mak = cfp[HAP_MA + last], mxk = last == HAP_MOE ? mx : 0;
+        for (int q = tid; q < PP * HAP_MAX_TYPES; q += nthreads) {
+            const int t = q % HAP_MAX_TYPES, d = q / HAP_MAX_TYPES + 1;
+            u32 word = 0;
+            if (cl.flat[d] && ((cl.tmask[d] >> t) & 1u)) {
+                const i64 room = dc.cap_eff[t] - ((d == 1 ? mpre : 0) + (d == PP ? mpost : 0) + mxk);
+                const int inflight = PP - d + 1, most = cl.wmax[d] < len_cap ? cl.wmax[d] : len_cap;
+                const i64 ma = (i64)(pc.M < inflight ? pc.M : inflight) * mak;
+                const float room_f = (float)room, mw_f = (float)mwk, ma_f = (float)ma * 9.765625e-4f;
+                for (int r = 0; r < R; ++r) {
+                    if (!((all_levels >> r) & 1u)) continue;
+                    // longest length n with n mwk + floor(xi n ma / 1024) <= room: the quotient, then exact steps from there
+                    const i64 xm = (i64)dc.xi_q[r] * ma;
+                    auto fits = [&](int n) { return (i64)n * mwk + (((i64)n * xm) >> 10) <= room; };
+                    const float guess = room_f / (mw_f + (float)dc.xi_q[r] * ma_f);
+                    int lo = guess < 0.0f ? 0 : guess > (float)most ? most : (int)guess;             // (a zero divisor: most, or NaN: 0)
+                    while (lo < most && fits(lo + 1)) ++lo;
+                    while (lo > 0 && !fits(lo)) --lo;
+                    word |= (u32)lo << (8 * r);
+                }
+            }
+            w4[q] = word;
+        }
+    }
+    __syncthreads();
+    // ---- policies that cannot be feasible: the longest stages that fit do not add up to N (every warp, for itself) ----
+    u32 dead = 0;
+    {
+        u32 longest = 0;                                                                      // of this lane's depth, a byte per level
+        if (lane < PP) {
+            const uint4 w = reinterpret_cast<const uint4 *>(w4)[lane];                         // (0 where the depth has no such type)
+            longest = cl.flat[lane + 1] ? __vmaxu4(__vmaxu4(w.x, w.y), __vmaxu4(w.z, w.w)) : 0x01010101u * cl.wmax[lane + 1];
+        }
+        for (int pos = 0; pos < dc.n_rc; ++pos) {
+            const u32 levels = dc.rc_masks[dc.rc_order[pos]] * 0x00204081u & 0x01010101u;     // a bit per byte
+            u32 v = longest & levels * 255u;
+            v = __vmaxu4(v, v >> 16);
+            const int most = (int)(max(v & 255u, v >> 8 & 255u));
+            const int none = __any_sync(0xffffffffu, lane < PP && most == 0);
+            if (none || __reduce_add_sync(0xffffffffu, most) < N) dead |= 1u << pos;
+        }
+    }
+    const bool any = dead != (1u << dc.n_rc) - 1u;                                            // else nothing reads the rows
+    // ---- prefix rows of the stage time: per row group the slowest member type of every layer, one warp per group ---
+    if (any) {
+        double *rows = reinterpret_cast<double *>(rec + cl.o_rows);
+        // a lane sums two consecutive layers itself, so that 64 layers take one scan (four spill registers)
+        constexpr int kRun = 2;
+        const int RW = NL ? 2 : R;
+        for (int mr = wib; mr < cl.n_mrows; mr += nwarps) {
+            const u32 mk = cl.mask_of_row[mr];
+            double *row = rows + (size_t)(mr * RW) * n1;
+            double preC = 0.0, preF = 0.0;                                                    // fwd + bwd, fwd of the layers before
+            for (int base = 0; base < N; base += 32 * kRun) {
+                const int run = N - base < 32 * kRun ? (N - base + 31) / 32 : kRun, l0 = base + lane * run;
+                double vC[kRun], vF[kRun], sumC = 0.0, sumF = 0.0;
+#pragma unroll
+                for (int i = 0; i < kRun; ++i)
+                    if (i < run) {
+                        double F = 0.0, B = 0.0;
+                        if (l0 + i < N) {
+                            const double2 *c = sC + l0 + i;
+                            for (u32 m = mk; m; m &= m - 1) { const double2 q = c[(__ffs((int)m) - 1) * N]; F = q.x > F ? q.x : F; B = q.y > B ? q.y : B; }
+                        }
+                        sumC += F + B; sumF += F;
+                        vC[i] = sumC; vF[i] = sumF;
+                    }
+                double upC = sumC, upF = sumF;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const double tC = __shfl_up_sync(0xffffffffu, upC, o), tF = __shfl_up_sync(0xffffffffu, upF, o);
+                    if (lane >= o) { upC += tC; upF += tF; }
+                }
+                const double tC = __shfl_up_sync(0xffffffffu, upC, 1), tF = __shfl_up_sync(0xffffffffu, upF, 1);
+                const double befC = lane ? preC + tC : preC, befF = lane ? preF + tF : preF;
+                double *dst = row + 1 + l0;
+#pragma unroll
+                for (int i = 0; i < kRun; ++i)
+                    if (i < run && l0 + i < N) {
+                        const double c = befC + vC[i], f = befF + vF[i];
+                        if (NL) { dst[i] = c; dst[n1 + i] = f; }
+                        else {
+#pragma unroll
+                            for (int r = 0; r < HAP_MAX_RC; ++r) if (r < R) dst[r * n1 + i] = c + in.tau[r] * f;
+                        }
+                    }
+                preC += __shfl_sync(0xffffffffu, upC, 31); preF += __shfl_sync(0xffffffffu, upF, 31);
+            }
+            if (lane < RW) row[lane * n1] = 0.0;
+        }
+    }
+    // ---- lower bound on the summed stage time: the cheapest type's time of every layer (pruning searches) ----------
+    if (lb_sum && !F64) {
+        i64 lmin = 0;
+        for (int l = tid; l < N; l += nthreads) {
+            double m = 0.0;
+            for (int h = 0; h < T; ++h) { const double2 q = sC[(size_t)h * N + l]; const double v = q.x + q.y; m = (h == 0 || v < m) ? v : m; }
+            lmin += (i64)m;
+        }
+        lmin = warp_sum_i64(lmin);
+        if (lane == 0 && lmin) atomicAdd(reinterpret_cast<unsigned long long *>(lb_sum), (unsigned long long)lmin);
+    }
+    // ---- the other depths' thresholds: per (type, level, end layer) the longest span ending there that fits; feasibility is
+    // monotone in the span, so a thread sweeps a segment of end layers with a split pointer that only moves forward
+    if (any && !cl.all_flat) {
+        uint8_t *nf = rec + cl.o_thr_nf;
+        constexpr int kSeg = 4;
+        for (int d = 1; d <= PP; ++d) {
+            if (cl.flat[d]) continue;
+            const int w = (int)cl.nf_w[d], nseg = (w + kSeg - 1) / kSeg;
+            for (int e = tid; e < T * R * nseg; e += nthreads) {
+                const int seg = e % nseg, q = e / nseg, r = q % R, t = q / R;
+                uint8_t *row = nf + cl.nf_off[d] + (size_t)q * w - cl.jlo[d];
+                const int j0 = cl.jlo[d] + seg * kSeg;
+                int j1 = j0 + kSeg - 1; if (j1 > cl.jhi[d]) j1 = cl.jhi[d];
+                const bool want = ((all_levels >> r) & 1u) && ((cl.tmask[d] >> t) & 1u);
+                const i64 extra = (d == 1 ? mpre : 0) + (d == PP ? mpost : 0);
+                const int inflight = PP - d + 1;
+                const i64 mstore = pc.M < inflight ? pc.M : inflight, cap = dc.cap_eff[t], xi = dc.xi_q[r];
+                int k = cl.kmin[d];
+                for (int j = j0; j <= j1; ++j) {
+                    if (!want) { row[j] = 0; continue; }
+                    if (k < j - (int)cl.wmax[d]) k = j - (int)cl.wmax[d];
+                    const int kcap = (int)cl.kmax[d] < j - 1 ? (int)cl.kmax[d] : j - 1;      // no cell looks at a split beyond this
+                    while (k <= kcap && !span_fits(sW, sA, sK, extra, mx, mstore, cap, xi, k, j)) ++k;
+                    row[j] = (uint8_t)(k <= kcap ? j - k : 0);
+                }
+            }
+        }
+    }
+    if (lb_sum) __syncthreads();
+    if (tid == 0) {
+        TreeHead h{};
+        h.offset = pc.offset; h.m1 = (i64)pc.M - 1; h.p = p; h.dead_policies = dead;
+        h.S = lb_sum ? *lb_sum : 0;
+        h.lb = h.S + h.m1 * ((h.S + PP - 1) / PP);
+        *reinterpret_cast<TreeHead *>(rec) = h;
+    }
+}
+
 // Persistent blocks over the configurations on the classes' lists: entry i of a class's list becomes its record i.  What
 // bounds a configuration is a chain of dependent steps (constants, layer costs, scans), hidden by the resident blocks.
-constexpr int kTreePrepThreads = 128;
 constexpr int kTreePrepBlocksPerSm = 9;
 template <bool F64, bool NL>
 __global__ void __launch_bounds__(kTreePrepThreads, kTreePrepBlocksPerSm)
-tree_prep_kernel(const DevConst dc, const TreeArgs ta, const TypeConst *__restrict__ tcg, const i64 *__restrict__ coef,
-                 const double *__restrict__ coeff, const void *__restrict__ c2v, DpOut out, int search)
+tree_prep_kernel(const __grid_constant__ DevConst dc, const __grid_constant__ TreeArgs ta, const __grid_constant__ TreeInput in, DpOut out, int search)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ TreeClass cl;
@@ -286,9 +524,6 @@ tree_prep_kernel(const DevConst dc, const TreeArgs ta, const TypeConst *__restri
     }
     if (tid == 0) s_lb = 0;
     __syncthreads();
-    unsigned all_levels = 0;
-    for (int q = 0; q < dc.n_rc; ++q) all_levels |= dc.rc_masks[q];
-    const int N = dc.N, T = dc.T, R = dc.R, n1 = N + 1;
     const u32 n_live = s_first[ta.n_cls];
     int loaded = -1;
   for (u32 item = blockIdx.x; item < n_live; item += gridDim.x) {
@@ -305,216 +540,28 @@ tree_prep_kernel(const DevConst dc, const TreeArgs ta, const TypeConst *__restri
         __syncthreads();
     }
     const hap_pconf pc = dc.pconf[p];
-    const int PP = pc.PP;
-    const i64 *cfp = coef + (size_t)p * T * HAP_NCOEF;                                        // integer coefficients (bytes)
-    auto cv = [&](int h, int q) -> double {                                                  // time coefficients
-        const size_t at = ((size_t)p * T + h) * HAP_NCOEF + q;
-        return F64 ? coeff[at] : (double)coef[at];
-    };
-
-    double2 *sC = reinterpret_cast<double2 *>(smem_raw);                                      // [T][N] forward, backward
-    uint8_t *sThr = reinterpret_cast<uint8_t *>(sC + (size_t)T * N);                          // flat words, then the other depths' bytes
-    const u32 thr_bytes = cl.rec_bytes - cl.o_thr;
-    i64 *sW = reinterpret_cast<i64 *>(sThr + (thr_bytes + 15) / 16 * 16);                     // byte prefixes (mixed kinds only)
-    i64 *sA = sW + n1;
-    uint8_t *sK = reinterpret_cast<uint8_t *>(sA + n1);
-
-    // ---- Eq. 2 for every (device type, layer), with the arithmetic of layer_cost_kernel -------------------------
-    if (c2v) {                                                                                // a preceding launch left them
-        for (int q = tid; q < T * N; q += nthreads) {
-            if (F64) sC[q] = reinterpret_cast<const double2 *>(c2v)[(size_t)p * T * N + q];
-            else { const longlong2 v = reinterpret_cast<const longlong2 *>(c2v)[(size_t)p * T * N + q]; sC[q] = make_double2((double)v.x, (double)v.y); }
-        }
-    } else {
-        const size_t row = ((size_t)pc.itp * dc.ncp + pc.icp) * dc.nmb + pc.ib;              // the same table row for every type
-        const size_t stride_h = (size_t)dc.ntp * dc.ncp * dc.nmb * N * 2;                     // 16-byte pairs between device types
-        const double2 *tab = reinterpret_cast<const double2 *>(dc.tab4) + row * N * 2;
-        const TypeConst *tcp = tcg + (size_t)p * T;
-        bool bad = false;
-        for (int q = tid; q < T * N; q += nthreads) {
-            const int h = q / N, l = q - h * N;
-            const bool dense = layer_kind(dc, l) == HAP_DENSE;
-            const double2 *tp = tab + (size_t)h * stride_h + (size_t)l * 2;
-            const double2 tb = __ldg(tp);
-            const double2 tf = dense ? make_double2(0.0, 0.0) : __ldg(tp + 1);
-            double cf, cb;
-            layer_cost_pair(reinterpret_cast<const double2 *>(tcp + h), tb, tf, dense, dc.kappa, cf, cb);
-            bad |= !(cf < 6.8719e10) | !(cb < 6.8719e10);                                     // 2^36 ns per layer
-            sC[q] = F64 ? make_double2(cf, cb) : make_double2((double)__double2ll_rn(cf), (double)__double2ll_rn(cb));
-        }
-        if (bad) atomicOr(out.range_flag, 1ull);
-    }
-    if (!cl.all_flat) {
-        for (int l = tid; l <= N; l += nthreads) sK[l] = (uint8_t)moe_before(dc, l);
-        for (int l = tid; l <= N; l += nthreads) {                                            // byte prefixes from the counts of layers per kind
-            const i64 nm = moe_before(dc, l), nd = (i64)l - nm;
-            sW[l] = nd * cfp[HAP_MW] + nm * cfp[HAP_MW + 1];
-            sA[l] = nd * cfp[HAP_MA] + nm * cfp[HAP_MA + 1];
+    tree_record<F64, NL>(dc, cl, p, pc, in, out.range_flag, smem_raw, smem_raw + cl.rec_bytes, search ? &s_lb : nullptr);
+    if (tid == 0) {
+        const i64 sum = s_lb;
+        if (search && out.prune) {
+            // candidates are counted as pruned until a part is evaluated
+            const u64 c1 = pc.offset + pc.nmap * (u64)dc.n_rc, a = pc.offset > out.first ? pc.offset : out.first;
+            const u64 b = c1 < out.first + out.count ? c1 : out.first + out.count;
+            if (a < b) atomicAdd(&ta.state->n_pruned, b - a);
+            if (ta.order) {
+                const int bk = order_bucket(sum + (i64)(pc.M - 1) * ((sum + pc.PP - 1) / pc.PP));
+                const u64 before = atomicAdd(ta.hist + bk, (u64)cl.items_per_conf << 32 | 1ull);
+                __stcg(ta.order_key + item, make_uint4((u32)ci | (u32)bk << 8, s_slot, (u32)before, (u32)(before >> 32)));
+            }
         }
     }
     __syncthreads();
-    unsigned char *rec = ta.rec + cl.rec_off + (u64)s_slot * cl.rec_bytes;
-
-    // ---- prefix rows of the stage time: per row group the slowest member type of every layer, one warp per group ---
-    double *rows = reinterpret_cast<double *>(rec + cl.o_rows);
-    for (int mr = wib; mr < cl.n_mrows; mr += nwarps) {
-        const int mk = cl.mask_of_row[mr];
-        double runC = 0.0, runF = 0.0;
-        for (int base = 0; base < N; base += 32) {
-            const int l = base + lane;
-            double vC = 0.0, vF = 0.0;                                                        // fwd + bwd, fwd
-            if (l < N) {
-                double F = 0.0, B = 0.0;
-                for (int h = 0; h < T; ++h)
-                    if (mk >> h & 1) { const double2 q = sC[(size_t)h * N + l]; F = q.x > F ? q.x : F; B = q.y > B ? q.y : B; }
-                vC = F + B; vF = F;
-            }
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const double tC = __shfl_up_sync(0xffffffffu, vC, o), tF = __shfl_up_sync(0xffffffffu, vF, o);
-                if (lane >= o) { vC += tC; vF += tF; }
-            }
-            vC += runC; vF += runF;
-            if (l < N) {
-                if (NL) { rows[(size_t)(mr * 2) * n1 + l + 1] = vC; rows[(size_t)(mr * 2 + 1) * n1 + l + 1] = vF; }
-                else for (int r = 0; r < R; ++r) rows[(size_t)(mr * R + r) * n1 + l + 1] = vC + (double)(dc.tau_q[r] >> 10) * vF;
-            }
-            runC = __shfl_sync(0xffffffffu, vC, 31); runF = __shfl_sync(0xffffffffu, vF, 31);
-        }
-        const int RW = NL ? 2 : R;
-        if (lane < RW) rows[(size_t)(mr * RW + lane) * n1] = 0.0;
-    }
-    // ---- lower bound on the summed stage time: the cheapest type's time of every layer (pruning searches) ----------
-    if (search && !F64) {
-        i64 lmin = 0;
-        for (int l = tid; l < N; l += nthreads) {
-            double m = 0.0;
-            for (int h = 0; h < T; ++h) { const double2 q = sC[(size_t)h * N + l]; const double v = q.x + q.y; m = (h == 0 || v < m) ? v : m; }
-            lmin += (i64)m;
-        }
-        lmin = warp_sum_i64(lmin);
-        if (lane == 0 && lmin) atomicAdd(reinterpret_cast<unsigned long long *>(&s_lb), (unsigned long long)lmin);
-    }
-    // ---- memory thresholds -------------------------------------------------------------------------------------------
     {
-        const i64 mx = cfp[HAP_MX], mpre = cfp[HAP_MPRE], mpost = cfp[HAP_MPOST];
-        // Depths whose spans are of one kind: the longest length that fits, a byte per level in one word per (depth, type)
-        const i64 mwk = cfp[HAP_MW + layer_kind(dc, N - 1)], mak = cfp[HAP_MA + layer_kind(dc, N - 1)];
-        const i64 mxk = layer_kind(dc, N - 1) == HAP_MOE ? mx : 0;
-        const int len_cap = N - dc.kind_uniform_from;
-        u32 *w4 = reinterpret_cast<u32 *>(sThr);
-        for (int q = tid; q < PP * T; q += nthreads) {
-            const int t = q % T, d = q / T + 1;
-            u32 word = 0;
-            if (cl.flat[d] && ((cl.tmask[d] >> t) & 1u)) {
-                const i64 base = (d == 1 ? mpre : 0) + (d == PP ? mpost : 0) + mxk, cap = dc.cap_eff[t];
-                const int inflight = PP - d + 1;
-                const i64 ma = (i64)(pc.M < inflight ? pc.M : inflight) * mak;
-                for (int r = 0; r < R; ++r) {
-                    if (!((all_levels >> r) & 1u)) continue;
-                    const i64 xi = dc.xi_q[r];
-                    // longest length n with n mwk + base + floor(xi n ma / 1024) <= cap: the quotient, then exact steps from there
-                    const int most = cl.wmax[d] < len_cap ? cl.wmax[d] : len_cap;
-                    auto fits = [&](int n) { return (i64)n * mwk + base + ((xi * ((i64)n * ma)) >> 10) <= cap; };
-                    const float guess = (float)(cap - base) / ((float)mwk + (float)xi * (float)ma * 9.765625e-4f);
-                    int lo = guess < 0.0f ? 0 : guess > (float)most ? most : (int)guess;             // (a zero divisor: most, or NaN: 0)
-                    while (lo < most && fits(lo + 1)) ++lo;
-                    while (lo > 0 && !fits(lo)) --lo;
-                    word |= (u32)lo << (8 * r);
-                }
-            }
-            w4[q] = word;
-        }
-        if (!cl.all_flat) {
-            // other depths: per (type, level, end layer) the longest span ending there that fits; feasibility is monotone in
-            // the span, so a thread sweeps a segment of end layers with a split pointer that only moves forward
-            uint8_t *nf = sThr + (cl.o_thr_nf - cl.o_thr);
-            constexpr int kSeg = 8;
-            for (int d = 1; d <= PP; ++d) {
-                if (cl.flat[d]) continue;
-                const int w = (int)cl.nf_w[d], nseg = (w + kSeg - 1) / kSeg;
-                for (int e = tid; e < T * R * nseg; e += nthreads) {
-                    const int seg = e % nseg, q = e / nseg, r = q % R, t = q / R;
-                    uint8_t *row = nf + cl.nf_off[d] + (size_t)q * w - cl.jlo[d];
-                    const int j0 = cl.jlo[d] + seg * kSeg;
-                    int j1 = j0 + kSeg - 1; if (j1 > cl.jhi[d]) j1 = cl.jhi[d];
-                    const bool want = ((all_levels >> r) & 1u) && ((cl.tmask[d] >> t) & 1u);
-                    const i64 extra = (d == 1 ? mpre : 0) + (d == PP ? mpost : 0);
-                    const int inflight = PP - d + 1;
-                    const i64 mstore = pc.M < inflight ? pc.M : inflight, cap = dc.cap_eff[t], xi = dc.xi_q[r];
-                    int k = cl.kmin[d];
-                    for (int j = j0; j <= j1; ++j) {
-                        if (!want) { row[j] = 0; continue; }
-                        if (k < j - (int)cl.wmax[d]) k = j - (int)cl.wmax[d];
-                        const int kcap = (int)cl.kmax[d] < j - 1 ? (int)cl.kmax[d] : j - 1;      // no cell looks at a split beyond this
-                        while (k <= kcap && !span_fits(sW, sA, sK, extra, mx, mstore, cap, xi, k, j)) ++k;
-                        row[j] = (uint8_t)(k <= kcap ? j - k : 0);
-                    }
-                }
-            }
-        }
+        const uint4 *src = reinterpret_cast<const uint4 *>(smem_raw);
+        uint4 *dst = reinterpret_cast<uint4 *>(ta.rec + cl.rec_off + (u64)s_slot * cl.rec_bytes);
+        for (u32 q = (u32)tid; q < cl.rec_bytes / 16; q += nthreads) dst[q] = src[q];
     }
-    // ---- stage constants ---------------------------------------------------------------------------------------------
-    {
-        double *ktab = reinterpret_cast<double *>(rec + kTreeOffKtab), *mi = reinterpret_cast<double *>(rec + cl.o_minfo);
-        for (int q = tid; q < cl.n_mrows * kTreeMinfo; q += nthreads) {
-            const int mr = q / kTreeMinfo, e = q % kTreeMinfo, mk = cl.mask_of_row[mr];
-            // the slowest member of a stage of several types
-            const int col = e == 0 ? HAP_SLAT : e <= 2 ? HAP_SBW + e - 1 : e <= 4 ? HAP_OPT + e - 3 : e == 5 ? HAP_KXD : HAP_KPOST;
-            double v = 0.0, pre = 0.0;
-            for (int h = 0; h < T; ++h)
-                if (mk >> h & 1) { const double x = cv(h, col); v = x > v ? x : v; const double y = cv(h, HAP_KPRE); pre = y > pre ? y : pre; }
-            if (e == 5 && !(dc.het_dispatch && (mk & (mk - 1)) != 0)) v = 0.0;
-            mi[q] = v;
-            if (e == 7) ktab[mr] = pre;
-        }
-        for (int q = tid; q < T * 6; q += nthreads) ktab[16 + q] = cv(q / 6, HAP_KP2P_INTRA + q % 6);   // intra, inter, cross[0..3]
-    }
-    __syncthreads();
-    // ---- policies that cannot be feasible: the longest stages that fit do not add up to N ------------------------------
-    {
-        const uint4 *src = reinterpret_cast<const uint4 *>(sThr);
-        uint4 *dst = reinterpret_cast<uint4 *>(rec + cl.o_thr);
-        for (int q = tid; q < (int)(thr_bytes / 16); q += nthreads) dst[q] = src[q];
-    }
-    if (wib == 0) {
-        u32 dead = 0;
-        for (int pos = 0; pos < dc.n_rc; ++pos) {
-            const unsigned mask = dc.rc_masks[dc.rc_order[pos]];
-            int most = 0;
-            if (lane < PP) {
-                const int d = lane + 1;
-                if (!cl.flat[d]) most = cl.wmax[d];
-                else
-                    for (int t = 0; t < T; ++t) {
-                        const u32 w = reinterpret_cast<const u32 *>(sThr)[lane * T + t];
-                        for (int r = 0; r < R; ++r) if ((mask >> r) & 1u) { const int v = (int)((w >> (8 * r)) & 255u); most = v > most ? v : most; }
-                    }
-            }
-            const int none = __any_sync(0xffffffffu, lane < PP && most == 0);
-            most = __reduce_add_sync(0xffffffffu, most);
-            if (none || most < N) dead |= 1u << pos;
-        }
-        if (lane == 0) {
-            TreeHead h{};
-            h.offset = pc.offset; h.m1 = (i64)pc.M - 1; h.p = p; h.dead_policies = dead;
-            h.S = s_lb;
-            h.lb = s_lb + h.m1 * ((s_lb + PP - 1) / PP);
-            *reinterpret_cast<TreeHead *>(rec) = h;
-            s_lb = 0;
-            if (search && out.prune) {
-                // candidates are counted as pruned until a part is evaluated
-                const u64 c1 = pc.offset + pc.nmap * (u64)dc.n_rc, a = pc.offset > out.first ? pc.offset : out.first;
-                const u64 b = c1 < out.first + out.count ? c1 : out.first + out.count;
-                if (a < b) atomicAdd(&ta.state->n_pruned, b - a);
-                if (ta.order) {
-                    const int bk = order_bucket(h.lb);
-                    const u64 before = atomicAdd(ta.hist + bk, (u64)cl.items_per_conf << 32 | 1ull);
-                    __stcg(ta.order_key + item, make_uint4((u32)ci | (u32)bk << 8, s_slot, (u32)before, (u32)(before >> 32)));
-                }
-            }
-        }
-    }
+    if (tid == 0) s_lb = 0;                             // (added to behind the next record's first barrier)
     __syncthreads();                                    // the shared arrays are free for the next configuration
   }
     if (search) {
@@ -578,9 +625,16 @@ tree_prep_kernel(const DevConst dc, const TreeArgs ta, const TypeConst *__restri
 // stage that fits at all = nx.  A level that is not allowed or never the lowest that fits has the bound of the one before it.
 struct TreeLevels { int b0, b1, b2, nx; };
 
+template <int RK>
 __device__ __forceinline__ TreeLevels tree_levels(int R, unsigned rc_mask, u32 len4)
 {
     TreeLevels lv;
+    if (RK == 2) {                                  // two levels at most (a level that does not exist has length 0)
+        const int l0 = (int)(len4 & 255u), l1 = (int)(len4 >> 8 & 255u);
+        lv.b0 = rc_mask & 1u ? l0 : -1;
+        lv.b1 = lv.b2 = lv.nx = rc_mask & 2u && l1 > lv.b0 ? l1 : lv.b0;
+        return lv;
+    }
     int run = -1;                                   // (level 0 not allowed: every length is above it)
     auto step = [&](int r) { if ((rc_mask >> r) & 1u) { const int l = (int)((len4 >> (8 * r)) & 255u); run = l > run ? l : run; } return run; };
     lv.b0 = step(0);
@@ -759,9 +813,10 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
     __shared__ double s_zero[2 * kTreePad + 1];             // the row before the first stage: 0 at layer 0
     __shared__ i64 s_cost[kTreeWarps];
     __shared__ u64 s_index[kTreeWarps];
-    __shared__ int s_last;
+    __shared__ int s_last, s_pos[2];
     const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
-    const int N = ta.N, T = ta.T, R = ta.R, n1 = N + 1, n_rc = ta.n_rc, RW = NL ? 2 : R;
+    const int N = ta.N, R = ta.R, n1 = N + 1, n_rc = ta.n_rc, RW = NL ? 2 : R;
+    const int kind_last = layer_kind(dc, N - 1);
     const i64 inf_bits = F64 ? 0x7ff0000000000000ll : kInf;
     const double dInfOut = F64 ? __longlong_as_double(0x7ff0000000000000ll) : kTreeInf;
 
@@ -783,8 +838,8 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
         u32 t = 0;                          // items before class c (in order of the bounds: configurations)
         for (int c = ta.c_lo; c < ta.c_hi; ++c) {
             s_total[c - ta.c_lo] = t;
-            const u32 live = __ldcg(&ta.state->live[c]), cpi = (u32)ta.cls[c].conf_per_item;
-            t += ordered ? live : (live + cpi - 1) / cpi * (u32)ta.cls[c].items_per_conf;
+            const u32 live = __ldcg(&ta.state->live[c]);
+            t += ordered ? live : live * (u32)(ta.cls[c].items_per_conf * (ta.by_policy ? ta.cls[c].policy_items : 1));
         }
         s_total[ta.c_hi - ta.c_lo] = t;
         s_item = blockIdx.x;
@@ -823,42 +878,48 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
         if (ordered) ci = (int)(s_entry.y & 255u);
         else while (item >= s_total[ci + 1 - ta.c_lo]) ++ci;
         const TreeClass *cl = ta.cls + ci;
-        const u32 local = ordered ? item - s_entry.x : item - s_total[ci - ta.c_lo], ipc = (u32)cl->items_per_conf, cpi = ordered ? 1u : (u32)cl->conf_per_item;
-        const u32 live = __ldcg(&ta.state->live[ci]);
-        const u32 conf0 = ordered ? s_entry.z : local / ipc * cpi, sub = local % ipc;
-        const u32 n_confs = conf0 + cpi <= live ? cpi : live - conf0;
+        const u32 ipc = (u32)cl->items_per_conf;
+        u32 local = ordered ? item - s_entry.x : item - s_total[ci - ta.c_lo];
+        {
+            int lo = 0, hi = n_rc;
+            if (!ordered && ta.by_policy && cl->policy_items > 1) {
+                // items of one policy each: the first policy's come first (they take longest)
+                const u32 items = __ldcg(&ta.state->live[ci]) * ipc;
+                lo = (int)(local / items); hi = lo + 1; local -= (u32)lo * items;
+            }
+            if (tid == 0) { s_pos[0] = lo; s_pos[1] = hi; }     // (in shared memory: registers are short below)
+        }
+        const u32 conf = ordered ? s_entry.z : local / ipc, sub = local % ipc;
         const u32 n_parts = (u32)cl->n_parts, part0 = n_parts * sub / ipc, part1 = n_parts * (sub + 1) / ipc;
         const u32 rec_bytes = cl->rec_bytes;
         const int PP = cl->PP;
-        // records of the item's configurations into shared memory
+        // the configuration's record into shared memory
+        if (tid == 0) s_unit = 0;
         {
-            const unsigned char *src = ta.rec + cl->rec_off + (u64)conf0 * rec_bytes;
-            const u32 total = n_confs * rec_bytes, dst = smem_u32(smem_raw);
-            for (u32 q = (u32)tid * 16u; q < total; q += kTreeThreads * 16u)
+            const unsigned char *src = ta.rec + cl->rec_off + (u64)conf * rec_bytes;
+            const u32 dst = smem_u32(smem_raw);
+            for (u32 q = (u32)tid * 16u; q < rec_bytes; q += kTreeThreads * 16u)
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + q), "l"(src + q) : "memory");
-            if (tid == 0) s_unit = 0;
             asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
         }
         __syncthreads();
         const u32 slice_bytes = (cl->buf_cells[0] + cl->buf_cells[1]) * 8u + cl->ch_bytes;
-        const u32 a_slice = smem_u32(smem_raw) + cpi * rec_bytes + (u32)wib * slice_bytes;
+        const u32 a_slice = smem_u32(smem_raw) + rec_bytes + (u32)wib * slice_bytes;
         const u32 a_buf[2] = {a_slice, a_slice + cl->buf_cells[0] * 8u};
         const u32 a_ch = a_buf[1] + cl->buf_cells[1] * 8u;
-        const u32 o_thr = cl->o_thr, o_nf = cl->o_thr_nf, o_rows = cl->o_rows, o_minfo = cl->o_minfo;
         const bool all_flat = cl->all_flat != 0;
         const bool packed = ta.kind_uniform && cl->n_mrows <= 4;       // sync and optimizer terms from the longest stage per row group
-        const u32 units = n_confs * (part1 - part0), row_stride = (u32)n1 * 8u, row_group = (u32)RW * row_stride;
+        const u32 row_stride = (u32)n1 * 8u, row_group = (u32)RW * row_stride;
 
         while (true) {
             u32 u = 0;
             if (lane == 0) u = atomicAdd(&s_unit, 1u);
             u = __shfl_sync(0xffffffffu, u, 0);
-            if (u >= units) break;
-            const u32 conf = u / (part1 - part0);
-            const TreePart *pt = cl->parts + part0 + u % (part1 - part0);
-            const unsigned char *rec = smem_raw + conf * rec_bytes;
+            if (u >= part1 - part0) break;
+            const TreePart *pt = cl->parts + part0 + u;
+            const unsigned char *rec = smem_raw;
             const TreeHead *hd = reinterpret_cast<const TreeHead *>(rec);
-            const u32 a_rec = smem_u32(rec);
+            const u32 a_rec = smem_u32(rec), a_rows = a_rec + cl->o_rows;
             const u32 nmap = pt->nmap;
             const u64 c_lo = hd->offset + (u64)pt->m_lo * (u64)n_rc, c_hi = c_lo + (u64)nmap * (u64)n_rc;
             const u64 w_lo = out.first, w_hi = out.first + out.count;
@@ -876,16 +937,16 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
             unsigned without_plan = 0;          // positions in rc_order under which no mapping was feasible
             const TreeTask *tasks = pt->tasks;
 
-            for (int pos = 0; pos < n_rc; ++pos) {
+            for (int pos = s_pos[0]; pos < s_pos[1]; ++pos) {
                 const int rc_idx = ta.rc_order[pos];
                 const unsigned rc_mask = ta.rc_masks[rc_idx];
                 bool dead = ((hd->dead_policies >> pos) & 1u) || (ta.rc_sup[pos] & without_plan) != 0;
                 // levels at a depth whose spans mix layer kinds: per end layer
                 auto nf_levels = [&](int d, int capt, int j) {
-                    const u32 w = cl->nf_w[d], a = a_rec + o_nf + cl->nf_off[d] + (u32)(capt * R) * w + (u32)(j - (int)cl->jlo[d]);
+                    const u32 w = cl->nf_w[d], a = a_rec + cl->o_thr_nf + cl->nf_off[d] + (u32)(capt * R) * w + (u32)(j - (int)cl->jlo[d]);
                     u32 len4 = 0;
                     for (int r = 0; r < R; ++r) len4 |= (u32)lds_u8(a + (u32)r * w) << (8 * r);
-                    return tree_levels(R, rc_mask, len4);
+                    return tree_levels<NL ? 4 : RK>(R, rc_mask, len4);
                 };
 
                 // ---- rows of the tree, depth by depth ------------------------------------------------------
@@ -909,11 +970,11 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
                             const u32 kidx = t.z & 255u, mrow = (t.z >> 8) & 255u;
                             const int capt = (int)(t.z >> 16);
                             const double K = lds_f64(a_rec + kTreeOffKtab + 8u * kidx);
-                            const u32 a_row0 = a_rec + o_rows + mrow * row_group, slot = t.x >> 16;
+                            const u32 a_row0 = a_rows + mrow * row_group, slot = t.x >> 16;
                             const u32 a_prev = a_prv + 8u * (t.x & 0xffffu), a_out = a_cur + 8u * slot, a_cho = a_ch + cell0 + slot;
                             constexpr int J = NL && kTreeJ > 2 ? kTreeJ / 2 : kTreeJ;
                             if (flat) {
-                                const TreeLevels lv = tree_levels(R, rc_mask, lds_u32(a_rec + o_thr + 4u * (u32)((d - 1) * T + capt)));
+                                const TreeLevels lv = tree_levels<NL ? 4 : RK>(R, rc_mask, lds_u32(a_rec + kTreeOffThr + 4u * (u32)((d - 1) * HAP_MAX_TYPES + capt)));
 #pragma unroll
                                 for (int h = 0; h < kTreeJ; h += J) {
                                     if (h && h >= cnt) break;
@@ -974,12 +1035,12 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
                         const u32 kidx = (pw >> 20) & 63u, mrow = (pw >> 26) & 15u;
                         const int capt = (int)(pw >> 30);
                         if (a <= b) {
-                            const double K = lds_f64(a_rec + kTreeOffKtab + 8u * kidx) + lds_f64(a_rec + o_minfo + (mrow * kTreeMinfo + 6) * 8u);
-                            const TreeLevels lv = all_flat || cl->flat[PP] ? tree_levels(R, rc_mask, lds_u32(a_rec + o_thr + 4u * (u32)((PP - 1) * T + capt)))
+                            const double K = lds_f64(a_rec + kTreeOffKtab + 8u * kidx) + lds_f64(a_rec + kTreeOffMinfo + (mrow * kTreeMinfo + 6) * 8u);
+                            const TreeLevels lv = all_flat || cl->flat[PP] ? tree_levels<NL ? 4 : RK>(R, rc_mask, lds_u32(a_rec + kTreeOffThr + 4u * (u32)((PP - 1) * HAP_MAX_TYPES + capt)))
                                                                            : nf_levels(PP, capt, N);
                             double best[1];
                             int arg[1];
-                            tree_scan<1, RK, F64, NL, COUNT>(ta, a_last + 8u * (pw & 0xfffffu), a_rec + o_rows + mrow * row_group, row_stride, N, 1, a, b, lv, K,
+                            tree_scan<1, RK, F64, NL, COUNT>(ta, a_last + 8u * (pw & 0xfffffu), a_rows + mrow * row_group, row_stride, N, 1, a, b, lv, K,
                                                              best, arg, splits);
                             bott = best[0]; n = arg[0];
                         }
@@ -1006,13 +1067,13 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
                         const u32 mrow = (pw >> 26) & 15u;
                         if (!HAP_CHECK_OK(5, n >= 1 && n <= b && b <= N)) break;
                         double K = lds_f64(a_rec + kTreeOffKtab + 8u * (u32)kidx);
-                        const u32 a_mi = a_rec + o_minfo + mrow * (kTreeMinfo * 8u);
+                        const u32 a_mi = a_rec + kTreeOffMinfo + mrow * (kTreeMinfo * 8u);
                         if (d == PP) K += lds_f64(a_mi + 48u);
                         // lowest allowed level whose longest stage holds n layers
-                        const TreeLevels lv = all_flat || cl->flat[d] ? tree_levels(R, rc_mask, lds_u32(a_rec + o_thr + 4u * (u32)((d - 1) * T + capt)))
+                        const TreeLevels lv = all_flat || cl->flat[d] ? tree_levels<NL ? 4 : RK>(R, rc_mask, lds_u32(a_rec + kTreeOffThr + 4u * (u32)((d - 1) * HAP_MAX_TYPES + capt)))
                                                                       : nf_levels(d, capt, b);
                         const int r = RK == 2 && !NL ? (int)(n > lv.b0) : (n > lv.b0) + (n > lv.b1) + (n > lv.b2);
-                        const u32 a_row = a_rec + o_rows + mrow * row_group + (NL ? 0u : (u32)r * row_stride);
+                        const u32 a_row = a_rows + mrow * row_group + (NL ? 0u : (u32)r * row_stride);
                         double cst = lds_f64(a_row + 8u * (u32)b) - lds_f64(a_row + 8u * (u32)(b - n));
                         if (NL) {
                             const double t = (lds_f64(a_row + 8u * (u32)(n1 + b)) - lds_f64(a_row + 8u * (u32)(n1 + b - n))) * ta.tau[r];
@@ -1025,7 +1086,8 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
                             most = __vmaxu4(most, (u32)n << (8u * mrow));
                             n_moe = ta.kind0 == HAP_MOE ? n : 0;
                         } else {
-                            n_moe = moe_before(dc, b) - moe_before(dc, b - n);
+                            // (behind the last change of kind the count needs no look at the layers)
+                            n_moe = b - n >= dc.kind_uniform_from ? (kind_last == HAP_MOE ? n : 0) : moe_before(dc, b) - moe_before(dc, b - n);
                             const double dm = (double)n_moe, dd = (double)(n - n_moe);
                             const double sy = lds_f64(a_mi) + dd * lds_f64(a_mi + 8u) + dm * lds_f64(a_mi + 16u);
                             const double op = dd * lds_f64(a_mi + 24u) + dm * lds_f64(a_mi + 32u);
@@ -1059,7 +1121,7 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
                     if (packed)
                         for (int g = 0; g < cl->n_mrows; ++g) {                // the terms grow with the stage: the longest one of a row group counts
                             const u32 len = (most >> (8 * g)) & 255u;
-                            const u32 a_mi = a_rec + o_minfo + (u32)(g * kTreeMinfo) * 8u;
+                            const u32 a_mi = a_rec + kTreeOffMinfo + (u32)(g * kTreeMinfo) * 8u;
                             const double dn = (double)len;
                             const double sy = lds_f64(a_mi) + dn * lds_f64(a_mi + 8u + 8u * (u32)ta.kind0), op = dn * lds_f64(a_mi + 24u + 8u * (u32)ta.kind0);
                             if (len) { t_sync = sy > t_sync ? sy : t_sync; t_opt = op > t_opt ? op : t_opt; }
@@ -1121,7 +1183,7 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
                         at = (u64)shfl_i64((i64)at, 0) + (u64)__popc(kept & ((1u << lane) - 1u));
                         if (keep && at < ta.max_surv) {
                             Survivor sv;
-                            sv.c = c_lo + (u64)m * (u64)n_rc + (u64)rc_idx; sv.lb = lb; sv.bott = (i64)bott; sv.ci = (u32)ci; sv.slot = conf0 + conf;
+                            sv.c = c_lo + (u64)m * (u64)n_rc + (u64)rc_idx; sv.lb = lb; sv.bott = (i64)bott; sv.ci = (u32)ci; sv.slot = conf;
                             ta.surv[at] = sv;
                         }
                     }
@@ -1243,7 +1305,7 @@ tree_refine_kernel(const TreeArgs ta, const DevConst dc, int exact, int max_pp)
         const i64 M1 = hd->m1;
         const u64 loc = c - pc.offset, map_idx = loc / (u64)n_rc;
         const unsigned rc_mask = ta.rc_masks[loc - map_idx * (u64)n_rc];
-        const double *ktab = reinterpret_cast<const double *>(rec + kTreeOffKtab), *minfo = reinterpret_cast<const double *>(rec + cl->o_minfo);
+        const double *ktab = reinterpret_cast<const double *>(rec + kTreeOffKtab), *minfo = reinterpret_cast<const double *>(rec + kTreeOffMinfo);
         const double *row0 = reinterpret_cast<const double *>(rec + cl->o_rows);
 
         // ---- this lane's stage: row group, capacity type, constant, window, band (the formulas of pipeline_dp_kernel) -----
@@ -1288,10 +1350,10 @@ tree_refine_kernel(const TreeArgs ta, const DevConst dc, int exact, int max_pp)
         }
         auto levels = [&](int d, int ct, int j) {
             u32 len4 = 0;
-            if (cl->flat[d]) len4 = __ldg(reinterpret_cast<const u32 *>(rec + cl->o_thr) + (d - 1) * dc.T + ct);
+            if (cl->flat[d]) len4 = __ldg(reinterpret_cast<const u32 *>(rec + kTreeOffThr) + (d - 1) * HAP_MAX_TYPES + ct);
             else if (HAP_CHECK_OK(6, j >= (int)cl->jlo[d] && j <= (int)cl->jhi[d]))
                 for (int r = 0; r < R; ++r) len4 |= (u32)__ldg(rec + cl->o_thr_nf + cl->nf_off[d] + (u32)(ct * R + r) * cl->nf_w[d] + (u32)(j - (int)cl->jlo[d])) << (8 * r);
-            return tree_levels(R, rc_mask, len4);
+            return tree_levels<4>(R, rc_mask, len4);
         };
         auto span = [&](int mr, int r, int k, int j, double kk) {
             if (!HAP_CHECK_OK(5, k >= 0 && k <= j && j <= N && r < R)) return kk;

@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <memory>
 #include <vector>
 
 namespace hap {
@@ -20,6 +21,7 @@ struct TreeClassHost {
     bool ok = false;                        // false: the class runs one warp per candidate
     unsigned masks_used = 0xffffffffu;      // type masks that occur (the general kernel builds rows for those only)
     TreeClass cls{};
+    double work = 0, chain = 0;             // instructions of a configuration's parts, of its longest part (one policy)
     std::vector<TreePartHost> parts;
 };
 
@@ -27,11 +29,37 @@ struct TreeInputs {
     const DevConst *dc;                     // N, T, m, node_size, P, cap_eff, kind_uniform_from, delta_q, uniform, R, tau_linear
     hap_pconf rep;                          // any configuration of the class
     size_t n_conf;
+    int n_sm;
     bool want_tree;
 };
 
 constexpr u64 kTreeMaxMappings = 1u << 18;
-constexpr size_t kTreeSliceBytes = 9216;  // a warp's rows and choices: what lets five blocks of four warps share an SM
+constexpr size_t kSmemPerSm = 227 * 1024;
+constexpr size_t kTreeSmemMost = 200 * 1024;     // dynamic part of a block
+constexpr size_t kTreeSmemFixed = 64, kTreeSmemStatic = 1024 + 256;     // behind the slices; static variables and the system's part
+
+// shared memory that computing a record takes beside it: layer costs of every type, byte prefixes (mixed kinds)
+inline size_t tree_record_scratch(const TreeClass &cl, int N, int T) { return (size_t)T * N * 16 + (cl.all_flat ? 0 : ((size_t)(N + 1) * 17 + 15) / 16 * 16); }
+
+// Cycles a class takes, roughly, in a given number of parts: its instructions at the rate at which the busy warps of an SM issue
+// them, then the chain of one item.  Measured on B200: a warp of these kernels issues an instruction every six to seven cycles
+// (7.3 warps stand for every issue), an SM 2.3 a cycle when all its warps are busy (57 % of the slots); warps of a block without
+// a part still hold their registers.  About two fifths of a class's configurations are feasible (1,024 devices: 27 %, 256
+// devices: 41 %).  An item's record comes in between two barriers of its block, 1,500 cycles and one per 16 bytes.  At 1,024 devices
+// without a homogeneous class 4 parts of 6 mappings each, all warps busy: 243 us a pass; 2 and 3 parts, which share more
+// prefixes, 273 and 271.  Negative: no block fits.
+struct TreeWork { double total = 0, longest = 0, n_conf = 0; size_t slice = 0; u32 rec_bytes = 0; int n_parts = 0, n_sm = 0; };
+constexpr double kTreeIssue = 2.3, kTreeWarpIssue = 0.15, kTreeLive = 0.4;
+constexpr double kTreeIteration = 150.0, kTreePerLength = 42.0, kTreeLeaf = 150.0, kTreePerStage = 100.0;      // warp instructions
+inline double tree_time(const TreeWork &w)
+{
+    const size_t smem = w.rec_bytes + kTreeWarps * w.slice + kTreeSmemFixed;
+    const int per_sm = (int)std::min<size_t>(kTreeBlocksPerSm, kSmemPerSm / (smem + kTreeSmemStatic)), items = (w.n_parts + kTreeWarps - 1) / kTreeWarps;
+    if (per_sm < 1 || smem > kTreeSmemMost) return -1.0;
+    const double busy = (double)w.n_parts / items, copy = 1500.0 + w.rec_bytes / 16;
+    const double issue = std::min(kTreeIssue, per_sm * busy * kTreeWarpIssue), live = kTreeLive * w.n_conf;
+    return live * (w.total + copy * kTreeWarpIssue * w.n_parts) / (w.n_sm * issue) + w.longest / kTreeWarpIssue + copy;
+}
 
 class TreeBuilder {
 public:
@@ -260,10 +288,8 @@ private:
         }
         auto up16 = [](u32 v) { return (v + 15) / 16 * 16; };
         const int RW = dc_.tau_linear ? R : 2;
-        cl.o_minfo = kTreeOffMinfo;
-        cl.o_rows = up16(cl.o_minfo + (u32)(cl.n_mrows * kTreeMinfo * 8));
-        cl.o_thr = up16(cl.o_rows + (u32)(cl.n_mrows * RW * (N_ + 1) * 8));
-        cl.o_thr_nf = cl.o_thr + up16((u32)(PP_ * T_ * 4));
+        cl.o_rows = kTreeOffMinfo + (u32)(cl.n_mrows * kTreeMinfo * 8);
+        cl.o_thr_nf = up16(cl.o_rows + (u32)(cl.n_mrows * RW * (N_ + 1) * 8));
         cl.rec_bytes = up16(cl.o_thr_nf + nf);
         return true;
     }
@@ -282,44 +308,44 @@ private:
                 w = std::max(w, (int)nd.nmax - (int)nd.nmin + 1);
             }
             cells[d & 1] = std::max(cells[d & 1], c); ch += c;
-            total += (double)((n_tasks + 31) / 32) * (150.0 + 42.0 * std::min(w, d == 1 ? kTreeJ : w));
+            total += (double)((n_tasks + 31) / 32) * (kTreeIteration + kTreePerLength * std::min(w, d == 1 ? kTreeJ : w));
         }
-        total += (double)((pt.m1 - pt.m0 + 31) / 32) * (150.0 + 50.0 * PP_);
+        total += (double)((pt.m1 - pt.m0 + 31) / 32) * (kTreeLeaf + kTreePerStage * PP_);
         slice = ((size_t)((cells[0] + 1) / 2 * 2) + (cells[1] + 1) / 2 * 2) * 8 + (ch + 15) / 16 * 16;
     }
 
     bool split(TreeClassHost &out)
     {
         // Parts over contiguous ranges of mappings: the few nodes near the root that two parts share are computed by both, so
-        // smaller parts cost little; more parts shorten the longest chain, fewer fill the lanes of a warp better.  Score =
-        // work of the class spread over the chip + the chain of one part.
+        // smaller parts cost little; more parts shorten the longest chain and fill the warps of a block, fewer fill the lanes
+        // of a warp better.  How many is what tree_time says.
         TreeClass &cl = out.cls;
-        int best_np = 0;
         double best = 0;
-        size_t best_slice = 0;
+        cl.n_parts = 0;
         for (u64 np : {1, 2, 3, 4, 6, 8, 12, 16, 20, 24, 28, 32, 40, 48, 56, 64, 80, 96, 128, 192, 256, 384, 512, 768, 1024, 2048, 4096, 8192}) {
             if (np > nmap_) break;
             std::vector<Part> parts((size_t)np);
             for (u64 q = 0; q < np; ++q) nodes(nmap_ * q / np, nmap_ * (q + 1) / np, parts[(size_t)q]);
-            double work = 0, longest = 0;
-            size_t slice = 0;
+            TreeWork w;
+            w.n_conf = (double)in_.n_conf; w.n_sm = in_.n_sm; w.n_parts = (int)np; w.rec_bytes = cl.rec_bytes;
             for (const Part &pt : parts) {
                 double c; size_t s;
                 cost(pt, c, s);
-                work += c; longest = std::max(longest, c); slice = std::max(slice, s);
+                w.total += c; w.longest = std::max(w.longest, c); w.slice = std::max(w.slice, s);
             }
-            const double score = work * (double)in_.n_conf / 380.0 + 4.0 * longest;
-            const bool fits = slice <= kTreeSliceBytes, best_fits = best_np && best_slice <= kTreeSliceBytes;
-            if (!best_np || (fits && (!best_fits || score < best)) || (!fits && !best_fits && slice < best_slice)) {
-                best_np = (int)np; best = score; best_slice = slice;
-            }
-            if (best_slice <= kTreeSliceBytes && best_np != (int)np && score > 1.5 * best) break;
+            const double t = tree_time(w);
+            if (t > 0 && (!cl.n_parts || t < best)) { best = t; cl.n_parts = (int)np; out.work = w.total; out.chain = w.longest; }
+            // finer parts share no more prefixes: what they all cost only grows, and a chain has an iteration a depth at least
+            const double least = w.total * kTreeLive * w.n_conf / (w.n_sm * kTreeIssue) + (PP_ - 1) * kTreeIteration / kTreeWarpIssue;
+            if (cl.n_parts && least > best) break;
         }
-        cl.n_parts = best_np;
-        out.parts.resize((size_t)best_np);
-        for (int q = 0; q < best_np; ++q) {
+        if (!cl.n_parts) return false;                          // no part leaves room for a block
+        cl.items_per_conf = (cl.n_parts + kTreeWarps - 1) / kTreeWarps;
+        cl.policy_items = 1;
+        out.parts.resize((size_t)cl.n_parts);
+        for (int q = 0; q < cl.n_parts; ++q) {
             Part pt;
-            nodes(nmap_ * q / best_np, nmap_ * (q + 1) / best_np, pt);
+            nodes(nmap_ * q / cl.n_parts, nmap_ * (q + 1) / cl.n_parts, pt);
             if (!emit(pt, cl, out.parts[(size_t)q])) return false;
         }
         return true;
@@ -396,30 +422,26 @@ private:
     int capt_[1 << HAP_MAX_TYPES] = {0};
 };
 
-// How the parts of a class are handed out: an item is a group of a configuration's parts, or all parts of several
-// configurations (classes of few parts); its parts fill the warps of a block a whole number of times.
-inline void tree_items(TreeClass &cl)
-{
-    cl.items_per_conf = 1; cl.conf_per_item = 1;
-    const size_t units = (size_t)cl.n_conf * cl.n_parts, all_warps = (size_t)148 * kTreeBlocksPerSm * kTreeWarps;
-    if (cl.n_parts > kTreeWarps) cl.items_per_conf = (cl.n_parts + kTreeWarps - 1) / kTreeWarps;
-    else if (units > all_warps && cl.n_parts < kTreeWarps) {
-        // as many configurations as fill the warps, where their records fit
-        const u32 slice = (cl.buf_cells[0] + cl.buf_cells[1]) * 8 + cl.ch_bytes;
-        const u32 budget = 220 * 1024 / kTreeBlocksPerSm;
-        const u32 room = budget > kTreeWarps * slice ? budget - kTreeWarps * slice : 0;
-        cl.conf_per_item = std::max<int>(1, std::min<int>(kTreeWarps / cl.n_parts, (int)(room / cl.rec_bytes)));
-    }
-}
-
 inline size_t tree_smem_bytes(const TreeClass &cl)
 {
-    return (size_t)cl.conf_per_item * cl.rec_bytes + kTreeWarps * ((size_t)(cl.buf_cells[0] + cl.buf_cells[1]) * 8 + cl.ch_bytes) + 64;
+    return (size_t)cl.rec_bytes + kTreeWarps * ((size_t)(cl.buf_cells[0] + cl.buf_cells[1]) * 8 + cl.ch_bytes) + kTreeSmemFixed;
 }
 
 inline size_t tree_prep_smem_bytes(const TreeClass &cl, int N, int T)
 {
-    return (size_t)T * N * 16 + (cl.rec_bytes - cl.o_thr + 15) / 16 * 16 + (size_t)(N + 1) * 17 + 32;
+    return cl.rec_bytes + tree_record_scratch(cl, N, T);
+}
+
+// Classes whose items take one policy each in a pass: those whose chain, walked policy after policy, is a good part of the pass.
+// Measured at 1,024 devices with two policies, six classes of 24 mappings / four of them and one of 840 mappings: no such items
+// 290 / 433 us, where a chain is more than a half of what the pass takes at the rate the chip issues 269 / 433, a quarter
+// 253 / 423, a tenth 249 / 416, a fiftieth the same.
+inline void tree_policy_items(std::vector<TreeClass> &cls, const std::vector<std::shared_ptr<const TreeClassHost>> &trees, int n_sm, int n_rc)
+{
+    double all = 0;
+    for (const auto &th : trees) all += th->work * kTreeLive * th->cls.n_conf / (n_sm * kTreeIssue);
+    for (size_t c = 0; c < cls.size(); ++c)
+        cls[c].policy_items = trees[c]->chain / kTreeWarpIssue > 0.1 * all ? n_rc : 1;
 }
 
 }  // namespace hap

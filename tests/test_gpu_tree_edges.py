@@ -85,3 +85,23 @@ def test_refined_search_over_listed_candidates(nodes, N, tau, policies, kinds, o
         with pytest.raises(hap.HapError):
             hap.hap_search_best(hp)
     hap.hap_problem_destroy(hp)
+
+
+@pytest.mark.parametrize("nodes,N,tau,policies,kinds", [CASES[2], CASES[4], ((2, 1, 1), 24, (0, 1024), (1, 3, 2), "uniform")])
+def test_ranges_of_a_pass_whose_items_take_one_policy(nodes, N, tau, policies, kinds):
+    """Ranges that begin and end between the policies of a mapping, and inside a configuration, against the oracle."""
+    import paper_2609_39350_b200 as hap
+    pb = problems.random_small(7 + N, N=N, T=len(nodes), nodes_per_type=nodes, node_size=2, window=True, first_dense=kinds == "dense_first")
+    R = len(tau)
+    pb.tau_q = np.array(tau, np.int32)
+    pb.xi_q = np.array([1024, 512, 200, 64][:R - 1] + [64], np.int32)
+    pb.rc_masks = np.array(policies, np.uint32)
+    o = Oracle(pb)
+    _, _, _, costs, _ = o.search_pconfs(0, 1, threads=NTHREADS, want_costs=True)
+    hp = hap.hap_problem_create(pb)
+    hap.hap_enumerate(hp)
+    cuts = sorted(np.random.default_rng(N).integers(1, hp.n_cand, 5).tolist())
+    for a, b in zip([0] + cuts, cuts + [hp.n_cand]):
+        if a < b:
+            assert np.array_equal(hap.hap_pipeline_dp(hp, a, b - a)["cost"].cpu().numpy(), costs[a:b]), (a, b)
+    hap.hap_problem_destroy(hp)
