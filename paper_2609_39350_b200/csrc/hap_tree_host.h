@@ -335,9 +335,11 @@ private:
             }
             const double t = tree_time(w);
             if (t > 0 && (!cl.n_parts || t < best)) { best = t; cl.n_parts = (int)np; out.work = w.total; out.chain = w.longest; }
-            // finer parts share no more prefixes: what they all cost only grows, and a chain has an iteration a depth at least
+            // finer parts share no more prefixes: what they all cost only grows, and a chain has an iteration a depth at least.  A
+            // sum of a growing and a falling term has one minimum, but for the rounding to whole warps: half as much again
+            // lies behind it
             const double least = w.total * kTreeLive * w.n_conf / (w.n_sm * kTreeIssue) + (PP_ - 1) * kTreeIteration / kTreeWarpIssue;
-            if (cl.n_parts && least > best) break;
+            if (cl.n_parts && (least > best || (t > 1.5 * best && cl.n_parts != (int)np))) break;
         }
         if (!cl.n_parts) return false;                          // no part leaves room for a block
         cl.items_per_conf = (cl.n_parts + kTreeWarps - 1) / kTreeWarps;
