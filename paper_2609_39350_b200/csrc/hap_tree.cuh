@@ -42,6 +42,7 @@ constexpr int kTreeThreads = kTreeWarps * 32;
 constexpr int kTreeBlocksPerSm = 5;       // (96 registers a thread)
 constexpr int kTreeJ = 4;                 // end layers of a task
 constexpr int kTreePad = kTreeJ - 1;      // infinite entries in front of every row and behind the last one
+constexpr int kTreeAhead = 1;             // and an entry in front of them all: a scan asks for the next one before it knows that it is done
 constexpr int kTreeKtab = 16 + HAP_MAX_TYPES * 6;    // stage constants: [0,16) pre-work by row group, then p2p [type][6]
 constexpr int kTreeMinfo = 8;             // doubles per row group: sync latency, sync bandwidth x 2, optimizer x 2, cross dispatch, post-work, pad
 
@@ -690,7 +691,7 @@ __device__ __forceinline__ void tree_scan(const TreeArgs &ta, u32 a_prev, u32 a_
         const u32 aj = a_row + 8u * (u32)j0;
 #pragma unroll
         for (int i = 0; i < J; ++i) {
-            C[i] = lds_f64(aj + 8u * i);                          // (entries past the last layer are other words of the record)
+            C[i] = lds_f64(aj + 8u * i);                          // (entries past the last layer are other words of the block)
             if (!F64) C[i] += K;
             F[i] = NL ? lds_f64(aj + 8u * i + stride) : 0.0;
             p[i] = lds_f64(pa + 8u * i);
@@ -810,7 +811,7 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ u32 s_item, s_unit, s_total[HAP_MAX_PP + 2];
     __shared__ uint4 s_entry;
-    __shared__ double s_zero[2 * kTreePad + 1];             // the row before the first stage: 0 at layer 0
+    __shared__ double s_zero[kTreeAhead + 2 * kTreePad + 1];    // the row before the first stage: 0 at layer 0
     __shared__ i64 s_cost[kTreeWarps];
     __shared__ u64 s_index[kTreeWarps];
     __shared__ int s_last, s_pos[2];
@@ -834,7 +835,7 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
     const bool ordered = SEARCH && !F64 && ta.order != nullptr;
     if (tid == 0) {
         if (blockIdx.x == 0 && ta.launch == 0) ta.report->stamp[1] = global_timer();
-        for (int q = 0; q < 2 * kTreePad + 1; ++q) s_zero[q] = q == kTreePad ? 0.0 : kTreeInf;
+        for (int q = 0; q < kTreeAhead + 2 * kTreePad + 1; ++q) s_zero[q] = q == kTreeAhead + kTreePad ? 0.0 : kTreeInf;
         u32 t = 0;                          // items before class c (in order of the bounds: configurations)
         for (int c = ta.c_lo; c < ta.c_hi; ++c) {
             s_total[c - ta.c_lo] = t;
@@ -972,6 +973,7 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
                             const double K = lds_f64(a_rec + kTreeOffKtab + 8u * kidx);
                             const u32 a_row0 = a_rows + mrow * row_group, slot = t.x >> 16;
                             const u32 a_prev = a_prv + 8u * (t.x & 0xffffu), a_out = a_cur + 8u * slot, a_cho = a_ch + cell0 + slot;
+                            (void)HAP_CHECK_OK(0, a > b || a_prev >= a_prv + 8u * (u32)(b - a + 1));      // the lowest entry a scan reads
                             constexpr int J = NL && kTreeJ > 2 ? kTreeJ / 2 : kTreeJ;
                             if (flat) {
                                 const TreeLevels lv = tree_levels<NL ? 4 : RK>(R, rc_mask, lds_u32(a_rec + kTreeOffThr + 4u * (u32)((d - 1) * HAP_MAX_TYPES + capt)));
@@ -1038,6 +1040,7 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
                             const double K = lds_f64(a_rec + kTreeOffKtab + 8u * kidx) + lds_f64(a_rec + kTreeOffMinfo + (mrow * kTreeMinfo + 6) * 8u);
                             const TreeLevels lv = all_flat || cl->flat[PP] ? tree_levels<NL ? 4 : RK>(R, rc_mask, lds_u32(a_rec + kTreeOffThr + 4u * (u32)((PP - 1) * HAP_MAX_TYPES + capt)))
                                                                            : nf_levels(PP, capt, N);
+                            (void)HAP_CHECK_OK(0, (pw & 0xfffffu) >= (u32)(b - a + 1));
                             double best[1];
                             int arg[1];
                             tree_scan<1, RK, F64, NL, COUNT>(ta, a_last + 8u * (pw & 0xfffffu), a_rows + mrow * row_group, row_stride, N, 1, a, b, lv, K,

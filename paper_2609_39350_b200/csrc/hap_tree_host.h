@@ -221,7 +221,7 @@ private:
             pt.lv[d].swap(sorted);
             if (d + 1 < PP_) for (auto &ch : pt.lv[d + 1]) ch.parent = newidx[ch.parent];
             else for (u64 m = m0; m < m1; ++m) if (!dead_[m]) pt.leaf_node[(size_t)(m - m0)] = newidx[pt.leaf_node[(size_t)(m - m0)]];
-            u32 c = 0;
+            u32 c = kTreeAhead;
             for (auto &nd : pt.lv[d]) { c += kTreePad; nd.rowoff = c; c += (u32)(nd.bh - nd.bl + 1); }
         }
     }
@@ -300,7 +300,7 @@ private:
         u32 cells[2] = {0, 0}, ch = 0;
         total = 0;
         for (int d = 1; d < PP_; ++d) {
-            u32 n_tasks = 0, c = kTreePad;
+            u32 n_tasks = 0, c = kTreeAhead + kTreePad;
             int w = 1;
             for (const Node &nd : pt.lv[d]) {
                 const int b = nd.bh - nd.bl + 1;
@@ -363,12 +363,12 @@ private:
         for (int d = 1; d < PP_; ++d) {
             tp.task_lo[d] = (u32)ph.tasks.size();
             tp.cell_lo[d] = cells;
-            u32 c = kTreePad;
+            u32 c = kTreeAhead + kTreePad;
             for (size_t ni = 0; ni < pt.lv[d].size(); ++ni) {
                 const Node &nd = pt.lv[d][ni];
                 const Node *pn = d > 1 ? &pt.lv[d - 1][nd.parent] : nullptr;
                 // slot of the parent's entry 0 (before the first stage: one row of layer 0 behind its padding)
-                const int pbl = pn ? pn->bl : 0, pbh = pn ? pn->bh : 0, porg = pn ? (int)pn->rowoff - pn->bl : kTreePad;
+                const int pbl = pn ? pn->bl : 0, pbh = pn ? pn->bh : 0, porg = pn ? (int)pn->rowoff - pn->bl : kTreeAhead + kTreePad;
                 for (int j = nd.bl; j <= nd.bh; j += kTreeJ) {
                     const int cnt = std::min(kTreeJ, nd.bh - j + 1);
                     const int a = std::max((int)nd.nmin, j - pbh);
@@ -406,7 +406,7 @@ private:
             if (a > b) continue;
             ph.leaf[m] = (u32)a | ((u32)b << 8);
             for (int d = PP_; d >= 1; --d) {
-                int org = PP_ > 1 ? 0 : kTreePad;
+                int org = PP_ > 1 ? 0 : kTreeAhead + kTreePad;
                 if (d == PP_) { if (PP_ > 1) { const Node &p = pt.lv[PP_ - 1][nd]; org = (int)p.rowoff - p.bl + N_ - a; } }
                 else { const Node &p = pt.lv[d][nd]; org = (int)tp.cell_lo[d] + (int)p.rowoff - p.bl + 256; nd = p.parent; }
                 ph.path[(size_t)(d - 1) * nmap + m] = (u32)org | ((u32)kidx(d, mask_[at + d - 1], link_[at + d - 1], cl) << 20) |
