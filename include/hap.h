@@ -16,6 +16,11 @@
  *  - `stream` is a cudaStream_t passed as void* (NULL = default stream).  Kernels are
  *    enqueued on it and the call returns without waiting, except where a function returns
  *    host values: that function synchronises `stream` (only that stream) before returning.
+ *    A problem's calls share its scratch memory: a call on another stream than the one before it waits for
+ *    that one's work on the device.
+ *  - Calls that return no host values may be made while `stream` is being captured, once a call of the same
+ *    kind has run (a first use may allocate).  They are then part of the graph: the caller orders the graph's
+ *    launches and the problem's other calls, before and after, and releases the graph before the problem.
  *  - A hap_problem is not thread safe; use one per thread or serialise calls.
  *  - Times are nanoseconds, memory is bytes, both as int64 after round-to-nearest-even of
  *    the fp64 formula value ("integer mode").  HAP_INF marks an infeasible candidate.
