@@ -45,11 +45,13 @@ inline size_t tree_record_scratch(const TreeClass &cl, int N, int T) { return (s
 // them, then the chain of one item.  Measured on B200: a warp of these kernels issues an instruction every six to seven cycles
 // (7.3 warps stand for every issue), an SM 2.3 a cycle when all its warps are busy (57 % of the slots); warps of a block without
 // a part still hold their registers.  About two fifths of a class's configurations are feasible (1,024 devices: 27 %, 256
-// devices: 41 %).  An item's record comes in between two barriers of its block, 1,500 cycles and one per 16 bytes.  At 1,024 devices
+// devices: 41 %).  An item's record comes in between two barriers of its block, 1,500 cycles and one per 16 bytes.  Other
+// items fill about half of a chain: counted in full, 32 devices of three types (31 layers) take 79 us instead of 71, a third of it
+// 1,024 devices 416 instead of 390, the rest the same.  At 1,024 devices
 // without a homogeneous class 4 parts of 6 mappings each, all warps busy: 243 us a pass; 2 and 3 parts, which share more
 // prefixes, 273 and 271.  Negative: no block fits.
 struct TreeWork { double total = 0, longest = 0, n_conf = 0; size_t slice = 0; u32 rec_bytes = 0; int n_parts = 0, n_sm = 0; };
-constexpr double kTreeIssue = 2.3, kTreeWarpIssue = 0.15, kTreeLive = 0.4;
+constexpr double kTreeIssue = 2.3, kTreeWarpIssue = 0.15, kTreeLive = 0.4, kTreeChain = 0.5;
 constexpr double kTreeIteration = 150.0, kTreePerLength = 42.0, kTreeLeaf = 150.0, kTreePerStage = 100.0;      // warp instructions
 inline double tree_time(const TreeWork &w)
 {
@@ -58,7 +60,7 @@ inline double tree_time(const TreeWork &w)
     if (per_sm < 1 || smem > kTreeSmemMost) return -1.0;
     const double busy = (double)w.n_parts / items, copy = 1500.0 + w.rec_bytes / 16;
     const double issue = std::min(kTreeIssue, per_sm * busy * kTreeWarpIssue), live = kTreeLive * w.n_conf;
-    return live * (w.total + copy * kTreeWarpIssue * w.n_parts) / (w.n_sm * issue) + w.longest / kTreeWarpIssue + copy;
+    return live * (w.total + copy * kTreeWarpIssue * w.n_parts) / (w.n_sm * issue) + kTreeChain * (w.longest / kTreeWarpIssue + copy);
 }
 
 class TreeBuilder {
@@ -338,7 +340,7 @@ private:
             // finer parts share no more prefixes: what they all cost only grows, and a chain has an iteration a depth at least.  A
             // sum of a growing and a falling term has one minimum, but for the rounding to whole warps: half as much again
             // lies behind it
-            const double least = w.total * kTreeLive * w.n_conf / (w.n_sm * kTreeIssue) + (PP_ - 1) * kTreeIteration / kTreeWarpIssue;
+            const double least = w.total * kTreeLive * w.n_conf / (w.n_sm * kTreeIssue) + kTreeChain * (PP_ - 1) * kTreeIteration / kTreeWarpIssue;
             if (cl.n_parts && (least > best || (t > 1.5 * best && cl.n_parts != (int)np))) break;
         }
         if (!cl.n_parts) return false;                          // no part leaves room for a block
