@@ -1276,9 +1276,9 @@ static hap_status ensure_general(hap_problem *p)
 }
 
 // per (configuration, type) constants and stage coefficients, then the layer costs of `n_conf` configurations from
-// `p_first` on (all by default); index_dev: of the one configuration that owns the candidate index stored there
+// `p_first` on (all by default)
 static hap_status launch_layer_kernel(hap_problem *p, i64 *c2, double *c2f, bool quant, cudaStream_t st, i64 *lb_sum,
-                                      const i64 *index_dev, unsigned p_first, unsigned n_conf, bool dependent)
+                                      unsigned p_first, unsigned n_conf, bool dependent)
 {
     const unsigned thr = (unsigned)((p->model.N + 31) / 32 * 32);
     // programmatic dependent launch: the blocks start while type_const_kernel drains and wait inside the kernel
@@ -1292,15 +1292,15 @@ static hap_status launch_layer_kernel(hap_problem *p, i64 *c2, double *c2f, bool
     i64 *no_i = nullptr; double *no_d = nullptr;
     // layer kinds: 0 all dense, 1 all MoE (uniform branch compiled away), 2 mixed
     const int kind = !p->dc.kind_uniform ? 2 : (p->kind[0] == HAP_MOE ? 1 : 0);
-    using Fn = void (*)(const DevConst, const TypeConst *, i64 *, double *, i64 *, u64 *, const i64 *, unsigned);
+    using Fn = void (*)(const DevConst, const TypeConst *, i64 *, double *, i64 *, u64 *, unsigned);
     if (quant) {
         static const Fn fns[3][2] = {{layer_cost_kernel<true, 0, false>, layer_cost_kernel<true, 0, true>},
                                      {layer_cost_kernel<true, 1, false>, layer_cost_kernel<true, 1, true>},
                                      {layer_cost_kernel<true, 2, false>, layer_cost_kernel<true, 2, true>}};
-        CUDA_TRY(p, cudaLaunchKernelEx(&cfg, fns[kind][lb_sum ? 1 : 0], p->dc, tcg, c2, no_d, lb_sum, p->d_range, index_dev, p_first));
+        CUDA_TRY(p, cudaLaunchKernelEx(&cfg, fns[kind][lb_sum ? 1 : 0], p->dc, tcg, c2, no_d, lb_sum, p->d_range, p_first));
     } else {
         static const Fn fns[3] = {layer_cost_kernel<false, 0, false>, layer_cost_kernel<false, 1, false>, layer_cost_kernel<false, 2, false>};
-        CUDA_TRY(p, cudaLaunchKernelEx(&cfg, fns[kind], p->dc, tcg, no_i, c2f, no_i, p->d_range, index_dev, p_first));
+        CUDA_TRY(p, cudaLaunchKernelEx(&cfg, fns[kind], p->dc, tcg, no_i, c2f, no_i, p->d_range, p_first));
     }
     return HAP_OK;
 }
@@ -1349,7 +1349,7 @@ static hap_status launch_layer_costs(hap_problem *p, i64 *c2, i64 *coef, double 
     if ((n_conf + per - 1) / per > 3 * (unsigned)sm_count(p->device)) {
         hap_status s = launch_type_consts(p, quant ? coef : nullptr, quant ? nullptr : coeff, st, p_lo, p_hi);
         if (s != HAP_OK) return s;
-        return launch_layer_kernel(p, c2, c2f, quant, st, lb_sum, nullptr, p_lo, n_conf, true);
+        return launch_layer_kernel(p, c2, c2f, quant, st, lb_sum, p_lo, n_conf, true);
     }
     const int kind = !p->dc.kind_uniform ? 2 : (p->kind[0] == HAP_MOE ? 1 : 0);      // layer kinds: all dense, all MoE, mixed
     using Fn = void (*)(const DevConst, i64 *, double *, i64 *, double *, i64 *, u64 *, unsigned, unsigned);
@@ -1481,8 +1481,8 @@ static hap_status launch_trees(hap_problem *p, const DpOut &out_in, bool search,
     if ((s = launch_type_consts(p, p->d_coef, f64 ? p->d_coeff : nullptr, st, p_lo, p_hi, &p->largs)) != HAP_OK) return s;
     const void *c2v = nullptr;
     if (separate || !p->all_trees) {
-        if (f64) { if ((s = launch_layer_kernel(p, nullptr, p->d_c2f, false, st, nullptr, nullptr, p_lo, p_hi - p_lo, true)) != HAP_OK) return s; }
-        else if ((s = launch_layer_kernel(p, p->d_c2, nullptr, true, st, p->d_lb, nullptr, p_lo, p_hi - p_lo, true)) != HAP_OK) return s;
+        if (f64) { if ((s = launch_layer_kernel(p, nullptr, p->d_c2f, false, st, nullptr, p_lo, p_hi - p_lo, true)) != HAP_OK) return s; }
+        else if ((s = launch_layer_kernel(p, p->d_c2, nullptr, true, st, p->d_lb, p_lo, p_hi - p_lo, true)) != HAP_OK) return s;
         if (separate) c2v = f64 ? (const void *)p->d_c2f : (const void *)p->d_c2;
     }
     const bool nl = !p->dc.tau_linear;
@@ -1629,7 +1629,7 @@ static hap_status run_pass(hap_problem *p, DpOut &out, bool f64, cudaStream_t st
         // the memory model stays on the integer byte coefficients in fp64 mode; times stay unrounded
         if (f64) {
             if ((s = launch_type_consts(p, p->d_coef, p->d_coeff, st, p_lo, p_hi)) != HAP_OK) return s;
-            if ((s = launch_layer_kernel(p, nullptr, p->d_c2f, false, st, nullptr, nullptr, p_lo, p_hi - p_lo, true)) != HAP_OK) return s;
+            if ((s = launch_layer_kernel(p, nullptr, p->d_c2f, false, st, nullptr, p_lo, p_hi - p_lo, true)) != HAP_OK) return s;
         } else if ((s = launch_layer_costs(p, p->d_c2, p->d_coef, nullptr, nullptr, true, st, nullptr, p_lo, p_hi)) != HAP_OK) return s;
     }
     CUDA_TRY(p, cudaEventRecord(p->ev[1], st));
@@ -1749,7 +1749,7 @@ extern "C" hap_status hap_search_range_f64(hap_problem *p, uint64_t first, uint6
     {   // the pass may have left the layer-cost array untouched: the winner's configuration is evaluated here
         size_t lo = 0, hi = p->pconfs.size();
         while (hi - lo > 1) { const size_t mid = (lo + hi) / 2; if (p->pconfs[mid].offset <= win) lo = mid; else hi = mid; }
-        if ((s = launch_layer_kernel(p, nullptr, p->d_c2f, false, st, nullptr, nullptr, (unsigned)lo, 1, false)) != HAP_OK) return s;
+        if ((s = launch_layer_kernel(p, nullptr, p->d_c2f, false, st, nullptr, (unsigned)lo, 1, false)) != HAP_OK) return s;
     }
     if ((s = launch_dp(p, one, false, st, true)) != HAP_OK) return s;
     decode_kernel<<<1, 32, 0, st>>>(p->dc, win, 1, &d1->cand, nullptr);
@@ -1934,7 +1934,7 @@ static hap_status joint_setup(hap_problem *p)
         if (!ent[w].empty()) std::memcpy(img.data() + o_ent, ent[w].data(), ent[w].size() * sizeof(unsigned));
         CUDA_TRY(p, cudaMemcpy(rh.d, img.data(), total, cudaMemcpyHostToDevice));
     }
-    p->joint_grid = 2 * 148;
+    p->joint_grid = 2 * sm_count(p->device);
     if (lmax_all) {
         const size_t bytes = (size_t)p->joint_grid * 2 * lmax_all * T * (N + 1) * sizeof(i64);
         CUDA_TRY(p, cached_malloc(p->device, (void **)&p->d_joint_scratch, bytes));

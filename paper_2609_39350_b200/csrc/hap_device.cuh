@@ -485,19 +485,12 @@ __device__ __forceinline__ void type_const_role(const DevConst &dc, TypeConst *t
 template <bool QUANT, int KIND, bool WANT_LB>
 __global__ void __launch_bounds__(256)
 layer_cost_kernel(const DevConst dc, const TypeConst *__restrict__ tcg, i64 *__restrict__ c2, double *__restrict__ c2f,
-                  i64 *__restrict__ lb_sum, u64 *range_flag, const i64 *index_dev, unsigned p_first)
+                  i64 *__restrict__ lb_sum, u64 *range_flag, unsigned p_first)
 {
     __shared__ TypeConst tcs[HAP_MAX_TYPES];
     __shared__ i64 s_lb[8];
     const int N = dc.N, T = dc.T;
-    // block b works on configuration p_first + b; or, when a preceding kernel left a candidate index in device
-    // memory, on the configuration that owns it (negative: none)
-    unsigned p = p_first + blockIdx.x;
-    if (index_dev) {
-        const i64 f = *index_dev;
-        if (f < 0) return;
-        p = (unsigned)find_pconf(dc, (u64)f);
-    }
+    const unsigned p = p_first + blockIdx.x;
     const int l = threadIdx.x;
     const bool dense = KIND == 0 || (KIND == 2 && l < N && layer_kind(dc, l) == HAP_DENSE);
     double2 ta[HAP_MAX_TYPES], tf[HAP_MAX_TYPES];           // (t_dense fwd, bwd), (t_ffn fwd, bwd) of the layer per type

@@ -51,7 +51,7 @@ constexpr int kTreeMinfo = 8;             // doubles per row group: sync latency
 //   x = slot of prev[j0 - a] in the previous depth's buffer | slot of j0's value in this depth's << 16
 //   y = j0 | a << 8 | b << 16 | (cnt - 1) << 24 | first of its row << 26 | last of the depth << 27
 //   z = stage constant index | row group of the stage's types << 8 | capacity type << 16
-//   w = unused
+//   w = 0 (a task is one load of 16 bytes)
 typedef uint4 TreeTask;
 
 // A contiguous range of a class's mappings with the tree of their prefixes.
@@ -238,9 +238,6 @@ __device__ __forceinline__ void sts_u8(u32 a, u32 v)
     if (!smem_addr_ok(a, 1)) return;
     asm volatile("st.shared.u8 [%0], %1;" :: "r"(a), "r"(v) : "memory");
 }
-
-template <typename T> struct IsF64 { static constexpr bool value = false; };
-template <> struct IsF64<double> { static constexpr bool value = true; };
 
 constexpr double kTreeInf = 4611686018427387904.0;        // 2^62, the integer INF: above every finite value
 constexpr double kTreeBound = 2305843009213693952.0;      // 2^61: every finite value is below
