@@ -1839,9 +1839,7 @@ static bool joint_reach_class(const hap_problem *p, int PP, int64_t G, const Joi
                 ent.push_back(e);
             }
     }
-    // few cells: the value form's chain (a level each) is shorter than a dozen tests of it (32 devices, 19 layers: 244 us
-    // against 418 us; 48 devices, 29 layers: 185 against 332; the line lies between those and 16 stages at 1,024 devices)
-    if (words > 2 || (i64)jc.S * T * N < 16384) return false;
+    if (words > 2) return false;
     jr.words = words;
     return reach_smem(N, T, p->prof.R, p->dc.tau_linear ? p->prof.R : 2, PP, jc.lmax, jr.nwin, words).total <= 110 * 1024;
 }
@@ -1855,6 +1853,19 @@ static hap_status joint_setup(hap_problem *p)
     for (const auto &r : p->pconfs) if (std::find(pps.begin(), pps.end(), r.PP) == pps.end()) pps.push_back(r.PP);
     std::sort(pps.begin(), pps.end(), std::greater<int>());      // the longest configurations start first
     std::vector<unsigned> ent[2];
+    // Where every class has few cells (states x types x layers) the value form is faster, whose chain is a level each where a
+    // search is a dozen tests of it (64 devices, 32 layers, at most 18,496 cells: 297 us against 488; 32 devices, 24 layers, 16,200:
+    // 208 against 340).  One class of many makes the search worth it (16 stages at 1,024 devices, 32,400 cells: 666 us against
+    // 990; 32 stages at 32 devices, 132,192: 471 against 531, two policies 480 against 981), and then the others do better beside it in the
+    // same launch than in launches of their own (32 devices, 32 layers: 492 us, 554 with the classes below 16,384 cells apart, 758
+    // without a search).
+    bool search = false;
+    for (int PP : pps) {
+        const int64_t G = p->W / PP;
+        double cells = (double)T * N;
+        for (int h = 0; h < T; ++h) cells = p->m[h] % G ? 0.0 : cells * (double)(p->m[h] / G + 1);
+        search = search || cells >= 20480.0;
+    }
     for (int PP : pps) {
         const int64_t G = p->W / PP;
         bool homog = true;
@@ -1885,7 +1896,7 @@ static hap_status joint_setup(hap_problem *p)
         jc.lmax = lmax;
         JointReach jr;
         std::vector<unsigned> en;
-        if (joint_reach_class(p, PP, G, jc, lvl_off, st_idx, slot, jr, en)) {
+        if (search && joint_reach_class(p, PP, G, jc, lvl_off, st_idx, slot, jr, en)) {
             const int w = jr.words - 1;
             hap_problem::ReachHost &rh = p->reach[w];
             for (int i = 0; i <= HAP_MAX_PP; ++i) jr.ent_off[i] += (unsigned)ent[w].size();

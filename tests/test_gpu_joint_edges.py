@@ -40,3 +40,13 @@ def test_joint_bottleneck_words(nodes, N, window, tau, dense_first):
             seen += 1
     assert seen > 0
     hap.hap_problem_destroy(hp)
+
+
+@pytest.mark.parametrize("nodes,N,window,tau,dense_first", [
+    ((2, 1, 1), 151, False, (0, 1024), True),         # 20,385 cells: every class in the form with a value per end layer
+    ((2, 1, 1), 152, False, (0, 1024), True),         # 20,520: the classes of few cells beside the large one, in bits where they fit
+    ((2, 2, 2, 2), 130, False, (0, 1024), True),      # two words, a dense first layer
+])
+def test_joint_bottleneck_forms(nodes, N, window, tau, dense_first):
+    """Both sides of the line between the forms, which one class draws for all."""
+    test_joint_bottleneck_words(nodes, N, window, tau, dense_first)
