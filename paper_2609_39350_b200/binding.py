@@ -5,6 +5,7 @@ import ctypes as C
 import operator
 import weakref
 import os
+import struct
 from typing import Optional
 
 import numpy as np
@@ -177,94 +178,90 @@ def _field_address(memo: dict, pb, name: str, dtype, keep: list) -> int:
     array that owns the memory is appended to `keep`."""
     a = getattr(pb, name)
     hit = memo.get(name)
-    if hit is not None and hit[0] is a:
-        keep.append(hit[1])
-        return hit[2]
     c = a
     if not (type(c) is np.ndarray and c.dtype == dtype and c.flags.c_contiguous):     # (no copy in the usual case)
         c = np.ascontiguousarray(np.asarray(c, dtype=dtype))
+        if hit is not None and hit[0] is a and np.array_equal(hit[1], c):             # (a list may have changed in place)
+            c = hit[1]
+    if hit is None or hit[1] is not c:
+        hit = memo[name] = (a, c, c.ctypes.data)
     keep.append(c)
-    memo[name] = (a, c, c.ctypes.data)
-    return memo[name][2]
+    return hit[2]
 
 
-_FIELDS = ("N", "S", "H", "E", "k", "n_shared", "F_dense", "F_exp", "nq", "nkv", "V", "GB", "beta", "kind", "P", "C", "node_size", "bw_intra",
-           "node_type", "node_bw_inter", "tp_list", "cp_list", "mb_list", "ep_list", "xi_q", "tau_q", "tdf", "tdb", "tff", "tfb", "tpre",
-           "tpost", "eta", "croute", "alpha", "rho", "act_coef", "copt", "kappa", "chi", "gamma", "ovl_tp", "ovl_cp", "ovl_dp", "capf",
-           "cap_eff", "fsize", "feff", "pp_list", "tpe_list", "tp_max", "delta_q", "map_cap", "rc_masks", "uniform", "het_coll", "eta_q")
-_MISSING = object()
+# the four descriptors one behind the other (each is a multiple of eight bytes long)
+_PARTS = (_Model, _Cluster, _Profile, _Opts)
+_CODES = {C.c_int32: "i", C.c_uint64: "Q", C.c_double: "d", C.c_void_p: "P"}
+_PACKED = struct.Struct("@" + "".join("".join(_CODES[t] for _, t in p._fields_) + "0P" for p in _PARTS))
+_OFFSETS = tuple(sum(C.sizeof(q) for q in _PARTS[:i]) for i in range(4))
+_Descriptors = C.c_char * _PACKED.size
+assert _PACKED.size == sum(map(C.sizeof, _PARTS))
 
 
-def _descriptors(pb):
-    """The C descriptors of a problem (their arrays' owners beside them).  Filling them costs 16 us, an eighth of a small
-    replan, so they are remembered beside the problem object for as long as each of its fields holds the same object;
-    the library reads the arrays' contents anew on every call."""
+_NUMBERS = operator.attrgetter("N", "S", "H", "E", "k", "n_shared", "F_dense", "F_exp", "nq", "nkv", "V", "GB", "beta",
+                               "kappa", "chi", "gamma", "ovl_tp", "ovl_cp", "ovl_dp", "capf", "tp_max", "delta_q", "map_cap")
+# the array fields in the order in which the descriptors hold their addresses
+_ARRAY_TYPES = (("kind", np.uint8), ("P", np.int64), ("C", np.int64), ("node_size", np.int32), ("bw_intra", np.float64), ("node_type", np.int32),
+                ("node_bw_inter", np.float64), ("tp_list", np.int32), ("cp_list", np.int32), ("mb_list", np.int32), ("ep_list", np.int32),
+                ("tdf", np.float64), ("tdb", np.float64), ("tff", np.float64), ("tfb", np.float64), ("tpre", np.float64), ("tpost", np.float64),
+                ("eta", np.float64), ("croute", np.float64), ("alpha", np.float64), ("rho", np.float64), ("act_coef", np.float64),
+                ("copt", np.float64), ("cap_eff", np.int64), ("xi_q", np.int32), ("tau_q", np.int32), ("pp_list", np.int32),
+                ("tpe_list", np.int32), ("rc_masks", np.uint32))
+_ARRAYS = operator.attrgetter(*(n for n, _ in _ARRAY_TYPES))
+_DTYPE, _DTYPES = operator.attrgetter("dtype"), [np.dtype(t) for _, t in _ARRAY_TYPES]
+
+
+def _descriptors(pb, prune: int, flags: int):
+    """The C descriptors of a problem, one behind the other, and the arrays they point to.  Numbers, lengths and types are read
+    anew on every call; an array's address is remembered beside the problem object for as long as the field holds that array
+    (asking numpy for three dozen of them takes 20 us), and the packed descriptors serve again where all values are equal."""
     memo = _address_memo(pb)
-    own = getattr(pb, "__dict__", None)
-    now = [own.get(n, _MISSING) for n in _FIELDS] if own is not None else None
-    hit = memo.get("")
-    if hit is not None and now is not None and all(map(operator.is_, now, hit[0])):
-        return hit[1]
-    keep = []
-
-    # addresses of the problem's arrays, remembered per field for as long as the field holds the same array object; kept
-    # beside the object, not in it, so that copies of the problem start empty
-    def arr(name, dtype):
-        return _field_address(memo, pb, name, dtype, keep)
-
-    mo = _Model()
-    for n in ("N", "S", "H", "E", "k", "n_shared", "F_dense", "F_exp", "nq", "nkv", "V", "GB"):
-        setattr(mo, n, int(getattr(pb, n)))
-    mo.beta = float(pb.beta)
-    mo.kind = arr("kind", np.uint8)
-    cl = _Cluster()
-    cl.n_types = int(pb.P.shape[0])
-    cl.P, cl.C, cl.node_size = arr("P", np.int64), arr("C", np.int64), arr("node_size", np.int32)
-    cl.bw_intra = arr("bw_intra", np.float64)
-    cl.n_nodes = int(pb.node_type.shape[0])
-    cl.node_type, cl.node_bw_inter = arr("node_type", np.int32), arr("node_bw_inter", np.float64)
-    pf = _Profile()
-    pf.ntp, pf.ncp, pf.nmb, pf.nep = len(pb.tp_list), len(pb.cp_list), len(pb.mb_list), len(pb.ep_list)
-    for n in ("tp_list", "cp_list", "mb_list", "ep_list", "xi_q", "tau_q"):
-        setattr(pf, n, arr(n, np.int32))
-    for n in ("tdf", "tdb", "tff", "tfb", "tpre", "tpost", "eta", "croute", "alpha", "rho", "act_coef", "copt"):
-        setattr(pf, n, arr(n, np.float64))
-    for n in ("kappa", "chi", "gamma", "ovl_tp", "ovl_cp", "ovl_dp", "capf"):
-        setattr(pf, n, float(getattr(pb, n)))
-    pf.cap_eff = arr("cap_eff", np.int64)
-    pf.R = len(pb.xi_q)
-    fsize = np.ascontiguousarray(np.asarray(getattr(pb, "fsize", []), dtype=np.float64))
-    feff = np.ascontiguousarray(np.asarray(getattr(pb, "feff", []), dtype=np.float64))
-    keep += [fsize, feff]
-    pf.n_fsize = int(fsize.shape[0])
-    pf.fsize, pf.feff = (_ptr(fsize), _ptr(feff)) if pf.n_fsize else (None, None)
-    so = _Opts()
-    so.npp, so.ntpe = len(pb.pp_list), len(pb.tpe_list)
-    so.pp_list, so.tpe_list = arr("pp_list", np.int32), arr("tpe_list", np.int32)
-    so.tp_max, so.delta_q, so.map_cap = int(pb.tp_max), int(pb.delta_q), int(pb.map_cap)
-    so.n_rc = len(pb.rc_masks)
-    so.rc_masks = arr("rc_masks", np.uint32)
-    so.flags = (OPT_UNIFORM if int(getattr(pb, "uniform", 0)) else 0) | (OPT_HETERO_DISPATCH if int(getattr(pb, "het_coll", 0)) else 0)
-    so.eta_q = int(getattr(pb, "eta_q", 0))
-    got = (mo, cl, pf, so, keep)
-    # not remembered: a field that the class provides (a property may change without the object's own fields changing) and
-    # one whose contents were converted or copied here
-    held = {id(a) for a in keep}
-    if now is not None and all((v is _MISSING and not hasattr(type(pb), n)) or isinstance(v, (int, float, np.generic)) or id(v) in held
-                               for n, v in zip(_FIELDS, now)):
-        memo[""] = (now, got)
-    return got
+    arrays, numbers = _ARRAYS(pb), _NUMBERS(pb)
+    keep = [arrays]
+    last = memo.get("")                     # arrays of the last call that were passed as they are, and their addresses
+    if last is not None and all(map(operator.is_, arrays, last[0])) and list(map(_DTYPE, arrays)) == _DTYPES:
+        at = last[1]
+    else:
+        at = [_field_address(memo, pb, name, dtype, keep) for name, dtype in _ARRAY_TYPES]
+        memo.pop("", None)
+        memo.pop("packed", None)
+        if all(map(operator.is_, arrays, keep[1:])):
+            memo[""] = (arrays, at)
+    n_fsize = at_fsize = at_feff = 0
+    fsize = getattr(pb, "fsize", None)
+    if fsize is not None and len(fsize):
+        n_fsize, at_fsize, at_feff = len(fsize), _field_address(memo, pb, "fsize", np.float64, keep), _field_address(memo, pb, "feff", np.float64, keep)
+    if int(getattr(pb, "uniform", 0)):
+        flags |= OPT_UNIFORM
+    if int(getattr(pb, "het_coll", 0)):
+        flags |= OPT_HETERO_DISPATCH
+    n = list(map(len, arrays))
+    given = (numbers, n, n_fsize, at_fsize, at_feff, prune, flags, getattr(pb, "eta_q", 0))
+    packed = memo.get("packed")
+    if packed is not None and packed[0] == given:
+        return packed[1], keep
+    kappa, chi, gamma, ovl_tp, ovl_cp, ovl_dp, capf = numbers[13:20]
+    values = ((*map(int, numbers[:12]), numbers[12], at[0]), (n[1], *at[1:5], n[5], *at[5:7]),
+              (*n[7:11], *at[7:19], kappa, at[19], chi, at[20], gamma, ovl_tp, ovl_cp, ovl_dp, at[21], capf, *at[22:24], n[24], *at[24:26],
+               n_fsize, at_fsize, at_feff),
+              (*n[26:28], *at[26:28], *map(int, numbers[20:]), n[28], at[28], int(prune), int(flags), int(getattr(pb, "eta_q", 0))))
+    out = _Descriptors()
+    try:
+        _PACKED.pack_into(out, 0, *values[0], *values[1], *values[2], *values[3])
+    except struct.error:                    # a number outside of its field: passed on as C would, for the library to judge
+        for part, offset, v in zip(_PARTS, _OFFSETS, values):
+            C.memmove(C.byref(out, offset), C.byref(part(*v)), C.sizeof(part))
+    if "" in memo:
+        memo["packed"] = (given, out)
+    return out, keep
 
 
 def hap_problem_create(pb, prune: int = 0, flags: int = 0) -> HapProblem:
     """Marshals a plain-data problem (see gen.problems.Problem) into the C descriptors."""
     L = load_library()
-    mo, cl, pf, base, keep = _descriptors(pb)      # (`keep` holds the arrays until the call has read them)
-    so = _Opts.from_buffer_copy(base)
-    so.prune = int(prune)
-    so.flags = int(flags) | base.flags
+    descriptors, keep = _descriptors(pb, prune, flags)      # (`keep` holds the arrays until the call has read them)
     out = C.c_void_p(0)
-    st = L.hap_problem_create(C.byref(mo), C.byref(cl), C.byref(pf), C.byref(so), C.byref(out))
+    st = L.hap_problem_create(*(C.byref(descriptors, offset) for offset in _OFFSETS), C.byref(out))
     if st != 0:
         raise HapError(st, "hap_problem_create")
     return HapProblem(out.value, pb)

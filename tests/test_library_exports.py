@@ -78,3 +78,44 @@ def test_binding_remembers_array_addresses_per_problem_object_only():
     del other, m2
     gc.collect()
     assert key not in b._ADDRESSES
+
+
+def _fields_of(b, pb):
+    raw, keep = b._descriptors(pb, 1, 4)
+    return [{n: getattr(t.from_buffer_copy(raw, at), n) for n, _ in t._fields_} for t, at in zip(b._PARTS, b._OFFSETS)], keep
+
+
+def test_descriptors_follow_the_problem_object():
+    """What changes between two calls on the same object -- numbers, lengths, a list's contents, an array's -- is in the
+    second call's descriptors."""
+    import numpy as np
+    from gen import problems
+    from paper_2609_39350_b200 import binding as b
+    pb = problems.small()
+    (mo, cl, pf, so), _ = _fields_of(b, pb)
+    assert (mo["N"], mo["GB"], mo["beta"], cl["n_types"], cl["n_nodes"]) == (pb.N, pb.GB, pb.beta, len(pb.P), len(pb.node_type))
+    assert (pf["kappa"], pf["chi"], pf["gamma"], pf["ovl_tp"], pf["ovl_cp"], pf["ovl_dp"], pf["capf"], pf["R"]) == (
+        pb.kappa, pb.chi, pb.gamma, pb.ovl_tp, pb.ovl_cp, pb.ovl_dp, pb.capf, len(pb.xi_q))
+    for name, f in [(n, mo) for n in ("kind",)] + [(n, cl) for n in ("P", "C", "node_size", "bw_intra", "node_type", "node_bw_inter")] + [
+            (n, pf) for n in ("tp_list", "cp_list", "mb_list", "ep_list", "tdf", "tdb", "tff", "tfb", "tpre", "tpost", "eta", "croute", "alpha", "rho",
+                              "act_coef", "copt", "cap_eff", "xi_q", "tau_q")] + [(n, so) for n in ("pp_list", "tpe_list", "rc_masks")]:
+        assert f[name] == getattr(pb, name).ctypes.data, name
+    assert (so["npp"], so["n_rc"], so["prune"], so["flags"], so["map_cap"], so["delta_q"]) == (len(pb.pp_list), len(pb.rc_masks), 1, 4, pb.map_cap, pb.delta_q)
+    pb.GB, pb.kappa, pb.eta_q = 2 * pb.GB, 3.0, 77
+    pb.mb_list = [1, 2]
+    first, keep = _fields_of(b, pb)
+    assert (first[0]["GB"], first[2]["kappa"], first[3]["eta_q"], first[2]["nmb"]) == (pb.GB, 3.0, 77, 2)
+    pb.mb_list.append(4)                              # the same list, longer
+    second, keep = _fields_of(b, pb)
+    assert second[2]["nmb"] == 3
+    assert np.ctypeslib.as_array(ctypes.cast(second[2]["mb_list"], ctypes.POINTER(ctypes.c_int32)), (3,)).tolist() == [1, 2, 4]
+    pb.tdf = pb.tdf.astype(np.float32)                # converted, and read anew when its contents change
+    third, keep = _fields_of(b, pb)
+    pb.tdf *= 2.0
+    fourth, keep = _fields_of(b, pb)
+    n = pb.tdf.size
+    got = np.ctypeslib.as_array(ctypes.cast(fourth[2]["tdf"], ctypes.POINTER(ctypes.c_double)), (n,))
+    assert np.array_equal(got, pb.tdf.ravel().astype(np.float64))
+    pb.map_cap, pb.GB = -1, (1 << 32) + 64            # outside of their fields: wrapped, as C does
+    fifth, keep = _fields_of(b, pb)
+    assert (fifth[3]["map_cap"], fifth[0]["GB"], fifth[0]["beta"]) == ((1 << 64) - 1, 64, pb.beta)
