@@ -148,9 +148,9 @@ typedef struct {
 #define HAP_OPT_NO_MAPTAB 1   /* keep no table of decoded mappings on the device: the DP kernel unranks each mapping itself */
 #define HAP_OPT_NO_TRIE 16    /* keep no prefix tree of the mappings: every pass runs one warp per candidate (the tree form
                                  shares the DP rows of common stage prefixes between all mappings of a configuration) */
-#define HAP_OPT_NO_FUSE 32    /* passes that walk the prefix trees let every block compute the layer times of its configuration itself
-                                 (Eq. 2) instead of reading an array that a layer-cost launch wrote before; this flag keeps the
-                                 separate launch (identical results) */
+#define HAP_OPT_NO_FUSE 32    /* passes that walk the prefix trees compute the layer times of a configuration (Eq. 2) where they lay out
+                                 its record instead of reading an array that a layer-cost launch wrote before; this flag keeps
+                                 the separate launch (identical results) */
 #define HAP_OPT_COUNT_SPLITS 64 /* instrumentation: hap_pipeline_dp passes of this problem also count the splits (k, j) their kernels
                                  evaluate, after all early exits, for hap_get_timings; costs a few percent of the pass */
 #define HAP_OPT_HETERO_DISPATCH 128 /* Pruning 3 (Sec. 3.5 (3)) also counts, for every stage whose devices are of more than one
@@ -241,9 +241,13 @@ hap_status hap_release_cached_memory(void);
  * What depends on the model's dimensions, the cluster and the search options only -- the configuration table, the
  * work items and the prefix trees of the classes' stage mappings -- is kept per process (host memory, at most a few
  * hundred entries, keyed by exactly those inputs) and reused when a later problem has the same key: planning again on
- * the same cluster with new profiled tables skips the loop nest and the tree build.  The device copies are still the
- * problem's own; the table and the address-free part of the trees are uploaded straight from page-locked images of
- * them (one per key, the tree images at most 16 per process). */
+ * the same cluster with new profiled tables skips the loop nest and the tree build.  Their device copy is shared by the
+ * problems of a process with the same key, too (at most 16 copies).  The problem's own device memory holds the stage
+ * coefficients, scratch and a record per configuration for the passes: head, constants, the prefix rows of the stage time and
+ * the memory thresholds, about 1 KB + 8 (N + 1) bytes per level and set of device types that a stage can have (at most
+ * 2^n_types - 1, in practice 4 to 10).  That is 55 to 115 MB at 1,024 devices and 96 layers, and under 600 MB for the
+ * largest inputs of that cluster (255 layers, 4 levels).  Where the device has no room for the records, passes run
+ * without the trees, one warp per candidate. */
 hap_status hap_enumerate(hap_problem *, uint64_t *n_pconf, uint64_t *n_candidates);
 hap_status hap_get_pconfs(const hap_problem *, hap_pconf *host_out, uint64_t cap);
 
@@ -261,7 +265,7 @@ hap_status hap_eval_layer_costs_f64(hap_problem *, double *dev_c2, double *dev_c
 /* Sec. 3.5 (non-uniform layer assignment, Pruning 1 and 2) with the min-max recurrence
  * DP[i][j] = min_k max(DP[i-1][k], cost_i(k,j)), backtrace, and Eq. 4 in the closed form
  * sum_i c_i + (M-1) max_i c_i + T_dp-sync + T_opt, for candidates [first, first+count).
- * The layer costs (Eq. 2) are recomputed first: inside the blocks of the dynamic program where the pass walks the
+ * The layer costs (Eq. 2) are recomputed first: with the configurations' records where the pass walks the
  * classes' prefix trees (the default), into library-owned memory by a separate launch otherwise.  No candidate is
  * skipped.
  * dev_cost, dev_bottleneck: [count] (HAP_INF when infeasible)
@@ -289,15 +293,16 @@ hap_status hap_search_range_f64(hap_problem *, uint64_t first, uint64_t count, h
 /* Eq. 1: layer costs, dynamic program and argmin over candidates [first, first+count) with
  * ties going to the lowest index; writes the plan to host memory.  Synchronises `stream`.
  * host_stats is nullable.  Returns HAP_E_INFEASIBLE when no candidate is feasible.
- * With opts.prune, blocks whose configuration-level lower bound exceeds the incumbent are skipped (strict bound:
- * same plan).  Under HAP_OPT_REFINE / HAP_OPT_EXACT a plain pass first bounds every candidate from below by
- * S + (M-1) B* (B* its bottleneck, S the configuration's sum over layers of the cheapest type's time) and the
- * refinement runs only for candidates whose bound does not exceed the incumbent; host_stats->n_pruned counts the
- * candidates cut this way, candidates without a feasible partition count as evaluated.  The first such call
- * allocates 8 bytes per candidate of scratch.
+ * With opts.prune, configurations are taken in the order of a lower bound on their candidates and those whose bound exceeds the
+ * incumbent are skipped (strict bound: same plan).  Under HAP_OPT_REFINE / HAP_OPT_EXACT such a search lists the candidates
+ * whose bound S + (M-1) B* (B* the candidate's bottleneck, S the configuration's sum over layers of the cheapest type's
+ * time) does not exceed the smallest plain T_iter, and only those are refined; host_stats->n_pruned counts the others
+ * (candidates without a feasible partition count as evaluated).  Where the list does not decide, or a class has no
+ * prefix tree, a plain pass bounds every candidate and the general kernel refines those whose bound does not exceed the incumbent
+ * (the first such call allocates 8 bytes per candidate).
  * The plan (partition, levels, terms of Eq. 4) comes from the search itself when every class walks its prefix tree:
- * each block leaves the plan of its best candidate and the winner's is copied out (the first search of a problem
- * allocates 112 bytes per block for them); otherwise the winner is evaluated once more alone. */
+ * each block leaves the plan of its best candidate and the last one writes the winner's to the host; otherwise the
+ * winner is evaluated once more alone. */
 hap_status hap_search_range(hap_problem *, uint64_t first, uint64_t count, hap_plan *host_out,
                             hap_search_stats *host_stats, void *stream);
 /* The whole candidate space. */

@@ -820,7 +820,7 @@ static void enum_cache_insert(const std::string &key, std::shared_ptr<const Enum
 
 // Configuration table and trees on the problem's device: from the process's images when one of the same key exists, else
 // laid out and copied now (once per cluster, model dimensions and search options).
-static hap_status image_for(hap_problem *p, const std::string &ekey)
+static hap_status image_for(hap_problem *p, const std::string &ekey, bool allow_trees)
 {
     // the tree kernel holds times as doubles: exact while every prefix row stays below 2^52, which the per-layer limit of
     // 2^36 ns guarantees when N (2 + max tau) <= 2^16; rows that are not combined by level also form tau x forward time
@@ -835,7 +835,7 @@ static hap_status image_for(hap_problem *p, const std::string &ekey)
         for (int r = 0; r < p->prof.R; ++r)
             if ((mk >> r) & 1u) { ordered = ordered && p->tau_q[r] >= last; last = p->tau_q[r]; }
     }
-    const bool want_tree = !(p->opts.flags & (HAP_OPT_NO_TRIE | HAP_OPT_NO_MAPTAB)) && exact && ordered;
+    const bool want_tree = allow_trees && !(p->opts.flags & (HAP_OPT_NO_TRIE | HAP_OPT_NO_MAPTAB)) && exact && ordered;
     std::string key = ekey;
     const int32_t head[] = {p->device, want_tree, p->prof.R, p->opts.delta_q, (int32_t)(p->opts.flags & HAP_OPT_UNIFORM), p->dc.kind_uniform,
                             p->dc.kind_uniform_from, p->dc.tau_linear};
@@ -1041,10 +1041,10 @@ extern "C" hap_status hap_enumerate(hap_problem *p, uint64_t *n_pconf, uint64_t 
         p->tab_bytes = er->tab_bytes;
         p->n_cand = er->n_cand;
         const size_t np = p->pconfs.size();
-        {
-            hap_status is = image_for(p, ekey);
-            if (is != HAP_OK) return is;
-        }
+        // (a device without room for the records of the trees runs one warp per candidate)
+        for (bool trees : {true, false}) {
+        const hap_status is = image_for(p, ekey, trees);
+        if (is != HAP_OK) return is;
         const DeviceImage &im = *p->image;
         p->all_trees = true;
         for (size_t ci = 0; ci < p->classes.size(); ++ci) {
@@ -1079,7 +1079,9 @@ extern "C" hap_status hap_enumerate(hap_problem *p, uint64_t *n_pconf, uint64_t 
             const size_t o_order = o; o = up(o + (ordering ? (np + 1) * sizeof(uint4) : 0));
             const size_t o_surv = o; o = up(o + (refining ? n_surv * sizeof(Survivor) : 0));
             const size_t o_res = o; o = up(o + sizeof(TreeResult));
-            CUDA_TRY(p, cached_malloc(p->device, (void **)&p->d_arena, o));
+            const cudaError_t e = cached_malloc(p->device, (void **)&p->d_arena, o);
+            if (e == cudaErrorMemoryAllocation && trees && im.rec_total) { cudaGetLastError(); continue; }
+            CUDA_TRY(p, e);
             unsigned char *base = p->d_arena;
             p->d_coef = reinterpret_cast<i64 *>(base + o_coef);
             p->d_tc = reinterpret_cast<TypeConst *>(base + o_tc); p->d_lb = reinterpret_cast<i64 *>(base + o_lb);
@@ -1118,6 +1120,8 @@ extern "C" hap_status hap_enumerate(hap_problem *p, uint64_t *n_pconf, uint64_t 
         p->dc.pconf = im.d_pconf;
         p->dc.n_pconf = np;
         p->enumerated = true;
+        break;
+        }
     }
     if (n_pconf) *n_pconf = p->pconfs.size();
     if (n_candidates) *n_candidates = p->n_cand;
