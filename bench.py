@@ -486,8 +486,8 @@ def main():
                                "bands and early exits avoid, not utilisation; traffic: not measured by this run",
                           peak_source=f"{SM_COUNT} SMs x {SCHEDULERS_PER_SM} schedulers x {LANES} lanes x "
                           f"{sm_mhz} MHz (clock sampled during the timed region)", sm_mhz_seen=sm_mhz),
-            roofline_layer_cost=dict(bound="hbm", kernel="type_const_kernel + layer_cost_kernel (hap_eval_layer_costs alone; "
-                                     "the pass itself computes layer costs inside the DP blocks and writes none)",
+            roofline_layer_cost=dict(bound="hbm", kernel="type_const_plain_kernel + layer_cost_kernel (hap_eval_layer_costs alone; "
+                                     "the pass itself computes layer costs with the configurations' records and writes none)",
                                      achieved=lc_gbs, peak=peaks["hbm_gbs"],
                                      unit="GB/s", frac=lc_gbs / peaks["hbm_gbs"], traffic=None,
                                      bytes_per_launch=16 * units, ms_alone=lc_alone_ms, ms_before_dp_in_pass=lc_med,

@@ -104,7 +104,7 @@ constexpr u32 kTreeOffKtab = sizeof(TreeHead);
 constexpr u32 kTreeOffThr = kTreeOffKtab + kTreeKtab * 8;                  // [depth - 1][HAP_MAX_TYPES] words
 constexpr u32 kTreeOffMinfo = kTreeOffThr + HAP_MAX_PP * HAP_MAX_TYPES * 4;
 
-// What a search brings back, written by the last block (device memory and, if mapped, the host's copy).
+// What a search brings back, written by the last block: to the host's mapped copy where there is one, else to device memory.
 struct TreeResult {
     u64 range_flag, n_feasible, n_pruned, again;      // again: the listed candidates do not decide the search
     i64 cost; u64 index;
