@@ -47,9 +47,8 @@ inline size_t tree_record_scratch(const TreeClass &cl, int N, int T) { return (s
 // a part still hold their registers.  About two fifths of a class's configurations are feasible (1,024 devices: 27 %, 256
 // devices: 41 %).  An item's record comes in between two barriers of its block, 1,500 cycles and one per 16 bytes.  Other
 // items fill about half of a chain: counted in full, 32 devices of three types (31 layers) take 79 us instead of 71, a third of it
-// 1,024 devices 416 instead of 390, the rest the same.  At 1,024 devices
-// without a homogeneous class 4 parts of 6 mappings each, all warps busy: 243 us a pass; 2 and 3 parts, which share more
-// prefixes, 273 and 271.  Negative: no block fits.
+// 1,024 devices 416 instead of 390, the rest the same.  A pass at 1,024 devices without a homogeneous class, by the parts of
+// its 24 mappings at 32 stages (all policies an item): 1 part 527 us, 2 384, 3 351, 4 310, 6 329, 8 324.  Negative: no block fits.
 struct TreeWork { double total = 0, longest = 0, n_conf = 0; size_t slice = 0; u32 rec_bytes = 0; int n_parts = 0, n_sm = 0; };
 constexpr double kTreeIssue = 2.3, kTreeWarpIssue = 0.15, kTreeLive = 0.4, kTreeChain = 0.5;
 constexpr double kTreeIteration = 150.0, kTreePerLength = 42.0, kTreeLeaf = 150.0, kTreePerStage = 100.0;      // warp instructions
