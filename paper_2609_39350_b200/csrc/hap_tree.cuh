@@ -14,7 +14,8 @@
 //   tree_dp_kernel     persistent blocks of four warps that take (configuration, up to four of its tree's parts) items
 //                      from a counter; in a pass an item of a class with long chains is one policy's.  A warp owns a
 //                      part of the tree -- a few to some tens of mappings -- and walks it depth by depth on its own:
-//                      no block barrier inside an item.  A task is four consecutive end layers of a node; a lane keeps
+//                      no block barrier inside an item.  A task is one, two or four consecutive end layers of a node (four
+//                      where the lanes are full, fewer where lanes would idle); a lane keeps
 //                      their running minima and slides one window of the parent's row over the stage lengths
 //                      (tree_scan).  Then one lane per mapping evaluates the last stage, walks the choices back and
 //                      assembles Eq. 4.  A search leaves the plan of the best candidate; the last block to finish
@@ -40,18 +41,19 @@ namespace hap {
 constexpr int kTreeWarps = 4;             // warps of a DP block
 constexpr int kTreeThreads = kTreeWarps * 32;
 constexpr int kTreeBlocksPerSm = 5;       // (96 registers a thread)
-constexpr int kTreeJ = 4;                 // end layers of a task
+constexpr int kTreeJ = 4;                 // end layers of a task at most
+template <int J> struct TreeWidth { static constexpr int value = J; };
 constexpr int kTreePad = kTreeJ - 1;      // infinite entries in front of every row and behind the last one
-constexpr int kTreeAhead = 1;             // and an entry in front of them all: a scan asks for the next one before it knows that it is done
+constexpr int kTreeAhead = 2;             // and entries in front of them all: a scan asks for the next two before it knows that it is done
 constexpr int kTreeKtab = 16 + HAP_MAX_TYPES * 6;    // stage constants: [0,16) pre-work by row group, then p2p [type][6]
 constexpr int kTreeMinfo = 8;             // doubles per row group: sync latency, sync bandwidth x 2, optimizer x 2, cross dispatch, post-work, pad
 
-// A task: up to four consecutive end layers j0..j0+cnt-1 of one node (a stage prefix of depth d < PP) and the stage lengths
+// A task: one, two or up to four consecutive end layers j0..j0+cnt-1 of one node (a stage prefix of depth d < PP) and the stage lengths
 // a..b that reach the parent's row from any of them.
 //   x = slot of prev[j0 - a] in the previous depth's buffer | slot of j0's value in this depth's << 16
 //   y = j0 | a << 8 | b << 16 | (cnt - 1) << 24 | first of its row << 26 | last of the depth << 27
 //   z = stage constant index | row group of the stage's types << 8 | capacity type << 16
-//   w = 0 (a task is one load of 16 bytes)
+//   w = most end layers of a task in its iteration (1, 2, 4): the same for the 32 tasks a warp takes together
 typedef uint4 TreeTask;
 
 // A contiguous range of a class's mappings with the tree of their prefixes.
@@ -667,79 +669,92 @@ __device__ __forceinline__ int tree_bound(const TreeLevels &lv, int r) { return 
 // (smallest split) on ties.  The lane holds a window of J entries of prev and of the row, prev[j0 + i - n], that moves by
 // one entry per length: two loads serve J splits, and the J minima are independent chains.  Entries of prev outside the
 // parent's row are infinite (padding), so nothing is clipped per split; lengths run level by level, the bounds in lv.
-// What bounds it is instruction issue: eight instructions per split (one subtraction, two comparisons and five selects of
-// 64-bit values), five more per length for the window.
+// Lengths are taken in pairs without a branch between them: the second of a pair counts where the level has it, and both
+// entries a pair moves on by are asked for before its first split, so that their latency lies behind it.  What bounds it is
+// instruction issue: eight instructions a split, half of the arithmetic pipe's time for selects.  Pairs against a test and a branch
+// per length: 1,024 devices 378 us a pass (393), 256 devices 439 (452).
 //   a_prev: address of prev[j0 - a]; a_row0: address of entry 0 of the row group's first row, `stride` bytes per row
 template <int J, int RK, bool F64, bool NL, bool COUNT>
 __device__ __forceinline__ void tree_scan(const TreeArgs &ta, u32 a_prev, u32 a_row0, u32 stride, int j0, int cnt, int a, int b, const TreeLevels &lv,
                                           double K, double (&best)[J], int (&arg)[J], u32 &splits)
 {
+    static_assert(J == 1 || J % 2 == 0, "pairs of lengths");
 #pragma unroll
     for (int i = 0; i < J; ++i) { best[i] = kTreeBound; arg[i] = 0; }
     const int end = b < lv.nx ? b : lv.nx;
     if (a > end) return;
     int n = a, r = RK == 2 && !NL ? (int)(a > lv.b0) : (a > lv.b0) + (a > lv.b1) + (a > lv.b2);
-    int change = RK == 2 && !NL ? (r == 0 ? lv.b0 + 1 : kNever) : tree_bound(lv, r) + 1;     // first length of the next level
-    u32 a_row = a_row0 + (NL ? 0u : (u32)r * stride);
-    double tau = NL ? ta.tau[r] : 0.0;
-    double C[J], F[J], p[J], q[J], f[J];
-    u32 pa = a_prev, k0 = 8u * (u32)(j0 - a);                     // cell 0's entries: prev, and offset in a row
-    {
+    int seg = 0;                                                  // last length of the level at hand
+    u32 a_row = 0, pa = a_prev, k0 = 8u * (u32)(j0 - a);          // cell 0's entries: prev, and offset in a row
+    double tau = 0.0, C[J], F[J], p[J], q[J], f[J];
+    // a level begins at length n: rows of the level, the window of length n; cell i's entries lie in place (i - h) mod J
+    auto level = [&](const int h) {
+        const int top = tree_bound(lv, r);
+        seg = RK == 2 && !NL && r ? end : end < top ? end : top;
+        a_row = a_row0 + (NL ? 0u : (u32)r * stride);
+        if (NL) tau = ta.tau[r];
         const u32 aj = a_row + 8u * (u32)j0;
 #pragma unroll
         for (int i = 0; i < J; ++i) {
+            const int w = (i - h) & (J - 1);
             C[i] = lds_f64(aj + 8u * i);                          // (entries past the last layer are other words of the block)
-            if (!F64) C[i] += K;
             F[i] = NL ? lds_f64(aj + 8u * i + stride) : 0.0;
-            p[i] = lds_f64(pa + 8u * i);
-            q[i] = lds_f64(a_row + k0 + 8u * i);
-            f[i] = NL ? lds_f64(a_row + k0 + 8u * i + stride) : 0.0;
+            p[w] = lds_f64(pa + 8u * i);
+            q[w] = lds_f64(a_row + k0 + 8u * i);
+            f[w] = NL ? lds_f64(a_row + k0 + 8u * i + stride) : 0.0;
         }
-    }
+        if (!F64)
+#pragma unroll
+            for (int i = 0; i < J; ++i) C[i] += K;
+    };
+    level(0);
     while (true) {
         double last[J];
 #pragma unroll
-        for (int s = 0; s < J; ++s) {
-            if (s == 0 || n + s <= end) {
-                if (n + s == change) {                            // the next level's row: the whole window is read anew
-                    do { ++r; } while (RK != 2 && n + s > tree_bound(lv, r));
-                    change = RK == 2 ? kNever : tree_bound(lv, r) + 1;
-                    if (NL) tau = ta.tau[r];
-                    else {
-                        a_row = a_row0 + (u32)r * stride;
-                        const u32 aj = a_row + 8u * (u32)j0;
+        for (int h = 0; h < J; h += 2) {
+            double tp[2], tq[2], tf[2];                           // the entries below cell 0's
 #pragma unroll
-                        for (int i = 0; i < J; ++i) {
-                            C[i] = lds_f64(aj + 8u * i);
-                            if (!F64) C[i] += K;
-                            q[(i - s) & (J - 1)] = lds_f64(a_row + k0 + 8u * i - 8u * s);
-                        }
-                    }
-                }
+            for (int s = 0; s < 2; ++s) {
+                tp[s] = lds_f64(pa - 8u * (s + 1));
+                tq[s] = lds_f64(a_row + k0 - 8u * (s + 1));
+                tf[s] = NL ? lds_f64(a_row + k0 + stride - 8u * (s + 1)) : 0.0;
+            }
+            const bool both = n < seg;
+#pragma unroll
+            for (int s = 0; s < 2; ++s)
 #pragma unroll
                 for (int i = 0; i < J; ++i) {
-                    const int w = (i - s) & (J - 1);
-                    const double c = tree_span<F64, NL>(C[i], q[w], F[i], f[w], K, tau);
-                    const double v = p[w] > c ? p[w] : c;
-                    if (v <= best[i]) { best[i] = v; arg[i] = n + s; }
+                    const int w = (i - s - h) & (J - 1);
+                    const bool below = i < s;
+                    const double c = tree_span<F64, NL>(C[i], below ? tq[0] : q[w], F[i], below ? tf[0] : f[w], K, tau);
+                    const double x = below ? tp[0] : p[w], v = x > c ? x : c;
+                    if (v <= best[i] && (s == 0 || both)) { best[i] = v; arg[i] = n + s; }
                     last[i] = c;
-                    if (COUNT) splits += i < cnt ? 1u : 0u;
+                    if (COUNT) splits += i < cnt && (s == 0 || both) ? 1u : 0u;
                 }
-                // the entry that leaves the window is that of cell J-1; the next one lies below cell 0's
-                const int w = (J - 1 - s) & (J - 1);
-                p[w] = lds_f64(pa - 8u * (s + 1));
-                q[w] = lds_f64(a_row + k0 - 8u * (s + 1));
-                if (NL) f[w] = lds_f64(a_row + k0 + stride - 8u * (s + 1));
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                const int w = (-1 - s - h) & (J - 1);
+                p[w] = tp[s]; q[w] = tq[s];
+                if (NL) f[w] = tf[s];
+            }
+            n += 2; pa -= 16u; k0 -= 16u;
+            if (n > seg) {
+                if (seg >= end) return;
+                const u32 back = 8u * (u32)(n - seg - 1);         // to the first length of the next level
+                n = seg + 1; pa += back; k0 += back;
+                do ++r; while (RK != 2 && n > tree_bound(lv, r));
+                level((h + 2) & (J - 1));
+#pragma unroll
+                for (int i = 0; i < J; ++i) last[i] = 0.0;
             }
         }
-        n += J; pa -= 8u * J; k0 -= 8u * J;
-        if (n > end) break;
         // costs grow with the length (the host sends policies whose higher levels repeat less forward work to the general
         // kernel): once they exceed all the minima, longer stages cannot win
         bool over = true;
 #pragma unroll
         for (int i = 0; i < J; ++i) over = over && last[i] > best[i];
-        if (over) break;
+        if (over) return;
     }
 }
 
@@ -908,6 +923,7 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
         const bool all_flat = cl->all_flat != 0;
         const bool packed = ta.kind_uniform && cl->n_mrows <= 4;       // sync and optimizer terms from the longest stage per row group
         const u32 row_stride = (u32)n1 * 8u, row_group = (u32)RW * row_stride;
+        const u32 flat_depths = all_flat ? ~0u : __ballot_sync(0xffffffffu, lane < PP && cl->flat[lane] != 0);      // (depths below PP)
 
         while (true) {
             u32 u = 0;
@@ -934,6 +950,8 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
             }
             unsigned without_plan = 0;          // positions in rc_order under which no mapping was feasible
             const TreeTask *tasks = pt->tasks;
+            // by lane: where the tasks of depth lane + 1 and its choices start
+            const u32 lane_task = __ldg(pt->task_lo + 1 + lane), lane_cell = __ldg(pt->cell_lo + 1 + lane);
 
             for (int pos = s_pos[0]; pos < s_pos[1]; ++pos) {
                 const int rc_idx = ta.rc_order[pos];
@@ -949,55 +967,52 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
 
                 // ---- rows of the tree, depth by depth ------------------------------------------------------
                 if (!dead && PP > 1) {
-                    u32 e_end = pt->task_lo[2];
-                    u32 e = (u32)lane;
+                    u32 lo = __shfl_sync(0xffffffffu, lane_task, 0), hi = __shfl_sync(0xffffffffu, lane_task, 1);
                     TreeTask nxt = make_uint4(0, 0, 0, 0);
-                    if (e < e_end) nxt = __ldg(tasks + e);
+                    if (lo + (u32)lane < hi) nxt = __ldg(tasks + lo + lane);
                     for (int d = 1; d < PP; ++d) {
-                        const u32 cell0 = pt->cell_lo[d];
-                        const u32 next_end = d + 1 < PP ? pt->task_lo[d + 2] : e_end;
-                        const bool flat = all_flat || cl->flat[d];
+                        const u32 cell0 = __shfl_sync(0xffffffffu, lane_cell, d - 1);
+                        const u32 next_hi = d + 1 < PP ? __shfl_sync(0xffffffffu, lane_task, d + 1) : hi;
+                        const bool flat = (flat_depths >> d) & 1u;
                         const u32 a_cur = a_buf[d & 1];
                         const u32 a_prv = d == 1 ? a_zero : a_buf[(d & 1) ^ 1];
                         bool alive = false;
-                        while (e < e_end) {
+                        for (u32 base = lo; base < hi; base += 32u) {
                             const TreeTask t = nxt;
-                            e += 32u;
-                            if (e < e_end) nxt = __ldg(tasks + e);
+                            // the next tasks, those of the next depth behind the last of this one, come in behind this scan
+                            const bool wrap = base + 32u >= hi;
+                            const u32 e = (wrap ? hi : base + 32u) + (u32)lane;
+                            if (e < (wrap ? next_hi : hi)) nxt = __ldg(tasks + e);
+                            if (base + (u32)lane >= hi) continue;
                             const int j0 = (int)(t.y & 255u), a = (int)(t.y >> 8) & 255, b = (int)(t.y >> 16) & 255, cnt = ((int)(t.y >> 24) & 3) + 1;
                             const u32 kidx = t.z & 255u, mrow = (t.z >> 8) & 255u;
                             const int capt = (int)(t.z >> 16);
                             const double K = lds_f64(a_rec + kTreeOffKtab + 8u * kidx);
                             const u32 a_row0 = a_rows + mrow * row_group, slot = t.x >> 16;
                             const u32 a_prev = a_prv + 8u * (t.x & 0xffffu), a_out = a_cur + 8u * slot, a_cho = a_ch + cell0 + slot;
-                            (void)HAP_CHECK_OK(0, a > b || a_prev >= a_prv + 8u * (u32)(b - a + 1));      // the lowest entry a scan reads
-                            constexpr int J = NL && kTreeJ > 2 ? kTreeJ / 2 : kTreeJ;
-                            if (flat) {
-                                const TreeLevels lv = tree_levels<NL ? 4 : RK>(R, rc_mask, lds_u32(a_rec + kTreeOffThr + 4u * (u32)((d - 1) * HAP_MAX_TYPES + capt)));
+                            (void)HAP_CHECK_OK(0, a > b || a_prev >= a_prv + 8u * (u32)(b - a + 2));      // the lowest entry a scan reads
+                            auto put = [&](int i, double v, int n) {
+                                if (HAP_CHECK_OK(1, slot + i < cl->buf_cells[d & 1])) sts_f64(a_out + 8u * i, n ? v : kTreeInf);
+                                if (HAP_CHECK_OK(2, cell0 + slot + i < cl->ch_bytes)) sts_u8(a_cho + i, (u32)n);
+                                alive |= n != 0;
+                            };
+                            const TreeLevels lv = flat ? tree_levels<NL ? 4 : RK>(R, rc_mask, lds_u32(a_rec + kTreeOffThr + 4u * (u32)((d - 1) * HAP_MAX_TYPES + capt)))
+                                                       : nf_levels(d, capt, j0);          // (one end layer a task)
+                            auto scan = [&](auto width, int h) {
+                                constexpr int J = decltype(width)::value;
+                                double best[J];
+                                int arg[J];
+                                tree_scan<J, RK, F64, NL, COUNT>(ta, a_prev + 8u * h, a_row0, row_stride, j0 + h, cnt - h, a, b, lv, K, best, arg, splits);
 #pragma unroll
-                                for (int h = 0; h < kTreeJ; h += J) {
-                                    if (h && h >= cnt) break;
-                                    double best[J];
-                                    int arg[J];
-                                    tree_scan<J, RK, F64, NL, COUNT>(ta, a_prev + 8u * h, a_row0, row_stride, j0 + h, cnt - h, a, b, lv, K, best, arg, splits);
-#pragma unroll
-                                    for (int i = 0; i < J; ++i)
-                                        if (h + i < cnt) {
-                                            if (HAP_CHECK_OK(1, slot + h + i < cl->buf_cells[d & 1])) sts_f64(a_out + 8u * (h + i), arg[i] ? best[i] : kTreeInf);
-                                            if (HAP_CHECK_OK(2, cell0 + slot + h + i < cl->ch_bytes)) sts_u8(a_cho + h + i, (u32)arg[i]);
-                                            alive |= arg[i] != 0;
-                                        }
-                                }
-                            } else {
-                                for (int i = 0; i < cnt; ++i) {                     // thresholds by end layer
-                                    double best[1];
-                                    int arg[1];
-                                    const TreeLevels lv = nf_levels(d, capt, j0 + i);
-                                    tree_scan<1, RK, F64, NL, COUNT>(ta, a_prev + 8u * i, a_row0, row_stride, j0 + i, 1, a, b, lv, K, best, arg, splits);
-                                    if (HAP_CHECK_OK(1, slot + i < cl->buf_cells[d & 1])) sts_f64(a_out + 8u * i, arg[0] ? best[0] : kTreeInf);
-                                    if (HAP_CHECK_OK(2, cell0 + slot + i < cl->ch_bytes)) sts_u8(a_cho + i, (u32)arg[0]);
-                                    alive |= arg[0] != 0;
-                                }
+                                for (int i = 0; i < J; ++i)
+                                    if (h + i < cnt) put(h + i, best[i], arg[i]);
+                            };
+                            if (t.w == 1u) scan(TreeWidth<1>(), 0);
+                            else if (t.w == 2u) scan(TreeWidth<2>(), 0);
+                            else if (!NL) scan(TreeWidth<kTreeJ>(), 0);
+                            else {                                                  // (a window of two rows a level: two halves)
+                                scan(TreeWidth<kTreeJ / 2>(), 0);
+                                if (cnt > kTreeJ / 2) scan(TreeWidth<kTreeJ / 2>(), kTreeJ / 2);
                             }
                             if (t.y & (1u << 26)) {                                 // the row's padding
 #pragma unroll
@@ -1008,10 +1023,7 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
                                 for (int i = 0; i < kTreePad; ++i) sts_f64(a_out + 8u * (cnt + i), kTreeInf);
                             }
                         }
-                        // the first record of the next depth is requested before this depth is closed
-                        e = e_end + (u32)lane;
-                        e_end = next_end;
-                        if (d + 1 < PP && e < e_end) nxt = __ldg(tasks + e);
+                        lo = hi; hi = next_hi;
                         __syncwarp();
                         if (!__any_sync(0xffffffffu, alive)) { dead = true; break; }      // no cell of this depth is finite: nothing below is
                     }
@@ -1037,7 +1049,7 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
                             const double K = lds_f64(a_rec + kTreeOffKtab + 8u * kidx) + lds_f64(a_rec + kTreeOffMinfo + (mrow * kTreeMinfo + 6) * 8u);
                             const TreeLevels lv = all_flat || cl->flat[PP] ? tree_levels<NL ? 4 : RK>(R, rc_mask, lds_u32(a_rec + kTreeOffThr + 4u * (u32)((PP - 1) * HAP_MAX_TYPES + capt)))
                                                                            : nf_levels(PP, capt, N);
-                            (void)HAP_CHECK_OK(0, (pw & 0xfffffu) >= (u32)(b - a + 1));
+                            (void)HAP_CHECK_OK(0, (pw & 0xfffffu) >= (u32)(b - a + 2));
                             double best[1];
                             int arg[1];
                             tree_scan<1, RK, F64, NL, COUNT>(ta, a_last + 8u * (pw & 0xfffffu), a_rows + mrow * row_group, row_stride, N, 1, a, b, lv, K,

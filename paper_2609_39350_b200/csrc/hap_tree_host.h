@@ -51,7 +51,9 @@ inline size_t tree_record_scratch(const TreeClass &cl, int N, int T) { return (s
 // its 24 mappings at 32 stages (all policies an item): 1 part 527 us, 2 384, 3 351, 4 310, 6 329, 8 324.  Negative: no block fits.
 struct TreeWork { double total = 0, longest = 0, n_conf = 0; size_t slice = 0; u32 rec_bytes = 0; int n_parts = 0, n_sm = 0; };
 constexpr double kTreeIssue = 2.3, kTreeWarpIssue = 0.15, kTreeLive = 0.4, kTreeChain = 0.5;
-constexpr double kTreeIteration = 150.0, kTreePerLength = 42.0, kTreeLeaf = 150.0, kTreePerStage = 100.0;      // warp instructions
+// Warp instructions: of an iteration of tasks of 1, 2 or 4 end layers and of a length in it; of 32 last stages and of a stage
+// on the way back.
+constexpr double kTreeIteration[3] = {70.0, 90.0, 130.0}, kTreePerLength[3] = {15.0, 24.0, 41.0}, kTreeLeaf = 150.0, kTreePerStage = 100.0;
 inline double tree_time(const TreeWork &w)
 {
     const size_t smem = w.rec_bytes + kTreeWarps * w.slice + kTreeSmemFixed;
@@ -295,21 +297,72 @@ private:
         return true;
     }
 
+    // a task before it is laid out: end layers j .. j + cnt - 1 of a node, stage lengths a .. b
+    struct Piece { u32 node; int j, cnt, a, b; };
+
+    // the task of J end layers from j on
+    Piece piece(const Part &pt, int d, u32 ni, int j, int J) const
+    {
+        const Node &nd = pt.lv[d][ni];
+        const int pbl = d > 1 ? pt.lv[d - 1][nd.parent].bl : 0, pbh = d > 1 ? pt.lv[d - 1][nd.parent].bh : 0;
+        Piece q{ni, j, std::min(J, nd.bh - j + 1), std::max((int)nd.nmin, j - pbh), 0};
+        q.b = std::min((int)nd.nmax, j + q.cnt - 1 - pbl);
+        if (q.a > q.b) q.b = q.a - 1;
+        return q;
+    }
+
+    // The tasks of a depth, in the order a warp takes them, 32 an iteration, and the warp instructions they take.  Four end layers
+    // a task are cheapest where the lanes are full: a length's loads, tests and steps serve four splits.  What does not fill
+    // an iteration, often the whole depth, is cut into tasks of two or one, which take a fraction of the instructions on
+    // lanes that would idle.  Longest tasks first, so that an iteration's are alike.  Depths whose thresholds go by end layer take
+    // one each.  Against tasks of four everywhere (20 of 32 lanes active, now 25): a pass at 1,024 devices 390 -> 378 us, 256
+    // devices with partitions 473 -> 439, 64 devices with three levels 150 -> 130, search at 1,024 devices 233 -> 220.
+    double cut(const Part &pt, int d, bool flat, std::vector<Piece> &out) const
+    {
+        auto longer = [](const Piece &x, const Piece &y) { return x.b - x.a > y.b - y.a; };
+        auto cost = [](const std::vector<Piece> &v, size_t from, size_t to, int J) {
+            double t = 0;
+            for (; from < to; from += 32) t += kTreeIteration[J / 2] + kTreePerLength[J / 2] * std::max(1, v[from].b - v[from].a + 1);
+            return t;
+        };
+        out.clear();
+        for (u32 ni = 0; ni < pt.lv[d].size(); ++ni)
+            for (int j = pt.lv[d][ni].bl; j <= pt.lv[d][ni].bh; j += flat ? kTreeJ : 1) out.push_back(piece(pt, d, ni, j, flat ? kTreeJ : 1));
+        std::stable_sort(out.begin(), out.end(), longer);
+        if (!flat) return cost(out, 0, out.size(), 1);
+        const size_t n = out.size(), full = n / 32 * 32;
+        double best = cost(out, 0, n, kTreeJ);
+        std::vector<Piece> tail, keep;
+        size_t head = n;
+        for (size_t h : {full, (size_t)0}) {
+            for (int J : {2, 1}) {
+                if (h == n || (n - h) * (size_t)(kTreeJ / J) > 96) continue;            // (two full iterations more than one: no gain)
+                tail.clear();
+                for (size_t q = h; q < n; ++q)
+                    for (int j = out[q].j; j < out[q].j + out[q].cnt; j += J) {
+                        tail.push_back(piece(pt, d, out[q].node, j, std::min(J, out[q].j + out[q].cnt - j)));
+                    }
+                std::stable_sort(tail.begin(), tail.end(), longer);
+                const double t = cost(out, 0, h, kTreeJ) + cost(tail, 0, tail.size(), J);
+                if (t < best) { best = t; head = h; keep.swap(tail); }
+            }
+            if (full == 0) break;
+        }
+        if (head < n) { out.resize(head); out.insert(out.end(), keep.begin(), keep.end()); }
+        return best;
+    }
+
     // warp instructions of a part, roughly: what the split is chosen by
-    void cost(const Part &pt, double &total, size_t &slice) const
+    void cost(const Part &pt, const TreeClass &cl, double &total, size_t &slice) const
     {
         u32 cells[2] = {0, 0}, ch = 0;
         total = 0;
+        std::vector<Piece> tasks;
         for (int d = 1; d < PP_; ++d) {
-            u32 n_tasks = 0, c = kTreeAhead + kTreePad;
-            int w = 1;
-            for (const Node &nd : pt.lv[d]) {
-                const int b = nd.bh - nd.bl + 1;
-                n_tasks += (u32)((b + kTreeJ - 1) / kTreeJ); c += (u32)b + kTreePad;
-                w = std::max(w, (int)nd.nmax - (int)nd.nmin + 1);
-            }
+            u32 c = kTreeAhead + kTreePad;
+            for (const Node &nd : pt.lv[d]) c += (u32)(nd.bh - nd.bl + 1) + kTreePad;
             cells[d & 1] = std::max(cells[d & 1], c); ch += c;
-            total += (double)((n_tasks + 31) / 32) * (kTreeIteration + kTreePerLength * std::min(w, d == 1 ? kTreeJ : w));
+            total += cut(pt, d, cl.flat[d] != 0, tasks);
         }
         total += (double)((pt.m1 - pt.m0 + 31) / 32) * (kTreeLeaf + kTreePerStage * PP_);
         slice = ((size_t)((cells[0] + 1) / 2 * 2) + (cells[1] + 1) / 2 * 2) * 8 + (ch + 15) / 16 * 16;
@@ -331,7 +384,7 @@ private:
             w.n_conf = (double)in_.n_conf; w.n_sm = in_.n_sm; w.n_parts = (int)np; w.rec_bytes = cl.rec_bytes;
             for (const Part &pt : parts) {
                 double c; size_t s;
-                cost(pt, c, s);
+                cost(pt, cl, c, s);
                 w.total += c; w.longest = std::max(w.longest, c); w.slice = std::max(w.slice, s);
             }
             const double t = tree_time(w);
@@ -339,7 +392,7 @@ private:
             // finer parts share no more prefixes: what they all cost only grows, and a chain has an iteration a depth at least.  A
             // sum of a growing and a falling term has one minimum, but for the rounding to whole warps: half as much again
             // lies behind it
-            const double least = w.total * kTreeLive * w.n_conf / (w.n_sm * kTreeIssue) + kTreeChain * (PP_ - 1) * kTreeIteration / kTreeWarpIssue;
+            const double least = w.total * kTreeLive * w.n_conf / (w.n_sm * kTreeIssue) + kTreeChain * (PP_ - 1) * kTreeIteration[0] / kTreeWarpIssue;
             if (cl.n_parts && (least > best || (t > 1.5 * best && cl.n_parts != (int)np))) break;
         }
         if (!cl.n_parts) return false;                          // no part leaves room for a block
@@ -360,33 +413,32 @@ private:
         const u32 nmap = (u32)(pt.m1 - pt.m0);
         tp.nmap = nmap; tp.m_lo = (u32)pt.m0;
         u32 cells = 0, buf[2] = {0, 0};
-        std::vector<u32> cell_lo(PP_ + 1, 0);
+        std::vector<Piece> pieces;
         for (int d = 1; d < PP_; ++d) {
             tp.task_lo[d] = (u32)ph.tasks.size();
             tp.cell_lo[d] = cells;
             u32 c = kTreeAhead + kTreePad;
-            for (size_t ni = 0; ni < pt.lv[d].size(); ++ni) {
-                const Node &nd = pt.lv[d][ni];
+            for (const Node &nd : pt.lv[d]) c += (u32)(nd.bh - nd.bl + 1) + kTreePad;
+            cut(pt, d, cl.flat[d] != 0, pieces);
+            for (const Piece &q : pieces) {
+                const Node &nd = pt.lv[d][q.node];
                 const Node *pn = d > 1 ? &pt.lv[d - 1][nd.parent] : nullptr;
                 // slot of the parent's entry 0 (before the first stage: one row of layer 0 behind its padding)
-                const int pbl = pn ? pn->bl : 0, pbh = pn ? pn->bh : 0, porg = pn ? (int)pn->rowoff - pn->bl : kTreeAhead + kTreePad;
-                for (int j = nd.bl; j <= nd.bh; j += kTreeJ) {
-                    const int cnt = std::min(kTreeJ, nd.bh - j + 1);
-                    const int a = std::max((int)nd.nmin, j - pbh);
-                    int b = std::min((int)nd.nmax, j + cnt - 1 - pbl);
-                    if (a > b) b = a - 1;
-                    // (no length reaches the parent's row: the origin below only has to be a slot of it)
-                    const int src = a > b ? porg + pbl : porg + j - a, dst = (int)nd.rowoff + j - nd.bl;
-                    if (src < 0 || src > 65535 || dst > 65535) return false;
-                    TreeTask t;
-                    t.x = (u32)src | ((u32)dst << 16);
-                    t.y = (u32)j | ((u32)a << 8) | ((u32)b << 16) | ((u32)(cnt - 1) << 24) | (j == nd.bl ? 1u << 26 : 0u) |
-                          (ni + 1 == pt.lv[d].size() && j + kTreeJ > nd.bh ? 1u << 27 : 0u);
-                    t.z = (u32)kidx(d, nd.mask, nd.link, cl) | ((u32)cl.mrow_of[nd.mask] << 8) | ((u32)capt_[nd.mask] << 16);
-                    t.w = 0;
-                    ph.tasks.push_back(t);
-                }
-                c += (u32)(nd.bh - nd.bl + 1) + kTreePad;
+                const int pbl = pn ? pn->bl : 0, porg = pn ? (int)pn->rowoff - pn->bl : kTreeAhead + kTreePad;
+                // (no length reaches the parent's row: the origin below only has to be a slot of it)
+                const int src = q.a > q.b ? porg + pbl : porg + q.j - q.a, dst = (int)nd.rowoff + q.j - nd.bl;
+                if (src < 0 || src > 65535 || dst > 65535) return false;
+                TreeTask t;
+                t.x = (u32)src | ((u32)dst << 16);
+                t.y = (u32)q.j | ((u32)q.a << 8) | ((u32)q.b << 16) | ((u32)(q.cnt - 1) << 24) | (q.j == nd.bl ? 1u << 26 : 0u) |
+                      (q.node + 1 == pt.lv[d].size() && q.j + q.cnt > nd.bh ? 1u << 27 : 0u);
+                t.z = (u32)kidx(d, nd.mask, nd.link, cl) | ((u32)cl.mrow_of[nd.mask] << 8) | ((u32)capt_[nd.mask] << 16);
+                // tasks of an iteration are of the same number of end layers: that of its largest one
+                const size_t at = ph.tasks.size() - tp.task_lo[d], first = at / 32 * 32;
+                int J = 1;
+                for (size_t x = first; x < std::min(first + 32, pieces.size()); ++x) J = std::max(J, pieces[x].cnt);
+                t.w = (u32)(J > 2 ? 4 : J);
+                ph.tasks.push_back(t);
             }
             buf[d & 1] = std::max(buf[d & 1], c);
             cells += c;

@@ -1,0 +1,30 @@
+"""The tasks a warp takes together: of one width, every cell of a row once, the padding written by the right ones."""
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+@pytest.fixture(scope="session")
+def tasks(tmp_path_factory):
+    exe = str(tmp_path_factory.mktemp("tasks") / "tree_tasks")
+    subprocess.run([os.environ.get("NVCC", "nvcc"), "-gencode", "arch=compute_100a,code=sm_100a", "-std=c++17", "-O1", "-o", exe,
+                    os.path.join(ROOT, "tests", "tree_tasks.cu")], check=True)
+
+    def run(*args):
+        out = subprocess.run([exe, *map(str, args)], check=True, capture_output=True, text=True).stdout
+        return [tuple(map(int, line.split())) for line in out.splitlines()]
+    return run
+
+
+# a part that fills iterations of four end layers and more, rows of one cell, wide windows, mixed layer kinds in front (and past
+# the first depths), one device type, an odd layer count
+@pytest.mark.parametrize("layers,first_moe,delta,nodes,node_size", [(96, 0, 205, "64,32,16,16", 8), (60, 1, 205, "12,8,8,4", 8), (33, 0, 205, "4,4", 8),
+                                                                    (16, 0, -1, "1,1", 4), (255, 0, -1, "8", 8), (12, 5, 300, "3,1", 2), (29, 29, 205, "3,3,1", 8)])
+def test_tasks_cover_the_rows(tasks, layers, first_moe, delta, nodes, node_size):
+    rows = tasks(layers, first_moe, delta, nodes, node_size)
+    assert rows and all(faults == 0 for *_, faults in rows), rows
+    if layers >= 60 and delta > 0:                       # all three widths occur
+        assert all(sum(r[i] for r in rows) > 0 for i in (1, 2, 3)), rows

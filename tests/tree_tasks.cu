@@ -1,0 +1,72 @@
+// Checks the task lists of the prefix trees of a cluster (test_tree_tasks.py; no GPU is needed): prints, per PP class, stages,
+// iterations of 1, 2 and 4 end layers, and the faults found.  Arguments: layers, first MoE layer, window delta, nodes per type,
+// node size.
+#include "../paper_2609_39350_b200/csrc/hap_tree_host.h"
+
+#include <cstdio>
+#include <cstdlib>
+#include <map>
+
+using namespace hap;
+
+int main(int argc, char **argv)
+{
+    if (argc != 6) return 2;
+    const i64 P[4] = {400000, 300000, 250000, 150000}, cap[4] = {80ll << 30, 64ll << 30, 48ll << 30, 32ll << 30};
+    DevConst dc{};
+    dc.N = atoi(argv[1]); dc.kind_uniform_from = atoi(argv[2]); dc.kind_uniform = dc.kind_uniform_from == 0;
+    dc.delta_q = atoi(argv[3]); dc.R = 2; dc.tau_linear = 1;
+    i64 W = 0;
+    for (char *s = strtok(argv[4], ","); s && dc.T < HAP_MAX_TYPES; s = strtok(nullptr, ",")) {
+        const int h = dc.T++;
+        dc.node_size[h] = atoi(argv[5]); dc.m[h] = (i64)atoi(s) * dc.node_size[h]; dc.P[h] = P[h]; dc.cap_eff[h] = cap[h];
+        W += dc.m[h];
+    }
+    for (int PP = 1; PP <= HAP_MAX_PP && PP <= dc.N; PP *= 2) {
+        if (W % PP) continue;
+        hap_pconf q{};
+        q.PP = PP; q.G = (int)(W / PP); q.mode = HAP_MAP_MULTISET; q.nmap = 1;
+        int placed = 0;
+        for (int h = 0; h < dc.T; ++h) {
+            if (dc.m[h] % q.G) q.mode = HAP_MAP_BLOCK;
+            for (int c = 1; c <= dc.m[h] / q.G && q.nmap < (1u << 20); ++c) q.nmap = q.nmap * (u64)++placed / (u64)c;
+        }
+        if (q.nmap > 2048) q.mode = HAP_MAP_BLOCK;
+        if (q.mode == HAP_MAP_BLOCK) { q.nmap = 1; for (int h = 2; h <= dc.T; ++h) q.nmap *= (u64)h; }
+        TreeInputs in{};
+        in.dc = &dc; in.rep = q; in.n_conf = 1000; in.n_sm = 148; in.want_tree = true;
+        TreeClassHost th;
+        TreeBuilder(in).build(th);
+        if (!th.ok) return 3;
+        const TreeClass &c = th.cls;
+        long iters[5] = {0, 0, 0, 0, 0}, faults = 0;
+        for (const TreePartHost &ph : th.parts)
+            for (int d = 1; d < PP; ++d) {
+                // every row (a run of slots between padding) is covered slot by slot, once; its first task writes the padding in
+                // front, one task of the depth that behind the last row
+                std::map<u32, u32> cover;
+                std::vector<u32> first;
+                int last = 0;
+                u32 top = 0;
+                for (u32 e = ph.meta.task_lo[d]; e < ph.meta.task_lo[d + 1]; ++e) {
+                    const TreeTask &t = ph.tasks[e];
+                    const u32 cnt = (t.y >> 24 & 3u) + 1, slot = t.x >> 16;
+                    if ((e - ph.meta.task_lo[d]) % 32 == 0) ++iters[t.w];
+                    else faults += t.w != ph.tasks[e - 1].w;                        // alike in an iteration
+                    faults += !(t.w == 1 || t.w == 2 || t.w == 4) || cnt > t.w || (!c.flat[d] && t.w != 1);
+                    for (u32 i = 0; i < cnt; ++i) faults += ++cover[slot + i] != 1 || slot + i >= c.buf_cells[d & 1];
+                    if (t.y >> 26 & 1u) first.push_back(slot);
+                    if (t.y >> 27 & 1u) { ++last; top = slot + cnt; }
+                }
+                size_t runs = 0;
+                u32 behind = 0;
+                for (const auto &[s, n] : cover) {
+                    if (s != behind) { ++runs; faults += std::find(first.begin(), first.end(), s) == first.end() || (runs > 1 && s - behind != kTreePad); }
+                    behind = s + 1;
+                }
+                faults += first.size() != runs || (runs && (last != 1 || top != behind)) || behind + kTreePad > c.buf_cells[d & 1] + (runs ? 0 : kTreePad);
+            }
+        printf("%d %ld %ld %ld %ld\n", PP, iters[1], iters[2], iters[4], faults);
+    }
+    return 0;
+}
