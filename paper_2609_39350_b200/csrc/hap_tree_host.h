@@ -397,6 +397,7 @@ private:
         }
         if (!cl.n_parts) return false;                          // no part leaves room for a block
         cl.items_per_conf = (cl.n_parts + kTreeWarps - 1) / kTreeWarps;
+        cl.ipc_inverse = cl.items_per_conf > 1 ? (u32)(((1ull << 32) + cl.items_per_conf - 1) / (u64)cl.items_per_conf) : 0u;
         cl.policy_items = 1;
         out.parts.resize((size_t)cl.n_parts);
         for (int q = 0; q < cl.n_parts; ++q) {
@@ -407,44 +408,50 @@ private:
         return true;
     }
 
+    // nothing to do beside t (what the 32 tasks of an iteration share, and addresses that exist)
+    static TreeTask no_task(const TreeTask &t) { return make_uint4(t.x, (t.y & 255u) | 1u << 8, t.z, t.w); }
+
     bool emit(const Part &pt, TreeClass &cl, TreePartHost &ph) const
     {
         TreePart &tp = ph.meta;
         const u32 nmap = (u32)(pt.m1 - pt.m0);
         tp.nmap = nmap; tp.m_lo = (u32)pt.m0;
-        u32 cells = 0, buf[2] = {0, 0};
+        u32 cells = 0, buf[2] = {0, 0}, cell_lo[HAP_MAX_PP + 1] = {0};      // choices of depth d start at cell_lo[d]
         std::vector<Piece> pieces;
         for (int d = 1; d < PP_; ++d) {
-            tp.task_lo[d] = (u32)ph.tasks.size();
-            tp.cell_lo[d] = cells;
+            cell_lo[d] = cells;
+            const size_t first = ph.tasks.size();
             u32 c = kTreeAhead + kTreePad;
             for (const Node &nd : pt.lv[d]) c += (u32)(nd.bh - nd.bl + 1) + kTreePad;
             cut(pt, d, cl.flat[d] != 0, pieces);
-            for (const Piece &q : pieces) {
+            for (size_t at = 0; at < pieces.size(); ++at) {
+                const Piece &q = pieces[at];
                 const Node &nd = pt.lv[d][q.node];
                 const Node *pn = d > 1 ? &pt.lv[d - 1][nd.parent] : nullptr;
                 // slot of the parent's entry 0 (before the first stage: one row of layer 0 behind its padding)
                 const int pbl = pn ? pn->bl : 0, porg = pn ? (int)pn->rowoff - pn->bl : kTreeAhead + kTreePad;
                 // (no length reaches the parent's row: the origin below only has to be a slot of it)
                 const int src = q.a > q.b ? porg + pbl : porg + q.j - q.a, dst = (int)nd.rowoff + q.j - nd.bl;
-                if (src < 0 || src > 65535 || dst > 65535) return false;
+                if (src < 0 || src > 65535 || dst > 65535 || cells + (u32)dst > 65535) return false;
                 TreeTask t;
                 t.x = (u32)src | ((u32)dst << 16);
-                t.y = (u32)q.j | ((u32)q.a << 8) | ((u32)q.b << 16) | ((u32)(q.cnt - 1) << 24) | (q.j == nd.bl ? 1u << 26 : 0u) |
-                      (q.node + 1 == pt.lv[d].size() && q.j + q.cnt > nd.bh ? 1u << 27 : 0u);
-                t.z = (u32)kidx(d, nd.mask, nd.link, cl) | ((u32)cl.mrow_of[nd.mask] << 8) | ((u32)capt_[nd.mask] << 16);
+                t.y = (u32)q.j | ((u32)q.a << 8) | ((u32)q.b << 16) | ((u32)q.cnt << 24) | (q.j == nd.bl ? 1u << 27 : 0u) |
+                      (q.node + 1 == pt.lv[d].size() && q.j + q.cnt > nd.bh ? 1u << 28 : 0u);
+                t.z = (u32)kidx(d, nd.mask, nd.link, cl) | ((u32)cl.mrow_of[nd.mask] << 8) | ((u32)((d - 1) * HAP_MAX_TYPES + capt_[nd.mask]) << 16);
                 // tasks of an iteration are of the same number of end layers: that of its largest one
-                const size_t at = ph.tasks.size() - tp.task_lo[d], first = at / 32 * 32;
+                const size_t it = at / 32 * 32;
                 int J = 1;
-                for (size_t x = first; x < std::min(first + 32, pieces.size()); ++x) J = std::max(J, pieces[x].cnt);
-                t.w = (u32)(J > 2 ? 4 : J);
+                for (size_t x = it; x < std::min(it + 32, pieces.size()); ++x) J = std::max(J, pieces[x].cnt);
+                t.w = (cells + (u32)dst) | (u32)(J > 2 ? 4 : J) << 16 | (it + 32 >= pieces.size() ? kTaskEnds : 0u) | (cl.flat[d] ? 0u : kTaskByLayer);
                 ph.tasks.push_back(t);
             }
+            while ((ph.tasks.size() - first) % 32) ph.tasks.push_back(no_task(ph.tasks.back()));
             buf[d & 1] = std::max(buf[d & 1], c);
             cells += c;
         }
-        for (int d = PP_; d <= HAP_MAX_PP; ++d) { tp.task_lo[d] = (u32)ph.tasks.size(); tp.cell_lo[d] = cells; }
-        if (cells >= (1u << 19)) return false;
+        tp.n_iter = (u32)(ph.tasks.size() / 32);
+        const TreeTask behind = no_task(ph.tasks.empty() ? make_uint4(0, 0, 0, 1u << 16) : ph.tasks.back());
+        ph.tasks.insert(ph.tasks.end(), 32, behind);
         for (int q = 0; q < 2; ++q) cl.buf_cells[q] = std::max(cl.buf_cells[q], (buf[q] + 1) / 2 * 2);
         cl.ch_bytes = std::max(cl.ch_bytes, (cells + 15) / 16 * 16);
         ph.path.assign((size_t)nmap * PP_, 0);
@@ -461,7 +468,7 @@ private:
             for (int d = PP_; d >= 1; --d) {
                 int org = PP_ > 1 ? 0 : kTreeAhead + kTreePad;
                 if (d == PP_) { if (PP_ > 1) { const Node &p = pt.lv[PP_ - 1][nd]; org = (int)p.rowoff - p.bl + N_ - a; } }
-                else { const Node &p = pt.lv[d][nd]; org = (int)tp.cell_lo[d] + (int)p.rowoff - p.bl + 256; nd = p.parent; }
+                else { const Node &p = pt.lv[d][nd]; org = (int)cell_lo[d] + (int)p.rowoff - p.bl + 256; nd = p.parent; }
                 ph.path[(size_t)(d - 1) * nmap + m] = (u32)org | ((u32)kidx(d, mask_[at + d - 1], link_[at + d - 1], cl) << 20) |
                                                       ((u32)cl.mrow_of[mask_[at + d - 1]] << 26) | ((u32)capt_[mask_[at + d - 1]] << 30);
             }

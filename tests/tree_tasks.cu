@@ -40,7 +40,10 @@ int main(int argc, char **argv)
         if (!th.ok) return 3;
         const TreeClass &c = th.cls;
         long iters[5] = {0, 0, 0, 0, 0}, faults = 0;
-        for (const TreePartHost &ph : th.parts)
+        for (const TreePartHost &ph : th.parts) {
+            u32 e = 0, behind_choices = 0;
+            faults += ph.tasks.size() != 32u * (ph.meta.n_iter + 1);                  // the iteration behind the last is there to be asked for
+            for (u32 q = 32 * ph.meta.n_iter; q < ph.tasks.size(); ++q) faults += (ph.tasks[q].y >> 24 & 7u) != 0 || (ph.tasks[q].y >> 8 & 255u) <= (ph.tasks[q].y >> 16 & 255u);
             for (int d = 1; d < PP; ++d) {
                 // every row (a run of slots between padding) is covered slot by slot, once; its first task writes the padding in
                 // front, one task of the depth that behind the last row
@@ -48,16 +51,25 @@ int main(int argc, char **argv)
                 std::vector<u32> first;
                 int last = 0;
                 u32 top = 0;
-                for (u32 e = ph.meta.task_lo[d]; e < ph.meta.task_lo[d + 1]; ++e) {
+                u32 first_choice = ~0u, last_choice = 0;
+                bool ends = false;
+                for (; !ends || e % 32; ++e) {
+                    if (e >= 32 * ph.meta.n_iter) { ++faults; break; }
                     const TreeTask &t = ph.tasks[e];
-                    const u32 cnt = (t.y >> 24 & 3u) + 1, slot = t.x >> 16;
-                    if ((e - ph.meta.task_lo[d]) % 32 == 0) ++iters[t.w];
-                    else faults += t.w != ph.tasks[e - 1].w;                        // alike in an iteration
-                    faults += !(t.w == 1 || t.w == 2 || t.w == 4) || cnt > t.w || (!c.flat[d] && t.w != 1);
+                    const u32 cnt = t.y >> 24 & 7u, slot = t.x >> 16, J = t.w >> 16 & 7u;
+                    ends = t.w & kTaskEnds;
+                    if (e % 32 == 0) ++iters[J];
+                    else faults += t.w >> 16 != ph.tasks[e - 1].w >> 16;            // alike in an iteration
+                    faults += !(J == 1 || J == 2 || J == 4) || cnt > J || (t.w >> 20 & 1u) != !c.flat[d] || (!c.flat[d] && J != 1);
+                    if (cnt == 0) { faults += (t.y >> 27 & 3u) || (t.y >> 8 & 255u) <= (t.y >> 16 & 255u); continue; }      // fills up
+                    faults += (t.z >> 16) / HAP_MAX_TYPES != (u32)d - 1;
+                    first_choice = std::min(first_choice, (t.w & 0xffffu) - slot); last_choice = std::max(last_choice, (t.w & 0xffffu) + cnt);
+                    faults += (t.w & 0xffffu) - slot != first_choice || (t.w & 0xffffu) < behind_choices || (t.w & 0xffffu) + cnt > c.ch_bytes;
                     for (u32 i = 0; i < cnt; ++i) faults += ++cover[slot + i] != 1 || slot + i >= c.buf_cells[d & 1];
-                    if (t.y >> 26 & 1u) first.push_back(slot);
-                    if (t.y >> 27 & 1u) { ++last; top = slot + cnt; }
+                    if (t.y >> 27 & 1u) first.push_back(slot);
+                    if (t.y >> 28 & 1u) { ++last; top = slot + cnt; }
                 }
+                behind_choices = last_choice;
                 size_t runs = 0;
                 u32 behind = 0;
                 for (const auto &[s, n] : cover) {
@@ -66,6 +78,8 @@ int main(int argc, char **argv)
                 }
                 faults += first.size() != runs || (runs && (last != 1 || top != behind)) || behind + kTreePad > c.buf_cells[d & 1] + (runs ? 0 : kTreePad);
             }
+            faults += e != 32 * ph.meta.n_iter;
+        }
         printf("%d %ld %ld %ld %ld\n", PP, iters[1], iters[2], iters[4], faults);
     }
     return 0;
