@@ -1429,7 +1429,7 @@ static cudaError_t launch_dependent(const void *fn, unsigned grid, unsigned thre
 }
 
 // One launch of the tree kernel: classes [c_lo, c_hi) of the image.
-struct TreeLaunch { int c_lo, c_hi; size_t smem; unsigned grid; u64 items; };
+struct TreeLaunch { int c_lo, c_hi; size_t smem; unsigned grid; u64 items; int blocks; };
 
 // A pass runs the deep pipelines (long chains of small depths) and the others in launches of their own, deep ones first:
 // the blocks of each take the shared memory their own classes need.  From 16 stages on, measured against one launch and a line at
@@ -1441,7 +1441,7 @@ static std::vector<TreeLaunch> tree_launches(const hap_problem *p, bool search, 
     const auto &cls = p->image->cls;
     std::vector<TreeLaunch> ls;
     auto group = [&](int c_lo, int c_hi) {
-        TreeLaunch l{c_lo, c_hi, 0, 0, 0};
+        TreeLaunch l{c_lo, c_hi, 0, 0, 0, kTreeBlocksPerSm};
         for (int c = c_lo; c < c_hi; ++c) {
             const TreeClass &cl = cls[(size_t)c];
             const unsigned a = std::max(p_lo, cl.p_lo), b = std::min(p_hi, cl.p_lo + cl.n_conf);
@@ -1450,7 +1450,8 @@ static std::vector<TreeLaunch> tree_launches(const hap_problem *p, bool search, 
             l.smem = std::max(l.smem, tree_smem_bytes(cl));
         }
         if (!l.items) return;
-        const unsigned per_sm = (unsigned)std::max<size_t>(1, std::min<size_t>(kTreeBlocksPerSm, kSmemPerSm / (l.smem + kTreeSmemStatic)));
+        if (search && p->dc.tau_linear && kTreeLive * (double)l.items > 2.0 * kTreeBlocksPerSm * sm_count(p->device)) l.blocks = kTreeSearchBlocksPerSm;
+        const unsigned per_sm = (unsigned)std::max<size_t>(1, std::min<size_t>((size_t)l.blocks, kSmemPerSm / (l.smem + kTreeSmemStatic)));
         l.grid = (unsigned)std::min<u64>(l.items, std::min<u64>((u64)sm_count(p->device) * per_sm, kTreeSlots / 2));
         ls.push_back(l);
     };
@@ -1516,18 +1517,24 @@ static hap_status launch_trees(hap_problem *p, const DpOut &out_in, bool search,
     const int form = nl ? 2 : p->prof.R > 2 ? 1 : 0;
     using Fn = void (*)(const TreeArgs, const DevConst, DpOut);
     constexpr int kP = kTreePass, kS = kTreeSearch, kL = kTreeList;
-    static const Fn fns[6][3] = {
+    constexpr int kB = kTreeSearchBlocksPerSm;
+    static const Fn fns[9][3] = {
         {tree_dp_kernel<kP, false, 2, false, false>, tree_dp_kernel<kP, false, 4, false, false>, tree_dp_kernel<kP, false, 4, true, false>},
         {tree_dp_kernel<kS, false, 2, false, false>, tree_dp_kernel<kS, false, 4, false, false>, tree_dp_kernel<kS, false, 4, true, false>},
         {tree_dp_kernel<kP, true, 2, false, false>, tree_dp_kernel<kP, true, 4, false, false>, tree_dp_kernel<kP, true, 4, true, false>},
         {tree_dp_kernel<kS, true, 2, false, false>, tree_dp_kernel<kS, true, 4, false, false>, tree_dp_kernel<kS, true, 4, true, false>},
         {tree_dp_kernel<kP, false, 2, false, true>, tree_dp_kernel<kP, false, 4, false, true>, tree_dp_kernel<kP, false, 4, true, true>},
-        {tree_dp_kernel<kL, false, 2, false, false>, tree_dp_kernel<kL, false, 4, false, false>, tree_dp_kernel<kL, false, 4, true, false>}};
-    const void *fn = (const void *)fns[refine ? 5 : counting ? 4 : (f64 ? 2 : 0) + (search ? 1 : 0)][form];
+        {tree_dp_kernel<kL, false, 2, false, false>, tree_dp_kernel<kL, false, 4, false, false>, tree_dp_kernel<kL, false, 4, true, false>},
+        // four blocks an SM: search, fp64 search, listing
+        {tree_dp_kernel<kS, false, 2, false, false, kB>, tree_dp_kernel<kS, false, 4, false, false, kB>, nullptr},
+        {tree_dp_kernel<kS, true, 2, false, false, kB>, tree_dp_kernel<kS, true, 4, false, false, kB>, nullptr},
+        {tree_dp_kernel<kL, false, 2, false, false, kB>, tree_dp_kernel<kL, false, 4, false, false, kB>, nullptr}};
+    const int mode = refine ? 5 : counting ? 4 : (f64 ? 2 : 0) + (search ? 1 : 0);
     int n = 0;
     for (const auto &l : ls) {
         ta.c_lo = l.c_lo; ta.c_hi = l.c_hi; ta.launch = n;
         ta.slot_lo = n == 0 ? 0 : ls[0].grid;
+        const void *fn = (const void *)fns[l.blocks == kTreeBlocksPerSm ? mode : refine ? 8 : f64 ? 7 : 6][form];
         CUDA_TRY(p, raise_smem_limit(p->device, fn, l.smem));
         void *args[] = {(void *)&ta, (void *)&p->dc, (void *)&out};
         CUDA_TRY(p, launch_dependent(fn, l.grid, kTreeThreads, l.smem, st, args));

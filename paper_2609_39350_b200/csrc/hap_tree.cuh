@@ -40,7 +40,12 @@ namespace hap {
 
 constexpr int kTreeWarps = 4;             // warps of a DP block
 constexpr int kTreeThreads = kTreeWarps * 32;
-constexpr int kTreeBlocksPerSm = 5;       // (96 registers a thread)
+// Blocks an SM: five (96 registers a thread), or four (128) for searches of several waves of items, whose last chains run faster beside
+// fewer warps and with what a plan takes in registers: pruned search at 1,024 devices 195 us against 214, its unpruned plan from host
+// tables 440 against 455, exact search at 256 devices 248 against 262.  Where the feasible items are two waves at most, every chain
+// begins at once or nearly so: 64 devices 130 us against 135.  A pass is bound by the issue slots (256 devices 419 against 424, 1,024
+// devices 359 against 352), and rows that are not combined by level need no more than 96 registers (126 against 139).
+constexpr int kTreeBlocksPerSm = 5, kTreeSearchBlocksPerSm = 4;
 constexpr int kTreeJ = 4;                 // end layers of a task at most
 template <int J> struct TreeWidth { static constexpr int value = J; };
 constexpr int kTreePad = kTreeJ - 1;      // infinite entries in front of every row and behind the last one
@@ -821,8 +826,8 @@ __device__ __forceinline__ void tree_finish(const TreeArgs &ta, const DevConst &
     __threadfence_system();
 }
 
-template <int MODE, bool F64, int RK, bool NL, bool COUNT>
-__global__ void __launch_bounds__(kTreeThreads, kTreeBlocksPerSm)
+template <int MODE, bool F64, int RK, bool NL, bool COUNT, int BLOCKS = kTreeBlocksPerSm>
+__global__ void __launch_bounds__(kTreeThreads, BLOCKS)
 tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
 {
     constexpr bool SEARCH = MODE != kTreePass, LIST = MODE == kTreeList;
