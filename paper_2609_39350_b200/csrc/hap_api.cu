@@ -117,7 +117,7 @@ struct hap_problem {
     int joint_grid = 0;
     // ... in the form of a search over reachable end layers: by 64-bit words per state
     struct ReachHost { std::vector<JointReach> classes; std::vector<unsigned> ids; unsigned char *d = nullptr; size_t o_ids = 0, smem = 0; };
-    ReachHost reach[2];
+    ReachHost reach[kReachWords];
     bool joint_ready = false;
     TreeResult *host_result = nullptr;     // page-locked, mapped: the last block of a search writes the plan here
     int timed = 0;                         // 1: events around the last pass, 2: the tree kernels' own time stamps
@@ -1833,7 +1833,13 @@ static bool joint_reach_class(const hap_problem *p, int PP, int64_t G, const Joi
         }
         jr.base[i] = top < 0 ? (i ? jr.base[i - 1] : 0) : base;
         jr.width[i] = top < 0 ? 0 : top - base + 1;
-        if (i >= 1 && i < PP && top >= 0) words = std::max(words, (top - base + 64) / 64);
+        if (i >= 1 && i < PP && top >= 0) {
+            if (top - base + 1 > 128) return false;
+            // a level's lengths are summed up from the shortest one's place and moved down from there where the level begins higher
+            int down = 0;
+            for (int h = 0; h < T && i >= 2; ++h) if (jc.cnt[h] > 0) down = std::max(down, jr.base[i] - jr.base[i - 1] - jr.nmin[h]);
+            words = std::max(words, (jr.width[i] + down + 63) / 64);
+        }
         jr.ent_off[i] = (unsigned)ent.size();
         if (i == 1)
             for (int h = 0; h < T; ++h) jr.first[h] = jc.cnt[h] > 0 ? (unsigned)slot[jc.stride[h]] : 0u;
@@ -1852,9 +1858,9 @@ static bool joint_reach_class(const hap_problem *p, int PP, int64_t G, const Joi
                 ent.push_back(e);
             }
     }
-    if (words > 2) return false;
+    if (words > kReachWords) return false;
     jr.words = words;
-    return reach_smem(N, T, p->prof.R, p->dc.tau_linear ? p->prof.R : 2, PP, jc.lmax, jr.nwin, words).total <= 110 * 1024;
+    return reach_smem(N, T, p->prof.R, p->dc.tau_linear ? p->prof.R : 2, PP, jc.lmax, jr.nwin, words).total <= (words > 2 ? 140 : 110) * 1024;
 }
 
 static hap_status joint_setup(hap_problem *p)
@@ -1865,7 +1871,7 @@ static hap_status joint_setup(hap_problem *p)
     std::vector<int> pps;
     for (const auto &r : p->pconfs) if (std::find(pps.begin(), pps.end(), r.PP) == pps.end()) pps.push_back(r.PP);
     std::sort(pps.begin(), pps.end(), std::greater<int>());      // the longest configurations start first
-    std::vector<unsigned> ent[2];
+    std::vector<unsigned> ent[kReachWords];
     // Where every class has few cells (states x types x layers) the value form is faster, whose chain is a level each where a
     // search is a dozen tests of it (64 devices, 32 layers, at most 18,496 cells: 297 us against 488; 32 devices, 24 layers, 16,200:
     // 208 against 340).  One class of many makes the search worth it (16 stages at 1,024 devices, 32,400 cells: 666 us against
@@ -1943,7 +1949,7 @@ static hap_status joint_setup(hap_problem *p)
         if (jh.smem > 227 * 1024) return fail(p, HAP_E_RANGE, "shared memory need of the joint recurrence exceeds the SM");
         p->joint.push_back(jh);
     }
-    for (int w = 0; w < 2; ++w) {
+    for (int w = 0; w < kReachWords; ++w) {
         // classes | ids | entries
         hap_problem::ReachHost &rh = p->reach[w];
         if (rh.classes.empty()) continue;
@@ -1978,11 +1984,12 @@ extern "C" hap_status hap_joint_bottleneck(hap_problem *p, int64_t *dev_out, voi
     CUDA_TRY(p, cudaMemsetAsync(dev_out, 0xff, np * p->opts.n_rc * sizeof(int64_t), st));     // -1: stages not homogeneous
     if ((s = launch_layer_costs(p, p->d_c2, p->d_coef, nullptr, nullptr, true, st)) != HAP_OK) return s;
     const bool lin = p->dc.tau_linear != 0;
-    for (int w = 0; w < 2; ++w) {
+    for (int w = 0; w < kReachWords; ++w) {
         const hap_problem::ReachHost &rh = p->reach[w];
         if (rh.classes.empty()) continue;
         using Fn = void (*)(const DevConst, const JointReach *, int, const unsigned *, const i64 *, const i64 *, i64 *);
-        static const Fn fns[2][2] = {{joint_reach_kernel<false, 1>, joint_reach_kernel<false, 2>}, {joint_reach_kernel<true, 1>, joint_reach_kernel<true, 2>}};
+        static const Fn fns[2][kReachWords] = {{joint_reach_kernel<false, 1>, joint_reach_kernel<false, 2>, joint_reach_kernel<false, 3>},
+                                               {joint_reach_kernel<true, 1>, joint_reach_kernel<true, 2>, joint_reach_kernel<true, 3>}};
         const Fn fn = fns[lin][w];
         CUDA_TRY(p, raise_smem_limit(p->device, (const void *)fn, rh.smem));
         fn<<<(unsigned)rh.ids.size(), kReachThreads, rh.smem, st>>>(p->dc, reinterpret_cast<const JointReach *>(rh.d), (int)rh.classes.size(),

@@ -6,19 +6,24 @@
 //     reach[u][t] = OR over stage lengths n, OR over types t' of the stage before,
 //                   (reach[u - e_t][t'] AND ok[t][t'][n]) << n
 // where bit k of ok says that layers (k, k + n] on type t cost at most B behind a stage of type t' and fit the memory of
-// this depth.  All bits of a state sit in one or two 64-bit words (bits count from the smallest end layer of the level), so
+// this depth.  All bits of a state sit in one to three 64-bit words (bits count from the smallest end layer of the level), so
 // a level of every state takes a few logic instructions per (type, type before, length) and both levels of the recurrence
 // stay in shared memory.  The stage costs are finitely many numbers: after a test, B moves to the nearest of them, so the
-// bisection ends after about a dozen tests, each exact.
+// bisection ends after about a dozen tests, each exact.  It starts at a guess: the B at which stages of mean cost would add up
+// to all layers (capacity); the answer lies within 2 % of it for half of the configurations, within 30 % for nine in ten.
 //
-// Lengths whose masks are full or empty at a depth (most, once B is near the answer) need no mask at all.
+// Lengths whose masks are full at a depth (most, once B is near the answer) need no mask at all.
 //
 // 1,024 devices, 3,114 homogeneous configurations of up to 3,825 states: 38.4 ms with a value per end layer in global memory,
-// 2.9 ms in this form.  128 threads a block: 3.6 ms, 192: 3.2 ms (few configurations are feasible, and each is a chain of
-// levels and tests); a lane for all next types of a state instead of one: 4.4 ms.
+// 2.83 ms in this form, 2.17 ms since the tests start at the guess instead of a lower bound (12 tests a feasible configuration
+// instead of 16 to 18), lengths are summed up in one direction and transfers that cannot occur are left out.  Five blocks an SM
+// instead of four (48 registers a thread, spilled): 2.36 ms.  128 threads a block: 3.6 ms, 192: 3.2 ms against 2.83 (few
+// configurations are feasible, and each is a chain of levels and tests); a lane for all next types of a state instead of one: 4.4 ms.
+// Measured on other tables, where this form took 2.40 ms: a warp that keeps to one type 2.50 (types of long stages hold up the
+// others); first a search with the least transfer of each type, whose states need no type before, 2.72 (its tests cost as much).
 //
 // One block per configuration.  Bound by instruction issue of the level loop: per (state, type) four logic operations per
-// (type before, length).  The value form -- a 64-bit minimum per end layer and split, rows in
+// (type before, length), and by the barrier of each level.  The value form -- a 64-bit minimum per end layer and split, rows in
 // global memory -- is kept for classes whose bits or masks do not fit (joint_dp_kernel).
 #pragma once
 #include "hap_device.cuh"
@@ -26,6 +31,7 @@
 namespace hap {
 
 constexpr int kReachThreads = 256;
+constexpr int kReachWords = 3;                    // 64-bit words of a state at most
 constexpr int kReachKc = 2 + HAP_MAX_TYPES;       // transfer into a stage: same type intra / inter node, from type 0..3
 constexpr int kReachOk = 2 * HAP_MAX_TYPES;       // masks of a (depth, type, length): [same-type link][type before]
 
@@ -48,24 +54,24 @@ template <int W>
 __device__ __forceinline__ Bits<W> bits_shift(const Bits<W> &x, int s)      // by s towards higher end layers (s < 0: lower)
 {
     Bits<W> y;
-    if (W == 1) y.w[0] = s >= 0 ? (s < 64 ? x.w[0] << s : 0) : (s > -64 ? x.w[0] >> -s : 0);
-    else {
-        const u64 lo = x.w[0], hi = x.w[W - 1];
-        if (s >= 0) {
-            y.w[0] = s < 64 ? lo << s : 0;
-            y.w[W - 1] = s == 0 ? hi : s < 64 ? (hi << s) | (lo >> (64 - s)) : s < 128 ? lo << (s - 64) : 0;
-        } else {
-            const int r = -s;
-            y.w[W - 1] = r < 64 ? hi >> r : 0;
-            y.w[0] = r < 64 ? (lo >> r) | (hi << (64 - r)) : r < 128 ? hi >> (r - 64) : 0;
+    if (W == 1) { y.w[0] = s >= 0 ? (s < 64 ? x.w[0] << s : 0) : (s > -64 ? x.w[0] >> -s : 0); return y; }
+    const int r = s >= 0 ? s : -s, words = r >> 6, b = r & 63;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        u64 near = 0, far = 0;                                  // the words that a word takes its bits from
+#pragma unroll
+        for (int v = 0; v < W; ++v) {
+            if (v == (s >= 0 ? w - words : w + words)) near = x.w[v];
+            if (v == (s >= 0 ? w - words - 1 : w + words + 1)) far = x.w[v];
         }
+        y.w[w] = s >= 0 ? (b ? near << b | far >> (64 - b) : near) : (b ? near >> b | far << (64 - b) : near);
     }
     return y;
 }
 
 __host__ __device__ inline int reach_mask_words(int N) { return (N + 31) / 32; }
 
-struct ReachSmem { u32 rows, wa, sk, m, a, reach, span, least, lvl, fin, total; };
+struct ReachSmem { u32 rows, wa, sk, m, a, reach, span, least, mean, lvl, fin, total; };
 __host__ __device__ inline ReachSmem reach_smem(int N, int T, int R, int RW, int PP, int lmax, int nwin, int words)
 {
     auto up = [](size_t v) { return (u32)((v + 15) / 16 * 16); };
@@ -80,6 +86,7 @@ __host__ __device__ inline ReachSmem reach_smem(int N, int T, int R, int RW, int
     s.m = (u32)o; o = up(o + (size_t)T * nwin * R * kReachKc * reach_mask_words(N) * 4);
     s.span = (u32)o; o = up(o + (size_t)T * nwin * R * 16);
     s.least = (u32)o; o = up(o + (size_t)T * nwin * R * 8);
+    s.mean = (u32)o; o = up(o + (size_t)T * nwin * R * 8);
     s.fin = (u32)o; o = up(o + (size_t)T * nwin * 4);
     s.lvl = (u32)o; o = up(o + (size_t)PP * T * nwin);
     s.total = (u32)(o > 0xffffffffull ? 0xffffffffull : o);
@@ -96,11 +103,13 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
     __shared__ i64 sP2P[HAP_MAX_TYPES][6];
     __shared__ i64 szero[1];
     __shared__ u64 s_dn, s_up;                              // bounds that a test leaves: next stage costs around B
-    __shared__ u64 s_low;
+    __shared__ int s_enough[kReachThreads / 32];
+    __shared__ Bits<W> s_level[HAP_MAX_PP + 1];             // all end layers of a level
     __shared__ i64 s_res[HAP_MAX_RC_MASKS];
     __shared__ int s_end[3][HAP_MAX_TYPES], s_full[3][HAP_MAX_TYPES];      // by depth % 3 and type: lengths from s_end on have empty
                                                             // masks, those before s_full have full ones
     __shared__ i64 s_k2[HAP_MAX_TYPES][2], s_kmin[HAP_MAX_TYPES];
+    __shared__ u32 s_via[HAP_MAX_TYPES];                    // transfers that can occur into a stage of the type, a bit each
     __shared__ u32 s_used[HAP_MAX_TYPES];                   // per type: levels of stages between the first and the last
     const int tid = threadIdx.x, wib = tid >> 5, lane = tid & 31;
     constexpr int nwarps = kReachThreads / 32;
@@ -126,6 +135,7 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
     u32 *sM = reinterpret_cast<u32 *>(smem_raw + lay.m);              // [type][length][level][transfer][word]: bit k: (k, k + n] costs at most B
     longlong2 *sSpan = reinterpret_cast<longlong2 *>(smem_raw + lay.span);    // [type][length][level]: least and most that n layers cost
     i64 *sLeast = reinterpret_cast<i64 *>(smem_raw + lay.least);              // ... least, first and last stages included
+    i64 *sMean = reinterpret_cast<i64 *>(smem_raw + lay.mean);                // ... mean
     u32 *sFin = reinterpret_cast<u32 *>(smem_raw + lay.fin);          // [type][length]: transfers under which the last stage costs at most B
     dp_prologue_rows<i64, LINEAR>(dc, p, c2, coef, coef, true, T, RW, 0xffffffffu, nwarps, sR, sW, sA, sK, minfo, sP2P, szero);
     for (int e = tid; e < 2 * HAP_MAX_TYPES * lmax; e += kReachThreads)             // (types that do not exist stay empty)
@@ -141,10 +151,11 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
     };
     for (int g = wib; g < T * nwin * R; g += nwarps) {
         const int r = g % R, q = (g / R) % nwin, t = g / (R * nwin), n = jc.nmin[t] + q;
-        i64 a = kInf, b = -1, any = kInf;                     // of the stages between the first and the last; of all
+        i64 a = kInf, b = -1, any = kInf, sum = 0;            // of the stages between the first and the last; of all
         for (int k = lane; k + n <= N; k += 32) {
             const i64 c = cost(t, r, k, k + n);
             any = c < any ? c : any;
+            sum += c;
             if (k > 0 && k + n < N) { a = c < a ? c : a; b = c > b ? c : b; }
         }
 #pragma unroll
@@ -154,17 +165,26 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
             const i64 z = __shfl_xor_sync(0xffffffffu, any, o);
             any = z < any ? z : any;
         }
-        if (lane == 0) { sSpan[g] = make_longlong2(a, b); sLeast[g] = any; }
+        sum = warp_sum_i64(sum);
+        if (lane == 0) { sSpan[g] = make_longlong2(a, b); sLeast[g] = any; sMean[g] = n <= N ? sum / (N - n + 1) : kInf; }
     }
     __syncthreads();
+    if (tid <= PP)
+#pragma unroll
+        for (int w = 0; w < W; ++w) { const int n = jc.width[tid] - 64 * w; s_level[tid].w[w] = n >= 64 ? ~0ull : n > 0 ? (1ull << n) - 1ull : 0ull; }
     // least and most of the transfers into a stage of a type 
     i64 *sK2 = &s_k2[0][0];
     if (tid < T) {                                            // (a type on its own with one stage has none)
-        i64 a = kInf, b = 0;
-        for (int e = 0; e < kReachKc; ++e) {
-            const int from = e < 2 ? tid : e - 2;
-            if (from < T && jc.cnt[from] > 0) { const i64 v = sP2P[tid][e]; a = v < a ? v : a; b = v > b ? v : b; }
+        u32 via = 0;
+        for (int h = 0; h < T; ++h) if (h != tid && jc.cnt[h] > 0) via |= 4u << h;
+        for (int q = 1; q < jc.cnt[tid]; ++q) {
+            const i64 first = (i64)q * pc.G;
+            via |= (first - 1) / dc.node_size[tid] == first / dc.node_size[tid] ? 1u : 2u;
         }
+        s_via[tid] = via;
+        i64 a = kInf, b = 0;
+        for (int e = 0; e < kReachKc; ++e)
+            if ((via >> e) & 1u) { const i64 v = sP2P[tid][e]; a = v < a ? v : a; b = v > b ? v : b; }
         sK2[2 * tid] = a; sK2[2 * tid + 1] = b;
         const i64 pre = minfo[(1 << tid) - 1].kpre;
         s_kmin[tid] = pre < a ? pre : a;
@@ -228,10 +248,10 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
                             // all of them or none: most lengths, once B is near the answer
                             see(most <= B ? most : least);
                             for (int e = lane; e < kReachKc * mw; e += 32) {
-                                const int f = e / mw, w = e - f * mw, from = f < 2 ? t : f - 2;
+                                const int f = e / mw, w = e - f * mw;
                                 // bits 1 .. N - n - 1
                                 const int top = N - n - w * 32;
-                                u32 v = most > B || from >= T || jc.cnt[from] == 0 || top <= 0 ? 0u : top >= 32 ? ~0u : (1u << top) - 1u;
+                                u32 v = most > B || !((s_via[t] >> f) & 1u) || top <= 0 ? 0u : top >= 32 ? ~0u : (1u << top) - 1u;
                                 if (w == 0) v &= ~1u;
                                 sM[(size_t)g * kReachKc * mw + e] = v;
                             }
@@ -239,6 +259,7 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
                         }
                         see(B + 1 - 4294967296ll);                            // (costs further away than that are not looked at)
                         up = B + 4294967296ll < up ? B + 4294967296ll : up;
+                        const u32 via = s_via[t];
                         for (int w = 0; w < mw; ++w) {
                             const int k = w * 32 + lane;
                             const bool in = k >= 1 && k + n < N;              // a stage that is neither the first nor the last
@@ -246,8 +267,7 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
                             u32 mine = 0;
 #pragma unroll
                             for (int e = 0; e < kReachKc; ++e) {
-                                const int from = e < 2 ? t : e - 2;
-                                if (from >= T || jc.cnt[from] == 0) continue;
+                                if (!((via >> e) & 1u)) continue;
                                 const i64 x = c + sP2P[t][e];
                                 const int hi = (int)(x >> 32);
                                 const u32 lw = (u32)x;
@@ -268,7 +288,7 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
                             if (lv != 255) {
                                 const i64 c = cost(t, lv, N - n, N) + minfo[(1 << t) - 1].kpost;
                                 for (int f = 0; f < 2 + T; ++f)
-                                    if (see(c + sP2P[t][f])) okl |= 1u << f;
+                                    if (((s_via[t] >> f) & 1u) && see(c + sP2P[t][f])) okl |= 1u << f;
                             }
                             const int l1 = sLvl[(size_t)t * nwin + q];
                             if (l1 != 255 && see(cost(t, l1, 0, n) + minfo[(1 << t) - 1].kpre)) okl |= 1u << 16;
@@ -286,15 +306,9 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
                     if (lane == 0) { atomicMax(&s_dn, (u64)dn); atomicMin(&s_up, (u64)up); }
                     __syncthreads();
                     // masks of a depth: the words of the level that its memory allows, from the first end layer of the level before
-                    auto level_mask = [&](int i) {
-                        Bits<W> b;
-#pragma unroll
-                        for (int w = 0; w < W; ++w) { const int n = jc.width[i] - 64 * w; b.w[w] = n >= 64 ? ~0ull : n > 0 ? (1ull << n) - 1ull : 0ull; }
-                        return b;
-                    };
-                    auto masks_of = [&](int i) {
+                    auto masks_of = [&](int i, int turn) {
                         const int at = jc.base[i - 1], w0 = at >> 5, s = at & 31;
-                        const Bits<W> all = level_mask(i - 1);
+                        const Bits<W> all = s_level[i - 1];
                         const int per_t = (nwin * kReachOk + 31) & ~31;
                         for (int e0 = wib * 32; e0 < T * per_t; e0 += kReachThreads) {          // (a warp stays inside one type)
                             const int t = e0 / per_t, e = e0 - t * per_t + lane;
@@ -302,7 +316,7 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
                             Bits<W> b;
 #pragma unroll
                             for (int w = 0; w < W; ++w) b.w[w] = 0;
-                            const bool in = q < nwin, there = in && jc.cnt[t] > 0 && h < T && jc.cnt[h] > 0;
+                            const bool in = q < nwin, there = in && jc.cnt[t] > 0 && ((s_via[t] >> f) & 1u);
                             const int lv = there ? sLvl[((size_t)(i - 1) * T + t) * nwin + q] : 255;
                             if (lv != 255) {
                                 const u32 *m = sM + ((size_t)((t * nwin + q) * R + lv) * kReachKc + f) * mw;
@@ -320,15 +334,15 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
                             if (in) {
                                 sOk[(size_t)((i & 1) * T + t) * nwin * kReachOk + e] = b;
                                 if ((lane & (kReachOk - 1)) == 0) {
-                                    if ((some >> lane) & 0xffu) atomicMax(&s_end[i % 3][t], q + 1);
-                                    if ((not_full >> lane) & 0xffu) atomicMin(&s_full[i % 3][t], q);
+                                    if ((some >> lane) & 0xffu) atomicMax(&s_end[turn][t], q + 1);
+                                    if ((not_full >> lane) & 0xffu) atomicMin(&s_full[turn][t], q);
                                 }
                             }
                         }
                     };
                     if (tid < 3 * HAP_MAX_TYPES) { s_end[tid / HAP_MAX_TYPES][tid % HAP_MAX_TYPES] = 0; s_full[tid / HAP_MAX_TYPES][tid % HAP_MAX_TYPES] = nwin; }
                     __syncthreads();
-                    if (PP > 2) masks_of(2);
+                    if (PP > 2) masks_of(2, 2);
                     // level 1
                     for (unsigned e = (unsigned)tid; e < jc.n_states[1] * (unsigned)T; e += kReachThreads) {
                         const unsigned t = e / jc.n_states[1], sl = e - t * jc.n_states[1];
@@ -344,17 +358,25 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
                         sReach[(size_t)t * lmax + sl] = b;
                     }
                     __syncthreads();
-                    for (int i = 2; i < PP; ++i) {
+                    for (int i = 2, turn = 2; i < PP; ++i, turn = turn == 2 ? 0 : turn + 1) {       // turn: i % 3
                         const Bits<W> *prv = sReach + (size_t)(i & 1 ? HAP_MAX_TYPES * lmax : 0);          // level 1 lies in the first buffer
                         Bits<W> *cur = sReach + (size_t)(i & 1 ? 0 : HAP_MAX_TYPES * lmax);
                         const unsigned ns = jc.n_states[i], total = ns * (unsigned)T;
                         const unsigned *ent = jc.ent + jc.ent_off[i];
                         const int d = jc.base[i] - jc.base[i - 1];
                         const Bits<W> *okd = sOk + (size_t)(i & 1) * T * nwin * kReachOk;
-                        const Bits<W> lm = level_mask(i);
-                        if (i + 1 < PP) masks_of(i + 1);
-                        if (tid < HAP_MAX_TYPES) { s_end[(i + 2) % 3][tid] = 0; s_full[(i + 2) % 3][tid] = nwin; }
+                        const Bits<W> lm = s_level[i];
+                        const int turn_next = turn == 2 ? 0 : turn + 1, turn_free = 3 - turn - turn_next;
+                        if (i + 1 < PP) masks_of(i + 1, turn_next);
+                        if (tid < HAP_MAX_TYPES) { s_end[turn_free][tid] = 0; s_full[turn_free][tid] = nwin; }
                         int some = 0;
+                        // lengths are gathered by Horner's rule from the longest on, one position a step; a bit that leaves the words at
+                        // the top lies outside the level (joint_reach_class); those before nf are all alike
+                        auto step_up = [&](Bits<W> &acc, const Bits<W> &x) {
+#pragma unroll
+                            for (int w = W - 1; w > 0; --w) acc.w[w] = acc.w[w] << 1 | acc.w[w - 1] >> 63 | x.w[w];
+                            acc.w[0] = acc.w[0] << 1 | x.w[0];
+                        };
                         for (unsigned e = (unsigned)tid; e < total; e += kReachThreads) {
                             const unsigned en = __ldg(ent + e), up_sl = en & 0xffffu;
                             const int t = (int)(en >> 16) & 3, cls = (int)(en >> 18) & 1;
@@ -373,43 +395,19 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
                                     none = none && any.w[w] == 0;
                                 }
                                 if (!none) {
-                                    // lengths are gathered by Horner's rule: the ones that move a bit down from the shortest on,
-                                    // the others from the longest on, one position a step
                                     const Bits<W> *ok = okd + (size_t)t * nwin * kReachOk + cls * HAP_MAX_TYPES;
-                                    const int lo = jc.nmin[t] - d, nl = s_end[i % 3][t], nf = s_full[i % 3][t], q0 = lo < 0 ? -lo : 0;
-                                    auto gather = [&](int q) {
+                                    const int nf = s_full[turn][t];
+                                    int q = s_end[turn][t] - 1;
+                                    for (; q >= nf; --q) {
                                         const Bits<W> *o = ok + q * kReachOk;
                                         Bits<W> x;
 #pragma unroll
                                         for (int w = 0; w < W; ++w)
                                             x.w[w] = (from[0].w[w] & o[0].w[w]) | (from[1].w[w] & o[1].w[w]) | (from[2].w[w] & o[2].w[w]) | (from[3].w[w] & o[3].w[w]);
-                                        return x;
-                                    };
-                                    auto step_up = [&](const Bits<W> &x) {
-                                        if (W > 1) acc.w[W - 1] = acc.w[W - 1] << 1 | acc.w[0] >> 63 | x.w[W - 1];
-                                        acc.w[0] = acc.w[0] << 1 | x.w[0];
-                                    };
-                                    int q = nl - 1;
-                                    for (; q >= q0 && q >= nf; --q) step_up(gather(q));
-                                    for (; q >= q0; --q) step_up(any);
-                                    if (lo > 0) acc = bits_shift<W>(acc, lo);
-                                    if (q0 > 0) {
-                                        Bits<W> down;
-#pragma unroll
-                                        for (int w = 0; w < W; ++w) down.w[w] = 0;
-                                        for (q = 0; q < q0; ++q) {
-                                            if (q < nl) {
-                                                const Bits<W> x = q < nf ? any : gather(q);
-#pragma unroll
-                                                for (int w = 0; w < W; ++w) down.w[w] |= x.w[w];
-                                            }
-                                            if (W > 1) down.w[0] = down.w[0] >> 1 | down.w[W - 1] << 63;
-                                            else down.w[0] >>= 1;
-                                            if (W > 1) down.w[W - 1] >>= 1;
-                                        }
-#pragma unroll
-                                        for (int w = 0; w < W; ++w) acc.w[w] |= down.w[w];
+                                        step_up(acc, x);
                                     }
+                                    for (; q >= 0; --q) step_up(acc, any);
+                                    acc = bits_shift<W>(acc, jc.nmin[t] - d);
 #pragma unroll
                                     for (int w = 0; w < W; ++w) { acc.w[w] &= lm.w[w]; some |= acc.w[w] != 0; }
                                 }
@@ -433,46 +431,90 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
                     }
                     return __syncthreads_or(done) != 0;
                 };
-                // lower bound: every type's longest stages that cost at most B somewhere have to add up to N
-                if (tid == 0) s_low = (u64)kInf;
-                __syncthreads();
-                for (int e = tid; e < T * nwin * R; e += kReachThreads) {
-                    const int r = e % R, t = e / (R * nwin);
-                    if (!((rc_mask >> r) & 1u) || jc.cnt[t] == 0 || sLeast[e] >= kInf) continue;
-                    const i64 B = sLeast[e] + s_kmin[t];
-                    int room = 0;
-                    for (int h = 0; h < T; ++h) {
-                        int most = 0;
-                        for (int q = 0; jc.cnt[h] > 0 && q <= jc.nmax[h] - jc.nmin[h]; ++q)
-                            for (int x = 0; x < R; ++x)
-                                if (((rc_mask >> x) & 1u) && sLeast[(h * nwin + q) * R + x] + s_kmin[h] <= B) most = jc.nmin[h] + q;
-                        room += most * jc.cnt[h];
-                    }
-                    if (room >= N) atomicMin(&s_low, (u64)B);
-                }
-                __syncthreads();
-                const i64 low = (i64)s_low;
-                // between lo (no smaller stage cost can do) and hi (does): the next test lies a little above the lower bound
-                // first, then halfway
-                i64 lo = floor_b, hi;
-                bool ok = true;
-                if (floor_b > 0) ok = !test(floor_b);                // the larger choice of levels did not help: same answer
-                if (!ok) result = floor_b;
-                else {
-                    if (floor_b > 0) lo = (i64)s_up;
-                    if (test(kInf - 1)) {
-                        hi = (i64)s_dn;
-                        if (low > lo) lo = low;
-                        i64 step = lo / 64;
-                        bool gallop = true;
-                        while (lo < hi) {
-                            i64 B = lo + (hi - lo) / 2;
-                            if (gallop && step > 0 && lo + step < B) B = lo + step;
-                            if (test(B)) { hi = (i64)s_dn; gallop = false; }
-                            else { lo = (i64)s_up; step *= 2; }
+                // The longest stages that cost at most B, at the level that the depth's memory asks for, have to add up to N, with the best
+                // type at every depth and with the best depth for every type.  With the least cost of a length anywhere, that is a lower
+                // bound on the answer -- where even the largest does not do, nothing is feasible --; with its mean cost, a guess at it.
+                // The sums grow with B in steps at those costs; a warp per trial, eight a round.
+                auto capacity = [&](const i64 *costs) -> i64 {
+                    i64 a, b;                                         // a smallest and largest cost that may be the one
+                    auto around = [&](i64 B, i64 &below, i64 &above) {       // the largest cost at most B, the smallest above
+                        below = 0; above = kInf;
+                        for (int t = 0; t < T; ++t)
+                            for (int e = lane; jc.cnt[t] > 0 && e < nwin * R; e += 32) {
+                                const i64 v = costs[t * nwin * R + e] + s_kmin[t];
+                                if (v <= B) below = v > below ? v : below; else above = v < above ? v : above;
+                            }
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) {
+                            const i64 x = __shfl_xor_sync(0xffffffffu, below, o), y = __shfl_xor_sync(0xffffffffu, above, o);
+                            below = x > below ? x : below; above = y < above ? y : above;
                         }
-                        result = hi;
+                    };
+                    i64 x, y;
+                    around(kInf - 1, b, y);
+                    around(-1, x, a);
+                    bool first = true;
+                    while (first || a < b) {
+                        // trials at (b - a) (1 .. 8) / 8 behind a: the last one is b
+                        const i64 step = (b - a) / nwarps, m = wib == nwarps - 1 ? b : a + step * (wib + 1);
+                        int best = 0, sum = 0;
+                        for (int h = 0; h < T; ++h) {
+                            int most = 0;
+                            if (jc.cnt[h] > 0 && lane < PP) {
+                                const uint8_t *lv = sLvl + ((size_t)lane * T + h) * nwin;
+                                const i64 *c = costs + (size_t)h * nwin * R, limit = m - s_kmin[h];
+                                for (int q = jc.nmax[h] - jc.nmin[h]; q >= 0; --q)
+                                    if (lv[q] != 255 && c[q * R + lv[q]] <= limit) { most = jc.nmin[h] + q; break; }
+                            }
+                            best = most > best ? most : best;
+                            sum += jc.cnt[h] * (int)__reduce_max_sync(0xffffffffu, (unsigned)most);
+                        }
+                        const bool enough = sum >= N && (int)__reduce_add_sync(0xffffffffu, (unsigned)best) >= N && !__any_sync(0xffffffffu, lane < PP && best == 0);
+                        if (lane == 0) s_enough[wib] = enough;
+                        __syncthreads();
+                        int k = 0;
+                        while (k < nwarps && !s_enough[k]) ++k;
+                        __syncthreads();
+                        if (k == nwarps) return kInf;                 // (the first round's last trial is the largest cost)
+                        first = false;
+                        const i64 lo = a + step * k, hi = k == nwarps - 1 ? b : a + step * (k + 1);      // not enough at lo (k > 0), enough at hi
+                        around(hi, b, y);
+                        if (k > 0) { around(lo, x, y); a = y; }
+                        else if (step == 0) b = a;
                     }
+                    return b;
+                };
+                __syncthreads();                                      // (the levels of the stages)
+                const i64 low = capacity(sLeast), guess = low < kInf ? capacity(sMean) : kInf;
+                // Between lo (no smaller stage cost can do) and hi (does; kInf: not known): from the guess on in growing steps, then
+                // halfway.  Whether anything is feasible at all is asked once three tests have failed.  An answer under a larger
+                // choice of levels is tested first: mostly it remains.  (One place calls the test: it is long.)
+                enum { kHalve, kUp, kDown };
+                int way = kUp, failed = 0;
+                i64 lo = low > floor_b ? low : floor_b, hi = kInf, step = guess / 64 + 1;
+                bool at_floor = floor_b > 0 && lo == floor_b;
+                i64 B = !at_floor && guess > lo ? guess : lo;
+                while (low < kInf) {
+                    const bool can = test(B);
+                    const i64 dn = (i64)s_dn, up = (i64)s_up;
+                    if (at_floor) {
+                        if (can) { result = floor_b; break; }
+                        at_floor = false;
+                        lo = up;
+                        if (lo >= kInf) break;
+                        B = guess > lo ? guess : lo;
+                        continue;
+                    }
+                    if (B == kInf - 1) {
+                        if (!can) break;
+                        hi = dn;
+                    } else if (can) { hi = dn; way = way == kDown || (way == kUp && failed == 0) ? kDown : kHalve; }
+                    else { lo = up; ++failed; way = way == kDown ? kHalve : way; }
+                    if (lo >= hi) { result = lo >= kInf ? kInf : lo; break; }      // (a test that succeeds at lo is the answer)
+                    if (hi == kInf && failed == 3) { B = kInf - 1; continue; }
+                    B = lo + (hi - lo) / 2;
+                    if (way == kUp) { B = lo + step < B ? lo + step : B; step *= 2; }
+                    else if (way == kDown) { B = hi - step > B ? hi - step : B; step *= 2; }
                 }
             }
         }

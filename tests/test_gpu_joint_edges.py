@@ -50,3 +50,11 @@ def test_joint_bottleneck_words(nodes, N, window, tau, dense_first):
 def test_joint_bottleneck_forms(nodes, N, window, tau, dense_first):
     """Both sides of the line between the forms, which one class draws for all."""
     test_joint_bottleneck_words(nodes, N, window, tau, dense_first)
+
+
+@pytest.mark.parametrize("nodes,N", [((1, 1, 1, 1), 131),      # at most 64 end layers a level, 71 with what lengths move down by: two words
+                                     ((2, 1, 1), 226),         # 91 and 133: three words
+                                     ((2, 2, 2, 2), 119)])     # eight and sixteen stages, 60 / 65 and 64 / 67
+def test_joint_bottleneck_levels_that_begin_higher(nodes, N):
+    """A level whose first end layer lies further up than the shortest stage of a type: its lengths are summed up below it."""
+    test_joint_bottleneck_words(nodes, N, True, (0, 1024), False)
