@@ -1110,7 +1110,7 @@ extern "C" hap_status hap_enumerate(hap_problem *p, uint64_t *n_pconf, uint64_t 
             }
             ta.res_dev = reinterpret_cast<TreeResult *>(base + o_res);
             ta.N = N; ta.T = T; ta.R = p->prof.R; ta.n_rc = p->opts.n_rc; ta.RW = p->dc.tau_linear ? p->prof.R : 2;
-            ta.eta_q = p->dc.eta_q; ta.kind_uniform = p->dc.kind_uniform; ta.kind0 = p->kind[0];
+            ta.eta_q = p->dc.eta_q;
             for (int i = 0; i < p->opts.n_rc; ++i) { ta.rc_masks[i] = p->dc.rc_masks[i]; ta.rc_sup[i] = p->dc.rc_sup[i]; ta.rc_order[i] = p->dc.rc_order[i]; }
             for (int r = 0; r < p->prof.R; ++r) ta.tau[r] = p->tau_q[r] / 1024.0;
             ta.cls = im.d_cls;
