@@ -1436,7 +1436,7 @@ struct TreeLaunch { int c_lo, c_hi; size_t smem; unsigned grid; u64 items; int b
 // 8 stages: 1,024 devices, classes of 24 mappings, two policies 244 us (251, 246), 60 layers 247 (275, 261), one policy 206
 // (194, 200); a class of 840 mappings 390 (389, 394); 256 devices with partitions 474 (464, 466).  A search is one launch where it
 // may prune (its items go in order of their bounds) or where everything starts at once.
-static std::vector<TreeLaunch> tree_launches(const hap_problem *p, bool search, bool prune, unsigned p_lo, unsigned p_hi)
+static std::vector<TreeLaunch> tree_launches(const hap_problem *p, bool search, bool prune, bool grouped, unsigned p_lo, unsigned p_hi)
 {
     const auto &cls = p->image->cls;
     std::vector<TreeLaunch> ls;
@@ -1446,11 +1446,11 @@ static std::vector<TreeLaunch> tree_launches(const hap_problem *p, bool search, 
             const TreeClass &cl = cls[(size_t)c];
             const unsigned a = std::max(p_lo, cl.p_lo), b = std::min(p_hi, cl.p_lo + cl.n_conf);
             if (a >= b) continue;
-            l.items += (u64)(b - a) * cl.items_per_conf * (prune ? 1 : cl.policy_items);
-            l.smem = std::max(l.smem, tree_smem_bytes(cl));
+            l.items += (u64)(grouped ? (b - a + cl.group - 1) / cl.group : b - a) * cl.items_per_conf * (prune ? 1 : cl.policy_items);
+            l.smem = std::max(l.smem, tree_smem_bytes(cl, grouped));
         }
         if (!l.items) return;
-        if (search && p->dc.tau_linear && kTreeLive * (double)l.items > 2.0 * kTreeBlocksPerSm * sm_count(p->device)) l.blocks = kTreeSearchBlocksPerSm;
+        if (search && !grouped && p->dc.tau_linear && kTreeLive * (double)l.items > 2.0 * kTreeBlocksPerSm * sm_count(p->device)) l.blocks = kTreeSearchBlocksPerSm;
         const unsigned per_sm = (unsigned)std::max<size_t>(1, std::min<size_t>((size_t)l.blocks, kSmemPerSm / (l.smem + kTreeSmemStatic)));
         l.grid = (unsigned)std::min<u64>(l.items, std::min<u64>((u64)sm_count(p->device) * per_sm, kTreeSlots / 2));
         ls.push_back(l);
@@ -1482,7 +1482,10 @@ static hap_status launch_trees(hap_problem *p, const DpOut &out_in, bool search,
     p->state_dirty = true;
     if (refine) out.prune = 1;
     const bool prune = search && !f64 && out.prune;
-    const std::vector<TreeLaunch> ls = tree_launches(p, search, prune, p_lo, p_hi);
+    const bool counting = (p->opts.flags & HAP_OPT_COUNT_SPLITS) && !f64 && !search;
+    bool grouped = false;
+    for (const auto &cl : p->image->cls) grouped = grouped || (cl.group > 1 && !prune && !counting);
+    const std::vector<TreeLaunch> ls = tree_launches(p, search, prune, grouped, p_lo, p_hi);
     const bool ordered = prune && ls.size() == 1 && ls[0].items > ls[0].grid;      // (in one wave everything starts at once)
     p->largs.n_hist = ordered ? kOrderBuckets : 0;
     if ((s = launch_type_consts(p, p->d_coef, f64 ? p->d_coeff : nullptr, st, p_lo, p_hi, &p->largs)) != HAP_OK) return s;
@@ -1512,13 +1515,12 @@ static hap_status launch_trees(hap_problem *p, const DpOut &out_in, bool search,
     for (const auto &l : ls) ta.blocks_total += l.grid;
     if (!final_reduce) ta.res_dev = nullptr;
     ta.res_host = final_reduce ? p->host_result : nullptr;
-    const bool counting = (p->opts.flags & HAP_OPT_COUNT_SPLITS) && !f64 && !search;
     // two row entries are held where there are at most two levels, else they are read by level
     const int form = nl ? 2 : p->prof.R > 2 ? 1 : 0;
     using Fn = void (*)(const TreeArgs, const DevConst, DpOut);
     constexpr int kP = kTreePass, kS = kTreeSearch, kL = kTreeList;
-    constexpr int kB = kTreeSearchBlocksPerSm;
-    static const Fn fns[9][3] = {
+    constexpr int kB = kTreeSearchBlocksPerSm, kG = kTreeBlocksPerSm;
+    static const Fn fns[13][3] = {
         {tree_dp_kernel<kP, false, 2, false, false>, tree_dp_kernel<kP, false, 4, false, false>, tree_dp_kernel<kP, false, 4, true, false>},
         {tree_dp_kernel<kS, false, 2, false, false>, tree_dp_kernel<kS, false, 4, false, false>, tree_dp_kernel<kS, false, 4, true, false>},
         {tree_dp_kernel<kP, true, 2, false, false>, tree_dp_kernel<kP, true, 4, false, false>, tree_dp_kernel<kP, true, 4, true, false>},
@@ -1528,13 +1530,18 @@ static hap_status launch_trees(hap_problem *p, const DpOut &out_in, bool search,
         // four blocks an SM: search, fp64 search, listing
         {tree_dp_kernel<kS, false, 2, false, false, kB>, tree_dp_kernel<kS, false, 4, false, false, kB>, nullptr},
         {tree_dp_kernel<kS, true, 2, false, false, kB>, tree_dp_kernel<kS, true, 4, false, false, kB>, nullptr},
-        {tree_dp_kernel<kL, false, 2, false, false, kB>, tree_dp_kernel<kL, false, 4, false, false, kB>, nullptr}};
+        {tree_dp_kernel<kL, false, 2, false, false, kB>, tree_dp_kernel<kL, false, 4, false, false, kB>, nullptr},
+        // grouped: pass, search, and both in fp64
+        {tree_dp_kernel<kP, false, 2, false, false, kG, true>, tree_dp_kernel<kP, false, 4, false, false, kG, true>, tree_dp_kernel<kP, false, 4, true, false, kG, true>},
+        {tree_dp_kernel<kS, false, 2, false, false, kG, true>, tree_dp_kernel<kS, false, 4, false, false, kG, true>, tree_dp_kernel<kS, false, 4, true, false, kG, true>},
+        {tree_dp_kernel<kP, true, 2, false, false, kG, true>, tree_dp_kernel<kP, true, 4, false, false, kG, true>, tree_dp_kernel<kP, true, 4, true, false, kG, true>},
+        {tree_dp_kernel<kS, true, 2, false, false, kG, true>, tree_dp_kernel<kS, true, 4, false, false, kG, true>, tree_dp_kernel<kS, true, 4, true, false, kG, true>}};
     const int mode = refine ? 5 : counting ? 4 : (f64 ? 2 : 0) + (search ? 1 : 0);
     int n = 0;
     for (const auto &l : ls) {
         ta.c_lo = l.c_lo; ta.c_hi = l.c_hi; ta.launch = n;
         ta.slot_lo = n == 0 ? 0 : ls[0].grid;
-        const void *fn = (const void *)fns[l.blocks == kTreeBlocksPerSm ? mode : refine ? 8 : f64 ? 7 : 6][form];
+        const void *fn = (const void *)fns[grouped ? 9 + mode : l.blocks == kTreeBlocksPerSm ? mode : refine ? 8 : f64 ? 7 : 6][form];
         CUDA_TRY(p, raise_smem_limit(p->device, fn, l.smem));
         void *args[] = {(void *)&ta, (void *)&p->dc, (void *)&out};
         CUDA_TRY(p, launch_dependent(fn, l.grid, kTreeThreads, l.smem, st, args));
@@ -2253,7 +2260,7 @@ extern "C" hap_status hap_launches_per_pass(hap_problem *p, uint32_t *host_count
     const bool trees = pass_uses_trees(p, out);
     uint32_t n = 1 + 2;                                     // type constants; argmin partial and final
     if (!trees || !p->all_trees || (p->opts.flags & HAP_OPT_NO_FUSE)) n += 1;              // layer-cost array
-    if (trees) n += 1 + (uint32_t)tree_launches(p, false, false, 0, (unsigned)p->pconfs.size()).size();     // records, recurrence
+    if (trees) n += 1 + (uint32_t)tree_launches(p, false, false, false, 0, (unsigned)p->pconfs.size()).size();     // records, recurrence
     for (const auto &cl : p->classes) if (!trees || cl.tree < 0) n += 1;                    // one warp per candidate
     *host_count = n;
     return HAP_OK;

@@ -91,6 +91,7 @@ struct TreeClass {
     u32 ipc_inverse;                        // 2^32 / items_per_conf, rounded up (0: one item)
     int items_per_conf;                     // an item is a group of the configuration's parts (at most a part a warp) ...
     int policy_items;                       // ... under all policies (1) or, in passes, under one (then: the number of policies)
+    int group;                              // ... or, in the kernel's grouped form, of this many configurations whose parts all fit a block's warps
     uint8_t mrow_of[16], mask_of_row[16];   // type mask <-> row group
     uint8_t first_min[HAP_MAX_TYPES];       // per capacity type: shortest first stage (255: no first stage on it)
     uint8_t wmax[HAP_MAX_PP + 1];           // longest stage of depth d
@@ -171,6 +172,9 @@ __device__ __forceinline__ u64 global_timer()
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
 }
+
+// items of a class's listed configurations, a part each
+__device__ __forceinline__ u32 tree_groups(u32 live, int group) { return group == 1 ? live : (live + (u32)group - 1u) / (u32)group; }
 
 __device__ u32 *tree_state_live(TreeState *state) { return state->live; }
 __device__ void tree_stamp_begin(TreeReport *report) { report->stamp[0] = global_timer(); }
@@ -826,7 +830,9 @@ __device__ __forceinline__ void tree_finish(const TreeArgs &ta, const DevConst &
     __threadfence_system();
 }
 
-template <int MODE, bool F64, int RK, bool NL, bool COUNT, int BLOCKS = kTreeBlocksPerSm>
+// GROUP: items of several configurations (TreeClass::group), in a form of its own because the record's place in shared memory is then
+// an address in a register: 2 % of a pass whose classes have no use for it.
+template <int MODE, bool F64, int RK, bool NL, bool COUNT, int BLOCKS = kTreeBlocksPerSm, bool GROUP = false>
 __global__ void __launch_bounds__(kTreeThreads, BLOCKS)
 tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
 {
@@ -863,7 +869,7 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
         for (int c = ta.c_lo; c < ta.c_hi; ++c) {
             s_total[c - ta.c_lo] = t;
             const u32 live = __ldcg(&ta.state->live[c]);
-            t += ordered ? live : live * (u32)(ta.cls[c].items_per_conf * (ta.by_policy ? ta.cls[c].policy_items : 1));
+            t += ordered ? live : tree_groups(live, GROUP ? ta.cls[c].group : 1) * (u32)(ta.cls[c].items_per_conf * (ta.by_policy ? ta.cls[c].policy_items : 1));
         }
         s_total[ta.c_hi - ta.c_lo] = t;
         s_item = blockIdx.x;
@@ -908,7 +914,7 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
             int lo = 0, hi = n_rc;
             if (!ordered && ta.by_policy && cl->policy_items > 1) {
                 // items of one policy each: the first policy's come first (they take longest)
-                const u32 items = __ldcg(&ta.state->live[ci]) * ipc;
+                const u32 items = tree_groups(__ldcg(&ta.state->live[ci]), GROUP ? cl->group : 1) * ipc;
                 lo = (int)(local / items); hi = lo + 1; local -= (u32)lo * items;
             }
             if (tid == 0) { s_pos[0] = lo; s_pos[1] = hi; }     // (in shared memory: registers are short below)
@@ -916,7 +922,12 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
         // (quotients by the inverse: one too large at most; divisions took a tenth of an item's instructions)
         u32 conf = ipc == 1 ? local : __umulhi(local, cl->ipc_inverse), sub = local - conf * ipc;
         if ((int)sub < 0) { --conf; sub += ipc; }
+        u32 n_rec = 1;                                          // configurations of the item: their records follow one another
         if (ordered) conf = s_entry.z;
+        else if (GROUP) {
+            conf *= (u32)cl->group;
+            n_rec = min((u32)cl->group, __ldcg(&ta.state->live[ci]) - conf);
+        }
         const u32 n_parts = (u32)cl->n_parts, per = ipc == 1 ? n_parts : __umulhi(n_parts, cl->ipc_inverse), more = n_parts - per * ipc;
         const u32 part0 = sub * per + (sub < more ? sub : more), part1 = part0 + per + (sub < more ? 1u : 0u);
         const u32 rec_bytes = cl->rec_bytes;
@@ -926,13 +937,13 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
         {
             const unsigned char *src = ta.rec + cl->rec_off + (u64)conf * rec_bytes;
             const u32 dst = smem_u32(smem_raw);
-            for (u32 q = (u32)tid * 16u; q < rec_bytes; q += kTreeThreads * 16u)
+            for (u32 q = (u32)tid * 16u; q < n_rec * rec_bytes; q += kTreeThreads * 16u)
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + q), "l"(src + q) : "memory");
             asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
         }
         __syncthreads();
         const u32 slice_bytes = (cl->buf_cells[0] + cl->buf_cells[1]) * 8u + cl->ch_bytes;
-        const u32 a_slice = smem_u32(smem_raw) + rec_bytes + (u32)wib * slice_bytes;
+        const u32 a_slice = smem_u32(smem_raw) + (GROUP ? (u32)cl->group : 1u) * rec_bytes + (u32)wib * slice_bytes;
         const u32 a_buf[2] = {a_slice, a_slice + cl->buf_cells[0] * 8u};
         const u32 a_ch = a_buf[1] + cl->buf_cells[1] * 8u;
         const bool all_flat = cl->all_flat != 0;
@@ -945,9 +956,11 @@ tree_dp_kernel(const TreeArgs ta, const DevConst dc, DpOut out)
             u32 u = 0;
             if (lane == 0) u = atomicAdd(&s_unit, 1u);
             u = __shfl_sync(0xffffffffu, u, 0);
-            if (u >= part1 - part0) break;
-            const TreePart *pt = cl->parts + part0 + u;
+            if (u >= n_rec * (part1 - part0)) break;
             const unsigned char *rec = smem_raw;
+            if (GROUP)
+                for (; u >= part1 - part0; u -= part1 - part0) rec += rec_bytes;
+            const TreePart *pt = cl->parts + part0 + u;
             const TreeHead *hd = reinterpret_cast<const TreeHead *>(rec);
             const u32 a_rec = smem_u32(rec), a_rows = a_rec + cl->o_rows;
             const u32 nmap = pt->nmap;

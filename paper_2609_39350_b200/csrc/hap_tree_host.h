@@ -399,6 +399,7 @@ private:
         cl.items_per_conf = (cl.n_parts + kTreeWarps - 1) / kTreeWarps;
         cl.ipc_inverse = cl.items_per_conf > 1 ? (u32)(((1ull << 32) + cl.items_per_conf - 1) / (u64)cl.items_per_conf) : 0u;
         cl.policy_items = 1;
+        cl.group = 1;
         out.parts.resize((size_t)cl.n_parts);
         for (int q = 0; q < cl.n_parts; ++q) {
             Part pt;
@@ -484,9 +485,9 @@ private:
     int capt_[1 << HAP_MAX_TYPES] = {0};
 };
 
-inline size_t tree_smem_bytes(const TreeClass &cl)
+inline size_t tree_smem_bytes(const TreeClass &cl, bool grouped = false)
 {
-    return (size_t)cl.rec_bytes + kTreeWarps * ((size_t)(cl.buf_cells[0] + cl.buf_cells[1]) * 8 + cl.ch_bytes) + kTreeSmemFixed;
+    return (size_t)(grouped ? cl.group : 1) * cl.rec_bytes + kTreeWarps * ((size_t)(cl.buf_cells[0] + cl.buf_cells[1]) * 8 + cl.ch_bytes) + kTreeSmemFixed;
 }
 
 inline size_t tree_prep_smem_bytes(const TreeClass &cl, int N, int T)
@@ -504,6 +505,19 @@ inline void tree_policy_items(std::vector<TreeClass> &cls, const std::vector<std
     for (const auto &th : trees) all += th->work * kTreeLive * th->cls.n_conf / (n_sm * kTreeIssue);
     for (size_t c = 0; c < cls.size(); ++c)
         cls[c].policy_items = trees[c]->chain / kTreeWarpIssue > 0.1 * all ? n_rc : 1;
+    // Configurations of one or two parts share a block, a warp per part, where most items are of such classes and there are more than
+    // one wave of them; else they do better on SMs of their own, and the others without the grouped form.  64 devices, three
+    // levels: 109 us a pass against 127.
+    double items = 0, few = 0;
+    for (const TreeClass &cl : cls) {
+        const double n = kTreeLive * cl.n_conf * cl.items_per_conf * cl.policy_items;
+        items += n; few += cl.n_parts <= kTreeWarps / 2 ? n : 0.0;
+    }
+    if (items <= (double)n_sm * kTreeBlocksPerSm || 2.0 * few < items) return;
+    for (TreeClass &cl : cls) {
+        cl.group = std::max(1, kTreeWarps / cl.n_parts);
+        if (tree_smem_bytes(cl, true) + kTreeSmemStatic > kSmemPerSm / kTreeBlocksPerSm) cl.group = 1;
+    }
 }
 
 }  // namespace hap

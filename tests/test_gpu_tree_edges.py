@@ -105,3 +105,31 @@ def test_ranges_of_a_pass_whose_items_take_one_policy(nodes, N, tau, policies, k
         if a < b:
             assert np.array_equal(hap.hap_pipeline_dp(hp, a, b - a)["cost"].cpu().numpy(), costs[a:b]), (a, b)
     hap.hap_problem_destroy(hp)
+
+
+@pytest.mark.parametrize("tau,policies", [((0, 1024), (3,)), ((0, 307, 1024), (1, 3, 7)), ((0, 1024, 2048), (7, 1))])
+def test_items_of_several_configurations(tau, policies):
+    """64 devices: classes of one or two parts share blocks, the last block of a class with fewer configurations; whole passes, ranges
+    that begin inside a block's configurations, searches, and the fp64 pass."""
+    import paper_2609_39350_b200 as hap
+    pb = problems.mixtral()
+    R = len(tau)
+    pb.tau_q = np.array(tau, np.int32)
+    pb.xi_q = np.array([1024, 400, 64][:R - 1] + [64], np.int32)
+    pb.rc_masks = np.array(policies, np.uint32)
+    o = Oracle(pb)
+    _, best, index, costs, _ = o.search_pconfs(0, 1, threads=NTHREADS, want_costs=True)
+    hp = hap.hap_problem_create(pb)
+    hap.hap_enumerate(hp)
+    assert np.array_equal(hap.hap_pipeline_dp(hp, 0, hp.n_cand)["cost"].cpu().numpy(), costs)
+    for a in np.random.default_rng(R).integers(0, hp.n_cand - 5000, 4).tolist():
+        assert np.array_equal(hap.hap_pipeline_dp(hp, a, 4999)["cost"].cpu().numpy(), costs[a:a + 4999]), a
+    plan, _ = hap.hap_search_best(hp)
+    assert (plan["index"], plan["T_iter"]) == (index, best)
+    whole = hap.hap_pipeline_dp(hp, 0, hp.n_cand)["bottleneck"].cpu().numpy()
+    f64 = hap.hap_pipeline_dp_f64(hp, 0, hp.n_cand)["bottleneck"].cpu().numpy()
+    fin = whole < INF
+    # a stage cost is a sum of numbers rounded to whole nanoseconds: forward and backward of at most N layers (half each), the repeated
+    # forward of at most twice that, its floor, three transfers and ends
+    assert np.array_equal(np.isfinite(f64), fin) and np.max(np.abs(f64[fin] - whole[fin])) <= 2 * pb.N + 4
+    hap.hap_problem_destroy(hp)
