@@ -13,7 +13,8 @@
 //                      warp each writes their results.
 //   tree_dp_kernel     persistent blocks of four warps that take (configuration, up to four of its tree's parts) items
 //                      from a counter; in a pass an item of a class with long chains is one policy's.  A warp owns a
-//                      part of the tree -- a few to some tens of mappings -- and walks it depth by depth on its own:
+//                      part of the tree -- a few to some tens of mappings -- and walks it depth by depth on its own
+//                      (parts of one configuration, or of a few where they have one or two):
 //                      no block barrier inside an item.  A task is one, two or four consecutive end layers of a node (four
 //                      where the lanes are full, fewer where lanes would idle); a lane keeps
 //                      their running minima and slides one window of the parent's row over the stage lengths
@@ -21,14 +22,15 @@
 //                      assembles Eq. 4.  A search leaves the plan of the best candidate; the last block to finish
 //                      reduces the blocks' minima and decodes the winner.
 //
-// Bounds and figures (B200).  1,024 devices, 96 layers, 2.4 million candidates: a pass takes 389 us (435 with a block per
-// configuration and a barrier per depth); the same devices where no stage size is homogeneous, 374 thousand candidates in
-// classes of 24 mappings: 244 us (274 in that form, 371 while one to three of a block's warps had a part); 256 devices
-// with partitions 474 us (985).  The recurrence is bound by instruction issue and by the chain of a part: a warp issues an
-// instruction every six to seven cycles, 15 to 20 of 32 lanes active; its row entries never leave shared memory.  A deeper
+// Bounds and figures (B200).  1,024 devices, 96 layers, 2.4 million candidates: a pass takes 358 us (435 with a block per
+// configuration and a barrier per depth); 256 devices with partitions 410 us (985); 64 devices with three levels 109 us.  The same
+// 1,024 devices where no stage size is homogeneous, 374 thousand candidates in classes of 24 mappings: 244 us when a pass took 390
+// (274 with that barrier, 371 while one to three of a block's warps had a part).  The recurrence is bound by instruction issue and by
+// the chain of a part: a warp issues an instruction every seven to eight cycles, 20 to 25 of 32 lanes active; half of them are the
+// scans', a fifth the ways' back; its row entries never leave shared memory.  A deeper
 // split into blocks that share a tree needs a barrier per depth (31 of them at 32 stages); a warp of its own per part needs
-// none.  Measured earlier in this form: two end layers per task and eight blocks an SM 475 us, one end layer 536, eight parts an
-// item instead of four 405.  Four blocks an SM, without the few spilled registers that five (96 a thread) cost, were no faster.
+// none.  Measured while a pass took 400 us: two end layers per task and eight blocks an SM 475 us, one end layer 536, eight parts an
+// item instead of four 405 (373 against 359 now).
 // Records computed by the items themselves instead of tree_prep_kernel: 270 us instead of 284 in classes of few mappings,
 // but 513 instead of 475 at 256 devices, because the recurrence then has fewer registers; not kept.
 //
@@ -41,8 +43,8 @@ namespace hap {
 constexpr int kTreeWarps = 4;             // warps of a DP block
 constexpr int kTreeThreads = kTreeWarps * 32;
 // Blocks an SM: five (96 registers a thread), or four (128) for searches of several waves of items, whose last chains run faster beside
-// fewer warps and with what a plan takes in registers: pruned search at 1,024 devices 195 us against 214, its unpruned plan from host
-// tables 440 against 455, exact search at 256 devices 248 against 262.  Where the feasible items are two waves at most, every chain
+// fewer warps and with what a plan takes in registers: pruned search at 1,024 devices 195 us against 214, an unpruned plan from host
+// tables 440 against 455, exact search at 256 devices 250 against 271.  Where the feasible items are two waves at most, every chain
 // begins at once or nearly so: 64 devices 130 us against 135.  A pass is bound by the issue slots (256 devices 419 against 424, 1,024
 // devices 359 against 352), and rows that are not combined by level need no more than 96 registers (126 against 139).
 constexpr int kTreeBlocksPerSm = 5, kTreeSearchBlocksPerSm = 4;
