@@ -48,6 +48,54 @@ struct JointReach {
     const unsigned *ent;
 };
 
+// Which limits are tested, and when the answer is known.  The answer lies between lo (no smaller stage cost can do) and hi (does; kInf:
+// not known that any does).  From a guess on in steps that double while they are taken, then halfway; whether anything is feasible at all
+// is asked once three tests have failed.  An answer under a larger choice of levels is tested first: mostly it remains.
+// Every limit lies in [lo, hi): a step is taken only where it is shorter than the way to the halving point, and never again once it was
+// not, so that it neither overflows nor leaves the interval, and each test makes that smaller -- whatever the stage costs are, those
+// beyond the supported range included.  At most 128 tests: 62 steps, 62 halvings, the larger choice's answer, the largest limit, one of each that
+// is not taken.
+struct LimitSearch {
+    enum Way { kHalve, kUp, kDown };
+    i64 lo, hi, B, step, guess;                   // B: the limit to be tested
+    int way, failed;
+    bool at_floor;                                // B is the answer under a larger choice of levels
+
+    // low: a lower bound on the answer; floor_b: the answer under a larger choice of levels (0: none); mean: the guess
+    __host__ __device__ void begin(i64 low, i64 floor_b, i64 mean)
+    {
+        lo = low > floor_b ? low : floor_b; hi = kInf;
+        at_floor = floor_b > 0 && lo == floor_b;
+        guess = mean > lo && mean < kInf ? mean : lo;
+        way = kUp; failed = 0; step = guess / 64 + 1;
+        B = at_floor ? lo : guess;
+    }
+
+    // Whether B can do, and the nearest stage costs: the largest at most B, the smallest above (kInf: none).  False: the answer is lo (kInf: infeasible).
+    __host__ __device__ bool next(bool can, i64 dn, i64 up)
+    {
+        if (can && at_floor) return false;
+        if (can) {
+            hi = dn < B ? dn : B;
+            if (B != kInf - 1) way = way != kHalve && (way == kDown || failed == 0) ? kDown : kHalve;
+        } else {
+            lo = up > B ? up : B + 1;
+            if (lo > kInf) lo = kInf;
+            if (!at_floor) { ++failed; if (way == kDown) way = kHalve; }
+        }
+        if (lo >= hi) return false;               // (a test that succeeds at lo is the answer)
+        if (at_floor) { at_floor = false; B = guess > lo ? guess : lo; return true; }
+        if (hi == kInf && failed == 3) { B = kInf - 1; return true; }
+        B = lo + (hi - lo) / 2;
+        if (way != kHalve) {
+            const i64 room = way == kUp ? B - lo : hi - B;
+            if (step < room) { B = way == kUp ? lo + step : hi - step; step *= 2; }
+            else way = kHalve;
+        }
+        return true;
+    }
+};
+
 template <int W> struct Bits { u64 w[W]; };
 
 template <int W>
@@ -486,35 +534,15 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
                 };
                 __syncthreads();                                      // (the levels of the stages)
                 const i64 low = capacity(sLeast), guess = low < kInf ? capacity(sMean) : kInf;
-                // Between lo (no smaller stage cost can do) and hi (does; kInf: not known): from the guess on in growing steps, then
-                // halfway.  Whether anything is feasible at all is asked once three tests have failed.  An answer under a larger
-                // choice of levels is tested first: mostly it remains.  (One place calls the test: it is long.)
-                enum { kHalve, kUp, kDown };
-                int way = kUp, failed = 0;
-                i64 lo = low > floor_b ? low : floor_b, hi = kInf, step = guess / 64 + 1;
-                bool at_floor = floor_b > 0 && lo == floor_b;
-                i64 B = !at_floor && guess > lo ? guess : lo;
-                while (low < kInf) {
-                    const bool can = test(B);
-                    const i64 dn = (i64)s_dn, up = (i64)s_up;
-                    if (at_floor) {
-                        if (can) { result = floor_b; break; }
-                        at_floor = false;
-                        lo = up;
-                        if (lo >= kInf) break;
-                        B = guess > lo ? guess : lo;
-                        continue;
+                // (one place calls the test: it is long)
+                if (low < kInf) {
+                    LimitSearch search;
+                    search.begin(low, floor_b, guess);
+                    while (true) {
+                        const bool can = test(search.B);
+                        if (!search.next(can, (i64)s_dn, (i64)s_up)) break;
                     }
-                    if (B == kInf - 1) {
-                        if (!can) break;
-                        hi = dn;
-                    } else if (can) { hi = dn; way = way == kDown || (way == kUp && failed == 0) ? kDown : kHalve; }
-                    else { lo = up; ++failed; way = way == kDown ? kHalve : way; }
-                    if (lo >= hi) { result = lo >= kInf ? kInf : lo; break; }      // (a test that succeeds at lo is the answer)
-                    if (hi == kInf && failed == 3) { B = kInf - 1; continue; }
-                    B = lo + (hi - lo) / 2;
-                    if (way == kUp) { B = lo + step < B ? lo + step : B; step *= 2; }
-                    else if (way == kDown) { B = hi - step > B ? hi - step : B; step *= 2; }
+                    result = search.lo;
                 }
             }
         }
