@@ -7,6 +7,7 @@
 #include <algorithm>
 #include <cstring>
 #include <memory>
+#include <unordered_map>
 #include <vector>
 
 namespace hap {
@@ -54,14 +55,17 @@ constexpr double kTreeIssue = 2.3, kTreeWarpIssue = 0.15, kTreeLive = 0.4, kTree
 // Warp instructions: of an iteration of tasks of 1, 2 or 4 end layers and of a length in it; of 32 last stages and of a stage
 // on the way back.
 constexpr double kTreeIteration[3] = {70.0, 90.0, 130.0}, kTreePerLength[3] = {15.0, 24.0, 41.0}, kTreeLeaf = 150.0, kTreePerStage = 100.0;
+inline double tree_time(const TreeWork &w, double busy_issue)
+{
+    const double copy = 1500.0 + w.rec_bytes / 16, live = kTreeLive * w.n_conf;
+    return live * (w.total + copy * kTreeWarpIssue * w.n_parts) / (w.n_sm * busy_issue) + kTreeChain * (w.longest / kTreeWarpIssue + copy);
+}
 inline double tree_time(const TreeWork &w)
 {
     const size_t smem = w.rec_bytes + kTreeWarps * w.slice + kTreeSmemFixed;
     const int per_sm = (int)std::min<size_t>(kTreeBlocksPerSm, kSmemPerSm / (smem + kTreeSmemStatic)), items = (w.n_parts + kTreeWarps - 1) / kTreeWarps;
     if (per_sm < 1 || smem > kTreeSmemMost) return -1.0;
-    const double busy = (double)w.n_parts / items, copy = 1500.0 + w.rec_bytes / 16;
-    const double issue = std::min(kTreeIssue, per_sm * busy * kTreeWarpIssue), live = kTreeLive * w.n_conf;
-    return live * (w.total + copy * kTreeWarpIssue * w.n_parts) / (w.n_sm * issue) + kTreeChain * (w.longest / kTreeWarpIssue + copy);
+    return tree_time(w, std::min(kTreeIssue, per_sm * ((double)w.n_parts / items) * kTreeWarpIssue));
 }
 
 class TreeBuilder {
@@ -81,7 +85,12 @@ public:
 
 private:
     struct Node { u32 parent, rowoff; uint8_t mask, link, nmin, nmax; int bl, bh; };
-    struct Part { u64 m0, m1; std::vector<std::vector<Node>> lv; std::vector<u32> leaf_node; };
+    struct Part {
+        u64 m0, m1;
+        std::vector<std::vector<Node>> lv;
+        std::vector<u32> leaf_node;
+        std::vector<u64> order; std::vector<u32> place; std::vector<Node> sorted;      // (kept: a cluster asks for thousands of parts)
+    };
 
     // the class's mappings in enumeration order (decode_stage unranks single ones; here they follow one another)
     void decode()
@@ -176,6 +185,17 @@ private:
                 bl_[at + s] = (uint8_t)std::max(0, std::min(255, a)); bh_[at + s] = (uint8_t)std::max(0, std::min(255, b));
             }
         }
+        shared_.assign((size_t)nmap_, 0);
+        for (u64 m = 0, before = nmap_; m < nmap_; ++m) {
+            if (dead_[m]) continue;
+            if (before < nmap_) {
+                const size_t a = (size_t)before * PP_, b = (size_t)m * PP_;
+                int d = 0;
+                while (d < PP_ && mask_[a + d] == mask_[b + d] && link_[a + d] == link_[b + d] && nmin_[a + d] == nmin_[b + d] && nmax_[a + d] == nmax_[b + d]) ++d;
+                shared_[m] = (uint8_t)d;
+            }
+            before = m;
+        }
         return true;
     }
 
@@ -184,48 +204,47 @@ private:
     void nodes(u64 m0, u64 m1, Part &pt) const
     {
         pt.m0 = m0; pt.m1 = m1;
-        pt.lv.assign(PP_ + 1, {});
+        pt.lv.resize(PP_ + 1);
+        for (auto &v : pt.lv) v.clear();
         pt.leaf_node.assign((size_t)(m1 - m0), 0);
-        std::vector<u32> path(PP_ + 1, 0);
-        std::vector<size_t> key(PP_ + 1, 0);                    // position of the stage the path's node was made from
-        bool have = false;
+        u32 path[HAP_MAX_PP + 1] = {0};
+        uint8_t lo[HAP_MAX_PP], hi[HAP_MAX_PP];                 // bands of the path's nodes, by stage
+        int open = 0;                                           // stages of the path that have a node
+        auto close = [&](int from) { for (int s = from; s < open; ++s) { Node &nd = pt.lv[s + 1][path[s + 1]]; nd.bl = lo[s]; nd.bh = hi[s]; } };
         for (u64 m = m0; m < m1; ++m) {
             if (dead_[m]) continue;
             const size_t at = (size_t)m * PP_;
-            int d0 = 1;
-            if (have)
-                for (; d0 < PP_; ++d0) {
-                    const size_t a = key[d0], b = at + d0 - 1;
-                    if (mask_[a] != mask_[b] || link_[a] != link_[b] || nmin_[a] != nmin_[b] || nmax_[a] != nmax_[b]) break;
-                }
-            for (int d = d0; d < PP_; ++d) {
-                const size_t b = at + d - 1;
-                path[d] = (u32)pt.lv[d].size(); key[d] = b;
-                pt.lv[d].push_back(Node{d > 1 ? path[d - 1] : 0, 0, mask_[b], link_[b], nmin_[b], nmax_[b], 1 << 20, -1});
+            const int same = std::min(open, (int)shared_[m]);
+            close(same);
+            for (int s = 0; s < same; ++s) { lo[s] = std::min(lo[s], bl_[at + s]); hi[s] = std::max(hi[s], bh_[at + s]); }
+            for (int s = same; s < PP_ - 1; ++s) {
+                lo[s] = bl_[at + s]; hi[s] = bh_[at + s];
+                path[s + 1] = (u32)pt.lv[s + 1].size();
+                pt.lv[s + 1].push_back(Node{s ? path[s] : 0, 0, mask_[at + s], link_[at + s], nmin_[at + s], nmax_[at + s], 0, 0});
             }
-            have = true;
-            for (int d = 1; d < PP_; ++d) {
-                Node &nd = pt.lv[d][path[d]];
-                nd.bl = std::min(nd.bl, (int)bl_[at + d - 1]); nd.bh = std::max(nd.bh, (int)bh_[at + d - 1]);
-            }
+            open = PP_ - 1;
             pt.leaf_node[(size_t)(m - m0)] = PP_ > 1 ? path[PP_ - 1] : 0;
         }
+        close(0);
         // nodes of a depth by the width of their band, then of their window (widest first): the lanes of a warp get runs of
         // similar length
         for (int d = 1; d < PP_; ++d) {
-            std::vector<u32> ord(pt.lv[d].size()), newidx(pt.lv[d].size());
-            for (size_t i = 0; i < ord.size(); ++i) ord[i] = (u32)i;
-            std::stable_sort(ord.begin(), ord.end(), [&](u32 a, u32 b) {
-                const Node &x = pt.lv[d][a], &y = pt.lv[d][b];
-                const int wx = x.bh - x.bl, wy = y.bh - y.bl;
-                return wx != wy ? wx > wy : (int)x.nmax - (int)x.nmin > (int)y.nmax - (int)y.nmin; });
-            std::vector<Node> sorted(pt.lv[d].size());
-            for (size_t i = 0; i < ord.size(); ++i) { sorted[i] = pt.lv[d][ord[i]]; newidx[ord[i]] = (u32)i; }
-            pt.lv[d].swap(sorted);
-            if (d + 1 < PP_) for (auto &ch : pt.lv[d + 1]) ch.parent = newidx[ch.parent];
-            else for (u64 m = m0; m < m1; ++m) if (!dead_[m]) pt.leaf_node[(size_t)(m - m0)] = newidx[pt.leaf_node[(size_t)(m - m0)]];
+            std::vector<Node> &lv = pt.lv[d];
+            const size_t n = lv.size();
+            pt.order.resize(n); pt.place.resize(n); pt.sorted.resize(n);
+            for (size_t i = 0; i < n; ++i)
+                pt.order[i] = (u64)(512 - (lv[i].bh - lv[i].bl)) << 48 | (u64)(512 - ((int)lv[i].nmax - (int)lv[i].nmin)) << 32 | i;
+            std::sort(pt.order.begin(), pt.order.end());
             u32 c = kTreeAhead;
-            for (auto &nd : pt.lv[d]) { c += kTreePad; nd.rowoff = c; c += (u32)(nd.bh - nd.bl + 1); }
+            for (size_t i = 0; i < n; ++i) {
+                const u32 from = (u32)pt.order[i];
+                Node &nd = pt.sorted[i];
+                nd = lv[from]; pt.place[from] = (u32)i;
+                c += kTreePad; nd.rowoff = c; c += (u32)(nd.bh - nd.bl + 1);
+            }
+            lv.swap(pt.sorted);
+            if (d + 1 < PP_) for (auto &ch : pt.lv[d + 1]) ch.parent = pt.place[ch.parent];
+            else for (u64 m = m0; m < m1; ++m) if (!dead_[m]) pt.leaf_node[(size_t)(m - m0)] = pt.place[pt.leaf_node[(size_t)(m - m0)]];
         }
     }
 
@@ -297,75 +316,208 @@ private:
         return true;
     }
 
-    // a task before it is laid out: end layers j .. j + cnt - 1 of a node, stage lengths a .. b
-    struct Piece { u32 node; int j, cnt, a, b; };
+    // a task before it is laid out: end layers j .. j + cnt - 1 of a node, stage lengths a .. b (b = a - 1: none)
+    struct Piece {
+        u32 node;
+        uint8_t j, cnt, a, b;
+        int length() const { return (int)b + 1 - (int)a; }
+    };
 
-    // the task of J end layers from j on
-    Piece piece(const Part &pt, int d, u32 ni, int j, int J) const
+    // What one depth after the other is cut with.
+    struct Cutter {
+        std::vector<Piece> tasks, rest, scratch;
+        std::vector<int16_t> len[3];                            // lengths of tasks of 1, 2 and 4 end layers, room for eight behind the last
+        size_t n[3];
+        u32 of[257] = {0};                                      // how many are of a length: all zero between uses
+        std::unordered_map<u64, double> known;                  // times by a hash of the depth's nodes (of which parts have many in common)
+
+        // Warp instructions of the first `most` of the tasks of J end layers, the longest ones first, 32 an iteration.
+        double time(int J, size_t most)
+        {
+            const int16_t *v = len[J / 2].data(), *end = v + n[J / 2];
+            const double it = kTreeIteration[J / 2], per = kTreePerLength[J / 2];
+            int16_t hi = 0;
+            for (const int16_t *l = v; l < end; ++l) hi = std::max(hi, *l);
+            if (n[J / 2] <= 32) return most ? it + per * std::max<int>(1, hi) : 0.0;
+            for (const int16_t *l = v; l < end; ++l) ++of[*l];
+            double t = 0;
+            size_t at = 0, next = 0;                            // tasks of length l or more; the first of the next iteration
+            for (int l = hi; l >= 0; --l) {
+                for (at += of[l]; next < at && next < most; next += 32) t += it + per * std::max(1, l);
+                of[l] = 0;
+            }
+            return t;
+        }
+
+        // longest first, equal ones in the order they had
+        void sort(std::vector<Piece> &v, size_t from)
+        {
+            int hi = 0;
+            for (size_t q = from; q < v.size(); ++q) { const int l = v[q].length(); ++of[l]; hi = std::max(hi, l); }
+            u32 at = 0;
+            for (int l = hi; l >= 0; --l) { const u32 k = of[l]; of[l] = at; at += k; }
+            scratch.resize(v.size() - from);
+            for (size_t q = from; q < v.size(); ++q) scratch[of[v[q].length()]++] = v[q];
+            std::copy(scratch.begin(), scratch.end(), v.begin() + (std::ptrdiff_t)from);
+            std::memset(of, 0, ((size_t)hi + 1) * sizeof(u32));
+        }
+    };
+
+    // a node with the end layers of the one before it
+    struct Reach {
+        int nmin, nmax, pbl, pbh;
+        // shortest and longest stage that end at j .. j + J - 1 and reach the row before
+        int a(int j) const { return std::max(nmin, j - pbh); }
+        int b(int j, int J) const { return std::min(nmax, j + J - 1 - pbl); }
+        int length(int j, int J) const { return std::max(0, b(j, J) - a(j) + 1); }
+        Piece piece(u32 node, int j, int J) const { return Piece{node, (uint8_t)j, (uint8_t)J, (uint8_t)a(j), (uint8_t)(a(j) + length(j, J) - 1)}; }
+    };
+    static Reach reach(const Part &pt, int d, u32 ni)
     {
         const Node &nd = pt.lv[d][ni];
-        const int pbl = d > 1 ? pt.lv[d - 1][nd.parent].bl : 0, pbh = d > 1 ? pt.lv[d - 1][nd.parent].bh : 0;
-        Piece q{ni, j, std::min(J, nd.bh - j + 1), std::max((int)nd.nmin, j - pbh), 0};
-        q.b = std::min((int)nd.nmax, j + q.cnt - 1 - pbl);
-        if (q.a > q.b) q.b = q.a - 1;
-        return q;
+        if (d == 1) return Reach{nd.nmin, nd.nmax, 0, 0};
+        const Node &pn = pt.lv[d - 1][nd.parent];
+        return Reach{nd.nmin, nd.nmax, pn.bl, pn.bh};
     }
 
-    // The tasks of a depth, in the order a warp takes them, 32 an iteration, and the warp instructions they take.  Four end layers
-    // a task are cheapest where the lanes are full: a length's loads, tests and steps serve four splits.  What does not fill
-    // an iteration, often the whole depth, is cut into tasks of two or one, which take a fraction of the instructions on
-    // lanes that would idle.  Longest tasks first, so that an iteration's are alike.  Depths whose thresholds go by end layer take
-    // one each.  Against tasks of four everywhere (20 of 32 lanes active, now 25): a pass at 1,024 devices 390 -> 378 us, 256
-    // devices with partitions 473 -> 439, 64 devices with three levels 150 -> 130, search at 1,024 devices 233 -> 220.
-    double cut(const Part &pt, int d, bool flat, std::vector<Piece> &out) const
+    // lengths of the tasks of J end layers of a depth, node by node (eight at a time: what lies behind a node's last one is written over)
+    template <int J>
+    static void lengths(const Part &pt, int d, Cutter &c)
     {
-        auto longer = [](const Piece &x, const Piece &y) { return x.b - x.a > y.b - y.a; };
-        auto cost = [](const std::vector<Piece> &v, size_t from, size_t to, int J) {
-            double t = 0;
-            for (; from < to; from += 32) t += kTreeIteration[J / 2] + kTreePerLength[J / 2] * std::max(1, v[from].b - v[from].a + 1);
-            return t;
-        };
-        out.clear();
-        for (u32 ni = 0; ni < pt.lv[d].size(); ++ni)
-            for (int j = pt.lv[d][ni].bl; j <= pt.lv[d][ni].bh; j += flat ? kTreeJ : 1) out.push_back(piece(pt, d, ni, j, flat ? kTreeJ : 1));
-        std::stable_sort(out.begin(), out.end(), longer);
-        if (!flat) return cost(out, 0, out.size(), 1);
-        const size_t n = out.size(), full = n / 32 * 32;
-        double best = cost(out, 0, n, kTreeJ);
-        std::vector<Piece> tail, keep;
-        size_t head = n;
-        for (size_t h : {full, (size_t)0}) {
-            for (int J : {2, 1}) {
-                if (h == n || (n - h) * (size_t)(kTreeJ / J) > 96) continue;            // (two full iterations more than one: no gain)
-                tail.clear();
-                for (size_t q = h; q < n; ++q)
-                    for (int j = out[q].j; j < out[q].j + out[q].cnt; j += J) {
-                        tail.push_back(piece(pt, d, out[q].node, j, std::min(J, out[q].j + out[q].cnt - j)));
-                    }
-                std::stable_sort(tail.begin(), tail.end(), longer);
-                const double t = cost(out, 0, h, kTreeJ) + cost(tail, 0, tail.size(), J);
-                if (t < best) { best = t; head = h; keep.swap(tail); }
+        size_t n = 0;
+        for (const Node &nd : pt.lv[d]) n += (size_t)std::max(0, nd.bh - nd.bl + J) / J;
+        c.n[J / 2] = n;
+        if (c.len[J / 2].size() < n + 8) c.len[J / 2].resize(2 * n + 8);
+        int16_t *o = c.len[J / 2].data();
+        for (u32 ni = 0; ni < pt.lv[d].size(); ++ni) {
+            const Reach r = reach(pt, d, ni);
+            const int16_t bh = (int16_t)pt.lv[d][ni].bh, nmin = (int16_t)(r.nmin - 1), nmax = (int16_t)r.nmax, pbl = (int16_t)r.pbl, pbh = (int16_t)(r.pbh + 1);
+            for (int j = pt.lv[d][ni].bl; j <= bh; j += 8 * J) {
+                for (int k = 0; k < 8; ++k) {
+                    const int16_t first = (int16_t)(j + k * J), last = std::min<int16_t>((int16_t)(first + J - 1), bh);
+                    const int16_t b = std::min<int16_t>(nmax, (int16_t)(last - pbl)), a = std::max<int16_t>(nmin, (int16_t)(first - pbh));
+                    o[k] = std::max<int16_t>(0, (int16_t)(b - a));
+                }
+                o += std::min(8, (bh - j + J) / J);
             }
-            if (full == 0) break;
         }
-        if (head < n) { out.resize(head); out.insert(out.end(), keep.begin(), keep.end()); }
+    }
+
+    // lengths of the last `left` tasks of four end layers, in the order of their lengths, as tasks of one and two: the shortest ones, the
+    // last of the list where they are alike
+    static void rest_lengths(const Part &pt, int d, Cutter &c, size_t left)
+    {
+        const int16_t *len = c.len[2].data() + c.n[2];
+        int most = 0, hi = 0;
+        for (size_t q = 0; q < c.n[2]; ++q) { const int l = c.len[2][q]; ++c.of[l]; hi = std::max(hi, l); }
+        size_t equal = left;                                    // of length `most`
+        for (; c.of[most] < equal; ++most) equal -= c.of[most];
+        std::memset(c.of, 0, ((size_t)hi + 1) * sizeof(u32));
+        for (int J : {1, 2}) if (c.len[J / 2].size() < (size_t)kTreeJ / J * left + 8) c.len[J / 2].resize((size_t)kTreeJ / J * left + 8);
+        int16_t *one = c.len[0].data(), *two = c.len[1].data();
+        for (u32 ni = (u32)pt.lv[d].size(); left && ni-- > 0;) {
+            const Reach r = reach(pt, d, ni);
+            const int bl = pt.lv[d][ni].bl, bh = pt.lv[d][ni].bh;
+            for (int j = bl + (bh - bl) / kTreeJ * kTreeJ; left && j >= bl; j -= kTreeJ) {
+                const int l = *--len;
+                if (l > most || (l == most && equal == 0)) continue;
+                if (l == most) --equal;
+                --left;
+                const int end = std::min(bh, j + kTreeJ - 1);
+                for (int i = j; i <= end; i += 2) {
+                    *two++ = (int16_t)r.length(i, std::min(2, end - i + 1));
+                    *one++ = (int16_t)r.length(i, 1);
+                    if (i < end) *one++ = (int16_t)r.length(i + 1, 1);
+                }
+            }
+        }
+        c.n[0] = (size_t)(one - c.len[0].data()); c.n[1] = (size_t)(two - c.len[1].data());
+    }
+
+    // The tasks of a depth, 32 an iteration, and the warp instructions they take.  Four end layers a task are cheapest where the lanes are
+    // full: a length's loads, tests and steps serve four splits.  What does not fill an iteration, often the whole depth, is cut
+    // into tasks of two or one, which take a fraction of the instructions on lanes that would idle.  Longest tasks first, so
+    // that an iteration's are alike.  Depths whose thresholds go by end layer take one each.  Against tasks of four everywhere (20
+    // of 32 lanes active, now 25): a pass at 1,024 devices 390 -> 378 us, 256 devices with partitions 473 -> 439, 64 devices with three
+    // levels 150 -> 130, search at 1,024 devices 233 -> 220.
+    // `lay`: leaves the tasks in the order a warp takes them.  The search for the number of parts asks for the time alone, thousands of
+    // times a cluster: it follows from how many tasks are of a length, and nothing is put in order.
+    double cut(const Part &pt, int d, bool flat, Cutter &c, bool lay) const
+    {
+        u64 hash = flat ? 1469598103934665603ull : 1099511628211ull;
+        if (!lay) {
+            for (u32 ni = 0; ni < pt.lv[d].size(); ++ni) {
+                const Reach r = reach(pt, d, ni);
+                const Node &nd = pt.lv[d][ni];
+                hash = (hash ^ ((u64)r.nmin << 40 | (u64)r.nmax << 32 | (u64)r.pbl << 24 | (u64)r.pbh << 16 | (u64)nd.bl << 8 | (u64)nd.bh)) * 0x9e3779b97f4a7c15ull;
+                hash ^= hash >> 29;
+            }
+            const auto it = c.known.find(hash);
+            if (it != c.known.end()) return it->second;
+        }
+        const int J0 = flat ? kTreeJ : 1;
+        if (flat) lengths<kTreeJ>(pt, d, c);
+        else lengths<1>(pt, d, c);
+        const size_t n = c.n[J0 / 2], full = n / 32 * 32;
+        double best = c.time(J0, n);
+        size_t head = n;
+        int width = kTreeJ;
+        if (flat)
+            for (size_t h : {full, (size_t)0}) {                // tasks of four end layers that stay: whole iterations, or none
+                if (h < n && (n - h) * 2 <= 96) {               // (two full iterations more than one: no gain)
+                    if (h) rest_lengths(pt, d, c, n - h);
+                    else {
+                        if (n * 4 <= 96) lengths<1>(pt, d, c);
+                        lengths<2>(pt, d, c);
+                    }
+                    const double before = h ? c.time(kTreeJ, h) : 0.0;
+                    for (int J : {2, 1}) {
+                        if ((n - h) * (size_t)(kTreeJ / J) > 96) continue;
+                        const double t = before + c.time(J, c.n[J / 2]);
+                        if (t < best) { best = t; head = h; width = J; }
+                    }
+                }
+                if (full == 0) break;
+            }
+        if (!lay) { c.known.emplace(hash, best); return best; }
+        std::vector<Piece> &out = c.tasks;
+        out.clear();
+        for (u32 ni = 0; ni < pt.lv[d].size(); ++ni) {
+            const Reach r = reach(pt, d, ni);
+            const int bh = pt.lv[d][ni].bh;
+            for (int j = pt.lv[d][ni].bl; j <= bh; j += J0) out.push_back(r.piece(ni, j, std::min(J0, bh - j + 1)));
+        }
+        c.sort(out, 0);
+        if (head < n) {
+            c.rest.assign(out.begin() + (std::ptrdiff_t)head, out.end());
+            out.resize(head);
+            for (const Piece &t : c.rest) {
+                const Reach r = reach(pt, d, t.node);
+                for (int i = 0; i < t.cnt; i += width) out.push_back(r.piece(t.node, t.j + i, std::min(width, t.cnt - i)));
+            }
+            c.sort(out, head);
+        }
         return best;
     }
 
     // warp instructions of a part, roughly: what the split is chosen by
-    void cost(const Part &pt, const TreeClass &cl, double &total, size_t &slice) const
+    double cost(const Part &pt, const TreeClass &cl, Cutter &cutter) const
+    {
+        double total = (double)((pt.m1 - pt.m0 + 31) / 32) * (kTreeLeaf + kTreePerStage * PP_);
+        for (int d = 1; d < PP_; ++d) total += cut(pt, d, cl.flat[d] != 0, cutter, false);
+        return total;
+    }
+
+    // a warp's row buffers and choices for it, in bytes
+    size_t slice(const Part &pt) const
     {
         u32 cells[2] = {0, 0}, ch = 0;
-        total = 0;
-        std::vector<Piece> tasks;
         for (int d = 1; d < PP_; ++d) {
             u32 c = kTreeAhead + kTreePad;
             for (const Node &nd : pt.lv[d]) c += (u32)(nd.bh - nd.bl + 1) + kTreePad;
             cells[d & 1] = std::max(cells[d & 1], c); ch += c;
-            total += cut(pt, d, cl.flat[d] != 0, tasks);
         }
-        total += (double)((pt.m1 - pt.m0 + 31) / 32) * (kTreeLeaf + kTreePerStage * PP_);
-        slice = ((size_t)((cells[0] + 1) / 2 * 2) + (cells[1] + 1) / 2 * 2) * 8 + (ch + 15) / 16 * 16;
+        return ((size_t)((cells[0] + 1) / 2 * 2) + (cells[1] + 1) / 2 * 2) * 8 + (ch + 15) / 16 * 16;
     }
 
     bool split(TreeClassHost &out)
@@ -374,26 +526,30 @@ private:
         // smaller parts cost little; more parts shorten the longest chain and fill the warps of a block, fewer fill the lanes
         // of a warp better.  How many is what tree_time says.
         TreeClass &cl = out.cls;
+        Cutter cutter;
+        Part pt;
         double best = 0;
         cl.n_parts = 0;
         for (u64 np : {1, 2, 3, 4, 6, 8, 12, 16, 20, 24, 28, 32, 40, 48, 56, 64, 80, 96, 128, 192, 256, 384, 512, 768, 1024, 2048, 4096, 8192}) {
             if (np > nmap_) break;
-            std::vector<Part> parts((size_t)np);
-            for (u64 q = 0; q < np; ++q) nodes(nmap_ * q / np, nmap_ * (q + 1) / np, parts[(size_t)q]);
             TreeWork w;
             w.n_conf = (double)in_.n_conf; w.n_sm = in_.n_sm; w.n_parts = (int)np; w.rec_bytes = cl.rec_bytes;
-            for (const Part &pt : parts) {
-                double c; size_t s;
-                cost(pt, cl, c, s);
-                w.total += c; w.longest = std::max(w.longest, c); w.slice = std::max(w.slice, s);
+            for (u64 q = 0; q < np && tree_time(w) > 0; ++q) {
+                nodes(nmap_ * q / np, nmap_ * (q + 1) / np, pt);
+                w.slice = std::max(w.slice, slice(pt));
+                const double c = cost(pt, cl, cutter);
+                w.total += c; w.longest = std::max(w.longest, c);
             }
             const double t = tree_time(w);
-            if (t > 0 && (!cl.n_parts || t < best)) { best = t; cl.n_parts = (int)np; out.work = w.total; out.chain = w.longest; }
-            // finer parts share no more prefixes: what they all cost only grows, and a chain has an iteration a depth at least.  A
-            // sum of a growing and a falling term has one minimum, but for the rounding to whole warps: half as much again
-            // lies behind it
-            const double least = w.total * kTreeLive * w.n_conf / (w.n_sm * kTreeIssue) + kTreeChain * (PP_ - 1) * kTreeIteration[0] / kTreeWarpIssue;
-            if (cl.n_parts && (least > best || (t > 1.5 * best && cl.n_parts != (int)np))) break;
+            if (t <= 0) continue;                               // (no block has room for a part of that size)
+            if (!cl.n_parts || t < best) { best = t; cl.n_parts = (int)np; out.work = w.total; out.chain = w.longest; }
+            // finer parts share no more prefixes: what they all cost only grows, but for how full their iterations are, and a chain has an
+            // iteration a depth, an end and a way back at least.  A sum of a growing and a falling term has one minimum, but for the
+            // rounding to whole warps: half as much again lies behind it
+            TreeWork finer = w;
+            finer.total *= 0.85;
+            finer.longest = (PP_ - 1) * (kTreeIteration[0] + kTreePerLength[0]) + kTreeLeaf + kTreePerStage * PP_;
+            if (tree_time(finer, kTreeIssue) > best || (t > 1.5 * best && cl.n_parts != (int)np)) break;
         }
         if (!cl.n_parts) return false;                          // no part leaves room for a block
         cl.items_per_conf = (cl.n_parts + kTreeWarps - 1) / kTreeWarps;
@@ -402,9 +558,8 @@ private:
         cl.group = 1;
         out.parts.resize((size_t)cl.n_parts);
         for (int q = 0; q < cl.n_parts; ++q) {
-            Part pt;
             nodes(nmap_ * q / cl.n_parts, nmap_ * (q + 1) / cl.n_parts, pt);
-            if (!emit(pt, cl, out.parts[(size_t)q])) return false;
+            if (!emit(pt, cl, cutter, out.parts[(size_t)q])) return false;
         }
         return true;
     }
@@ -412,19 +567,20 @@ private:
     // nothing to do beside t (what the 32 tasks of an iteration share, and addresses that exist)
     static TreeTask no_task(const TreeTask &t) { return make_uint4(t.x, (t.y & 255u) | 1u << 8, t.z, t.w); }
 
-    bool emit(const Part &pt, TreeClass &cl, TreePartHost &ph) const
+    bool emit(const Part &pt, TreeClass &cl, Cutter &cutter, TreePartHost &ph) const
     {
         TreePart &tp = ph.meta;
         const u32 nmap = (u32)(pt.m1 - pt.m0);
         tp.nmap = nmap; tp.m_lo = (u32)pt.m0;
         u32 cells = 0, buf[2] = {0, 0}, cell_lo[HAP_MAX_PP + 1] = {0};      // choices of depth d start at cell_lo[d]
-        std::vector<Piece> pieces;
+        const std::vector<Piece> &pieces = cutter.tasks;
         for (int d = 1; d < PP_; ++d) {
             cell_lo[d] = cells;
             const size_t first = ph.tasks.size();
             u32 c = kTreeAhead + kTreePad;
             for (const Node &nd : pt.lv[d]) c += (u32)(nd.bh - nd.bl + 1) + kTreePad;
-            cut(pt, d, cl.flat[d] != 0, pieces);
+            cut(pt, d, cl.flat[d] != 0, cutter, true);
+            int J = 1;
             for (size_t at = 0; at < pieces.size(); ++at) {
                 const Piece &q = pieces[at];
                 const Node &nd = pt.lv[d][q.node];
@@ -441,8 +597,10 @@ private:
                 t.z = (u32)kidx(d, nd.mask, nd.link, cl) | ((u32)cl.mrow_of[nd.mask] << 8) | ((u32)((d - 1) * HAP_MAX_TYPES + capt_[nd.mask]) << 16);
                 // tasks of an iteration are of the same number of end layers: that of its largest one
                 const size_t it = at / 32 * 32;
-                int J = 1;
-                for (size_t x = it; x < std::min(it + 32, pieces.size()); ++x) J = std::max(J, pieces[x].cnt);
+                if (at == it) {
+                    J = 1;
+                    for (size_t x = it; x < std::min(it + 32, pieces.size()); ++x) J = std::max(J, (int)pieces[x].cnt);
+                }
                 t.w = (cells + (u32)dst) | (u32)(J > 2 ? 4 : J) << 16 | (it + 32 >= pieces.size() ? kTaskEnds : 0u) | (cl.flat[d] ? 0u : kTaskByLayer);
                 ph.tasks.push_back(t);
             }
@@ -482,6 +640,7 @@ private:
     const int N_, PP_, T_;
     u64 nmap_ = 0;
     std::vector<uint8_t> mask_, link_, nmin_, nmax_, bl_, bh_, dead_;
+    std::vector<uint8_t> shared_;           // stages that a mapping has in common with the one before it
     int capt_[1 << HAP_MAX_TYPES] = {0};
 };
 

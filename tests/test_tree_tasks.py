@@ -26,5 +26,7 @@ def tasks(tmp_path_factory):
 def test_tasks_cover_the_rows(tasks, layers, first_moe, delta, nodes, node_size):
     rows = tasks(layers, first_moe, delta, nodes, node_size)
     assert rows and all(faults == 0 for *_, faults in rows), rows
+    # the split is searched for without laying out, or putting in order, the tasks of the numbers of parts that are not taken
+    assert all(allocated <= 100 * parts + 60 * PP for PP, *_, parts, allocated, _ in rows), rows
     if layers >= 60 and delta > 0:                       # all three widths occur
         assert all(sum(r[i] for r in rows) > 0 for i in (1, 2, 3)), rows

@@ -1,6 +1,6 @@
 // Checks the task lists of the prefix trees of a cluster (test_tree_tasks.py; no GPU is needed): prints, per PP class, stages,
-// iterations of 1, 2 and 4 end layers, and the faults found.  Arguments: layers, first MoE layer, window delta, nodes per type,
-// node size.
+// iterations of 1, 2 and 4 end layers, parts, memory allocations of the build, and the faults found.  Arguments: layers, first MoE
+// layer, window delta, nodes per type, node size.
 #include "../paper_2609_39350_b200/csrc/hap_tree_host.h"
 
 #include <cstdio>
@@ -8,6 +8,13 @@
 #include <map>
 
 using namespace hap;
+
+static long allocations;
+#ifndef __CUDA_ARCH__
+void *operator new(size_t n) { ++allocations; return malloc(n); }
+void operator delete(void *p) noexcept { free(p); }
+void operator delete(void *p, size_t) noexcept { free(p); }
+#endif
 
 int main(int argc, char **argv)
 {
@@ -36,12 +43,24 @@ int main(int argc, char **argv)
         TreeInputs in{};
         in.dc = &dc; in.rep = q; in.n_conf = 1000; in.n_sm = 148; in.want_tree = true;
         TreeClassHost th;
+        allocations = 0;
         TreeBuilder(in).build(th);
+        const long allocated = allocations;
         if (!th.ok) return 3;
         const TreeClass &c = th.cls;
         long iters[5] = {0, 0, 0, 0, 0}, faults = 0;
+        double work = 0, chain = 0;                                                  // instructions, from the tasks as they are laid out
         for (const TreePartHost &ph : th.parts) {
             u32 e = 0, behind_choices = 0;
+            double part = (double)((ph.meta.nmap + 31) / 32) * (kTreeLeaf + kTreePerStage * PP);
+            for (u32 q = 0; q < 32 * ph.meta.n_iter; q += 32) {
+                int most = 1;
+                for (u32 i = q; i < q + 32; ++i)
+                    if (ph.tasks[i].y >> 24 & 7u) most = std::max(most, (int)(ph.tasks[i].y >> 16 & 255u) - (int)(ph.tasks[i].y >> 8 & 255u) + 1);
+                const u32 J = ph.tasks[q].w >> 16 & 7u;
+                part += kTreeIteration[J / 2] + kTreePerLength[J / 2] * most;
+            }
+            work += part; chain = std::max(chain, part);
             faults += ph.tasks.size() != 32u * (ph.meta.n_iter + 1);                  // the iteration behind the last is there to be asked for
             for (u32 q = 32 * ph.meta.n_iter; q < ph.tasks.size(); ++q) faults += (ph.tasks[q].y >> 24 & 7u) != 0 || (ph.tasks[q].y >> 8 & 255u) <= (ph.tasks[q].y >> 16 & 255u);
             for (int d = 1; d < PP; ++d) {
@@ -80,7 +99,9 @@ int main(int argc, char **argv)
             }
             faults += e != 32 * ph.meta.n_iter;
         }
-        printf("%d %ld %ld %ld %ld\n", PP, iters[1], iters[2], iters[4], faults);
+        // the estimate that the parts were chosen by (an iteration whose tasks all came out narrower than planned takes less)
+        faults += work > th.work || work < 0.95 * th.work || chain > th.chain || chain < 0.95 * th.chain;
+        printf("%d %ld %ld %ld %zu %ld %ld\n", PP, iters[1], iters[2], iters[4], th.parts.size(), allocated, faults);
     }
     return 0;
 }
