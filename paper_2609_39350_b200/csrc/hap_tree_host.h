@@ -80,7 +80,8 @@ public:
         out.masks_used = 0;
         for (size_t q = 0; q < mask_.size(); ++q) out.masks_used |= 1u << mask_[q];
         if (!in_.want_tree || !windows()) return;
-        out.ok = class_fields(out.cls) && split(out);
+        Part all;
+        out.ok = class_fields(out.cls, all) && split(out, all);
     }
 
 private:
@@ -231,16 +232,22 @@ private:
         for (int d = 1; d < PP_; ++d) {
             std::vector<Node> &lv = pt.lv[d];
             const size_t n = lv.size();
-            pt.order.resize(n); pt.place.resize(n); pt.sorted.resize(n);
-            for (size_t i = 0; i < n; ++i)
-                pt.order[i] = (u64)(512 - (lv[i].bh - lv[i].bl)) << 48 | (u64)(512 - ((int)lv[i].nmax - (int)lv[i].nmin)) << 32 | i;
-            std::sort(pt.order.begin(), pt.order.end());
+            auto key = [&](size_t i) { return (u32)(512 - (lv[i].bh - lv[i].bl)) << 16 | (u32)(512 - ((int)lv[i].nmax - (int)lv[i].nmin)); };
             u32 c = kTreeAhead;
+            auto put = [&](Node &nd) { c += kTreePad; nd.rowoff = c; c += (u32)(nd.bh - nd.bl + 1); };
+            size_t sorted = 1;
+            while (sorted < n && key(sorted - 1) <= key(sorted)) ++sorted;
+            if (sorted >= n) {                                  // (as they come)
+                for (Node &nd : lv) put(nd);
+                continue;
+            }
+            pt.order.resize(n); pt.place.resize(n); pt.sorted.resize(n);
+            for (size_t i = 0; i < n; ++i) pt.order[i] = (u64)key(i) << 32 | i;
+            std::sort(pt.order.begin(), pt.order.end());
             for (size_t i = 0; i < n; ++i) {
                 const u32 from = (u32)pt.order[i];
-                Node &nd = pt.sorted[i];
-                nd = lv[from]; pt.place[from] = (u32)i;
-                c += kTreePad; nd.rowoff = c; c += (u32)(nd.bh - nd.bl + 1);
+                put(pt.sorted[i] = lv[from]);
+                pt.place[from] = (u32)i;
             }
             lv.swap(pt.sorted);
             if (d + 1 < PP_) for (auto &ch : pt.lv[d + 1]) ch.parent = pt.place[ch.parent];
@@ -255,7 +262,7 @@ private:
     }
 
     // row groups, windows, thresholds and the layout of a configuration's record
-    bool class_fields(TreeClass &cl)
+    bool class_fields(TreeClass &cl, Part &all)
     {
         const int R = dc_.R;
         cl.PP = PP_;
@@ -264,7 +271,6 @@ private:
         for (size_t q = 0; q < mask_.size(); ++q) used |= 1u << mask_[q];
         for (int mk = 1; mk < (1 << T_); ++mk)
             if ((used >> mk) & 1u) { cl.mrow_of[mk] = (uint8_t)cl.n_mrows; cl.mask_of_row[cl.n_mrows] = (uint8_t)mk; cl.n_mrows++; }
-        Part all;
         nodes(0, nmap_, all);
         std::memset(cl.first_min, 255, sizeof(cl.first_min));
         for (int d = 1; d <= PP_; ++d) { cl.jlo[d] = 255; cl.jhi[d] = 0; cl.kmin[d] = 255; cl.kmax[d] = 0; }
@@ -520,36 +526,59 @@ private:
         return ((size_t)((cells[0] + 1) / 2 * 2) + (cells[1] + 1) / 2 * 2) * 8 + (ch + 15) / 16 * 16;
     }
 
-    bool split(TreeClassHost &out)
+    bool split(TreeClassHost &out, const Part &all)
     {
         // Parts over contiguous ranges of mappings: the few nodes near the root that two parts share are computed by both, so
         // smaller parts cost little; more parts shorten the longest chain and fill the warps of a block, fewer fill the lanes
-        // of a warp better.  How many is what tree_time says.
+        // of a warp better.  How many is what tree_time says, climbed from a guess: every number that is looked at lays out all its prefixes
+        // (looking at each from one part on took 1.1 to 1.6 times as long a build; of 1,684 classes two came out otherwise, 2 and 4 % slower
+        // by tree_time).
         TreeClass &cl = out.cls;
         Cutter cutter;
         Part pt;
-        double best = 0;
+        constexpr int counts[] = {1, 2, 3, 4, 6, 8, 12, 16, 20, 24, 28, 32, 40, 48, 56, 64, 80, 96, 128, 192, 256, 384, 512, 768, 1024, 2048, 4096, 8192};
+        constexpr int n_counts = (int)(sizeof(counts) / sizeof(counts[0]));
+        int last = 0;
+        while (last + 1 < n_counts && (u64)counts[last + 1] <= nmap_) ++last;
+        TreeWork w;
+        w.n_conf = (double)in_.n_conf; w.n_sm = in_.n_sm; w.rec_bytes = cl.rec_bytes;
+        // what the whole tree takes says about where to look: parts take their share of it, and an iteration a depth, an end and a way back at
+        // least
+        const double whole = cost(all, cl, cutter), least = (PP_ - 1) * (kTreeIteration[0] + kTreePerLength[0]) + kTreeLeaf + kTreePerStage * PP_;
+        const size_t whole_slice = slice(all);
+        int at = last;
+        double guess = -1.0;
+        for (int i = 0; i <= last; ++i) {
+            w.n_parts = counts[i]; w.slice = whole_slice / (size_t)counts[i];
+            w.longest = whole / counts[i] + least; w.total = w.longest * counts[i];
+            const double t = tree_time(w);
+            if (t > 0 && (guess < 0 || t < guess)) { guess = t; at = i; }
+        }
+        bool seen[n_counts] = {false};
+        double best = -1.0;
+        int best_at = -1;
         cl.n_parts = 0;
-        for (u64 np : {1, 2, 3, 4, 6, 8, 12, 16, 20, 24, 28, 32, 40, 48, 56, 64, 80, 96, 128, 192, 256, 384, 512, 768, 1024, 2048, 4096, 8192}) {
-            if (np > nmap_) break;
-            TreeWork w;
-            w.n_conf = (double)in_.n_conf; w.n_sm = in_.n_sm; w.n_parts = (int)np; w.rec_bytes = cl.rec_bytes;
-            for (u64 q = 0; q < np && tree_time(w) > 0; ++q) {
+        auto look = [&](int i) {                                // takes counts[i] parts if that is faster than what is taken
+            if (i < 0 || i > last || seen[i]) return;
+            seen[i] = true;
+            const u64 np = (u64)counts[i];
+            w.n_parts = (int)np; w.slice = 0; w.total = w.longest = 0.0;
+            double t = tree_time(w);
+            for (u64 q = 0; q < np && t > 0 && (best < 0 || t <= best); ++q) {
                 nodes(nmap_ * q / np, nmap_ * (q + 1) / np, pt);
                 w.slice = std::max(w.slice, slice(pt));
                 const double c = cost(pt, cl, cutter);
                 w.total += c; w.longest = std::max(w.longest, c);
+                t = tree_time(w);
             }
-            const double t = tree_time(w);
-            if (t <= 0) continue;                               // (no block has room for a part of that size)
-            if (!cl.n_parts || t < best) { best = t; cl.n_parts = (int)np; out.work = w.total; out.chain = w.longest; }
-            // finer parts share no more prefixes: what they all cost only grows, but for how full their iterations are, and a chain has an
-            // iteration a depth, an end and a way back at least.  A sum of a growing and a falling term has one minimum, but for the
-            // rounding to whole warps: half as much again lies behind it
-            TreeWork finer = w;
-            finer.total *= 0.85;
-            finer.longest = (PP_ - 1) * (kTreeIteration[0] + kTreePerLength[0]) + kTreeLeaf + kTreePerStage * PP_;
-            if (tree_time(finer, kTreeIssue) > best || (t > 1.5 * best && cl.n_parts != (int)np)) break;
+            if (t <= 0 || (best > 0 && (t > best || (t == best && i > best_at)))) return;      // (t <= 0: no block has room for a part of that size)
+            best = t; best_at = i; cl.n_parts = (int)np; out.work = w.total; out.chain = w.longest;
+        };
+        look(at);
+        while (best_at < 0 && at < last) look(++at);
+        for (int from = -1; best_at != from;) {
+            from = best_at;
+            for (int i : {from + 1, from - 1, from + 2, from - 2}) look(i);
         }
         if (!cl.n_parts) return false;                          // no part leaves room for a block
         cl.items_per_conf = (cl.n_parts + kTreeWarps - 1) / kTreeWarps;
