@@ -530,9 +530,8 @@ private:
     {
         // Parts over contiguous ranges of mappings: the few nodes near the root that two parts share are computed by both, so
         // smaller parts cost little; more parts shorten the longest chain and fill the warps of a block, fewer fill the lanes
-        // of a warp better.  How many is what tree_time says, climbed from a guess: every number that is looked at lays out all its prefixes
-        // (looking at each from one part on took 1.1 to 1.6 times as long a build; of 1,684 classes two came out otherwise, 2 and 4 % slower
-        // by tree_time).
+        // of a warp better.  How many is what tree_time says: a guess, then every number from the first one that may be better.  (Climbing from
+        // the guess alone took a fifth less time and ended at other, slower numbers: how many blocks an SM holds grows in steps.)
         TreeClass &cl = out.cls;
         Cutter cutter;
         Part pt;
@@ -540,46 +539,54 @@ private:
         constexpr int n_counts = (int)(sizeof(counts) / sizeof(counts[0]));
         int last = 0;
         while (last + 1 < n_counts && (u64)counts[last + 1] <= nmap_) ++last;
+        // What the whole tree takes says where to look first, and which numbers are too small: parts take their share of it at least (but
+        // for how full their iterations are and how narrow their bands), and an iteration a depth, an end and a way back.
+        const double least = (PP_ - 1) * (kTreeIteration[0] + kTreePerLength[0]) + kTreeLeaf + kTreePerStage * PP_;
         TreeWork w;
         w.n_conf = (double)in_.n_conf; w.n_sm = in_.n_sm; w.rec_bytes = cl.rec_bytes;
-        // what the whole tree takes says about where to look: parts take their share of it, and an iteration a depth, an end and a way back at
-        // least
-        const double whole = cost(all, cl, cutter), least = (PP_ - 1) * (kTreeIteration[0] + kTreePerLength[0]) + kTreeLeaf + kTreePerStage * PP_;
+        const double whole = cost(all, cl, cutter);
         const size_t whole_slice = slice(all);
+        double bound[n_counts], guess = -1.0;
         int at = last;
-        double guess = -1.0;
         for (int i = 0; i <= last; ++i) {
             w.n_parts = counts[i]; w.slice = whole_slice / (size_t)counts[i];
             w.longest = whole / counts[i] + least; w.total = w.longest * counts[i];
             const double t = tree_time(w);
             if (t > 0 && (guess < 0 || t < guess)) { guess = t; at = i; }
+            w.slice = w.slice / 4 * 3;
+            w.longest = std::max(0.85 * whole / counts[i], least); w.total = 0.85 * whole;
+            bound[i] = tree_time(w);
         }
-        bool seen[n_counts] = {false};
         double best = -1.0;
         int best_at = -1;
         cl.n_parts = 0;
-        auto look = [&](int i) {                                // takes counts[i] parts if that is faster than what is taken
-            if (i < 0 || i > last || seen[i]) return;
-            seen[i] = true;
+        // takes counts[i] parts if that is faster than what is taken; true: more parts are not
+        auto look = [&](int i) {
             const u64 np = (u64)counts[i];
             w.n_parts = (int)np; w.slice = 0; w.total = w.longest = 0.0;
             double t = tree_time(w);
-            for (u64 q = 0; q < np && t > 0 && (best < 0 || t <= best); ++q) {
+            u64 q = 0;
+            while (q < np && t > 0 && (best < 0 || t <= best)) {
                 nodes(nmap_ * q / np, nmap_ * (q + 1) / np, pt);
                 w.slice = std::max(w.slice, slice(pt));
                 const double c = cost(pt, cl, cutter);
                 w.total += c; w.longest = std::max(w.longest, c);
                 t = tree_time(w);
+                ++q;
             }
-            if (t <= 0 || (best > 0 && (t > best || (t == best && i > best_at)))) return;      // (t <= 0: no block has room for a part of that size)
-            best = t; best_at = i; cl.n_parts = (int)np; out.work = w.total; out.chain = w.longest;
+            if (t <= 0) return false;                           // (no block has room for a part of that size)
+            if (best < 0 || (q == np && (t < best || (t == best && i < best_at)))) { best = t; best_at = i; cl.n_parts = (int)np; out.work = w.total; out.chain = w.longest; }
+            // finer parts share no more prefixes: what they all cost only grows, but for how full their iterations are.  A sum of a growing and
+            // a falling term has one minimum, but for the rounding to whole warps: half as much again lies behind it
+            TreeWork finer = w;
+            finer.total *= (double)np / (double)q;
+            t = std::max(t, tree_time(finer));
+            finer.total *= 0.85; finer.longest = least;
+            return tree_time(finer, kTreeIssue) > best || (t > 1.5 * best && best_at != i);
         };
         look(at);
-        while (best_at < 0 && at < last) look(++at);
-        for (int from = -1; best_at != from;) {
-            from = best_at;
-            for (int i : {from + 1, from - 1, from + 2, from - 2}) look(i);
-        }
+        for (int i = 0; i <= last; ++i)
+            if (i != at && bound[i] > 0 && (best < 0 || bound[i] < best) && look(i) && i > best_at) break;
         if (!cl.n_parts) return false;                          // no part leaves room for a block
         cl.items_per_conf = (cl.n_parts + kTreeWarps - 1) / kTreeWarps;
         cl.ipc_inverse = cl.items_per_conf > 1 ? (u32)(((1ull << 32) + cl.items_per_conf - 1) / (u64)cl.items_per_conf) : 0u;
