@@ -30,3 +30,27 @@ def test_tasks_cover_the_rows(tasks, layers, first_moe, delta, nodes, node_size)
     assert all(allocated <= 100 * parts + 60 * PP for PP, *_, parts, allocated, _ in rows), rows
     if layers >= 60 and delta > 0:                       # all three widths occur
         assert all(sum(r[i] for r in rows) > 0 for i in (1, 2, 3)), rows
+
+
+@pytest.fixture(scope="session")
+def walk(tmp_path_factory):
+    exe = str(tmp_path_factory.mktemp("walk") / "tree_walk")
+    subprocess.run([os.environ.get("NVCC", "nvcc"), "-gencode", "arch=compute_100a,code=sm_100a", "-std=c++17", "-O1", "-o", exe,
+                    os.path.join(ROOT, "tests", "tree_walk.cu")], check=True)
+
+    def run(*args):
+        out = subprocess.run([exe, *map(str, args)], check=True, capture_output=True, text=True).stdout
+        return [tuple(map(int, line.split())) for line in out.splitlines()]
+    return run
+
+
+# as above, and: 1,820 mappings at 16 stages, few configurations (other numbers of parts), a narrow window, no homogeneous stages
+@pytest.mark.parametrize("layers,first_moe,delta,nodes,node_size,n_conf", [
+    (96, 0, 205, "64,32,16,16", 8, 1000), (60, 1, 205, "12,8,8,4", 8, 1000), (33, 0, 205, "4,4", 8, 50), (16, 0, -1, "1,1", 4, 1000), (255, 0, -1, "8", 8, 1000),
+    (12, 5, 300, "3,1", 2, 1000), (29, 29, 205, "3,3,1", 8, 1000), (60, 0, 205, "24,8", 8, 728), (17, 0, 205, "1,1", 8, 10), (31, 2, 150, "2,1,1", 8, 200),
+    (255, 0, 205, "72,27,16,13", 8, 7)])
+def test_tasks_reach_every_split(walk, layers, first_moe, delta, nodes, node_size, n_conf):
+    """Walked on the host as the kernel walks them, tasks, last stages and ways back give every mapping's own bottleneck and partition, and
+    read nothing that was not written or lies outside of the row before."""
+    rows = walk(layers, first_moe, delta, nodes, node_size, n_conf)
+    assert rows and all(faults == 0 for *_, faults in rows), rows
