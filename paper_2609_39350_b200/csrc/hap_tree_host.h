@@ -700,19 +700,28 @@ inline void tree_policy_items(std::vector<TreeClass> &cls, const std::vector<std
     for (const auto &th : trees) all += th->work * kTreeLive * th->cls.n_conf / (n_sm * kTreeIssue);
     for (size_t c = 0; c < cls.size(); ++c)
         cls[c].policy_items = trees[c]->chain / kTreeWarpIssue > 0.1 * all ? n_rc : 1;
-    // Configurations of one or two parts share a block, a warp per part, where most items are of such classes and there are more than
-    // one wave of them; else they do better on SMs of their own, and the others without the grouped form.  64 devices, three
-    // levels: 109 us a pass against 127.
-    double items = 0, few = 0;
-    for (const TreeClass &cl : cls) {
-        const double n = kTreeLive * cl.n_conf * cl.items_per_conf * cl.policy_items;
-        items += n; few += cl.n_parts <= kTreeWarps / 2 ? n : 0.0;
-    }
-    if (items <= (double)n_sm * kTreeBlocksPerSm || 2.0 * few < items) return;
+    // how many configurations of one or two parts can share a block, a warp per part
     for (TreeClass &cl : cls) {
         cl.group = std::max(1, kTreeWarps / cl.n_parts);
         if (tree_smem_bytes(cl, true) + kTreeSmemStatic > kSmemPerSm / kTreeBlocksPerSm) cl.group = 1;
     }
+}
+
+// Whether a pass over configurations [p_lo, p_hi) takes the grouped form: where a quarter of its items or more are of classes that share
+// blocks, and there is more than half a wave of them (all configurations counted, feasible or not).  50 passes of 8 to 1,024 devices and their
+// halves to sixteenths, grouped against not: up to half a wave 0.95 to 1.06 times as fast, which is the noise, from there to a wave 3 to
+// 5 % faster, with more items 5 to 54 %; below a quarter of such items the same within 1 %.  64 devices, three levels and policies, a pass
+// 102 us against 121; 256 devices of two types, 400 configurations of 32 stages 56 against 80.
+inline bool tree_grouped(const std::vector<TreeClass> &cls, unsigned p_lo, unsigned p_hi, int n_sm)
+{
+    double items = 0, few = 0;
+    for (const TreeClass &cl : cls) {
+        const unsigned a = std::max(p_lo, cl.p_lo), b = std::min(p_hi, cl.p_lo + cl.n_conf);
+        if (a >= b) continue;
+        const double k = (double)(b - a) * cl.items_per_conf * cl.policy_items;
+        items += k; few += cl.group > 1 ? k : 0.0;
+    }
+    return items > 0.5 * n_sm * kTreeBlocksPerSm && 4.0 * few >= items;
 }
 
 }  // namespace hap

@@ -133,3 +133,68 @@ def test_items_of_several_configurations(tau, policies):
     # forward of at most twice that, its floor, three transfers and ends
     assert np.array_equal(np.isfinite(f64), fin) and np.max(np.abs(f64[fin] - whole[fin])) <= 2 * pb.N + 4
     hap.hap_problem_destroy(hp)
+
+
+@pytest.mark.parametrize("tau,policies", [((0, 1024), (3,)), ((0, 307, 1024), (1, 3, 7)), ((0, 1024, 2048), (7, 1))])
+def test_costs_of_items_of_several_configurations(tau, policies):
+    """As above with a dense first layer, and the unrounded costs, within 1e-9 relative of the fp64 oracle: sums, synchronisation and optimizer
+    terms of every configuration of a block.  (That these calls take the grouped form: test_calls_that_share_blocks_between_configurations.)"""
+    import paper_2609_39350_b200 as hap
+    pb = problems.mixtral()
+    R = len(tau)
+    pb.kind[0] = 0
+    pb.tau_q = np.array(tau, np.int32)
+    pb.xi_q = np.array([1024, 400, 64][:R - 1] + [64], np.int32)
+    pb.rc_masks = np.array(policies, np.uint32)
+    o = Oracle(pb)
+    _, best, index, costs, _ = o.search_pconfs(0, 1, threads=NTHREADS, want_costs=True)
+    _, costs_f, bn_f, _ = o.search_pconfs_f64(0, 1, threads=NTHREADS)
+    hp = hap.hap_problem_create(pb)
+    hap.hap_enumerate(hp)
+    assert np.array_equal(hap.hap_pipeline_dp(hp, 0, hp.n_cand)["cost"].cpu().numpy(), costs)
+    plan, _ = hap.hap_search_best(hp)
+    assert (plan["index"], plan["T_iter"]) == (index, best)
+    got = {k: v.cpu().numpy() for k, v in hap.hap_pipeline_dp_f64(hp, 0, hp.n_cand).items()}
+    for key, want in (("cost", costs_f), ("bottleneck", bn_f)):
+        fin = np.isfinite(want)
+        assert fin.any() and np.array_equal(fin, np.isfinite(got[key])), key
+        assert np.max(np.abs(got[key][fin] - want[fin]) / want[fin]) <= 1e-9, key
+    plan = hap.hap_search_range_f64(hp, 0, hp.n_cand)
+    two = np.sort(costs_f[np.isfinite(costs_f)])[:2]
+    assert plan["T_iter_f64"] == pytest.approx(two[0], rel=1e-9)
+    assert plan["index"] == int(np.argmin(costs_f)) or two[1] - two[0] <= 1e-9 * two[0]
+    hap.hap_problem_destroy(hp)
+
+
+def test_searches_of_several_waves_with_three_levels():
+    """256 devices, three levels combined into rows, one policy: some 13,000 items, of which two fifths are more than two waves, so that every
+    search takes the kernels of four blocks an SM -- unpruned, in the order of the bounds, listing for refinement, unrounded."""
+    import paper_2609_39350_b200 as hap
+    pb = problems.dsv2()
+    pb.tau_q = np.array((0, 1024, 2048), np.int32)
+    pb.xi_q = np.array((1024, 400, 64), np.int32)
+    pb.rc_masks = np.array((7,), np.uint32)
+    o = Oracle(pb)
+    _, best, index, _, _ = o.search_pconfs(0, 1, threads=NTHREADS, want_costs=True)
+    for prune in (0, 1):
+        hp = hap.hap_problem_create(pb, prune=prune)
+        hap.hap_enumerate(hp)
+        plan, st = hap.hap_search_best(hp)
+        assert (plan["index"], plan["T_iter"]) == (index, best), prune
+        want, _, _ = o.eval_index(index)
+        assert plan["n"] == want["n"] and plan["r"] == want["r"] and st["n_evaluated"] + st["n_pruned"] == hp.n_cand
+        if not prune:
+            costs = hap.hap_pipeline_dp_f64(hp, 0, hp.n_cand)["cost"].cpu().numpy()
+            got = hap.hap_search_range_f64(hp, 0, hp.n_cand)
+            assert (got["index"], got["T_iter_f64"]) == (int(np.argmin(costs)), float(costs.min()))
+            assert got["T_iter_f64"] == pytest.approx(o.eval_index_f64(got["index"])["T_iter"], rel=1e-9)
+        hap.hap_problem_destroy(hp)
+    for flag in (hap.OPT_REFINE, hap.OPT_EXACT):               # against one warp per candidate
+        plans = []
+        for more in (0, hap.OPT_NO_TRIE):
+            hp = hap.hap_problem_create(pb, flags=flag | more)
+            hap.hap_enumerate(hp)
+            plan, _ = hap.hap_search_best(hp)
+            plans.append((plan["index"], plan["T_iter"], plan["n"], plan["r"]))
+            hap.hap_problem_destroy(hp)
+        assert plans[0] == plans[1], flag
