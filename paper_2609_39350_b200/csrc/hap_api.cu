@@ -1883,13 +1883,16 @@ static hap_status joint_setup(hap_problem *p)
     // 208 against 340).  One class of many makes the search worth it (16 stages at 1,024 devices, 32,400 cells: 666 us against
     // 990; 32 stages at 32 devices, 132,192: 471 against 531, two policies 480 against 981), and then the others do better beside it in the
     // same launch than in launches of their own (32 devices, 32 layers: 492 us, 554 with the classes below 16,384 cells apart, 758
-    // without a search).
+    // without a search).  A class in three words is a launch of its own, which its own cells have to make worth it: 32 devices, 255 layers, 400
+    // configurations of four stages (9,180 cells) beside larger classes, 582 us in three words, 200 in the value form; 1,024 devices, 255
+    // layers, 32 stages (3.9 million cells), 1.5 ms against 44.
+    constexpr double kSearchCells = 20480.0;
     bool search = false;
     for (int PP : pps) {
         const int64_t G = p->W / PP;
         double cells = (double)T * N;
         for (int h = 0; h < T; ++h) cells = p->m[h] % G ? 0.0 : cells * (double)(p->m[h] / G + 1);
-        search = search || cells >= 20480.0;
+        search = search || cells >= kSearchCells;
     }
     for (int PP : pps) {
         const int64_t G = p->W / PP;
@@ -1921,7 +1924,7 @@ static hap_status joint_setup(hap_problem *p)
         jc.lmax = lmax;
         JointReach jr;
         std::vector<unsigned> en;
-        if (search && joint_reach_class(p, PP, G, jc, lvl_off, st_idx, slot, jr, en)) {
+        if (search && joint_reach_class(p, PP, G, jc, lvl_off, st_idx, slot, jr, en) && (jr.words <= 2 || (double)S * T * N >= kSearchCells)) {
             const int w = jr.words - 1;
             hap_problem::ReachHost &rh = p->reach[w];
             for (int i = 0; i <= HAP_MAX_PP; ++i) jr.ent_off[i] += (unsigned)ent[w].size();

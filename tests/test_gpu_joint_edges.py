@@ -58,3 +58,11 @@ def test_joint_bottleneck_forms(nodes, N, window, tau, dense_first):
 def test_joint_bottleneck_levels_that_begin_higher(nodes, N):
     """A level whose first end layer lies further up than the shortest stage of a type: its lengths are summed up below it."""
     test_joint_bottleneck_words(nodes, N, True, (0, 1024), False)
+
+
+@pytest.mark.parametrize("nodes,N", [((1, 1, 1, 1), 226),      # eight stages, 135: three words
+                                     ((2, 1, 1), 226)])        # four stages in three words would be 8,136 cells: a value per end layer, beside eight in bits
+def test_joint_bottleneck_three_words(nodes, N):
+    """Classes whose levels take three words, on both sides of the line between the forms."""
+    test_joint_bottleneck_words(nodes, N, True, (0, 1024), False)
+    test_joint_bottleneck_words(nodes, N, True, (0, 307, 1024), False)
