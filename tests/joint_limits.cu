@@ -13,10 +13,10 @@ using namespace hap;
 static int most, lost, wrong;
 
 // costs in order; the smallest limit that can do is `answer` (kInf: none)
-static void search(const std::vector<i64> &costs, i64 answer, i64 low, i64 floor_b, i64 guess)
+static void search(const std::vector<i64> &costs, i64 answer, i64 low, i64 floor_b, i64 guess, bool doubtful)
 {
     LimitSearch s;
-    s.begin(low, floor_b, guess);
+    s.begin(low, floor_b, guess, doubtful);
     for (int n = 1; ; ++n) {
         const i64 lo = s.lo, hi = s.hi;
         if (n > 128 || s.B < lo || s.B >= hi) { ++lost; return; }
@@ -49,7 +49,8 @@ static void report(const char *name, std::vector<i64> costs)
         for (i64 low : lows)
             for (i64 guess : guesses)
                 for (i64 floor_b : {(i64)0, low, a ? costs[a / 2 ? a / 2 : 0] : 0, answer < kInf ? answer : 0})
-                    if (floor_b <= answer) search(costs, answer, low, floor_b, guess);
+                    for (bool doubtful : {false, true})
+                        if (floor_b <= answer) search(costs, answer, low, floor_b, guess, doubtful);
         if (a == n) break;
     }
     printf("%s %d %d %d\n", name, most, lost, wrong);
