@@ -150,7 +150,7 @@ __host__ __device__ inline ReachSmem reach_smem(int N, int T, int R, int RW, int
 }
 
 template <bool LINEAR, int W>
-__global__ void __launch_bounds__(kReachThreads, 4)
+__global__ void __launch_bounds__(kReachThreads, W > 2 ? 2 : 4)      // (three words: 85 KB and more of shared memory a block)
 joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, const unsigned *ids, const i64 *c2, const i64 *coef, i64 *out)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
