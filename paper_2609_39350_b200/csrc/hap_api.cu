@@ -678,7 +678,6 @@ extern "C" hap_status hap_problem_create(const hap_model *mo, const hap_cluster 
     for (int l = 0; l < N; ++l) if (p->kind[l] == HAP_MOE) dc.kindbits[l >> 6] |= 1ull << (l & 63);
     dc.kind_uniform_from = N - 1;
     while (dc.kind_uniform_from > 0 && p->kind[dc.kind_uniform_from - 1] == p->kind[N - 1]) --dc.kind_uniform_from;
-    dc.kind_uniform = dc.kind_uniform_from == 0;
     dc.tab4 = p->d_tables + kRangeSlot / sizeof(double);
     dc.tpre = dc.tab4 + 4 * n5; dc.tpost = dc.tpre + n4;
 
@@ -740,7 +739,7 @@ static std::string tree_cache_key(const hap_problem *p, const hap_problem::PpCla
     const hap_pconf &rep = p->pconfs[p->items[cl.item_lo].p];
     const size_t n_conf = p->items[cl.item_hi - 1].p - p->items[cl.item_lo].p + 1;
     const int32_t head[] = {p->model.N, p->T, p->prof.R, cl.PP, rep.G, rep.mode, p->opts.delta_q, (int32_t)(p->opts.flags & HAP_OPT_UNIFORM),
-                            p->dc.kind_uniform, p->dc.kind_uniform_from, (int32_t)n_conf, p->dc.tau_linear, (int32_t)want_tree, sm_count(p->device)};
+                            p->dc.kind_uniform_from, (int32_t)n_conf, p->dc.tau_linear, (int32_t)want_tree, sm_count(p->device)};
     key_put(k, head);
     key_put(k, rep.nmap);
     for (int h = 0; h < p->T; ++h) { key_put(k, p->P[h]); key_put(k, p->cap_eff[h]); key_put(k, p->dc.m[h]); key_put(k, p->dc.node_size[h]); }
@@ -837,8 +836,8 @@ static hap_status image_for(hap_problem *p, const std::string &ekey, bool allow_
     }
     const bool want_tree = allow_trees && !(p->opts.flags & (HAP_OPT_NO_TRIE | HAP_OPT_NO_MAPTAB)) && exact && ordered;
     std::string key = ekey;
-    const int32_t head[] = {p->device, want_tree, p->prof.R, p->opts.delta_q, (int32_t)(p->opts.flags & HAP_OPT_UNIFORM), p->dc.kind_uniform,
-                            p->dc.kind_uniform_from, p->dc.tau_linear};
+    const int32_t head[] = {p->device, want_tree, p->prof.R, p->opts.delta_q, (int32_t)(p->opts.flags & HAP_OPT_UNIFORM), p->dc.kind_uniform_from,
+                            p->dc.tau_linear};
     key_put(key, head);
     for (int h = 0; h < p->T; ++h) { key_put(key, p->P[h]); key_put(key, p->cap_eff[h]); key_put(key, p->dc.node_size[h]); }
     ImageCache &ic = image_cache();
@@ -1295,7 +1294,7 @@ static hap_status launch_layer_kernel(hap_problem *p, i64 *c2, double *c2f, bool
     const TypeConst *tcg = p->d_tc;
     i64 *no_i = nullptr; double *no_d = nullptr;
     // layer kinds: 0 all dense, 1 all MoE (uniform branch compiled away), 2 mixed
-    const int kind = !p->dc.kind_uniform ? 2 : (p->kind[0] == HAP_MOE ? 1 : 0);
+    const int kind = p->dc.kind_uniform_from > 0 ? 2 : (p->kind[0] == HAP_MOE ? 1 : 0);
     using Fn = void (*)(const DevConst, const TypeConst *, i64 *, double *, i64 *, u64 *, unsigned);
     if (quant) {
         static const Fn fns[3][2] = {{layer_cost_kernel<true, 0, false>, layer_cost_kernel<true, 0, true>},
@@ -1355,7 +1354,7 @@ static hap_status launch_layer_costs(hap_problem *p, i64 *c2, i64 *coef, double 
         if (s != HAP_OK) return s;
         return launch_layer_kernel(p, c2, c2f, quant, st, lb_sum, p_lo, n_conf, true);
     }
-    const int kind = !p->dc.kind_uniform ? 2 : (p->kind[0] == HAP_MOE ? 1 : 0);      // layer kinds: all dense, all MoE, mixed
+    const int kind = p->dc.kind_uniform_from > 0 ? 2 : (p->kind[0] == HAP_MOE ? 1 : 0);      // layer kinds: all dense, all MoE, mixed
     using Fn = void (*)(const DevConst, i64 *, double *, i64 *, double *, i64 *, u64 *, unsigned, unsigned);
     static const Fn fns[3][3] = {{cost_kernel<false, 0, false>, cost_kernel<true, 0, false>, cost_kernel<true, 0, true>},
                                  {cost_kernel<false, 1, false>, cost_kernel<true, 1, false>, cost_kernel<true, 1, true>},
@@ -1541,6 +1540,7 @@ static hap_status launch_trees(hap_problem *p, const DpOut &out_in, bool search,
         ta.c_lo = l.c_lo; ta.c_hi = l.c_hi; ta.launch = n;
         ta.slot_lo = n == 0 ? 0 : ls[0].grid;
         const void *fn = (const void *)fns[grouped ? 9 + mode : l.blocks == kTreeBlocksPerSm ? mode : refine ? 8 : f64 ? 7 : 6][form];
+        if (!fn) return fail(p, HAP_E_STATE, "no tree kernel of this form");
         CUDA_TRY(p, raise_smem_limit(p->device, fn, l.smem));
         void *args[] = {(void *)&ta, (void *)&p->dc, (void *)&out};
         CUDA_TRY(p, launch_dependent(fn, l.grid, kTreeThreads, l.smem, st, args));

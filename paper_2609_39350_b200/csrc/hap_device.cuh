@@ -62,8 +62,7 @@ struct DevConst {
     int S, H, E, k, n_shared, F_dense, F_exp, nq, nkv, V, GB;
     int delta_q, tau_linear, eta_q, uniform;
     int het_dispatch;                 // Pruning 3 also counts the dispatch / combine traffic of stages that span device types
-    int kind_uniform;                 // every layer is of one kind (all MoE or all dense): a span's memory depends on its length only
-    int kind_uniform_from;            // first layer u such that layers u..N-1 are all of one kind (0 when kind_uniform)
+    int kind_uniform_from;            // first layer u such that layers u..N-1 are all of one kind (0: all are, and a span's memory depends on its length only)
     double beta, kappa, chi, gamma, ovl_tp, ovl_cp, ovl_dp, capf;
     double alpha[3];
     double eta[HAP_MAX_TYPES], croute[HAP_MAX_TYPES], copt[HAP_MAX_TYPES];

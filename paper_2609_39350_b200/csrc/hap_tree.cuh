@@ -43,10 +43,11 @@ namespace hap {
 constexpr int kTreeWarps = 4;             // warps of a DP block
 constexpr int kTreeThreads = kTreeWarps * 32;
 // Blocks an SM: five (96 registers a thread), or four (128) for searches of several waves of items, whose last chains run faster beside
-// fewer warps and with what a plan takes in registers: pruned search at 1,024 devices 195 us against 214, an unpruned plan from host
-// tables 440 against 455, exact search at 256 devices 250 against 271.  Where the feasible items are two waves at most, every chain
-// begins at once or nearly so: 64 devices 130 us against 135.  A pass is bound by the issue slots (256 devices 419 against 424, 1,024
-// devices 359 against 352), and rows that are not combined by level need no more than 96 registers (126 against 139).
+// fewer warps and with what a plan takes in registers: pruned search at 1,024 devices 195 us with four, 214 with five, an unpruned plan from
+// host tables 440 and 455, exact search at 256 devices 250 and 271.  Where the feasible items are two waves at most, every chain begins at
+// once or nearly so: 64 devices 135 us with four, 130 with five.  Passes take five: 256 devices with partitions 420 us with four, 410 with
+// five, against 355 and 358 at 1,024 devices.  Rows that are not combined by level need no more than 96 registers: 139 and 126.  (The number of
+// parts is planned for five blocks, whichever kernel runs.)
 constexpr int kTreeBlocksPerSm = 5, kTreeSearchBlocksPerSm = 4;
 constexpr int kTreeJ = 4;                 // end layers of a task at most
 template <int J> struct TreeWidth { static constexpr int value = J; };

@@ -36,7 +36,7 @@ def test_items_of_deep_classes_keep_their_block_busy(layout, layers, nodes):
 @pytest.mark.parametrize("layers,nodes,first_moe,delta,node_size", [(96, "72,27,16,13", 0, 205, 8), (60, "12,8,8,4", 1, 205, 8), (16, "1,1", 0, -1, 4),
                                                                     (32, "2,1,1", 0, 150, 8), (12, "3,1", 5, 300, 2), (255, "8", 0, -1, 8)])
 def test_scans_stay_inside_the_row_before(layout, layers, nodes, first_moe, delta, node_size):
-    """The window of a scan moves down by one entry a length and asks for one entry more than it uses: the lowest slot
+    """The window of a scan moves down by one entry a length and asks for two entries more than it uses: the lowest slot
     any task or last stage reads is one of its row buffer."""
     for c in layout(layers, nodes, first_moe, delta, 2, node_size):
         assert c["low"] >= 0, c

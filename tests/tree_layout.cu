@@ -12,7 +12,7 @@ int main(int argc, char **argv)
     if (argc != 8) return 2;
     const i64 P[4] = {400000, 300000, 250000, 150000}, cap[4] = {80ll << 30, 64ll << 30, 48ll << 30, 32ll << 30};
     DevConst dc{};
-    dc.N = atoi(argv[1]); dc.kind_uniform_from = atoi(argv[2]); dc.kind_uniform = dc.kind_uniform_from == 0;
+    dc.N = atoi(argv[1]); dc.kind_uniform_from = atoi(argv[2]);
     dc.delta_q = atoi(argv[3]); dc.R = atoi(argv[4]); dc.tau_linear = 1;
     i64 W = 0;
     for (char *s = strtok(argv[5], ","); s && dc.T < HAP_MAX_TYPES; s = strtok(nullptr, ",")) {
@@ -41,16 +41,16 @@ int main(int argc, char **argv)
         TreeBuilder(in).build(th);
         if (!th.ok) return 3;
         // entries of the row before that the scans read: the window of a task starts at its slot and moves down by one entry
-        // a length, one further than the last (tree_scan asks for the next entry before it knows that there is none)
+        // a length, two further than the last (tree_scan asks for the next two before it knows that there are none)
         long low = 1 << 20;
         for (const TreePartHost &ph : th.parts) {
             for (const TreeTask &t : ph.tasks) {
                 const long src = (long)(t.x & 0xffffu), a = t.y >> 8 & 255u, b = t.y >> 16 & 255u;
-                if (a <= b) low = std::min(low, src - (b - a + 1));
+                if (a <= b) low = std::min(low, src - (b - a + 2));
             }
             for (u32 m = 0; m < ph.meta.nmap; ++m) {
                 const long a = ph.leaf[m] & 255u, b = ph.leaf[m] >> 8 & 255u;
-                if (a <= b) low = std::min(low, (long)(ph.path[(size_t)(PP - 1) * ph.meta.nmap + m] & 0xfffffu) - (b - a + 1));
+                if (a <= b) low = std::min(low, (long)(ph.path[(size_t)(PP - 1) * ph.meta.nmap + m] & 0xfffffu) - (b - a + 2));
             }
         }
         const TreeClass &c = th.cls;

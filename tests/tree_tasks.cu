@@ -21,7 +21,7 @@ int main(int argc, char **argv)
     if (argc != 6) return 2;
     const i64 P[4] = {400000, 300000, 250000, 150000}, cap[4] = {80ll << 30, 64ll << 30, 48ll << 30, 32ll << 30};
     DevConst dc{};
-    dc.N = atoi(argv[1]); dc.kind_uniform_from = atoi(argv[2]); dc.kind_uniform = dc.kind_uniform_from == 0;
+    dc.N = atoi(argv[1]); dc.kind_uniform_from = atoi(argv[2]);
     dc.delta_q = atoi(argv[3]); dc.R = 2; dc.tau_linear = 1;
     i64 W = 0;
     for (char *s = strtok(argv[4], ","); s && dc.T < HAP_MAX_TYPES; s = strtok(nullptr, ",")) {
