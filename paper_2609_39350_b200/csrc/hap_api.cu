@@ -1482,7 +1482,7 @@ static hap_status launch_trees(hap_problem *p, const DpOut &out_in, bool search,
     if (refine) out.prune = 1;
     const bool prune = search && !f64 && out.prune;
     const bool counting = (p->opts.flags & HAP_OPT_COUNT_SPLITS) && !f64 && !search;
-    const bool grouped = !prune && !counting && tree_grouped(p->image->cls, p_lo, p_hi, sm_count(p->device));
+    const bool grouped = !prune && !counting && tree_grouped(p->image->cls, p_lo, p_hi, sm_count(p->device), search);
     const std::vector<TreeLaunch> ls = tree_launches(p, search, prune, grouped, p_lo, p_hi);
     const bool ordered = prune && ls.size() == 1 && ls[0].items > ls[0].grid;      // (in one wave everything starts at once)
     p->largs.n_hist = ordered ? kOrderBuckets : 0;

@@ -707,12 +707,14 @@ inline void tree_policy_items(std::vector<TreeClass> &cls, const std::vector<std
     }
 }
 
-// Whether a pass over configurations [p_lo, p_hi) takes the grouped form: where a quarter of its items or more are of classes that share
-// blocks, and there is more than half a wave of them (all configurations counted, feasible or not).  50 passes of 8 to 1,024 devices and their
+// Whether a call over configurations [p_lo, p_hi) takes the grouped form: where a quarter of a pass's items or more, or half of a search's, are
+// of classes that share blocks, and there is more than half a wave of items (all configurations counted, feasible or not).  50 passes of 8 to 1,024 devices and their
 // halves to sixteenths, grouped against not: up to half a wave 0.95 to 1.06 times as fast, which is the noise, from there to a wave 3 to
 // 5 % faster, with more items 5 to 54 %; below a quarter of such items the same within 1 %.  64 devices, three levels and policies, a pass
 // 102 us against 121; 256 devices of two types, 400 configurations of 32 stages 56 against 80.
-inline bool tree_grouped(const std::vector<TreeClass> &cls, unsigned p_lo, unsigned p_hi, int n_sm)
+// Searches of several waves lose four blocks an SM (kTreeSearchBlocksPerSm) by it: 149 unpruned ones of half a wave or more, 0.90 to 1.23 times as
+// fast where a quarter to a half of the items are such (24 of them), 0.89 to 1.36, on average 1.06, where more are.
+inline bool tree_grouped(const std::vector<TreeClass> &cls, unsigned p_lo, unsigned p_hi, int n_sm, bool search)
 {
     double items = 0, few = 0;
     for (const TreeClass &cl : cls) {
@@ -721,7 +723,7 @@ inline bool tree_grouped(const std::vector<TreeClass> &cls, unsigned p_lo, unsig
         const double k = (double)(b - a) * cl.items_per_conf * cl.policy_items;
         items += k; few += cl.group > 1 ? k : 0.0;
     }
-    return items > 0.5 * n_sm * kTreeBlocksPerSm && 4.0 * few >= items;
+    return items > 0.5 * n_sm * kTreeBlocksPerSm && (search ? 2.0 : 4.0) * few >= items;
 }
 
 }  // namespace hap

@@ -58,14 +58,16 @@ def test_tasks_reach_every_split(walk, layers, first_moe, delta, nodes, node_siz
 
 def test_calls_that_share_blocks_between_configurations(tmp_path):
     """64 devices, three policies: the classes of two mappings share blocks.  The whole pass and ranges of half a wave of items take the
-    grouped form; a rank's share with fewer, or whose items are mostly of other classes, does not."""
+    grouped form; a rank's share with fewer, or whose items are mostly of other classes, does not.  A search
+    asks for half of them, a pass for a quarter."""
     exe = str(tmp_path / "tree_groups")
     subprocess.run([os.environ.get("NVCC", "nvcc"), "-gencode", "arch=compute_100a,code=sm_100a", "-std=c++17", "-O1", "-o", exe,
                     os.path.join(ROOT, "tests", "tree_groups.cu")], check=True)
     conf = (1024, 900, 676, 400, 144, 36)
-    ranges = {(0, 3180): 1, (0, 300): 1, (0, 100): 0, (1024, 400): 1, (1924, 676): 0, (2600, 400): 0, (3144, 36): 0, (17, 0): 0}
+    ranges = {(0, 3180): (1, 1), (0, 300): (1, 1), (0, 100): (0, 0), (1024, 400): (1, 1), (2600, 580): (1, 0), (0, 1924): (1, 1), (1924, 676): (0, 0), (2600, 400): (0, 0),
+              (3144, 36): (0, 0), (17, 0): (0, 0)}
     out = subprocess.run([exe, "32", "205", "4,4", "8", "3", ",".join(map(str, conf)), *(str(x) for r in ranges for x in r)],
                          check=True, capture_output=True, text=True).stdout.split()
     parts, group = out[0:12:2], out[1:12:2]
     assert all((int(g) > 1) == (int(n) <= 2) for n, g in zip(parts, group)) and "4" in group
-    assert [int(v) for v in out[12:]] == list(ranges.values())
+    assert [int(v) for v in out[12:]] == [v for r in ranges.values() for v in r]

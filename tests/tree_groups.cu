@@ -1,6 +1,6 @@
 // Which calls take the grouped form of the tree kernel (test_tree_tasks.py; no GPU is needed).  Arguments: layers, window delta, nodes per
 // type, node size, policies, configurations of the classes (1, 2, 4, ... stages), then pairs: first configuration, how many.
-// Prints parts and group of every class, then 0 or 1 per pair.
+// Prints parts and group of every class, then per pair 0 or 1 for a pass and for a search.
 #include "../paper_2609_39350_b200/csrc/hap_tree_host.h"
 
 #include <cstdio>
@@ -46,6 +46,8 @@ int main(int argc, char **argv)
     }
     tree_policy_items(cls, trees, 148, atoi(argv[5]));
     for (const TreeClass &c : cls) printf("%d %d\n", c.n_parts, c.group);
-    for (int a = 7; a + 1 < argc; a += 2) printf("%d\n", (int)tree_grouped(cls, (unsigned)atoi(argv[a]), (unsigned)(atoi(argv[a]) + atoi(argv[a + 1])), 148));
+    for (int a = 7; a + 1 < argc; a += 2)
+        for (bool search : {false, true})
+            printf("%d\n", (int)tree_grouped(cls, (unsigned)atoi(argv[a]), (unsigned)(atoi(argv[a]) + atoi(argv[a + 1])), 148, search));
     return 0;
 }
