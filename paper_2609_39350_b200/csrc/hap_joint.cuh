@@ -150,7 +150,7 @@ __host__ __device__ inline ReachSmem reach_smem(int N, int T, int R, int RW, int
 }
 
 template <bool LINEAR, int W>
-__global__ void __launch_bounds__(kReachThreads, W > 2 ? 2 : 4)      // (three words: 85 KB and more of shared memory a block)
+__global__ void __launch_bounds__(kReachThreads, W > 2 ? 2 : 4)      // (three words: 85 KB and more of shared memory a block; 1,966 us against 2,368 with four and spilled registers)
 joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, const unsigned *ids, const i64 *c2, const i64 *coef, i64 *out)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -493,7 +493,7 @@ joint_reach_kernel(const DevConst dc, const JointReach *classes, int n_classes, 
                 // The sums grow with B in steps at those costs; a warp per trial, eight a round.  Where the largest B leaves less than a tenth of
                 // the layers to spare, whether anything is feasible is in doubt: of the configurations of 32, 256 and 1,024 devices that pass the bound,
                 // 95 % of the infeasible ones lie there and 3 % of the others.  Asked first there instead of after three tests: 256 devices, 220
-                // layers, nothing feasible 527 -> 283 us, 1,024 devices 2,201 -> 2,158; 1,024 devices, 255 layers 2,174 -> 2,368.
+                // layers, nothing feasible 527 -> 283 us, 1,024 devices 2,201 -> 2,158; 1,024 devices, 255 layers (ten of 6,228 feasible) 2,174 -> 2,368.
                 auto capacity = [&](const i64 *costs) -> i64 {
                     i64 a, b;                                         // a smallest and largest cost that may be the one
                     auto around = [&](i64 B, i64 &below, i64 &above) {       // the largest cost at most B, the smallest above
